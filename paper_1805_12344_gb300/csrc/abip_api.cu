@@ -483,9 +483,7 @@ size_t dense_solve_smem(int m, int n, bool mixed = false) {
   }
   return (size_t)(5 * m + 3 * n) * sizeof(double);
 }
-size_t dense_setup_smem(int m, int n) {
-  return std::max((size_t)(2 * 32 * 33), (size_t)(2 * m + n)) * sizeof(double);
-}
+size_t dense_setup_smem(int m, int n) { return (size_t)(2 * m + n) * sizeof(double); }
 
 // Allocate and fill the device descriptors of a set of dense instances.
 int dense_alloc(abip_handle* h, const std::vector<DenseHostInst>& hi, void** arena_out, DenseInst** dinst,
@@ -556,9 +554,10 @@ int dense_alloc(abip_handle* h, const std::vector<DenseHostInst>& hi, void** are
   return ABIP_OK;
 }
 
-int dense_run_setup(abip_handle* h, DenseInst* dinst, int* queue, int count, int grid, size_t smem, cudaStream_t st) {
+int dense_run_setup(abip_handle* h, DenseInst* dinst, int* queue, int count, int grid, size_t smem, int mmax, bool mixed,
+                    cudaStream_t st) {
   cudaMemsetAsync(queue, 0, 8, st);
-  cudaError_t e = abip::launch_dense_setup(dinst, count, queue, grid, smem, st);
+  cudaError_t e = abip::launch_dense_setup(dinst, count, queue, grid, smem, mmax, mixed, st);
   if (e != cudaSuccess) return fail(h, ABIP_E_CUDA, std::string("dense setup launch: ") + cudaGetErrorString(e));
   e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return fail(h, ABIP_E_CUDA, std::string("dense setup: ") + cudaGetErrorString(e));
@@ -955,7 +954,7 @@ int abip_setup(const abip_matrix* A, const double* b, const double* c, const abi
       if (rc == ABIP_OK) rc = dense_alloc(h, hi, &h->arena, &h->dinst, &h->queue, hd, h->mixed != 0, prm.bb_beta != 0);
       if (rc == ABIP_OK) {
         h->hinst = hd[0];
-        rc = dense_run_setup(h, h->dinst, h->queue, 1, 1, dense_setup_smem(m, n), 0);
+        rc = dense_run_setup(h, h->dinst, h->queue, 1, 1, dense_setup_smem(m, n), m, h->mixed != 0, 0);
       }
       if (rc == ABIP_OK) {
         cudaMemcpy(&h->hinst, h->dinst, sizeof(DenseInst), cudaMemcpyDeviceToHost);
@@ -1072,6 +1071,7 @@ int abip_solve_batch(int32_t count, const abip_matrix* A, const double* const* b
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   std::vector<DenseHostInst> hi(count);
   size_t smem_solve = 0, smem_setup = 0;
+  int mmax = 0;
   for (int k = 0; k < count; ++k) {
     int rc = validate_matrix(&tmp, &A[k]);
     if (rc) return fail(nullptr, rc, "instance " + std::to_string(k) + ": " + tmp.err);
@@ -1090,6 +1090,7 @@ int abip_solve_batch(int32_t count, const abip_matrix* A, const double* const* b
       return fail(nullptr, ABIP_E_INVALID_ARG, "instance " + std::to_string(k) + ": non-finite b or c");
     smem_solve = std::max(smem_solve, dense_solve_smem(m, n, mixed));
     smem_setup = std::max(smem_setup, dense_setup_smem(m, n));
+    mmax = std::max(mmax, m);
   }
   void* arena = nullptr;
   DenseInst* dinst = nullptr;
@@ -1116,7 +1117,7 @@ int abip_solve_batch(int32_t count, const abip_matrix* A, const double* const* b
   }
   const int sms = abip::dense_max_ctas(tmp.device);
   const DenseParams dp = dense_params(prm);
-  rc = dense_run_setup(&tmp, dinst, queue, count, std::min(count, sms * 4), smem_setup, st);
+  rc = dense_run_setup(&tmp, dinst, queue, count, std::min(count, sms * 4), smem_setup, mmax, mixed, st);
   // occupancy variant: 0, or the autotuner's (cached, or timed on this batch)
   int variant = 0, tuned = 0;
   if (!rc && prm.autotune) {

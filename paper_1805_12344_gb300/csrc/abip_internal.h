@@ -251,7 +251,13 @@ struct DenseParams {
 // global scratch of the Barzilai-Borwein selection per instance (DenseInst::work)
 inline size_t bb_work_doubles(int m, int n) { return 4 * (size_t)m + 6 * (size_t)n; }
 
-cudaError_t launch_dense_setup(DenseInst* inst, int count, int* queue, int grid, size_t smem, cudaStream_t st);
+// Gram and Cholesky factor of every instance (L), over the SMs; mmax: the largest m
+cudaError_t launch_dense_factor(DenseInst* inst, int count, int mmax, int sms, cudaStream_t st);
+// the FP32 explicit inverse of G (Ginvf) of every instance, from L
+cudaError_t launch_dense_inverse(DenseInst* inst, int count, int mmax, int sms, cudaStream_t st);
+// the whole setup: factor, embedding constants and M^{-1} H and, when `inverse`, Ginvf
+cudaError_t launch_dense_setup(DenseInst* inst, int count, int* queue, int grid, size_t smem, int mmax, bool inverse,
+                               cudaStream_t st);
 // Occupancy variants of the dense solve kernel (the batch autotuner's choice)
 constexpr int kDenseVariants = 3;
 cudaError_t launch_dense_solve(DenseInst* inst, int count, DenseParams prm, int* queue, const int* order,

@@ -213,6 +213,9 @@ __device__ void solve_M(const DenseInst& I, const double* a, const double* d, do
   __syncthreads();
 }
 
+// FACTOR: form and factor G here, in the one CTA (the allocation-free entry point); otherwise
+// launch_dense_factor has left L, and this kernel does the embedding constants and M^{-1} H.
+template <bool FACTOR>
 __global__ void __launch_bounds__(kThreads) dense_setup_kernel(DenseInst* insts, int count, int* queue) {
   extern __shared__ double sm[];
   __shared__ double red[32 * 8];
@@ -220,6 +223,7 @@ __global__ void __launch_bounds__(kThreads) dense_setup_kernel(DenseInst* insts,
     const int id = next_instance(queue, count);
     if (id < 0) return;
     DenseInst& I = insts[id];
+    if (!FACTOR && I.err != 0) continue;
     const int m = I.m, n = I.n;
     // embedding constants
     double acc[3] = {0.0, 0.0, 0.0};
@@ -236,10 +240,12 @@ __global__ void __launch_bounds__(kThreads) dense_setup_kernel(DenseInst* insts,
     }
     block_allsum<3>(acc, red);
     const double zbar = acc[0] + 1.0;
-    gram(I.A, I.ld, m, n, I.L, sm);
-    if (!cholesky(I.L, m)) {
-      if (threadIdx.x == 0) { I.err = DEV_ERR_CHOLESKY; I.status = 0; }
-      continue;
+    if (FACTOR) {
+      gram(I.A, I.ld, m, n, I.L, sm);
+      if (!cholesky(I.L, m)) {
+        if (threadIdx.x == 0) { I.err = DEV_ERR_CHOLESKY; I.status = 0; }
+        continue;
+      }
     }
     // M^{-1} h1, M^{-1} h2 with h1 = [-b; c], h2 = [bbar; -cbar]
     double* a = sm;            // m
@@ -273,17 +279,6 @@ __global__ void __launch_bounds__(kThreads) dense_setup_kernel(DenseInst* insts,
       I.err = isfinite(det) && det != 0.0 ? 0 : DEV_ERR_NONFINITE;
     }
     __syncthreads();
-    if (I.Ginvf) {   // mixed precision: the FP32 explicit inverse of G, column by column
-      double* w = sm;   // m
-      for (int col = 0; col < m; ++col) {
-        for (int i = threadIdx.x; i < m; i += kThreads) w[i] = i == col ? 1.0 : 0.0;
-        __syncthreads();
-        trsv_lower<double>(I.L, m, w);
-        trsv_lower_t<double>(I.L, m, w);
-        for (int i = threadIdx.x; i < m; i += kThreads) I.Ginvf[(size_t)col * I.ldtf + i] = (float)w[i];
-        __syncthreads();
-      }
-    }
   }
 }
 
@@ -1465,12 +1460,20 @@ __global__ void __launch_bounds__(kThreads) dense_backward_kernel(BackwardInst* 
 // dynamic shared memory of the solve kernel: 5m + 3n doubles, at most this many bytes
 constexpr size_t kDenseSmemMax = 200 * 1024;
 
-cudaError_t launch_dense_setup(DenseInst* inst, int count, int* queue, int grid, size_t smem, cudaStream_t st) {
-  // the caller sizes smem for the largest instance: max(2m + n, 2 * 32 * 33) doubles
-  cudaError_t e = cudaFuncSetAttribute(dense_setup_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDenseSmemMax);
+cudaError_t launch_dense_setup(DenseInst* inst, int count, int* queue, int grid, size_t smem, int mmax, bool inverse,
+                               cudaStream_t st) {
+  // the caller sizes smem for the largest instance: 2m + n doubles
+  cudaError_t e = cudaFuncSetAttribute(dense_setup_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDenseSmemMax);
   if (e != cudaSuccess) return e;
-  dense_setup_kernel<<<grid, kThreads, smem, st>>>(inst, count, queue);
-  return cudaGetLastError();
+  int dev = 0;
+  cudaGetDevice(&dev);
+  const int sms = dense_max_ctas(dev);
+  e = launch_dense_factor(inst, count, mmax, sms, st);
+  if (e != cudaSuccess) return e;
+  dense_setup_kernel<false><<<grid, kThreads, smem, st>>>(inst, count, queue);
+  e = cudaGetLastError();
+  if (e != cudaSuccess || !inverse) return e;
+  return launch_dense_inverse(inst, count, mmax, sms, st);
 }
 
 // the solve kernel of a precision and an occupancy variant (0, 1, 2: MINB 1, 2, 3 for FP64
@@ -1607,7 +1610,7 @@ extern "C" ABIP_API int abip_solve_dense_noalloc(int32_t m, int32_t n, const dou
   cudaMemcpyAsync(dinst, &I, sizeof(I), cudaMemcpyHostToDevice, st);
   cudaMemsetAsync(queue, 0, 2 * sizeof(int), st);
   const size_t smem_setup = std::max((size_t)(2 * 32 * 33), (size_t)(2 * m + n)) * sizeof(double);
-  abip::dense_setup_kernel<<<1, abip::kThreads, smem_setup, st>>>(dinst, 1, queue);
+  abip::dense_setup_kernel<true><<<1, abip::kThreads, smem_setup, st>>>(dinst, 1, queue);
   cudaMemsetAsync(queue, 0, 2 * sizeof(int), st);
   abip::DenseParams dp{prm.beta, prm.gamma, prm.alpha, prm.eps, prm.max_admm_iters, prm.warmstart,
                        prm.stop_rule, 0, 1, 0, 0, 0.0, 0.0, prm.gamma_max};

@@ -1,0 +1,56 @@
+"""The dense setup split over the SMs (Gram tiles, cluster Cholesky, column-tiled inverse) at the
+edges of its 32-wide blocks and of its dispatch: one instance (8-CTA clusters, 4-column inverse
+tiles), a few (8-column tiles) and more than twice the SMs (32-column tiles).
+
+FP64 iterates agree with the oracle to the 1e-10 of the parity tests.  A mixed update is formed
+from FP32 products of changes of order 1, each off by at most n 2^-24 relative: 4 updates at
+n <= 200 stay within 1e-4 of the FP64 iterate."""
+import numpy as np
+import pytest
+
+from oracle import abip_oracle as O
+from paper_1805_12344_gb300 import workloads as W
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+UPDATES = 4
+
+
+@pytest.fixture(scope="module")
+def abip():
+    if not torch.cuda.is_available():
+        pytest.skip("needs a GPU")
+    from paper_1805_12344_gb300 import build, abip as _abip
+    build.build()
+    _abip.lib()
+    return _abip
+
+
+def _rel(a, b):
+    return np.linalg.norm(a - b) / np.linalg.norm(b)
+
+
+@pytest.mark.parametrize("m", [1, 31, 32, 33, 64, 65, 97])
+def test_single_instance_first_iterates(abip, m):
+    lp = W.planted_dense(m, 2 * m + 3, seed=W.seed_for(W.DENSE_PLANTED, 700 + m))
+    ref = O.run_iterations(lp.A, lp.b, lp.c, UPDATES, O.Params(linsys=0))
+    for precision, tol in ((abip.ABIP_PREC_F64, 1e-10), (abip.ABIP_PREC_MIXED, 1e-4)):
+        s = abip.Solver(lp.A, lp.b, lp.c, precision=precision, max_admm_iters=UPDATES)
+        s.solve()
+        assert _rel(s.stacked_state(), ref) <= tol, (m, precision)
+        s.close()
+
+
+@pytest.mark.parametrize("count", [90, 320])
+def test_batch_first_iterates(abip, count):
+    sizes = [(1 + (7 * k) % 67, k) for k in range(count)]
+    lps = [W.planted_dense(m, 2 * m + k % 5, seed=W.seed_for(W.DENSE_PLANTED, 800 + k)) for m, k in sizes]
+    args = ([l.A for l in lps], [l.b for l in lps], [l.c for l in lps])
+    for precision, tol in ((abip.ABIP_PREC_F64, 1e-10), (abip.ABIP_PREC_MIXED, 1e-4)):
+        infos, xs, ys, ss = abip.abip_solve_batch(*args, abip.default_params(precision=precision, max_admm_iters=UPDATES))
+        for k in range(0, count, 13):
+            ref = O.run_iterations(lps[k].A, lps[k].b, lps[k].c, UPDATES, O.Params(linsys=0))
+            m, n = lps[k].A.shape
+            got = np.concatenate([ys[k], xs[k]]) * infos[k]["tau"]
+            assert _rel(got, ref[:m + n]) <= tol, (k, precision)
