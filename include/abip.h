@@ -119,7 +119,8 @@ typedef struct {
                                confirmations of the Sec. 4.1 tests (each screen pass that comes
                                sooner waits); 1 = confirm whenever the screen passes */
     int32_t grid_ctas;      /* 0: automatic; else the persistent grid size (tests) */
-    int64_t barrier_limit_ns; /* sparse paths: wall-clock limit of one grid-barrier wait in the
+    int64_t barrier_limit_ns; /* sparse paths, and one large dense LP in FP64 (solved by the whole
+                                 grid): wall-clock limit of one grid-barrier wait in the
                                  persistent kernel, and of one wait of the direct projection's
                                  factorisation and sweeps on an entry another warp computes; a
                                  wait past it ends the call with ABIP_E_TIMEOUT (the kernel

@@ -486,8 +486,9 @@ size_t dense_solve_smem(int m, int n, bool mixed = false) {
 size_t dense_setup_smem(int m, int n) { return (size_t)(2 * m + n) * sizeof(double); }
 
 // Allocate and fill the device descriptors of a set of dense instances.
+// group: with the arrays of the FP64 solve by a group of CTAs; h->gscratch for one instance.
 int dense_alloc(abip_handle* h, const std::vector<DenseHostInst>& hi, void** arena_out, DenseInst** dinst,
-                int** queue, std::vector<DenseInst>& hdesc, bool mixed = false, bool bb = false) {
+                int** queue, std::vector<DenseInst>& hdesc, bool mixed = false, bool bb = false, bool group = false) {
   const int count = (int)hi.size();
   auto layout = [&](Arena& ar, std::vector<DenseInst>& d) {
     DenseInst* di = ar.take<DenseInst>(count);
@@ -497,8 +498,11 @@ int dense_alloc(abip_handle* h, const std::vector<DenseHostInst>& hi, void** are
     for (int k = 0; k < count; ++k) {
       const int m = hi[k].m, n = hi[k].n;
       DenseInst& I = d[k];
-      I.m = m; I.n = n; I.ld = n;
-      I.A = ar.take<double>((size_t)m * n);
+      I.m = m; I.n = n;
+      I.ld = group ? n + (n & 1) : n;
+      I.A = ar.take<double>((size_t)m * I.ld);
+      I.AT = group ? ar.take<double>((size_t)n * (m + (m & 1))) : nullptr;
+      I.Ginv = group ? ar.take<double>((size_t)m * (m + (m & 1))) : nullptr;
       I.b = ar.take<double>(m); I.c = ar.take<double>(n);
       I.L = ar.take<double>((size_t)m * m);
       I.bbar = ar.take<double>(m); I.cbar = ar.take<double>(n);
@@ -516,6 +520,10 @@ int dense_alloc(abip_handle* h, const std::vector<DenseHostInst>& hi, void** are
         I.Af = nullptr; I.ATf = nullptr; I.Ginvf = nullptr;
       }
     }
+    if (group && count == 1) {
+      h->gscratch_len = abip::dense_group_scratch(hi[0].m, hi[0].n, abip::dense_max_ctas(h->device));
+      h->gscratch = ar.take<double>(h->gscratch_len);
+    }
   };
   Arena probe;
   std::vector<DenseInst> tmp;
@@ -531,7 +539,10 @@ int dense_alloc(abip_handle* h, const std::vector<DenseHostInst>& hi, void** are
   cudaMemset(mem, 0, probe.off);
   for (int k = 0; k < count; ++k) {
     const DenseInst& I = hdesc[k];
-    cudaMemcpy((void*)I.A, hi[k].A.data(), hi[k].A.size() * 8, cudaMemcpyHostToDevice);
+    if (I.ld == I.n)
+      cudaMemcpy((void*)I.A, hi[k].A.data(), hi[k].A.size() * 8, cudaMemcpyHostToDevice);
+    else
+      cudaMemcpy2D((void*)I.A, I.ld * 8, hi[k].A.data(), (size_t)I.n * 8, (size_t)I.n * 8, I.m, cudaMemcpyHostToDevice);
     cudaMemcpy((void*)I.b, hi[k].b.data(), hi[k].m * 8, cudaMemcpyHostToDevice);
     cudaMemcpy((void*)I.c, hi[k].c.data(), hi[k].n * 8, cudaMemcpyHostToDevice);
     if (mixed) {   // padded FP32 copies of A and A^T (padding stays 0 from the memset)
@@ -554,10 +565,10 @@ int dense_alloc(abip_handle* h, const std::vector<DenseHostInst>& hi, void** are
   return ABIP_OK;
 }
 
-int dense_run_setup(abip_handle* h, DenseInst* dinst, int* queue, int count, int grid, size_t smem, int mmax, bool mixed,
-                    cudaStream_t st) {
+int dense_run_setup(abip_handle* h, DenseInst* dinst, int* queue, int count, int grid, size_t smem, int mmax, int nmax,
+                    bool inverse, cudaStream_t st) {
   cudaMemsetAsync(queue, 0, 8, st);
-  cudaError_t e = abip::launch_dense_setup(dinst, count, queue, grid, smem, mmax, mixed, st);
+  cudaError_t e = abip::launch_dense_setup(dinst, count, queue, grid, smem, mmax, nmax, inverse, st);
   if (e != cudaSuccess) return fail(h, ABIP_E_CUDA, std::string("dense setup launch: ") + cudaGetErrorString(e));
   e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return fail(h, ABIP_E_CUDA, std::string("dense setup: ") + cudaGetErrorString(e));
@@ -570,21 +581,30 @@ DenseParams dense_params(const abip_params& p) {
                      p.bb_max_redo, p.eps_cor, p.eps_penalty, p.gamma_max};
 }
 
+// The solve launch: by groups of CTAs with h->gplan when h->group, else one CTA per instance.
 int dense_run_solve(abip_handle* h, DenseInst* dinst, int* queue, int count, int grid, size_t smem,
                     const DenseParams& dp, cudaStream_t st, const int* order = nullptr, int variant = 0) {
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
   cudaMemsetAsync(queue, 0, 8, st);
+  const bool grid_mode = h->group && h->gplan.grid_mode;
+  double* words = grid_mode ? h->gscratch + h->gscratch_len - 2 : nullptr;   // barrier counter, error word
+  if (words) cudaMemsetAsync(words, 0, 16, st);
   cudaEventRecord(e0, st);
-  cudaError_t e = abip::launch_dense_solve(dinst, count, dp, queue, order, grid, smem, variant, st);
+  cudaError_t e = h->group ? abip::launch_dense_group(dinst, count, dp, queue, order, h->gplan, variant, h->gscratch,
+                                                      h->gscratch_len, (unsigned long long)h->prm.barrier_limit_ns, st)
+                           : abip::launch_dense_solve(dinst, count, dp, queue, order, grid, smem, variant, st);
   cudaEventRecord(e1, st);
+  int derr = 0;
+  if (e == cudaSuccess && words) e = cudaMemcpyAsync(&derr, words + 1, sizeof(int), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   float ms = 0.f;
   if (e == cudaSuccess) cudaEventElapsedTime(&ms, e0, e1);
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   if (e != cudaSuccess) return fail(h, ABIP_E_CUDA, std::string("dense solve: ") + cudaGetErrorString(e));
+  if (derr != 0) return fail(h, device_error_code(derr), std::string("solve: ") + device_error_str(derr));
   h->kernel_s = ms * 1e-3;
   h->launches = 1;
   return ABIP_OK;
@@ -612,7 +632,7 @@ std::string tune_key(int device, bool mixed, const std::vector<DenseHostInst>& h
     std::strcpy(prop.name, "unknown");
   }
   double mn = 0.0;
-  int mmax = 0;
+  int mmax = 0, nmax = 0;
   for (const DenseHostInst& x : hi) {
     mn += (double)x.m * x.n;
     mmax = std::max(mmax, x.m);
@@ -951,10 +971,19 @@ int abip_setup(const abip_matrix* A, const double* b, const double* c, const abi
       hi[0].m = m; hi[0].n = n; hi[0].b = hb; hi[0].c = hc;
       rc = read_matrix_dense(h, A, hi[0].A);
       std::vector<DenseInst> hd;
-      if (rc == ABIP_OK) rc = dense_alloc(h, hi, &h->arena, &h->dinst, &h->queue, hd, h->mixed != 0, prm.bb_beta != 0);
+      h->group = !h->mixed && !prm.bb_beta &&
+                 abip::plan_dense_group(&m, &n, 1, abip::dense_max_ctas(h->device), h->gplan) != 0;
+      if (rc == ABIP_OK) {
+        rc = dense_alloc(h, hi, &h->arena, &h->dinst, &h->queue, hd, h->mixed != 0, prm.bb_beta != 0, h->group);
+        if (rc == ABIP_E_OOM && h->group) {   // without the group's copies of A^T and G^{-1}
+          h->group = false;
+          rc = dense_alloc(h, hi, &h->arena, &h->dinst, &h->queue, hd, false, false, false);
+        }
+      }
       if (rc == ABIP_OK) {
         h->hinst = hd[0];
-        rc = dense_run_setup(h, h->dinst, h->queue, 1, 1, dense_setup_smem(m, n), m, h->mixed != 0, 0);
+        rc = dense_run_setup(h, h->dinst, h->queue, 1, 1, dense_setup_smem(m, n), m, h->group ? n : 0,
+                             h->mixed || h->group, 0);
       }
       if (rc == ABIP_OK) {
         cudaMemcpy(&h->hinst, h->dinst, sizeof(DenseInst), cudaMemcpyDeviceToHost);
@@ -1071,7 +1100,7 @@ int abip_solve_batch(int32_t count, const abip_matrix* A, const double* const* b
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   std::vector<DenseHostInst> hi(count);
   size_t smem_solve = 0, smem_setup = 0;
-  int mmax = 0;
+  int mmax = 0, nmax = 0;
   for (int k = 0; k < count; ++k) {
     int rc = validate_matrix(&tmp, &A[k]);
     if (rc) return fail(nullptr, rc, "instance " + std::to_string(k) + ": " + tmp.err);
@@ -1091,12 +1120,24 @@ int abip_solve_batch(int32_t count, const abip_matrix* A, const double* const* b
     smem_solve = std::max(smem_solve, dense_solve_smem(m, n, mixed));
     smem_setup = std::max(smem_setup, dense_setup_smem(m, n));
     mmax = std::max(mmax, m);
+    nmax = std::max(nmax, n);
   }
   void* arena = nullptr;
   DenseInst* dinst = nullptr;
   int* queue = nullptr;
   std::vector<DenseInst> hd;
-  int rc = dense_alloc(&tmp, hi, &arena, &dinst, &queue, hd, mixed, prm.bb_beta != 0);
+  const int sms = abip::dense_max_ctas(tmp.device);
+  {
+    std::vector<int> ms(count), ns(count);
+    for (int k = 0; k < count; ++k) { ms[k] = hi[k].m; ns[k] = hi[k].n; }
+    tmp.group = !mixed && !prm.bb_beta && abip::plan_dense_group(ms.data(), ns.data(), count, sms, tmp.gplan) != 0;
+  }
+  tmp.prm = prm;
+  int rc = dense_alloc(&tmp, hi, &arena, &dinst, &queue, hd, mixed, prm.bb_beta != 0, tmp.group);
+  if (rc == ABIP_E_OOM && tmp.group) {   // without the group's copies of A^T and G^{-1}
+    tmp.group = false;
+    rc = dense_alloc(&tmp, hi, &arena, &dinst, &queue, hd, mixed, false, false);
+  }
   if (rc) return fail(nullptr, rc, tmp.err);
   // hand-out order: largest first (the batch's wall time is its slowest instance)
   int* order = nullptr;
@@ -1115,9 +1156,9 @@ int abip_solve_batch(int32_t count, const abip_matrix* A, const double* const* b
     }
     cudaMemcpy(order, ord.data(), count * sizeof(int), cudaMemcpyHostToDevice);
   }
-  const int sms = abip::dense_max_ctas(tmp.device);
   const DenseParams dp = dense_params(prm);
-  rc = dense_run_setup(&tmp, dinst, queue, count, std::min(count, sms * 4), smem_setup, mmax, mixed, st);
+  rc = dense_run_setup(&tmp, dinst, queue, count, std::min(count, sms * 4), smem_setup, mmax, tmp.group ? nmax : 0,
+                       mixed || tmp.group, st);
   // occupancy variant: 0, or the autotuner's (cached, or timed on this batch)
   int variant = 0, tuned = 0;
   if (!rc && prm.autotune) {
@@ -1136,7 +1177,8 @@ int abip_solve_batch(int32_t count, const abip_matrix* A, const double* const* b
       probe.bb = 0;
       double best_s = 1e300;
       for (int v = 0; v < abip::kDenseVariants && !rc; ++v) {
-        const int per_v = abip::dense_solve_ctas_per_sm(mixed, smem_solve, v);
+        const int per_v = tmp.group ? abip::dense_group_ctas_per_sm(tmp.gplan, v)
+                                    : abip::dense_solve_ctas_per_sm(mixed, smem_solve, v);
         if (per_v < 1) continue;
         rc = dense_run_solve(&tmp, dinst, queue, count, std::min(count, sms * per_v), smem_solve, probe, st, order, v);
         if (!rc && tmp.kernel_s < best_s) { best_s = tmp.kernel_s; variant = v; }
@@ -1147,7 +1189,8 @@ int abip_solve_batch(int32_t count, const abip_matrix* A, const double* const* b
       tune_store(tc);
     }
   }
-  const int per = std::max(1, abip::dense_solve_ctas_per_sm(mixed, smem_solve, variant));
+  const int per = std::max(1, tmp.group ? abip::dense_group_ctas_per_sm(tmp.gplan, variant)
+                                        : abip::dense_solve_ctas_per_sm(mixed, smem_solve, variant));
   const int grid = std::min(count, sms * per);
   if (!rc) rc = dense_run_solve(&tmp, dinst, queue, count, grid, smem_solve, dp, st, order, variant);
   if (!rc) {

@@ -198,6 +198,9 @@ struct DenseInst {
   // mixed precision (null on the FP64 path): FP32 A (rows padded to ldf), FP32 A^T
   // (rows padded to ldtf) and the FP32 explicit inverse of G = I + A A^T (m x ldtf)
   const float* Af; const float* ATf; float* Ginvf;
+  // FP64 path by a group of CTAs (null elsewhere): A^T (n rows) and the explicit inverse of G
+  // (m rows), rows padded with zeros to an even length; A's ld is even then
+  double* AT; double* Ginv;
   double zbar, nb, nc;
   double Kinv[4];
   // results
@@ -253,11 +256,31 @@ inline size_t bb_work_doubles(int m, int n) { return 4 * (size_t)m + 6 * (size_t
 
 // Gram and Cholesky factor of every instance (L), over the SMs; mmax: the largest m
 cudaError_t launch_dense_factor(DenseInst* inst, int count, int mmax, int sms, cudaStream_t st);
-// the FP32 explicit inverse of G (Ginvf) of every instance, from L
+// the explicit inverse of G (FP32 Ginvf or FP64 Ginv, where not null) of every instance, from L
 cudaError_t launch_dense_inverse(DenseInst* inst, int count, int mmax, int sms, cudaStream_t st);
-// the whole setup: factor, embedding constants and M^{-1} H and, when `inverse`, Ginvf
-cudaError_t launch_dense_setup(DenseInst* inst, int count, int* queue, int grid, size_t smem, int mmax, bool inverse,
-                               cudaStream_t st);
+// A^T of every instance (AT)
+cudaError_t launch_dense_transpose(DenseInst* inst, int count, int mmax, int nmax, int sms, cudaStream_t st);
+// the whole setup: factor, embedding constants and M^{-1} H and, when `inverse`, G's inverse;
+// nmax > 0: also AT
+cudaError_t launch_dense_setup(DenseInst* inst, int count, int* queue, int grid, size_t smem, int mmax, int nmax,
+                               bool inverse, cudaStream_t st);
+
+// FP64 solve by a group of CTAs per instance (dense_group.cu)
+struct DenseGroupPlan {
+  int ctas;                  // CTAs per instance: the cluster size, or the grid's CTAs
+  int grid_mode;             // 1: one instance over a cooperative grid
+  int cache_vec, cache_mat;  // shared-memory copies of the vectors and matrix rows a CTA reads
+  size_t smem;
+};
+// the plan for a batch (sizes m[k], n[k]); 0 if no group holds its vectors in shared memory
+int plan_dense_group(const int* m, const int* n, int count, int sms, DenseGroupPlan& plan);
+// doubles of scratch of the grid mode; its last two are the barrier counter and the error
+// word, zeroed by the caller before each launch
+size_t dense_group_scratch(int m, int n, int sms);
+cudaError_t launch_dense_group(DenseInst* inst, int count, const DenseParams& prm, int* queue, const int* order,
+                               const DenseGroupPlan& plan, int variant, double* scratch, size_t scratch_len,
+                               unsigned long long limit_ns, cudaStream_t st);
+int dense_group_ctas_per_sm(const DenseGroupPlan& plan, int variant);
 // Occupancy variants of the dense solve kernel (the batch autotuner's choice)
 constexpr int kDenseVariants = 3;
 cudaError_t launch_dense_solve(DenseInst* inst, int count, DenseParams prm, int* queue, const int* order,
@@ -353,6 +376,10 @@ struct abip_handle {
   int grid = 0;
   // dense path
   abip::DenseInst* dinst = nullptr;   // device, one entry
+  bool group = false;                 // FP64 solve by a group of CTAs (gplan)
+  abip::DenseGroupPlan gplan{};
+  double* gscratch = nullptr;         // its grid mode's scratch, gscratch_len doubles
+  size_t gscratch_len = 0;
   int* queue = nullptr;
   abip::DenseInst hinst{};            // host mirror of the descriptor
   double nb = 0, nc = 0;

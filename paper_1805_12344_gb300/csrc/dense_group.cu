@@ -1,0 +1,697 @@
+// Dense ABIP in FP64 with a group of CTAs per LP: a thread-block cluster (2 .. 16 CTAs) per
+// instance of a batch, or the whole cooperative grid for one large LP.
+//
+// What bounds it: the FP64 pipe, 2 FMA per clock and SM on this part, so an LP on one SM pays
+// its 3 m n + m^2 multiply-adds per update at 1/152 of the chip; and, for a small LP, the chain
+// of dependent phases.  Hence
+//  * the rows of A and G^{-1} and the columns of A (rows of the stored A^T) are dealt out to the
+//    CTAs of the group; every CTA keeps the vectors q, z_y, x and s whole in shared memory and
+//    publishes its part of each (distributed shared memory in a cluster, L2 in a grid);
+//  * z_y = G^{-1} q is one product with the explicit inverse instead of two triangular sweeps of
+//    m / 32 serial blocks (lambda_min(G) >= 1, so its error bound is that of the sweeps);
+//  * A^T y follows from the update's linearity, y <- alpha u_y + (1 - alpha) y, whose error does
+//    not grow (|1 - alpha| < 1) and which only the tests of Sec. 4.1 read: three products with
+//    the entries of A per update instead of four;
+//  * eight rows (or four with two vectors) per warp, their sums reduced together: 9 additions
+//    for 8 sums where butterflies take 40 -- a warp-wide FP64 addition costs 16 clocks here;
+//  * what a CTA reads every update (its rows of the matrices and of the vectors) is copied to
+//    shared memory when it fits.
+// One update has four barriers of the group: z_y | H^T z | x, s | products and test sums.
+// Measured, us per update, one CTA with triangular sweeps -> this kernel: 50 x 120 76.9 -> 11.1
+// (the chain of phases: 16 x 48 takes 10.0), 512 x 1154 1564 -> 26.4, the slowest of 64 LPs of
+// m 16 .. 256 621 -> 65.
+#include <algorithm>
+
+#include <cooperative_groups.h>
+
+#include "abip_device.cuh"
+#include "abip_internal.h"
+
+namespace cg = cooperative_groups;
+
+namespace abip {
+namespace {
+
+constexpr int kThr = 256;
+constexpr int kWarps = kThr / 32;
+constexpr int kSums = 9;
+
+enum Act : int { ACT_STEP = 0, ACT_WARM = 1, ACT_STOP = 2 };
+
+// Sums of P per-lane values over the warp, P a power of two <= 32: halving exchanges, then a
+// butterfly over the rest.  Lane l receives the sum of value l >> (5 - log2 P).
+template <int P>
+__device__ __forceinline__ double sum_together(double (&a)[P], int lane) {
+  int o = 16;
+#pragma unroll
+  for (int h = P / 2; h > 0; h >>= 1, o >>= 1) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int k = 0; k < h; ++k) {
+      const double send = up ? a[k] : a[k + h];
+      const double keep = up ? a[k + h] : a[k];
+      a[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+  double v = a[0];
+#pragma unroll
+  for (; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// out(which, i, sum_j M[row0 + i][j] v_which[j]) for i < rows: R rows per warp at a time, NV
+// vectors; rows of M are ld (even) doubles, 16-byte aligned and zero-padded like v0, v1.
+template <int R, int NV, typename F>
+__device__ __forceinline__ void dots(const double* M, int64_t ld, int rows, const double* v0, const double* v1, F out) {
+  constexpr int P = R * NV;
+  constexpr int kShift = P == 16 ? 1 : P == 8 ? 2 : P == 4 ? 3 : P == 2 ? 4 : 5;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int nq = (int)(ld >> 1);
+  for (int g = wid * R; g < rows; g += kWarps * R) {
+    double a[P];
+#pragma unroll
+    for (int k = 0; k < P; ++k) a[k] = 0.0;
+    const double2* r[R];
+#pragma unroll
+    for (int u = 0; u < R; ++u) r[u] = reinterpret_cast<const double2*>(M + (size_t)min(g + u, rows - 1) * ld);
+#pragma unroll(R >= 4 ? 1 : 4)
+    for (int t = lane; t < nq; t += 32) {
+      const double2 x = reinterpret_cast<const double2*>(v0)[t];
+      double2 z = x;
+      if (NV == 2) z = reinterpret_cast<const double2*>(v1)[t];
+#pragma unroll
+      for (int u = 0; u < R; ++u) {
+        const double2 w = r[u][t];
+        a[u] += w.x * x.x;
+        if (NV == 2) a[R + u] += w.x * z.x;
+        a[u] += w.y * x.y;
+        if (NV == 2) a[R + u] += w.y * z.y;
+      }
+    }
+    const double v = sum_together<P>(a, lane);
+    if ((lane & ((1 << kShift) - 1)) == 0) {
+      const int k = lane >> kShift, u = k % R;
+      if (g + u < rows) out(k / R, g + u, v);
+    }
+  }
+}
+
+// rows per warp by the rows of the CTA: all warps busy first, then more sums per reduction
+template <int NV, typename F>
+__device__ __forceinline__ void dots_any(const double* M, int64_t ld, int rows, const double* v0, const double* v1, F out) {
+  if (rows > 4 * kWarps) dots<8, NV>(M, ld, rows, v0, v1, out);
+  else if (rows > 2 * kWarps) dots<4, NV>(M, ld, rows, v0, v1, out);
+  else if (rows > kWarps) dots<2, NV>(M, ld, rows, v0, v1, out);
+  else dots<1, NV>(M, ld, rows, v0, v1, out);
+}
+
+// The group of CTAs that solves an LP: a cluster (GRID = false) or the cooperative grid.
+template <bool GRID>
+struct Group {
+  int rank, size;
+  GridBarrier gb;
+  unsigned long long target;
+  __device__ Group(const GridBarrier& b) : gb(b), target(0) {
+    if constexpr (GRID) {
+      rank = blockIdx.x;
+      size = gridDim.x;
+    } else {
+      cg::cluster_group cl = cg::this_cluster();
+      rank = (int)cl.block_rank();
+      size = (int)cl.num_blocks();
+    }
+  }
+  // all CTAs of the group; false (everywhere) after a grid wait past its limit
+  __device__ __forceinline__ bool sync() {
+    if constexpr (GRID) return grid_sync(gb, target);
+    cg::this_cluster().sync();
+    return true;
+  }
+  // entry i of a shared vector, in every CTA's copy (cluster) or in the L2 copy g (grid)
+  __device__ __forceinline__ void put(double* vec, double* g, int i, double v) const {
+    if constexpr (GRID) {
+      __stcg(g + i, v);
+    } else {
+      const cg::cluster_group cl = cg::this_cluster();
+      for (int r = 0; r < size; ++r) *cl.map_shared_rank(vec + i, r) = v;
+    }
+  }
+  // after a sync: the grid's copy comes into shared memory (the caller syncs the CTA)
+  __device__ __forceinline__ void fetch(double* vec, const double* g, int len) const {
+    if constexpr (GRID)
+      for (int i = threadIdx.x; i < len; i += kThr) vec[i] = __ldcg(g + i);
+  }
+};
+
+struct GroupArgs {
+  DenseInst* insts;
+  int count;
+  DenseParams P;
+  int* queue;
+  const int* order;
+  int cache_vec, cache_mat;       // copies in shared memory: the CTA's vectors, its matrix rows
+  // grid mode: published vectors (q, z_y: ldt each; x, s: ld each), partial sums, barrier
+  double* gvec;
+  double* gpart;                  // (kSums + 2) * grid
+  unsigned long long* bar;
+  int* err;
+  unsigned long long bar_limit_ns;
+};
+
+struct Scal {
+  double tau, kappa, theta, mu, t1, t2, itau, cmu, gk;
+  int action, status, outer, ok;
+  int64_t total;
+  double a[kSums];   // the test sums
+};
+
+// The block's sums of NS values per thread (only the first `act` warps hold any), published
+// in the partial slots of every CTA: slots[r * NS + k] is CTA r's sum k.
+template <int NS, int P, bool GRID>
+__device__ __forceinline__ void publish_sums(const Group<GRID>& G, double (&acc)[P], int act, double* wsum, double* slots,
+                                             double* gslots) {
+  constexpr int kShift = P == 16 ? 1 : 4;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  if (wid < act) {
+    const double v = sum_together<P>(acc, lane);
+    const int k = lane >> kShift;
+    if ((lane & ((1 << kShift) - 1)) == 0 && k < NS) wsum[k * kWarps + wid] = v;
+  }
+  __syncthreads();
+  if constexpr (GRID) {
+    if (threadIdx.x < NS) {
+      double v = wsum[threadIdx.x * kWarps];
+      for (int w = 1; w < act; ++w) v += wsum[threadIdx.x * kWarps + w];
+      __stcg(gslots + (size_t)threadIdx.x * G.size + G.rank, v);
+    }
+  } else {
+    const cg::cluster_group cl = cg::this_cluster();
+    for (int t = threadIdx.x; t < NS * G.size; t += kThr) {
+      const int k = t % NS, r = t / NS;
+      double v = wsum[k * kWarps];
+      for (int w = 1; w < act; ++w) v += wsum[k * kWarps + w];
+      *cl.map_shared_rank(slots + G.rank * NS + k, r) = v;
+    }
+  }
+}
+
+// After the barrier: the NS totals into out (shared), by warp 0, in the same order in every CTA.
+template <int NS, bool GRID>
+__device__ __forceinline__ void total_sums(const Group<GRID>& G, const double* slots, const double* gslots, double* out) {
+  const int lane = threadIdx.x & 31;
+  if constexpr (GRID) {
+    double v[16];
+#pragma unroll
+    for (int k = 0; k < 16; ++k) v[k] = 0.0;
+    for (int i = lane; i < G.size; i += 32)
+#pragma unroll
+      for (int k = 0; k < NS; ++k) v[k] += __ldcg(gslots + (size_t)k * G.size + i);
+    const double s = sum_together<16>(v, lane);
+    if ((lane & 1) == 0 && (lane >> 1) < NS) out[lane >> 1] = s;
+  } else {
+    const int k = lane >> 1, h = lane & 1;
+    double v = 0.0;
+    if (k < NS)
+      for (int r = h; r < G.size; r += 2) v += slots[r * NS + k];
+    v += __shfl_xor_sync(0xffffffffu, v, 1);
+    if (h == 0 && k < NS) out[k] = v;
+  }
+  __syncwarp();
+}
+
+__device__ __forceinline__ int even(int k) { return (k + 1) & ~1; }
+
+// Algorithm 2 (with the relaxation of Sec. 4.2) for one instance by the group.
+template <bool GRID>
+__device__ void solve_one(DenseInst& I, const GroupArgs& Q, Group<GRID>& G, double* sm, double* wsum, Scal& S) {
+  const DenseParams& P = Q.P;
+  const int m = I.m, n = I.n, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int mp = even(m), np = even(n);
+  const int mc = (m + G.size - 1) / G.size, nc_ = (n + G.size - 1) / G.size;
+  const int i0 = min(m, G.rank * mc), mr = min(m, i0 + mc) - i0;   // this CTA's rows
+  const int j0 = min(n, G.rank * nc_), nr = min(n, j0 + nc_) - j0; // this CTA's columns
+  double* q = sm;
+  double* zy = q + mp;
+  double* x = zy + mp;
+  double* s = x + np;
+  double* hslot = s + np;                               // 2 * size
+  double* rslot = hslot + 2 * (GRID ? 1 : G.size);      // kSums * size
+  double* y = rslot + kSums * (GRID ? 1 : G.size);      // own rows
+  double* Ax = y + mc;
+  double* As = Ax + mc;
+  double* aty = As + mc;                                // own columns
+  double* v = aty + nc_;
+  double* top = v + nc_;
+  double* gq = Q.gvec;
+  double* gzy = gq + mp;
+  double* gx = gzy + mp;
+  double* gs = gx + np;
+  double* ghs = Q.gpart;
+  double* grs = Q.gpart + 2 * G.size;
+  const double* b = I.b + i0;
+  const double* bbar = I.bbar + i0;
+  const double* g1y = I.g1 + i0;
+  const double* g2y = I.g2 + i0;
+  const double* c = I.c + j0;
+  const double* cbar = I.cbar + j0;
+  const double* g1x = I.g1 + m + j0;
+  const double* g2x = I.g2 + m + j0;
+  const double* Ar = I.A + (size_t)i0 * I.ld;
+  const double* ATr = I.AT + (size_t)j0 * mp;
+  const double* Gr = I.Ginv + (size_t)i0 * mp;
+  if (Q.cache_vec) {
+    double* d = top;
+    auto copy = [&](const double*& src, int len, int room) {
+      for (int i = threadIdx.x; i < len; i += kThr) d[i] = src[i];
+      src = d;
+      d += room;
+    };
+    copy(b, mr, mc); copy(bbar, mr, mc); copy(g1y, mr, mc); copy(g2y, mr, mc);
+    copy(c, nr, nc_); copy(cbar, nr, nc_); copy(g1x, nr, nc_); copy(g2x, nr, nc_);
+    top = sm + even((int)(d - sm));
+  }
+  if (Q.cache_mat) {
+    double* d = top;
+    auto copy = [&](const double*& src, int rows, int64_t ld, int room) {
+      for (int64_t e = threadIdx.x; e < rows * ld; e += kThr) d[e] = src[e];
+      src = d;
+      d += room * ld;
+    };
+    copy(Ar, mr, np, mc); copy(ATr, nr, mp, nc_); copy(Gr, mr, mp, mc);
+  }
+  const double alpha = P.alpha, eps = P.eps, a1 = 1.0 - alpha;
+  const double zbar = I.zbar, xi = -(double)n - 1.0, nb = I.nb, nc = I.nc;
+  const double Ki0 = I.Kinv[0], Ki1 = I.Kinv[1], Ki2 = I.Kinv[2], Ki3 = I.Kinv[3];
+  // screens of the Sec. 4.1 tests without square roots and divisions; a sum that passes is
+  // tested as written
+  const double tp = eps * (1.0 + nb) * (1.0 + 1e-12), td = eps * (1.0 + nc) * (1.0 + 1e-12);
+  // start of Algorithm 2, or a state loaded by abip_set_state
+  const bool resume = I.resume != 0;
+  for (int i = threadIdx.x; i < mp; i += kThr) {
+    q[i] = 0.0;
+    zy[i] = (resume && i < m) ? I.y[i] : 0.0;
+  }
+  for (int j = threadIdx.x; j < np; j += kThr) {
+    x[j] = j < n ? (resume ? I.x[j] : 1.0) : 0.0;
+    s[j] = j < n ? (resume ? I.s[j] : 1.0) : 0.0;
+  }
+  for (int i = threadIdx.x; i < mr; i += kThr) y[i] = resume ? I.y[i0 + i] : 0.0;
+  for (int j = threadIdx.x; j < nr; j += kThr) aty[j] = 0.0;
+  if (threadIdx.x == 0) {
+    S.tau = resume ? I.r_tau : 1.0;
+    S.kappa = resume ? I.r_kappa : 1.0;
+    S.theta = resume ? I.r_theta : 1.0;
+    S.mu = resume ? I.r_mu : P.beta;
+    S.total = resume ? I.r_iters : 0;
+    S.outer = resume ? I.r_outer : 0;
+    S.itau = 1.0 / S.tau;
+    S.status = 0;
+    S.ok = 1;
+  }
+  __syncthreads();
+  if (resume) {   // A^T y of the loaded state, once (z_y's buffer holds y)
+    dots_any<1>(ATr, mp, nr, zy, zy, [&](int, int j, double d) { aty[j] = d; });
+    __syncthreads();
+    for (int i = threadIdx.x; i < mp; i += kThr) zy[i] = 0.0;
+  }
+  const int items = nr + mr, act = min(kWarps, max(1, (items + 31) / 32));
+  bool first = true;   // the sums of a start or of a warm start: no test, no count
+  if (!G.sync()) return;   // nobody publishes into a CTA that is still filling its copies
+  for (;;) {
+    // ---- products of the state, its test sums (residual_sums' order of quantities), and q
+    dots_any<2>(Ar, np, mr, x, s, [&](int w, int i, double d) { (w == 0 ? Ax : As)[i] = d; });
+    __syncthreads();
+    {
+      double acc[16];
+#pragma unroll
+      for (int k = 0; k < 16; ++k) acc[k] = 0.0;
+      const double ta = S.tau, th = S.theta, it = S.itau;
+      for (int e = threadIdx.x; e < items; e += kThr) {
+        if (e < nr) {
+          const double at = aty[e], sj = s[j0 + e], cj = c[e], cb = cbar[e], xj = x[j0 + e];
+          const double as = at + sj;
+          const double rx = cj * ta - cb * th - as;
+          const double dr = as * it - cj;
+          acc[0] += rx * rx; acc[2] += dr * dr; acc[4] += as * as;
+          acc[7] += cj * xj; acc[8] += cb * xj;
+        } else {
+          const int i = e - nr;
+          const double ax = Ax[i], bi = b[i], bb = bbar[i], yi = y[i];
+          const double ry = ax - bi * ta + bb * th;
+          const double pr = ax * it - bi;
+          acc[0] += ry * ry; acc[1] += pr * pr; acc[3] += ax * ax;
+          acc[5] += bi * yi; acc[6] += bb * yi;
+          G.put(q, gq, i0 + i, yi - (ax + As[i]));
+        }
+      }
+      publish_sums<kSums, 16, GRID>(G, acc, act, wsum, rslot, grs);
+    }
+    if (!G.sync()) return;
+    G.fetch(q, gq, m);
+    if (wid == 0) {
+      total_sums<kSums, GRID>(G, rslot, grs, S.a);
+      if (lane == 0) {
+        const double* a = S.a;
+        const double tau = S.tau;
+        const double rt = a[5] - a[7] + zbar * S.theta - S.kappa;
+        const double rth = -a[6] + a[8] - zbar * tau - xi;
+        const double inner2 = a[0] + rt * rt + rth * rth;
+        int st = 0, action = ACT_STEP;
+        if (!isfinite(inner2)) {
+          S.ok = 0;
+          action = ACT_STOP;
+        } else {
+          if (!first) {
+            S.total += 1;
+            if (P.stop_rule == 0) {
+              if (a[1] <= tp * tp && a[2] <= td * td) {
+                const double ps = sqrt(a[1]) / (1.0 + nb), ds = sqrt(a[2]) / (1.0 + nc);
+                const double gp = fabs(a[7] / tau - a[5] / tau) / (1.0 + fabs(a[7] / tau) + fabs(a[5] / tau));
+                if (ps <= eps && ds <= eps && gp <= eps) st = ABIP_OPTIMAL;
+              }
+              const double pe = eps * a[5], de = eps * a[7];
+              if (st == 0 && a[5] > 0 && a[4] * (nb * nb) <= pe * pe * (1.0 + 1e-11) && sqrt(a[4]) <= pe / nb)
+                st = ABIP_PRIMAL_INFEASIBLE;
+              if (st == 0 && a[7] < 0 && a[3] * (nc * nc) <= de * de * (1.0 + 1e-11) && sqrt(a[3]) <= -de / nc)
+                st = ABIP_DUAL_INFEASIBLE;
+            }
+            if (st == 0 && S.total >= P.max_admm) st = ABIP_MAX_ITER;
+          }
+          if (st == 0 && inner2 <= S.mu) {
+            double rho = 0.0;
+            if (P.gamma_max > 0.0)
+              rho = fmax(sqrt(a[1]) / (1.0 + nb),
+                         fmax(sqrt(a[2]) / (1.0 + nc),
+                              fabs(a[7] / tau - a[5] / tau) / (1.0 + fabs(a[7] / tau) + fabs(a[5] / tau))));
+            S.gk = adaptive_gamma(P.gamma, P.gamma_max, eps, rho);
+            S.mu *= S.gk;
+            S.outer += 1;
+            action = ACT_WARM;
+            if (P.stop_rule == 1 && S.mu < eps) st = ABIP_OPTIMAL;
+            else if (S.outer >= kMaxOuter) st = ABIP_MAX_ITER;   // mu has underflowed
+          }
+          if (st != 0) {
+            S.status = st;
+            action = ACT_STOP;
+          }
+        }
+        S.action = action;
+      }
+    }
+    __syncthreads();
+    if (S.action == ACT_STOP) break;
+    if (S.action == ACT_WARM) {
+      const double gk = S.gk, sg = sqrt(gk);
+      for (int j = threadIdx.x; j < n; j += kThr) {   // every CTA its own copies of x and s
+        if (P.warmstart == 1) { x[j] *= sg; s[j] *= sg; }
+        else if (x[j] >= s[j]) s[j] *= gk;
+        else x[j] *= gk;
+      }
+      for (int i = threadIdx.x; i < mr; i += kThr) y[i] *= sg;
+      for (int j = threadIdx.x; j < nr; j += kThr) aty[j] *= sg;
+      if (threadIdx.x == 0) {
+        if (P.warmstart == 1) { S.tau *= sg; S.kappa *= sg; }
+        else if (S.tau >= S.kappa) S.kappa *= gk;
+        else S.tau *= gk;
+        S.theta *= sg;
+        S.itau = 1.0 / S.tau;
+      }
+      first = true;
+      // no CTA publishes q or its sums before all have read the last ones
+      if (!G.sync()) return;
+      continue;
+    }
+    first = false;
+    // ---- projection: z_y = G^{-1} (y - A (x + s)), z_x = x + s + A^T z_y, H^T z
+    dots_any<1>(Gr, mp, mr, q, q, [&](int, int i, double d) { G.put(zy, gzy, i0 + i, d); });
+    if (!G.sync()) return;
+    G.fetch(zy, gzy, m);
+    if constexpr (GRID) __syncthreads();
+    dots_any<1>(ATr, mp, nr, zy, zy, [&](int, int j, double d) { v[j] = d; });
+    __syncthreads();
+    {
+      double acc[2] = {0.0, 0.0};
+      for (int e = threadIdx.x; e < items; e += kThr) {
+        if (e < nr) {
+          const double z = x[j0 + e] + s[j0 + e] + v[e];
+          acc[0] += c[e] * z;
+          acc[1] -= cbar[e] * z;
+        } else {
+          const int i = e - nr;
+          const double z = zy[i0 + i];
+          acc[0] -= b[i] * z;
+          acc[1] += bbar[i] * z;
+        }
+      }
+      publish_sums<2, 2, GRID>(G, acc, act, wsum, hslot, ghs);
+    }
+    if (!G.sync()) return;
+    if (wid == 0) {
+      __shared__ double hz[2];
+      total_sums<2, GRID>(G, hslot, ghs, hz);
+      if (lane == 0) {
+        const double v1 = S.tau + S.kappa + hz[0], v2 = S.theta + xi + hz[1];
+        S.t1 = Ki0 * v1 + Ki1 * v2;
+        S.t2 = Ki2 * v1 + Ki3 * v2;
+        S.cmu = S.mu / P.beta;
+      }
+    }
+    __syncthreads();
+    // ---- relaxation, barrier and dual steps (Eqs. Simple-Update:*), and A^T y by linearity;
+    // the scalars' own step on the last warp
+    const double t1 = S.t1, t2 = S.t2, cmu = S.cmu;
+    for (int e = threadIdx.x; e < items; e += kThr) {
+      if (e < nr) {
+        const int j = j0 + e;
+        const double x0 = x[j], s0 = s[j];
+        const double ux = x0 + s0 + v[e] - g1x[e] * t1 - g2x[e] * t2;
+        double xn, sn;
+        barrier_step<double>(alpha * ux + a1 * x0 - s0, cmu, xn, sn);
+        G.put(x, gx, j, xn);
+        G.put(s, gs, j, sn);
+        // A^T g1y = g1x - c and A^T g2y = g2x + cbar (M g = h)
+        aty[e] = alpha * (v[e] - (g1x[e] - c[e]) * t1 - (g2x[e] + cbar[e]) * t2) + a1 * aty[e];
+      } else {
+        const int i = e - nr;
+        const double uy = zy[i0 + i] - g1y[i] * t1 - g2y[i] * t2;
+        y[i] = alpha * uy + a1 * y[i];
+      }
+    }
+    if (threadIdx.x == kThr - 1) {
+      const double th = alpha * t1 + a1 * S.tau;
+      double tn, kn;
+      barrier_step<double>(th - S.kappa, cmu, tn, kn);
+      S.tau = tn;
+      S.kappa = kn;
+      S.theta = alpha * t2 + a1 * S.theta;
+      S.itau = 1.0 / tn;
+    }
+    if (!G.sync()) return;
+    G.fetch(x, gx, n);
+    G.fetch(s, gs, n);
+    if constexpr (GRID) __syncthreads();
+  }
+  // outputs: raw state and the scaled candidate or certificate (Sec. 4.1)
+  const double bty = S.a[5], ctx = S.a[7], tau = S.tau;
+  const int status = S.status;
+  double sx = 1.0 / tau, sy = 1.0 / tau;
+  if (status == ABIP_PRIMAL_INFEASIBLE) { sx = 1.0; sy = 1.0 / bty; }
+  if (status == ABIP_DUAL_INFEASIBLE) { sx = -1.0 / ctx; sy = 1.0; }
+  for (int i = threadIdx.x; i < mr; i += kThr) {
+    I.y[i0 + i] = y[i];
+    if (I.out_y) I.out_y[i0 + i] = y[i] * sy;
+  }
+  for (int e = threadIdx.x; e < nr; e += kThr) {
+    const int j = j0 + e;
+    I.x[j] = x[j];
+    I.s[j] = s[j];
+    if (I.out_x) I.out_x[j] = x[j] * sx;
+    if (I.out_s) I.out_s[j] = s[j] * sy;
+  }
+  // the descriptor is read by every CTA until here
+  if (!G.sync()) return;
+  if (G.rank == 0 && threadIdx.x == 0) {
+    const double* a = S.a;
+    I.tau = tau; I.kappa = S.kappa; I.theta = S.theta; I.mu = S.mu;
+    I.resume = 0;
+    I.pres = sqrt(a[1]) / (1.0 + nb);
+    I.dres = sqrt(a[2]) / (1.0 + nc);
+    I.dgap = fabs(ctx / tau - bty / tau) / (1.0 + fabs(ctx / tau) + fabs(bty / tau));
+    I.ctx = ctx; I.bty = bty; I.obj = ctx / tau;
+    I.admm_iters = S.total; I.outer_iters = S.outer; I.status = status;
+    I.beta_last = P.beta;
+    if (!S.ok) I.err = DEV_ERR_NONFINITE;
+  }
+}
+
+template <int MINB>
+__global__ void __launch_bounds__(kThr, MINB) dense_cluster_kernel(GroupArgs Q) {
+  extern __shared__ __align__(16) double sm[];
+  __shared__ double wsum[kSums * kWarps];
+  __shared__ Scal S;
+  __shared__ int s_id;
+  cg::cluster_group cl = cg::this_cluster();
+  Group<false> G(GridBarrier{});
+  for (;;) {
+    if (G.rank == 0 && threadIdx.x == 0) {
+      const int k = atomicAdd(Q.queue, 1);
+      const int id = k < Q.count ? (Q.order ? Q.order[k] : k) : -1;
+      for (int r = 0; r < G.size; ++r) *cl.map_shared_rank(&s_id, r) = id;
+    }
+    cl.sync();
+    const int id = s_id;
+    if (id < 0) return;   // the same in every CTA, after which none writes to another
+    DenseInst& I = Q.insts[id];
+    if (I.err == 0) solve_one<false>(I, Q, G, sm, wsum, S);
+    cl.sync();            // every CTA has read s_id and its copies
+  }
+}
+
+__global__ void __launch_bounds__(kThr, 1) dense_grid_kernel(GroupArgs Q) {
+  extern __shared__ __align__(16) double sm[];
+  __shared__ double wsum[kSums * kWarps];
+  __shared__ Scal S;
+  Group<true> G(GridBarrier{Q.bar, Q.err, Q.bar_limit_ns});
+  if (Q.insts[0].err == 0) solve_one<true>(Q.insts[0], Q, G, sm, wsum, S);
+}
+
+using ClusterFn = void (*)(GroupArgs);
+ClusterFn cluster_fn(int variant) {
+  return variant == 2 ? dense_cluster_kernel<3> : variant == 1 ? dense_cluster_kernel<2> : dense_cluster_kernel<1>;
+}
+
+struct SmemPlan {
+  size_t bytes;
+  int cache_vec, cache_mat;
+};
+
+size_t base_doubles(int m, int n, int C, bool grid) {
+  const size_t mp = (m + 1) / 2 * 2, np = (n + 1) / 2 * 2, mc = (m + C - 1) / C, nc = (n + C - 1) / C;
+  return 2 * mp + 2 * np + (2 + kSums) * (size_t)(grid ? 1 : C) + 3 * mc + 2 * nc;
+}
+size_t vec_doubles(int m, int n, int C) { return 4 * (size_t)((m + C - 1) / C) + 4 * (size_t)((n + C - 1) / C) + 2; }
+size_t mat_doubles(int m, int n, int C) {
+  const size_t mp = (m + 1) / 2 * 2, np = (n + 1) / 2 * 2, mc = (m + C - 1) / C, nc = (n + C - 1) / C;
+  return mc * (np + mp) + nc * mp + 2;
+}
+
+// the shared memory of a launch for the given sizes: the copies that fit the budget
+SmemPlan plan_smem(const int* m, const int* n, int count, int C, bool grid, size_t budget) {
+  size_t base = 0, vec = 0, mat = 0;
+  for (int k = 0; k < count; ++k) {
+    const size_t b = base_doubles(m[k], n[k], C, grid), v = b + vec_doubles(m[k], n[k], C);
+    base = std::max(base, b);
+    vec = std::max(vec, v);
+    mat = std::max(mat, v + mat_doubles(m[k], n[k], C));
+  }
+  SmemPlan p{base * 8 + 16, 0, 0};
+  if (vec * 8 <= budget) { p.bytes = vec * 8 + 16; p.cache_vec = 1; }
+  if (p.cache_vec && mat * 8 <= budget) { p.bytes = mat * 8 + 16; p.cache_mat = 1; }
+  return p;
+}
+
+constexpr size_t kSmemMax = 224 * 1024;
+
+cudaError_t cluster_config(ClusterFn f, int C, size_t smem, cudaLaunchConfig_t& cfg, cudaLaunchAttribute* at) {
+  cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
+  if (e == cudaSuccess && C > 8) e = cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  cfg.blockDim = dim3(kThr);
+  cfg.gridDim = dim3((unsigned)C);
+  cfg.dynamicSmemBytes = smem;
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)C;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return e;
+}
+
+}  // namespace
+
+int plan_dense_group(const int* m, const int* n, int count, int sms, DenseGroupPlan& plan) {
+  plan = DenseGroupPlan{};
+  // FP64 operations of one update of the largest instance: its products, and about 80 a
+  // column and row for the steps and sums
+  int64_t wmax = 0;
+  for (int k = 0; k < count; ++k)
+    wmax = std::max(wmax, 3 * (int64_t)m[k] * n[k] + (int64_t)m[k] * m[k] + 80 * (int64_t)(m[k] + n[k]));
+  // CTAs per instance: up to two CTAs per SM over the batch, while a CTA keeps more than 5000
+  // operations (2.5k clocks; the four barriers cost about as much).  Measured, us per update
+  // with 1 / 2 / 4 / 8 / 16 CTAs: 16 x 48 11.6 / 10.6 / 10.0 / 10.1 / 10.9; 50 x 120 19.0 /
+  // 13.5 / 11.9 / 11.1 / 11.1; 100 x 300 53 / 31 / 19.7 / 14.5 / 13.1; 512 x 1154 578 / 298 /
+  // 153 / 83 / 51; 64 LPs of m 16 .. 256 222 / 117 / 65 / 98 / 163.
+  int C = 1;
+  while (C < 16 && 2 * C * (int64_t)count <= 2 * sms && wmax / C > 5000) C *= 2;
+  // One LP over the whole grid: its barriers cost more than a cluster's, its 152 SMs take over
+  // from 16 at about 8e5 operations (cluster of 16 / grid: 200 x 600 20.6 / 23.7 us, 256 x
+  // 1024 25.2 / 24.2, 300 x 900 30.8 / 24.5, 512 x 1154 50.7 / 26.4).
+  plan.grid_mode = count == 1 && wmax > 800000;
+  if (plan.grid_mode) {
+    const SmemPlan s = plan_smem(m, n, count, sms, true, kSmemMax - 16);
+    plan.ctas = sms;
+    plan.smem = s.bytes;
+    plan.cache_vec = s.cache_vec;
+    plan.cache_mat = s.cache_mat;
+    return 1;
+  }
+  for (;; C *= 2) {
+    const size_t budget = C * (int64_t)count > sms ? 100 * 1024 : kSmemMax - 16;
+    const SmemPlan s = plan_smem(m, n, count, C, false, budget);
+    plan.ctas = C;
+    plan.smem = s.bytes;
+    plan.cache_vec = s.cache_vec;
+    plan.cache_mat = s.cache_mat;
+    if (s.bytes <= kSmemMax) return 1;
+    if (C >= 8) return 0;
+  }
+}
+
+size_t dense_group_scratch(int m, int n, int sms) {
+  const size_t mp = (m + 1) / 2 * 2, np = (n + 1) / 2 * 2;
+  return 2 * mp + 2 * np + (size_t)(kSums + 2) * sms + 4;
+}
+
+cudaError_t launch_dense_group(DenseInst* inst, int count, const DenseParams& prm, int* queue, const int* order,
+                               const DenseGroupPlan& plan, int variant, double* scratch, size_t scratch_len,
+                               unsigned long long limit_ns, cudaStream_t st) {
+  GroupArgs Q{inst, count, prm, queue, order, plan.cache_vec, plan.cache_mat, nullptr, nullptr, nullptr, nullptr, limit_ns};
+  if (plan.grid_mode) {
+    // barrier counter and error word at the end of the scratch, zeroed by the caller
+    Q.bar = reinterpret_cast<unsigned long long*>(scratch + scratch_len - 2);
+    Q.err = reinterpret_cast<int*>(scratch + scratch_len - 1);
+    Q.gpart = scratch;
+    Q.gvec = scratch + (size_t)(kSums + 2) * plan.ctas + ((kSums + 2) * (size_t)plan.ctas & 1);
+    cudaError_t e = cudaFuncSetAttribute(dense_grid_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
+    if (e != cudaSuccess) return e;
+    void* args[] = {&Q};
+    return cudaLaunchCooperativeKernel((const void*)dense_grid_kernel, dim3(plan.ctas), dim3(kThr), args, plan.smem, st);
+  }
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[1];
+  ClusterFn f = cluster_fn(variant);
+  cudaError_t e = cluster_config(f, plan.ctas, plan.smem, cfg, at);
+  if (e != cudaSuccess) return e;
+  int ncl = 0;
+  e = cudaOccupancyMaxActiveClusters(&ncl, f, &cfg);
+  if (e != cudaSuccess) return e;
+  if (ncl < 1) return cudaErrorInvalidConfiguration;
+  cfg.gridDim = dim3((unsigned)(std::min(count, ncl) * plan.ctas));
+  cfg.stream = st;
+  return cudaLaunchKernelEx(&cfg, f, Q);
+}
+
+int dense_group_ctas_per_sm(const DenseGroupPlan& plan, int variant) {
+  int per = 0;
+  if (plan.grid_mode) {
+    cudaFuncSetAttribute(dense_grid_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, dense_grid_kernel, kThr, plan.smem);
+    return per;
+  }
+  ClusterFn f = cluster_fn(variant);
+  cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, f, kThr, plan.smem);
+  return per;
+}
+
+}  // namespace abip

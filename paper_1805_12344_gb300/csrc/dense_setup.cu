@@ -306,8 +306,28 @@ __global__ void __launch_bounds__(kThr) inverse_tiles_kernel(const DenseInst* __
     }
     for (int e = threadIdx.x; e < m * Q; e += kThr) {
       const int q = e / m, i = e % m;
-      if (c0 + q < m) I.Ginvf[(size_t)(c0 + q) * I.ldtf + i] = (float)W[i * Q + q];
+      if (c0 + q >= m) continue;
+      if (I.Ginvf) I.Ginvf[(size_t)(c0 + q) * I.ldtf + i] = (float)W[i * Q + q];
+      if (I.Ginv) I.Ginv[(size_t)(c0 + q) * (m + (m & 1)) + i] = W[i * Q + q];
     }
+    __syncthreads();
+  }
+}
+
+// A^T, rows padded to an even length (the padding is zero already), 32 x 32 tiles
+__global__ void __launch_bounds__(kThr) transpose_tiles_kernel(const DenseInst* __restrict__ insts) {
+  __shared__ double T[32][33];
+  const DenseInst& I = insts[blockIdx.y];
+  const int m = I.m, n = I.n, mp = m + (m & 1);
+  const int tm = (m + 31) / 32, tiles = tm * ((n + 31) / 32);
+  const int lane = threadIdx.x & 31, row = threadIdx.x >> 5;
+  for (int t = blockIdx.x; t < tiles; t += gridDim.x) {
+    const int i0 = (t % tm) * 32, j0 = (t / tm) * 32;
+    for (int r = row; r < 32; r += kThr / 32)
+      T[r][lane] = (i0 + r < m && j0 + lane < n) ? I.A[(size_t)(i0 + r) * I.ld + j0 + lane] : 0.0;
+    __syncthreads();
+    for (int r = row; r < 32; r += kThr / 32)
+      if (j0 + r < n && i0 + lane < m) I.AT[(size_t)(j0 + r) * mp + i0 + lane] = T[lane][r];
     __syncthreads();
   }
 }
@@ -352,6 +372,16 @@ cudaError_t launch_dense_factor(DenseInst* inst, int count, int mmax, int sms, c
   cfg.attrs = at;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, chol_cluster_kernel, inst, count);
+}
+
+cudaError_t launch_dense_transpose(DenseInst* inst, int count, int mmax, int nmax, int sms, cudaStream_t st) {
+  const int64_t tiles = (int64_t)((mmax + 31) / 32) * ((nmax + 31) / 32);
+  for (int k0 = 0; k0 < count; k0 += 32768) {
+    const int cnt = std::min(32768, count - k0);
+    const int gx = (int)std::max<int64_t>(1, std::min<int64_t>(tiles, (8 * sms + cnt - 1) / cnt));
+    transpose_tiles_kernel<<<dim3(gx, cnt), kThr, 0, st>>>(inst + k0);
+  }
+  return cudaGetLastError();
 }
 
 cudaError_t launch_dense_inverse(DenseInst* inst, int count, int mmax, int sms, cudaStream_t st) {

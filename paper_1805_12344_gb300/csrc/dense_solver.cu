@@ -1460,8 +1460,8 @@ __global__ void __launch_bounds__(kThreads) dense_backward_kernel(BackwardInst* 
 // dynamic shared memory of the solve kernel: 5m + 3n doubles, at most this many bytes
 constexpr size_t kDenseSmemMax = 200 * 1024;
 
-cudaError_t launch_dense_setup(DenseInst* inst, int count, int* queue, int grid, size_t smem, int mmax, bool inverse,
-                               cudaStream_t st) {
+cudaError_t launch_dense_setup(DenseInst* inst, int count, int* queue, int grid, size_t smem, int mmax, int nmax,
+                               bool inverse, cudaStream_t st) {
   // the caller sizes smem for the largest instance: 2m + n doubles
   cudaError_t e = cudaFuncSetAttribute(dense_setup_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDenseSmemMax);
   if (e != cudaSuccess) return e;
@@ -1472,8 +1472,9 @@ cudaError_t launch_dense_setup(DenseInst* inst, int count, int* queue, int grid,
   if (e != cudaSuccess) return e;
   dense_setup_kernel<false><<<grid, kThreads, smem, st>>>(inst, count, queue);
   e = cudaGetLastError();
-  if (e != cudaSuccess || !inverse) return e;
-  return launch_dense_inverse(inst, count, mmax, sms, st);
+  if (e == cudaSuccess && inverse) e = launch_dense_inverse(inst, count, mmax, sms, st);
+  if (e == cudaSuccess && nmax > 0) e = launch_dense_transpose(inst, count, mmax, nmax, sms, st);
+  return e;
 }
 
 // the solve kernel of a precision and an occupancy variant (0, 1, 2: MINB 1, 2, 3 for FP64
