@@ -502,7 +502,8 @@ int dense_alloc(abip_handle* h, const std::vector<DenseHostInst>& hi, void** are
       I.ld = group ? n + (n & 1) : n;
       I.A = ar.take<double>((size_t)m * I.ld);
       I.AT = group ? ar.take<double>((size_t)n * (m + (m & 1))) : nullptr;
-      I.Ginv = group ? ar.take<double>((size_t)m * (m + (m & 1))) : nullptr;
+      I.Li = group ? ar.take<double>((size_t)m * (m + (m & 1))) : nullptr;
+      I.LiT = group ? ar.take<double>((size_t)m * (m + (m & 1))) : nullptr;
       I.b = ar.take<double>(m); I.c = ar.take<double>(n);
       I.L = ar.take<double>((size_t)m * m);
       I.bbar = ar.take<double>(m); I.cbar = ar.take<double>(n);
@@ -592,8 +593,8 @@ int dense_run_solve(abip_handle* h, DenseInst* dinst, int* queue, int count, int
   double* words = grid_mode ? h->gscratch + h->gscratch_len - 2 : nullptr;   // barrier counter, error word
   if (words) cudaMemsetAsync(words, 0, 16, st);
   cudaEventRecord(e0, st);
-  cudaError_t e = h->group ? abip::launch_dense_group(dinst, count, dp, queue, order, h->gplan, variant, h->gscratch,
-                                                      h->gscratch_len, (unsigned long long)h->prm.barrier_limit_ns, st)
+  cudaError_t e = h->group ? abip::launch_dense_group(dinst, count, dp, queue, order, h->gplan, h->gsp, variant,
+                                                      h->gscratch, h->gscratch_len, (unsigned long long)h->prm.barrier_limit_ns, st)
                            : abip::launch_dense_solve(dinst, count, dp, queue, order, grid, smem, variant, st);
   cudaEventRecord(e1, st);
   int derr = 0;
@@ -607,6 +608,133 @@ int dense_run_solve(abip_handle* h, DenseInst* dinst, int* queue, int count, int
   if (derr != 0) return fail(h, device_error_code(derr), std::string("solve: ") + device_error_str(derr));
   h->kernel_s = ms * 1e-3;
   h->launches = 1;
+  return ABIP_OK;
+}
+
+// ---------------------------------------------------------------------------
+// Sparse direct projection of an LP with few rows: the dense path's group kernel with the
+// products over the CSR entries.  The setup launch of the sparse path (its factor and checks)
+// has run; this adds the inverse of G's Cholesky factor and a descriptor of the same vectors.
+// Where there is no room for it, or G's factorisation breaks down, the sweeps stay.
+// ---------------------------------------------------------------------------
+void setup_direct(abip_handle* h, const HostCSR& A) {
+  const int m = h->m, n = h->n, mp = m + (m & 1);
+  if (m > abip::kDirectMaxRows || A.rp[m] > (int64_t)INT32_MAX) return;
+  // A by columns with duplicate entries merged (row order within a column is increasing), and
+  // back by rows
+  HostCSR T = transpose(A), M;
+  M.m = n; M.n = m;
+  M.rp.assign(n + 1, 0);
+  for (int j = 0; j < n; ++j) {
+    for (int64_t k = T.rp[j]; k < T.rp[j + 1]; ++k) {
+      if (k > T.rp[j] && T.ci[k] == T.ci[k - 1]) M.v.back() += T.v[k];
+      else { M.ci.push_back(T.ci[k]); M.v.push_back(T.v[k]); }
+    }
+    M.rp[j + 1] = (int64_t)M.ci.size();
+  }
+  const HostCSR R = transpose(M);
+  const std::vector<int32_t> rp(R.rp.begin(), R.rp.end()), cp(M.rp.begin(), M.rp.end());
+  const size_t nz = M.ci.size();
+  const int sms = abip::dense_max_ctas(h->device);
+  abip::DenseGroupPlan plan;
+  abip::GroupSparse sp;
+  if (!abip::plan_sparse_group(m, n, rp.data(), cp.data(), sms, sp, plan)) return;
+  struct { int32_t *rp, *ci, *cp, *ri; double *va, *cv; } d;
+  DenseInst I{};
+  DenseInst* dinst = nullptr;
+  int* queue = nullptr;
+  double* scratch = nullptr;
+  const size_t scratch_len = abip::dense_group_scratch(m, n, sms);
+  auto layout = [&](Arena& ar) {
+    dinst = ar.take<DenseInst>(1);
+    queue = ar.take<int>(2);
+    I.L = ar.take<double>((size_t)m * m);
+    I.Li = ar.take<double>((size_t)m * mp);
+    I.LiT = ar.take<double>((size_t)m * mp);
+    I.g1 = ar.take<double>(m + n); I.g2 = ar.take<double>(m + n);
+    d.rp = ar.take<int32_t>(m + 1); d.ci = ar.take<int32_t>(nz); d.va = ar.take<double>(nz);
+    d.cp = ar.take<int32_t>(n + 1); d.ri = ar.take<int32_t>(nz); d.cv = ar.take<double>(nz);
+    scratch = ar.take<double>(scratch_len);
+  };
+  Arena probe;
+  layout(probe);
+  void* mem = nullptr;
+  if (cudaMalloc(&mem, probe.off) != cudaSuccess) { cudaGetLastError(); return; }
+  Arena ar;
+  ar.base = static_cast<char*>(mem);
+  layout(ar);
+  const GridData<double>& g = h->gd64;
+  cudaError_t e = cudaMemset(mem, 0, probe.off);
+  auto up = [&](void* dst, const void* src, size_t bytes, cudaMemcpyKind kind) {
+    if (e == cudaSuccess && bytes) e = cudaMemcpy(dst, src, bytes, kind);
+  };
+  up(d.rp, rp.data(), rp.size() * 4, cudaMemcpyHostToDevice);
+  up(d.ci, R.ci.data(), nz * 4, cudaMemcpyHostToDevice);
+  up(d.va, R.v.data(), nz * 8, cudaMemcpyHostToDevice);
+  up(d.cp, cp.data(), cp.size() * 4, cudaMemcpyHostToDevice);
+  up(d.ri, M.ci.data(), nz * 4, cudaMemcpyHostToDevice);
+  up(d.cv, M.v.data(), nz * 8, cudaMemcpyHostToDevice);
+  up(I.g1, g.g1y, m * 8, cudaMemcpyDeviceToDevice);
+  up(I.g1 + m, g.g1x, n * 8, cudaMemcpyDeviceToDevice);
+  up(I.g2, g.g2y, m * 8, cudaMemcpyDeviceToDevice);
+  up(I.g2 + m, g.g2x, n * 8, cudaMemcpyDeviceToDevice);
+  sp.rp = d.rp; sp.ci = d.ci; sp.va = d.va;
+  sp.cp = d.cp; sp.ri = d.ri; sp.cv = d.cv;
+  SolveCtl hc;
+  up(&hc, h->ctl, sizeof(hc), cudaMemcpyDeviceToHost);
+  I.m = m; I.n = n; I.ld = n;
+  I.b = g.b; I.c = g.c; I.bbar = g.bbar; I.cbar = g.cbar;
+  I.y = g.y; I.x = g.x; I.s = g.s;
+  I.out_x = h->stage; I.out_y = h->stage + n; I.out_s = h->stage + n + m;
+  I.zbar = hc.zbar; I.nb = hc.nb; I.nc = hc.nc;
+  for (int k = 0; k < 4; ++k) I.Kinv[k] = hc.Kinv[k];
+  up(dinst, &I, sizeof(I), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = abip::launch_sparse_factor(dinst, m, sp, sms, 0);
+  if (e == cudaSuccess) e = abip::launch_dense_inverse(dinst, 1, m, sms, 0);
+  DenseInst back{};
+  up(&back, dinst, sizeof(back), cudaMemcpyDeviceToHost);
+  if (e != cudaSuccess || back.err != 0) {
+    cudaGetLastError();
+    cudaFree(mem);
+    return;
+  }
+  h->arena2 = mem;
+  h->hinst = I;
+  h->dinst = dinst;
+  h->queue = queue;
+  h->gplan = plan;
+  h->gsp = sp;
+  h->gscratch = scratch;
+  h->gscratch_len = scratch_len;
+  h->group = true;
+}
+
+// The solve of a handle that setup_direct completed; its scalars go where the sparse path
+// keeps them (abip_get_state).
+int solve_direct(abip_handle* h, cudaStream_t st) {
+  const int m = h->m, n = h->n;
+  DenseInst I = h->hinst;
+  if (h->resume) {
+    const std::vector<double>& rs = h->resume_state;
+    cudaMemcpyAsync(I.y, rs.data(), m * 8, cudaMemcpyHostToDevice, st);
+    cudaMemcpyAsync(I.x, rs.data() + m, n * 8, cudaMemcpyHostToDevice, st);
+    cudaMemcpyAsync(I.s, rs.data() + m + n + 2, n * 8, cudaMemcpyHostToDevice, st);
+    I.resume = 1;
+    I.r_tau = rs[m + n]; I.r_theta = rs[m + n + 1]; I.r_kappa = rs[m + 2 * n + 2]; I.r_mu = rs[m + 2 * n + 3];
+    h->resume = false;
+  }
+  cudaMemcpyAsync(h->dinst, &I, sizeof(I), cudaMemcpyHostToDevice, st);
+  const int rc = dense_run_solve(h, h->dinst, h->queue, 1, 1, 0, dense_params(h->prm), st);
+  if (rc) return rc;
+  SolveCtl hc;
+  cudaError_t e = cudaMemcpy(&I, h->dinst, sizeof(I), cudaMemcpyDeviceToHost);
+  if (e == cudaSuccess) e = cudaMemcpy(&hc, h->ctl, sizeof(hc), cudaMemcpyDeviceToHost);
+  hc.tau = I.tau; hc.theta = I.theta; hc.kappa = I.kappa; hc.mu = I.mu;
+  hc.admm_iters = I.admm_iters; hc.cg_iters = 0; hc.outer_iters = I.outer_iters; hc.status = I.status;
+  hc.pres = I.pres; hc.dres = I.dres; hc.dgap = I.dgap; hc.ctx = I.ctx; hc.bty = I.bty;
+  hc.err = I.err;
+  if (e == cudaSuccess) e = cudaMemcpy(h->ctl, &hc, sizeof(hc), cudaMemcpyHostToDevice);
+  if (e != cudaSuccess) return fail(h, ABIP_E_CUDA, std::string("solve results: ") + cudaGetErrorString(e));
   return ABIP_OK;
 }
 
@@ -955,6 +1083,7 @@ int abip_setup(const abip_matrix* A, const double* b, const double* c, const abi
       } else {
         const std::vector<double> lx0 = abip::ldl_host::initial_values(hA, sym);
         rc = setup_grid_path(h, h->gd64, hA, hb, hc, !f32, abip::grid_solver_max_ctas(!f32, h->device), &sym, &lx0);
+        if (rc == ABIP_OK) setup_direct(h, hA);
       }
     } else if (rc == ABIP_OK) {
       if (h->mixed)   // FP32 values: exact for float input, rounded for double input (FP64 refreshes see them)
@@ -975,7 +1104,7 @@ int abip_setup(const abip_matrix* A, const double* b, const double* c, const abi
                  abip::plan_dense_group(&m, &n, 1, abip::dense_max_ctas(h->device), h->gplan) != 0;
       if (rc == ABIP_OK) {
         rc = dense_alloc(h, hi, &h->arena, &h->dinst, &h->queue, hd, h->mixed != 0, prm.bb_beta != 0, h->group);
-        if (rc == ABIP_E_OOM && h->group) {   // without the group's copies of A^T and G^{-1}
+        if (rc == ABIP_E_OOM && h->group) {   // without the group's copies of A^T and the factor's inverse
           h->group = false;
           rc = dense_alloc(h, hi, &h->arena, &h->dinst, &h->queue, hd, false, false, false);
         }
@@ -1016,7 +1145,7 @@ int abip_solve(abip_handle* h, double* x, double* y, double* s, abip_info* info,
   int rc;
   abip_info inf{};
   if (h->path == 0) {
-    rc = solve_grid_path(h, st);
+    rc = h->group ? solve_direct(h, st) : solve_grid_path(h, st);
     if (rc) return rc;
     SolveCtl hc;
     cudaMemcpy(&hc, h->ctl, sizeof(hc), cudaMemcpyDeviceToHost);
@@ -1030,13 +1159,15 @@ int abip_solve(abip_handle* h, double* x, double* y, double* s, abip_info* info,
     if (hc.status == ABIP_PRIMAL_INFEASIBLE) { sx = 1.0; sy = 1.0 / hc.bty; }
     if (hc.status == ABIP_DUAL_INFEASIBLE) { sx = -1.0 / hc.ctx; sy = 1.0; }
     double* stage = h->stage;
-    const double* gx = h->mixed ? h->gdd.x : h->gd64.x;
-    const double* gy = h->mixed ? h->gdd.y : h->gd64.y;
-    const double* gs = h->mixed ? h->gdd.s : h->gd64.s;
-    output_kernel<double><<<128, 256, 0, st>>>(gx, n, sx, stage);
-    output_kernel<double><<<128, 256, 0, st>>>(gy, m, sy, stage + n);
-    output_kernel<double><<<128, 256, 0, st>>>(gs, n, sy, stage + n + m);
-    h->launches += 3;
+    if (!h->group) {   // the group kernel has written the scaled outputs
+      const double* gx = h->mixed ? h->gdd.x : h->gd64.x;
+      const double* gy = h->mixed ? h->gdd.y : h->gd64.y;
+      const double* gs = h->mixed ? h->gdd.s : h->gd64.s;
+      output_kernel<double><<<128, 256, 0, st>>>(gx, n, sx, stage);
+      output_kernel<double><<<128, 256, 0, st>>>(gy, m, sy, stage + n);
+      output_kernel<double><<<128, 256, 0, st>>>(gs, n, sy, stage + n + m);
+      h->launches += 3;
+    }
     rc = copy_out(h, x, stage, n, st);
     if (!rc) rc = copy_out(h, y, stage + n, m, st);
     if (!rc) rc = copy_out(h, s, stage + n + m, n, st);
@@ -1134,7 +1265,7 @@ int abip_solve_batch(int32_t count, const abip_matrix* A, const double* const* b
   }
   tmp.prm = prm;
   int rc = dense_alloc(&tmp, hi, &arena, &dinst, &queue, hd, mixed, prm.bb_beta != 0, tmp.group);
-  if (rc == ABIP_E_OOM && tmp.group) {   // without the group's copies of A^T and G^{-1}
+  if (rc == ABIP_E_OOM && tmp.group) {   // without the group's copies of A^T and the factor's inverse
     tmp.group = false;
     rc = dense_alloc(&tmp, hi, &arena, &dinst, &queue, hd, mixed, false, false);
   }
@@ -1453,6 +1584,7 @@ int abip_set_state(abip_handle* h, const double* buf) {
 void abip_free(abip_handle* h) {
   if (!h) return;
   if (h->arena) cudaFree(h->arena);
+  if (h->arena2) cudaFree(h->arena2);
   if (h->ev0) cudaEventDestroy(h->ev0);
   if (h->ev1) cudaEventDestroy(h->ev1);
   delete h;

@@ -198,9 +198,9 @@ struct DenseInst {
   // mixed precision (null on the FP64 path): FP32 A (rows padded to ldf), FP32 A^T
   // (rows padded to ldtf) and the FP32 explicit inverse of G = I + A A^T (m x ldtf)
   const float* Af; const float* ATf; float* Ginvf;
-  // FP64 path by a group of CTAs (null elsewhere): A^T (n rows) and the explicit inverse of G
-  // (m rows), rows padded with zeros to an even length; A's ld is even then
-  double* AT; double* Ginv;
+  // FP64 path by a group of CTAs (null elsewhere): A^T (n rows), L^{-1} and L^{-T} (m rows
+  // each), rows padded with zeros to an even length; A's ld is even then
+  double* AT; double* Li; double* LiT;
   double zbar, nb, nc;
   double Kinv[4];
   // results
@@ -254,13 +254,22 @@ struct DenseParams {
 // global scratch of the Barzilai-Borwein selection per instance (DenseInst::work)
 inline size_t bb_work_doubles(int m, int n) { return 4 * (size_t)m + 6 * (size_t)n; }
 
-// Gram and Cholesky factor of every instance (L), over the SMs; mmax: the largest m
+// A by rows (rp, ci, va) and by columns (cp, ri, cv), device arrays, FP64 values, no duplicate
+// entries; room_a, room_at: most entries of one CTA's rows and columns.
+struct GroupSparse {
+  const int32_t* rp = nullptr; const int32_t* ci = nullptr; const double* va = nullptr;
+  const int32_t* cp = nullptr; const int32_t* ri = nullptr; const double* cv = nullptr;
+  int room_a = 0, room_at = 0;
+};
+// Gram and Cholesky factor of every instance (L), over the SMs; mmax: the largest m.  The
+// sparse form takes G = I + A A^T of one instance from A by rows and columns (L zeroed).
+cudaError_t launch_sparse_factor(DenseInst* inst, int m, const GroupSparse& sp, int sms, cudaStream_t st);
 cudaError_t launch_dense_factor(DenseInst* inst, int count, int mmax, int sms, cudaStream_t st);
-// the explicit inverse of G (FP32 Ginvf or FP64 Ginv, where not null) of every instance, from L
+// from L of every instance: the explicit inverse of G (FP32, Ginvf), or L^{-1} and L^{-T} (Li, LiT)
 cudaError_t launch_dense_inverse(DenseInst* inst, int count, int mmax, int sms, cudaStream_t st);
 // A^T of every instance (AT)
 cudaError_t launch_dense_transpose(DenseInst* inst, int count, int mmax, int nmax, int sms, cudaStream_t st);
-// the whole setup: factor, embedding constants and M^{-1} H and, when `inverse`, G's inverse;
+// the whole setup: factor, embedding constants and M^{-1} H and, when `inverse`, the inverse;
 // nmax > 0: also AT
 cudaError_t launch_dense_setup(DenseInst* inst, int count, int* queue, int grid, size_t smem, int mmax, int nmax,
                                bool inverse, cudaStream_t st);
@@ -271,15 +280,22 @@ struct DenseGroupPlan {
   int grid_mode;             // 1: one instance over a cooperative grid
   int cache_vec, cache_mat;  // shared-memory copies of the vectors and matrix rows a CTA reads
   size_t smem;
+  int sparse;                // 1: products with A over its CSR rows and columns (GroupSparse)
 };
 // the plan for a batch (sizes m[k], n[k]); 0 if no group holds its vectors in shared memory
 int plan_dense_group(const int* m, const int* n, int count, int sms, DenseGroupPlan& plan);
+// Rows up to which the sparse direct projection forms L^{-1}: m^2 multiply-adds over the SMs per
+// update against two sweeps along the elimination tree at about 2.8 us per dependent link
+// (grid flow, us per update, sweeps / inverse: m = 255 309 / 15, 1023 631 / 30, 1599 903 / 38), and a setup that grows by m^3 / 3 multiply-adds (1599: 24 ms more).
+constexpr int kDirectMaxRows = 1600;
+// the plan for one sparse LP (host rp, cp); 0 where the sweeps serve it
+int plan_sparse_group(int m, int n, const int32_t* rp, const int32_t* cp, int sms, GroupSparse& sp, DenseGroupPlan& plan);
 // doubles of scratch of the grid mode; its last two are the barrier counter and the error
 // word, zeroed by the caller before each launch
 size_t dense_group_scratch(int m, int n, int sms);
 cudaError_t launch_dense_group(DenseInst* inst, int count, const DenseParams& prm, int* queue, const int* order,
-                               const DenseGroupPlan& plan, int variant, double* scratch, size_t scratch_len,
-                               unsigned long long limit_ns, cudaStream_t st);
+                               const DenseGroupPlan& plan, const GroupSparse& sp, int variant, double* scratch,
+                               size_t scratch_len, unsigned long long limit_ns, cudaStream_t st);
 int dense_group_ctas_per_sm(const DenseGroupPlan& plan, int variant);
 // Occupancy variants of the dense solve kernel (the batch autotuner's choice)
 constexpr int kDenseVariants = 3;
@@ -380,6 +396,9 @@ struct abip_handle {
   abip::DenseGroupPlan gplan{};
   double* gscratch = nullptr;         // its grid mode's scratch, gscratch_len doubles
   size_t gscratch_len = 0;
+  // sparse direct projection of an LP with few rows: path 0 with group set, its own arena
+  abip::GroupSparse gsp;
+  void* arena2 = nullptr;
   int* queue = nullptr;
   abip::DenseInst hinst{};            // host mirror of the descriptor
   double nb = 0, nc = 0;

@@ -4,11 +4,14 @@
 // What bounds it: the FP64 pipe, 2 FMA per clock and SM on this part, so an LP on one SM pays
 // its 3 m n + m^2 multiply-adds per update at 1/152 of the chip; and, for a small LP, the chain
 // of dependent phases.  Hence
-//  * the rows of A and G^{-1} and the columns of A (rows of the stored A^T) are dealt out to the
-//    CTAs of the group; every CTA keeps the vectors q, z_y, x and s whole in shared memory and
-//    publishes its part of each (distributed shared memory in a cluster, L2 in a grid);
-//  * z_y = G^{-1} q is one product with the explicit inverse instead of two triangular sweeps of
-//    m / 32 serial blocks (lambda_min(G) >= 1, so its error bound is that of the sweeps);
+//  * the rows of A and of the factor's inverse and the columns of A (rows of the stored A^T)
+//    are dealt out to the CTAs of the group; every CTA keeps the vectors q, t, z_y, x and s
+//    whole in shared memory and publishes its part of each (distributed shared memory in a
+//    cluster, L2 in a grid);
+//  * z_y = G^{-1} q is two products, t = L^{-1} q and z_y = L^{-T} t, with the inverse of the
+//    factor formed at setup, instead of two sweeps of m / 32 serial blocks.  One product with
+//    G^{-1} itself would save a barrier, but its error is larger than the sweeps' (x of a 512 x
+//    1154 L1-SVM after 60 updates, relative: sweeps 5.0e-14, G^{-1} 6.1e-13, this 3.7e-14);
 //  * A^T y follows from the update's linearity, y <- alpha u_y + (1 - alpha) y, whose error does
 //    not grow (|1 - alpha| < 1) and which only the tests of Sec. 4.1 read: three products with
 //    the entries of A per update instead of four;
@@ -16,7 +19,9 @@
 //    for 8 sums where butterflies take 40 -- a warp-wide FP64 addition costs 16 clocks here;
 //  * what a CTA reads every update (its rows of the matrices and of the vectors) is copied to
 //    shared memory when it fits.
-// One update has four barriers of the group: z_y | H^T z | x, s | products and test sums.
+// The same kernel serves the sparse direct projection of an LP with few rows (SPARSE): the
+// products with A run over its CSR rows and columns, L^{-1} stays dense.
+// One update has five barriers of the group: t | z_y | H^T z | x, s | products and test sums.
 // Measured, us per update, one CTA with triangular sweeps -> this kernel: 50 x 120 76.9 -> 11.1
 // (the chain of phases: 16 x 48 takes 10.0), 512 x 1154 1564 -> 26.4, the slowest of 64 LPs of
 // m 16 .. 256 621 -> 65.
@@ -105,6 +110,51 @@ __device__ __forceinline__ void dots_any(const double* M, int64_t ld, int rows, 
   else dots<1, NV>(M, ld, rows, v0, v1, out);
 }
 
+// out(k, sum_j M[k][j] v[j]) for the CTA's rows k < rows of a triangular M, row k being row
+// rank + size k of the matrix at M + k * stride: dealt out in turn, since the rows grow (LOWER)
+// or shrink in length.  Only the triangle is read, in pairs of columns and to the longest of
+// the R rows that a warp has at once (the entries beyond are stored zeros).
+template <int R, bool LOWER, typename F>
+__device__ __forceinline__ void tri_dots(const double* M, int64_t stride, int rows, int rank, int size, int nq,
+                                         const double* v, F out) {
+  constexpr int kShift = R == 8 ? 2 : R == 4 ? 3 : R == 2 ? 4 : 5;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  for (int g = wid * R; g < rows; g += kWarps * R) {
+    double a[R];
+    const double2* r[R];
+#pragma unroll
+    for (int u = 0; u < R; ++u) {
+      a[u] = 0.0;
+      r[u] = reinterpret_cast<const double2*>(M + (size_t)min(g + u, rows - 1) * stride);
+    }
+    const int t0 = LOWER ? 0 : (rank + size * g) >> 1;
+    const int t1 = LOWER ? ((rank + size * min(g + R - 1, rows - 1)) >> 1) + 1 : nq;
+#pragma unroll(R >= 4 ? 1 : 4)
+    for (int t = t0 + lane; t < t1; t += 32) {
+      const double2 x = reinterpret_cast<const double2*>(v)[t];
+#pragma unroll
+      for (int u = 0; u < R; ++u) {
+        const double2 w = r[u][t];
+        a[u] += w.x * x.x;
+        a[u] += w.y * x.y;
+      }
+    }
+    const double d = sum_together<R>(a, lane);
+    if ((lane & ((1 << kShift) - 1)) == 0) {
+      const int u = lane >> kShift;
+      if (g + u < rows) out(g + u, d);
+    }
+  }
+}
+template <bool LOWER, typename F>
+__device__ __forceinline__ void tri_any(const double* M, int64_t stride, int rows, int rank, int size, int nq,
+                                        const double* v, F out) {
+  if (rows > 4 * kWarps) tri_dots<8, LOWER>(M, stride, rows, rank, size, nq, v, out);
+  else if (rows > 2 * kWarps) tri_dots<4, LOWER>(M, stride, rows, rank, size, nq, v, out);
+  else if (rows > kWarps) tri_dots<2, LOWER>(M, stride, rows, rank, size, nq, v, out);
+  else tri_dots<1, LOWER>(M, stride, rows, rank, size, nq, v, out);
+}
+
 // The group of CTAs that solves an LP: a cluster (GRID = false) or the cooperative grid.
 template <bool GRID>
 struct Group {
@@ -150,7 +200,8 @@ struct GroupArgs {
   int* queue;
   const int* order;
   int cache_vec, cache_mat;       // copies in shared memory: the CTA's vectors, its matrix rows
-  // grid mode: published vectors (q, z_y: ldt each; x, s: ld each), partial sums, barrier
+  GroupSparse sp;                 // SPARSE: A by rows and by columns
+  // grid mode: published vectors (q, t, z_y: even(m) each; x, s: even(n) each), partial sums, barrier
   double* gvec;
   double* gpart;                  // (kSums + 2) * grid
   unsigned long long* bar;
@@ -221,8 +272,43 @@ __device__ __forceinline__ void total_sums(const Group<GRID>& G, const double* s
 
 __device__ __forceinline__ int even(int k) { return (k + 1) & ~1; }
 
+// rp, ci, va: CSR rows (of the CTA).  out(which, i, sum_j A_ij v_which[j]) for i < rows, eight
+// lanes per row (the sums of the rows of a grid flow LP's incidence matrix are 4 to 8 long).
+template <typename F>
+__device__ __forceinline__ void sparse_rows2(const int32_t* rp, const int32_t* ci, const double* va, int rows,
+                                             const double* v0, const double* v1, F out) {
+  const int sub = threadIdx.x & 7;
+  const int per = kThr / 8, n8 = (rows + per - 1) / per * per;   // whole warps enter the shuffles
+  for (int i = threadIdx.x >> 3; i < n8; i += per) {
+    double a0 = 0.0, a1 = 0.0;
+    if (i < rows)
+      for (int e = rp[i] + sub; e < rp[i + 1]; e += 8) {
+        const double a = va[e];
+        const int j = ci[e];
+        a0 += a * v0[j];
+        a1 += a * v1[j];
+      }
+    // the two sums together: lanes 0-3 carry a0, 4-7 a1
+    const double send = sub < 4 ? a1 : a0, keep = sub < 4 ? a0 : a1;
+    double v = keep + __shfl_xor_sync(0xffffffffu, send, 4);
+    v += __shfl_xor_sync(0xffffffffu, v, 2);
+    v += __shfl_xor_sync(0xffffffffu, v, 1);
+    if (i < rows && (sub & 3) == 0) out(sub >> 2, i, v);
+  }
+}
+// out(j, sum_i A_ij v[i]) for the CTA's columns, a thread per column
+template <typename F>
+__device__ __forceinline__ void sparse_cols(const int32_t* cp, const int32_t* ri, const double* cv, int cols,
+                                            const double* v, F out) {
+  for (int j = threadIdx.x; j < cols; j += kThr) {
+    double a = 0.0;
+    for (int e = cp[j]; e < cp[j + 1]; ++e) a += cv[e] * v[ri[e]];
+    out(j, a);
+  }
+}
+
 // Algorithm 2 (with the relaxation of Sec. 4.2) for one instance by the group.
-template <bool GRID>
+template <bool GRID, bool SPARSE>
 __device__ void solve_one(DenseInst& I, const GroupArgs& Q, Group<GRID>& G, double* sm, double* wsum, Scal& S) {
   const DenseParams& P = Q.P;
   const int m = I.m, n = I.n, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -231,7 +317,8 @@ __device__ void solve_one(DenseInst& I, const GroupArgs& Q, Group<GRID>& G, doub
   const int i0 = min(m, G.rank * mc), mr = min(m, i0 + mc) - i0;   // this CTA's rows
   const int j0 = min(n, G.rank * nc_), nr = min(n, j0 + nc_) - j0; // this CTA's columns
   double* q = sm;
-  double* zy = q + mp;
+  double* tv = q + mp;
+  double* zy = tv + mp;
   double* x = zy + mp;
   double* s = x + np;
   double* hslot = s + np;                               // 2 * size
@@ -243,7 +330,8 @@ __device__ void solve_one(DenseInst& I, const GroupArgs& Q, Group<GRID>& G, doub
   double* v = aty + nc_;
   double* top = v + nc_;
   double* gq = Q.gvec;
-  double* gzy = gq + mp;
+  double* gtv = gq + mp;
+  double* gzy = gtv + mp;
   double* gx = gzy + mp;
   double* gs = gx + np;
   double* ghs = Q.gpart;
@@ -256,9 +344,17 @@ __device__ void solve_one(DenseInst& I, const GroupArgs& Q, Group<GRID>& G, doub
   const double* cbar = I.cbar + j0;
   const double* g1x = I.g1 + m + j0;
   const double* g2x = I.g2 + m + j0;
-  const double* Ar = I.A + (size_t)i0 * I.ld;
-  const double* ATr = I.AT + (size_t)j0 * mp;
-  const double* Gr = I.Ginv + (size_t)i0 * mp;
+  const double* Ar = SPARSE ? nullptr : I.A + (size_t)i0 * I.ld;
+  const double* ATr = SPARSE ? nullptr : I.AT + (size_t)j0 * mp;
+  const int32_t* rp = SPARSE ? Q.sp.rp + i0 : nullptr;   // entries [rp[i], rp[i + 1]) of ci, va
+  const int32_t* cp = SPARSE ? Q.sp.cp + j0 : nullptr;
+  const int32_t *ci = Q.sp.ci, *ri = Q.sp.ri;
+  const double *va = Q.sp.va, *cv = Q.sp.cv;
+  // L^{-1} and L^{-T}: rows rank, rank + size, ...
+  const int tr = G.rank < m ? (m - G.rank + G.size - 1) / G.size : 0;
+  int64_t tstride = (int64_t)G.size * mp;
+  const double* Lr = I.Li + (size_t)min(G.rank, m - 1) * mp;
+  const double* Ur = I.LiT + (size_t)min(G.rank, m - 1) * mp;
   if (Q.cache_vec) {
     double* d = top;
     auto copy = [&](const double*& src, int len, int room) {
@@ -272,12 +368,29 @@ __device__ void solve_one(DenseInst& I, const GroupArgs& Q, Group<GRID>& G, doub
   }
   if (Q.cache_mat) {
     double* d = top;
-    auto copy = [&](const double*& src, int rows, int64_t ld, int room) {
-      for (int64_t e = threadIdx.x; e < rows * ld; e += kThr) d[e] = src[e];
+    auto copy = [&](const double*& src, int rows, int ld, int64_t stride, int room) {
+      for (int e = threadIdx.x; e < rows * ld; e += kThr) d[e] = src[(int64_t)(e / ld) * stride + e % ld];
       src = d;
       d += room * ld;
     };
-    copy(Ar, mr, np, mc); copy(ATr, nr, mp, nc_); copy(Gr, mr, mp, mc);
+    if constexpr (!SPARSE) { copy(Ar, mr, np, np, mc); copy(ATr, nr, mp, mp, nc_); }
+    copy(Lr, tr, mp, tstride, mc);
+    copy(Ur, tr, mp, tstride, mc);
+    tstride = mp;
+    if constexpr (SPARSE) {
+      // the CTA's entries, offsets shifted to the copies
+      auto entries = [&](const int32_t*& ptr, const int32_t*& idx, const double*& val, int rows, int room, int prow) {
+        const int e0 = ptr[0], len = ptr[rows] - e0;
+        int32_t* di = reinterpret_cast<int32_t*>(d + room);
+        int32_t* dp = di + room;
+        for (int e = threadIdx.x; e < len; e += kThr) { d[e] = val[e0 + e]; di[e] = idx[e0 + e]; }
+        for (int r = threadIdx.x; r <= rows; r += kThr) dp[r] = ptr[r] - e0;
+        val = d; idx = di; ptr = dp;
+        d += room + (room + prow + 1 + 1) / 2;
+      };
+      entries(rp, ci, va, mr, Q.sp.room_a, mc);
+      entries(cp, ri, cv, nr, Q.sp.room_at, nc_);
+    }
   }
   const double alpha = P.alpha, eps = P.eps, a1 = 1.0 - alpha;
   const double zbar = I.zbar, xi = -(double)n - 1.0, nb = I.nb, nc = I.nc;
@@ -289,6 +402,7 @@ __device__ void solve_one(DenseInst& I, const GroupArgs& Q, Group<GRID>& G, doub
   const bool resume = I.resume != 0;
   for (int i = threadIdx.x; i < mp; i += kThr) {
     q[i] = 0.0;
+    tv[i] = 0.0;
     zy[i] = (resume && i < m) ? I.y[i] : 0.0;
   }
   for (int j = threadIdx.x; j < np; j += kThr) {
@@ -310,7 +424,8 @@ __device__ void solve_one(DenseInst& I, const GroupArgs& Q, Group<GRID>& G, doub
   }
   __syncthreads();
   if (resume) {   // A^T y of the loaded state, once (z_y's buffer holds y)
-    dots_any<1>(ATr, mp, nr, zy, zy, [&](int, int j, double d) { aty[j] = d; });
+    if constexpr (SPARSE) sparse_cols(cp, ri, cv, nr, zy, [&](int j, double d) { aty[j] = d; });
+    else dots_any<1>(ATr, mp, nr, zy, zy, [&](int, int j, double d) { aty[j] = d; });
     __syncthreads();
     for (int i = threadIdx.x; i < mp; i += kThr) zy[i] = 0.0;
   }
@@ -319,7 +434,8 @@ __device__ void solve_one(DenseInst& I, const GroupArgs& Q, Group<GRID>& G, doub
   if (!G.sync()) return;   // nobody publishes into a CTA that is still filling its copies
   for (;;) {
     // ---- products of the state, its test sums (residual_sums' order of quantities), and q
-    dots_any<2>(Ar, np, mr, x, s, [&](int w, int i, double d) { (w == 0 ? Ax : As)[i] = d; });
+    if constexpr (SPARSE) sparse_rows2(rp, ci, va, mr, x, s, [&](int w, int i, double d) { (w == 0 ? Ax : As)[i] = d; });
+    else dots_any<2>(Ar, np, mr, x, s, [&](int w, int i, double d) { (w == 0 ? Ax : As)[i] = d; });
     __syncthreads();
     {
       double acc[16];
@@ -423,11 +539,16 @@ __device__ void solve_one(DenseInst& I, const GroupArgs& Q, Group<GRID>& G, doub
     }
     first = false;
     // ---- projection: z_y = G^{-1} (y - A (x + s)), z_x = x + s + A^T z_y, H^T z
-    dots_any<1>(Gr, mp, mr, q, q, [&](int, int i, double d) { G.put(zy, gzy, i0 + i, d); });
+    tri_any<true>(Lr, tstride, tr, G.rank, G.size, mp >> 1, q, [&](int k, double d) { G.put(tv, gtv, G.rank + G.size * k, d); });
+    if (!G.sync()) return;
+    G.fetch(tv, gtv, m);
+    if constexpr (GRID) __syncthreads();
+    tri_any<false>(Ur, tstride, tr, G.rank, G.size, mp >> 1, tv, [&](int k, double d) { G.put(zy, gzy, G.rank + G.size * k, d); });
     if (!G.sync()) return;
     G.fetch(zy, gzy, m);
     if constexpr (GRID) __syncthreads();
-    dots_any<1>(ATr, mp, nr, zy, zy, [&](int, int j, double d) { v[j] = d; });
+    if constexpr (SPARSE) sparse_cols(cp, ri, cv, nr, zy, [&](int j, double d) { v[j] = d; });
+    else dots_any<1>(ATr, mp, nr, zy, zy, [&](int, int j, double d) { v[j] = d; });
     __syncthreads();
     {
       double acc[2] = {0.0, 0.0};
@@ -524,7 +645,7 @@ __device__ void solve_one(DenseInst& I, const GroupArgs& Q, Group<GRID>& G, doub
   }
 }
 
-template <int MINB>
+template <int MINB, bool SPARSE>
 __global__ void __launch_bounds__(kThr, MINB) dense_cluster_kernel(GroupArgs Q) {
   extern __shared__ __align__(16) double sm[];
   __shared__ double wsum[kSums * kWarps];
@@ -542,23 +663,27 @@ __global__ void __launch_bounds__(kThr, MINB) dense_cluster_kernel(GroupArgs Q) 
     const int id = s_id;
     if (id < 0) return;   // the same in every CTA, after which none writes to another
     DenseInst& I = Q.insts[id];
-    if (I.err == 0) solve_one<false>(I, Q, G, sm, wsum, S);
+    if (I.err == 0) solve_one<false, SPARSE>(I, Q, G, sm, wsum, S);
     cl.sync();            // every CTA has read s_id and its copies
   }
 }
 
+template <bool SPARSE>
 __global__ void __launch_bounds__(kThr, 1) dense_grid_kernel(GroupArgs Q) {
   extern __shared__ __align__(16) double sm[];
   __shared__ double wsum[kSums * kWarps];
   __shared__ Scal S;
   Group<true> G(GridBarrier{Q.bar, Q.err, Q.bar_limit_ns});
-  if (Q.insts[0].err == 0) solve_one<true>(Q.insts[0], Q, G, sm, wsum, S);
+  if (Q.insts[0].err == 0) solve_one<true, SPARSE>(Q.insts[0], Q, G, sm, wsum, S);
 }
 
 using ClusterFn = void (*)(GroupArgs);
-ClusterFn cluster_fn(int variant) {
-  return variant == 2 ? dense_cluster_kernel<3> : variant == 1 ? dense_cluster_kernel<2> : dense_cluster_kernel<1>;
+ClusterFn cluster_fn(int variant, bool sparse) {
+  if (sparse) return dense_cluster_kernel<1, true>;
+  return variant == 2 ? dense_cluster_kernel<3, false> : variant == 1 ? dense_cluster_kernel<2, false>
+                                                                      : dense_cluster_kernel<1, false>;
 }
+ClusterFn grid_fn(bool sparse) { return sparse ? dense_grid_kernel<true> : dense_grid_kernel<false>; }
 
 struct SmemPlan {
   size_t bytes;
@@ -567,22 +692,28 @@ struct SmemPlan {
 
 size_t base_doubles(int m, int n, int C, bool grid) {
   const size_t mp = (m + 1) / 2 * 2, np = (n + 1) / 2 * 2, mc = (m + C - 1) / C, nc = (n + C - 1) / C;
-  return 2 * mp + 2 * np + (2 + kSums) * (size_t)(grid ? 1 : C) + 3 * mc + 2 * nc;
+  return 3 * mp + 2 * np + (2 + kSums) * (size_t)(grid ? 1 : C) + 3 * mc + 2 * nc;
 }
 size_t vec_doubles(int m, int n, int C) { return 4 * (size_t)((m + C - 1) / C) + 4 * (size_t)((n + C - 1) / C) + 2; }
 size_t mat_doubles(int m, int n, int C) {
   const size_t mp = (m + 1) / 2 * 2, np = (n + 1) / 2 * 2, mc = (m + C - 1) / C, nc = (n + C - 1) / C;
-  return mc * (np + mp) + nc * mp + 2;
+  return mc * (np + 2 * mp) + nc * mp + 2;
+}
+
+size_t sparse_doubles(int m, int n, int C, int room_a, int room_at) {
+  const size_t mp = (m + 1) / 2 * 2, mc = (m + C - 1) / C, nc = (n + C - 1) / C;
+  return 2 * mc * mp + 2 + room_a + (room_a + mc + 2) / 2 + room_at + (room_at + nc + 2) / 2;
 }
 
 // the shared memory of a launch for the given sizes: the copies that fit the budget
-SmemPlan plan_smem(const int* m, const int* n, int count, int C, bool grid, size_t budget) {
+SmemPlan plan_smem(const int* m, const int* n, int count, int C, bool grid, size_t budget,
+                   const GroupSparse* sp = nullptr) {
   size_t base = 0, vec = 0, mat = 0;
   for (int k = 0; k < count; ++k) {
     const size_t b = base_doubles(m[k], n[k], C, grid), v = b + vec_doubles(m[k], n[k], C);
     base = std::max(base, b);
     vec = std::max(vec, v);
-    mat = std::max(mat, v + mat_doubles(m[k], n[k], C));
+    mat = std::max(mat, v + (sp ? sparse_doubles(m[k], n[k], C, sp->room_a, sp->room_at) : mat_doubles(m[k], n[k], C)));
   }
   SmemPlan p{base * 8 + 16, 0, 0};
   if (vec * 8 <= budget) { p.bytes = vec * 8 + 16; p.cache_vec = 1; }
@@ -647,29 +778,62 @@ int plan_dense_group(const int* m, const int* n, int count, int sms, DenseGroupP
   }
 }
 
+namespace {
+// most entries a CTA's share of the rows holds: ptr (len + 1) in shares of ceil(len / C) rows
+int share_room(const int32_t* ptr, int len, int C) {
+  const int per = (len + C - 1) / C;
+  int most = 0;
+  for (int r = 0; r < len; r += per) most = std::max(most, ptr[std::min(len, r + per)] - ptr[r]);
+  return most;
+}
+}  // namespace
+
+int plan_sparse_group(int m, int n, const int32_t* rp, const int32_t* cp, int sms, GroupSparse& sp, DenseGroupPlan& plan) {
+  plan = DenseGroupPlan{};
+  plan.sparse = 1;
+  if (m > kDirectMaxRows) return 0;
+  const int64_t w = 3 * (int64_t)rp[m] + (int64_t)m * m + 80 * (int64_t)(m + n);
+  plan.grid_mode = w > 800000;   // as for a dense LP
+  int C = 1;
+  while (C < 16 && w / C > 5000) C *= 2;
+  if (plan.grid_mode) C = sms;
+  for (;; C *= 2) {
+    sp.room_a = share_room(rp, m, C);
+    sp.room_at = share_room(cp, n, C);
+    const SmemPlan s = plan_smem(&m, &n, 1, C, plan.grid_mode != 0, kSmemMax - 16, &sp);
+    plan.ctas = C;
+    plan.smem = s.bytes;
+    plan.cache_vec = s.cache_vec;
+    plan.cache_mat = s.cache_mat;
+    if (s.bytes <= kSmemMax) return 1;
+    if (C >= 8) return 0;
+  }
+}
+
 size_t dense_group_scratch(int m, int n, int sms) {
   const size_t mp = (m + 1) / 2 * 2, np = (n + 1) / 2 * 2;
-  return 2 * mp + 2 * np + (size_t)(kSums + 2) * sms + 4;
+  return 3 * mp + 2 * np + (size_t)(kSums + 2) * sms + 4;
 }
 
 cudaError_t launch_dense_group(DenseInst* inst, int count, const DenseParams& prm, int* queue, const int* order,
-                               const DenseGroupPlan& plan, int variant, double* scratch, size_t scratch_len,
-                               unsigned long long limit_ns, cudaStream_t st) {
-  GroupArgs Q{inst, count, prm, queue, order, plan.cache_vec, plan.cache_mat, nullptr, nullptr, nullptr, nullptr, limit_ns};
+                               const DenseGroupPlan& plan, const GroupSparse& sp, int variant, double* scratch,
+                               size_t scratch_len, unsigned long long limit_ns, cudaStream_t st) {
+  GroupArgs Q{inst, count, prm, queue, order, plan.cache_vec, plan.cache_mat, sp, nullptr, nullptr, nullptr, nullptr, limit_ns};
   if (plan.grid_mode) {
     // barrier counter and error word at the end of the scratch, zeroed by the caller
     Q.bar = reinterpret_cast<unsigned long long*>(scratch + scratch_len - 2);
     Q.err = reinterpret_cast<int*>(scratch + scratch_len - 1);
     Q.gpart = scratch;
     Q.gvec = scratch + (size_t)(kSums + 2) * plan.ctas + ((kSums + 2) * (size_t)plan.ctas & 1);
-    cudaError_t e = cudaFuncSetAttribute(dense_grid_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
+    const ClusterFn f = grid_fn(plan.sparse != 0);
+    cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
     if (e != cudaSuccess) return e;
     void* args[] = {&Q};
-    return cudaLaunchCooperativeKernel((const void*)dense_grid_kernel, dim3(plan.ctas), dim3(kThr), args, plan.smem, st);
+    return cudaLaunchCooperativeKernel((const void*)f, dim3(plan.ctas), dim3(kThr), args, plan.smem, st);
   }
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute at[1];
-  ClusterFn f = cluster_fn(variant);
+  ClusterFn f = cluster_fn(variant, plan.sparse != 0);
   cudaError_t e = cluster_config(f, plan.ctas, plan.smem, cfg, at);
   if (e != cudaSuccess) return e;
   int ncl = 0;
@@ -684,11 +848,11 @@ cudaError_t launch_dense_group(DenseInst* inst, int count, const DenseParams& pr
 int dense_group_ctas_per_sm(const DenseGroupPlan& plan, int variant) {
   int per = 0;
   if (plan.grid_mode) {
-    cudaFuncSetAttribute(dense_grid_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, dense_grid_kernel, kThr, plan.smem);
+    cudaFuncSetAttribute(grid_fn(false), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, grid_fn(false), kThr, plan.smem);
     return per;
   }
-  ClusterFn f = cluster_fn(variant);
+  ClusterFn f = cluster_fn(variant, false);
   cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, f, kThr, plan.smem);
   return per;

@@ -1,6 +1,6 @@
 // Setup of the dense path spread over the SMs: G = I + A A^T (Sec. 4.4) by output tiles,
-// its Cholesky factor by a thread-block cluster per instance, and the FP32 explicit inverse
-// of the mixed-precision path by column tiles.
+// its Cholesky factor by a thread-block cluster per instance, and by column tiles the FP32
+// explicit inverse of the mixed-precision path or the inverse of the factor of the FP64 path.
 //
 // What bounds it: the FP64 pipe (2 FMA per clock and SM).  A Gram of 512 x 1154 is 151 MFMA:
 // 36 ms on one SM, 0.3 ms on 136 tiles over the SMs.  Every value is formed by the operations
@@ -67,6 +67,26 @@ __global__ void __launch_bounds__(kThr) gram_tiles_kernel(const DenseInst* __res
       const int gi = bi * 32 + tr * 4 + q, gk = bk * 32 + tc;
       if (gi < m && gk <= gi) I.L[(size_t)gi * m + gk] = acc[q] + (gi == gk ? 1.0 : 0.0);
     }
+  }
+}
+
+// G of a sparse A, lower triangle of the zeroed L: a warp per row i, over the entries (i, j) of
+// the row in order, its lanes over the entries (k, j) of column j (k distinct: no duplicates)
+__global__ void __launch_bounds__(kThr) gram_sparse_kernel(const DenseInst* __restrict__ inst, GroupSparse sp) {
+  const int m = inst->m, lane = threadIdx.x & 31;
+  for (int i = blockIdx.x * (kThr / 32) + (threadIdx.x >> 5); i < m; i += gridDim.x * (kThr / 32)) {
+    double* row = inst->L + (size_t)i * m;
+    for (int e = sp.rp[i]; e < sp.rp[i + 1]; ++e) {
+      const int j = sp.ci[e];
+      const double a = sp.va[e];
+      for (int t = sp.cp[j] + lane; t < sp.cp[j + 1]; t += 32) {
+        const int k = sp.ri[t];
+        if (k <= i) row[k] += a * sp.cv[t];
+      }
+      __syncwarp();
+    }
+    if (lane == 0) row[i] += 1.0;
+    __syncwarp();
   }
 }
 
@@ -195,7 +215,7 @@ __global__ void __launch_bounds__(kThr) chol_cluster_kernel(DenseInst* insts, in
 }
 
 // ---------------------------------------------------------------------------
-// Explicit inverse of G from L, Q columns per CTA: L z = e_col, L^T g = z with one column per
+// Inverses from L, Q columns per CTA: L z = e_col (L^{-1}) and L^T g = z (G^{-1}), one column per
 // lane (32 / Q rows side by side in a warp).  Same operations per column as trsv_lower and
 // trsv_lower_t: the 32 products of a block are summed in the order of their butterfly.
 // ---------------------------------------------------------------------------
@@ -263,6 +283,16 @@ __global__ void __launch_bounds__(kThr) inverse_tiles_kernel(const DenseInst* __
       }
       __syncthreads();
     }
+    if (I.Li) {   // column c0 + q of L^{-1} is z
+      const int mp = m + (m & 1);
+      for (int e = threadIdx.x; e < m * Q; e += kThr) {
+        if (c0 + e % Q < m) I.Li[(size_t)(e / Q) * mp + c0 + e % Q] = W[e];
+        const int q = e / m, i = e % m;
+        if (c0 + q < m) I.LiT[(size_t)(c0 + q) * mp + i] = W[i * Q + q];
+      }
+      __syncthreads();
+      continue;
+    }
     // L^T g = z
     for (int kb = ((m - 1) / kNB) * kNB; kb >= 0; kb -= kNB) {
       const int nb = min(kNB, m - kb);
@@ -306,9 +336,7 @@ __global__ void __launch_bounds__(kThr) inverse_tiles_kernel(const DenseInst* __
     }
     for (int e = threadIdx.x; e < m * Q; e += kThr) {
       const int q = e / m, i = e % m;
-      if (c0 + q >= m) continue;
-      if (I.Ginvf) I.Ginvf[(size_t)(c0 + q) * I.ldtf + i] = (float)W[i * Q + q];
-      if (I.Ginv) I.Ginv[(size_t)(c0 + q) * (m + (m & 1)) + i] = W[i * Q + q];
+      if (c0 + q < m) I.Ginvf[(size_t)(c0 + q) * I.ldtf + i] = (float)W[i * Q + q];
     }
     __syncthreads();
   }
@@ -344,22 +372,16 @@ cudaError_t launch_inverse(DenseInst* inst, int count, int mmax, int sms, cudaSt
   return cudaGetLastError();
 }
 
-}  // namespace
-
-cudaError_t launch_dense_factor(DenseInst* inst, int count, int mmax, int sms, cudaStream_t st) {
+cudaError_t launch_cholesky(DenseInst* inst, int count, int mmax, int sms, cudaStream_t st) {
   const int nt = (mmax + 31) / 32, tiles = nt * (nt + 1) / 2;
-  for (int k0 = 0; k0 < count; k0 += 32768) {
-    const int cnt = std::min(32768, count - k0);
-    // enough CTAs to fill the SMs a few times; the rest of an instance's tiles in a loop
-    const int gx = std::max(1, std::min(tiles, (8 * sms + cnt - 1) / cnt));
-    gram_tiles_kernel<<<dim3(gx, cnt), kThr, 0, st>>>(inst + k0);
-  }
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  // CTAs per factorisation: a power of two up to the portable cluster size while the SMs
-  // outnumber the CTAs and a CTA has more than one tile of the first trailing update
+  // CTAs per factorisation: a power of two up to 16 while the SMs outnumber the CTAs and a
+  // CTA has more than one tile of the first trailing update
   int C = 1;
-  while (C < 8 && 2 * C * count <= sms && 2 * C <= tiles) C *= 2;
+  while (C < 16 && 2 * C * count <= sms && 2 * C <= tiles) C *= 2;
+  if (C > 8) {
+    const cudaError_t e = cudaFuncSetAttribute(chol_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+  }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(std::min(count, 4 * sms) * C));
   cfg.blockDim = dim3(kThr);
@@ -372,6 +394,26 @@ cudaError_t launch_dense_factor(DenseInst* inst, int count, int mmax, int sms, c
   cfg.attrs = at;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, chol_cluster_kernel, inst, count);
+}
+
+}  // namespace
+
+cudaError_t launch_dense_factor(DenseInst* inst, int count, int mmax, int sms, cudaStream_t st) {
+  const int nt = (mmax + 31) / 32, tiles = nt * (nt + 1) / 2;
+  for (int k0 = 0; k0 < count; k0 += 32768) {
+    const int cnt = std::min(32768, count - k0);
+    // enough CTAs to fill the SMs a few times; the rest of an instance's tiles in a loop
+    const int gx = std::max(1, std::min(tiles, (8 * sms + cnt - 1) / cnt));
+    gram_tiles_kernel<<<dim3(gx, cnt), kThr, 0, st>>>(inst + k0);
+  }
+  const cudaError_t e = cudaGetLastError();
+  return e != cudaSuccess ? e : launch_cholesky(inst, count, mmax, sms, st);
+}
+
+cudaError_t launch_sparse_factor(DenseInst* inst, int m, const GroupSparse& sp, int sms, cudaStream_t st) {
+  gram_sparse_kernel<<<std::max(1, std::min(4 * sms, (m + 7) / 8)), kThr, 0, st>>>(inst, sp);
+  const cudaError_t e = cudaGetLastError();
+  return e != cudaSuccess ? e : launch_cholesky(inst, 1, m, sms, st);
 }
 
 cudaError_t launch_dense_transpose(DenseInst* inst, int count, int mmax, int nmax, int sms, cudaStream_t st) {
