@@ -227,6 +227,7 @@ void layout_ldl(Arena& ar, GridData<double>& g, const abip::ldl_host::Symbolic* 
   view.y = g.y; view.x = g.x; view.s = g.s; view.zy = g.zy; view.zx = g.zx;
   view.g1y = g.g1y; view.g1x = g.g1x; view.g2y = g.g2y; view.g2x = g.g2x;
   view.partials = g.partials;
+  view.bar = g.bar;
   view.ctl = g.ctl;
   g.ldlv = ar.take<abip::LdlView>(1);
   g.ldl_N = N;

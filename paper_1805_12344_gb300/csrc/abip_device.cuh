@@ -44,16 +44,33 @@ __device__ __forceinline__ unsigned long long ld_acquire_u64(const unsigned long
 }
 
 struct GridBarrier {
-  unsigned long long* count;   // total arrivals since the launch (host zeroes it)
+  unsigned long long* count;   // total arrivals since the launch (host zeroes it); kBarPoison once failed
   int* err;                    // first device error (0 = none)
   unsigned long long limit_ns; // wall-clock limit of one wait; 0 = kBarrierLimitNs
 };
 
+// Bit of the arrival counter that a failure sets: every wait on the counter then ends, so a
+// barrier needs no look at the error word.
+constexpr unsigned long long kBarPoison = 1ull << 62;
+
+// Record a device error (the first one stays) and let every barrier wait of the launch end.
+__device__ __forceinline__ void grid_fail(unsigned long long* count, int* err, int code) {
+  atomicCAS(err, 0, code);
+  __threadfence();
+  atomicOr(count, kBarPoison);
+}
+
+__device__ __forceinline__ void red_release_add_u64(unsigned long long* p, unsigned long long v) {
+  asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+
 // Grid-wide barrier for a cooperative launch (all CTAs co-resident).  The
 // arrival counter only grows: barrier number k of the launch completes when it
-// reaches k * gridDim.x, so no reset is needed.  Thread 0 of each CTA arrives
-// after a release fence and waits with a wall-clock limit (read on the first spin
-// and every 64th after it), leaving early if any CTA has flagged an error.
+// reaches k * gridDim.x, so no reset is needed.  Thread 0 of each CTA arrives by a
+// releasing reduction (nothing comes back) and polls by acquiring loads with a wall-clock
+// limit, leaving early once any CTA has failed (kBarPoison).  What it costs is the round
+// trips of the L2: one way in, one poll; no fences beside the two accesses and no load of
+// the error word after them.
 // `target` is this CTA's running count (all CTAs pass the same barriers).  Returns
 // false (in every thread) on timeout or error; the caller must then leave the kernel.
 __device__ __forceinline__ bool grid_sync(const GridBarrier& gb, unsigned long long& target) {
@@ -61,26 +78,21 @@ __device__ __forceinline__ bool grid_sync(const GridBarrier& gb, unsigned long l
   __syncthreads();
   target += gridDim.x;
   if (threadIdx.x == 0) {
-    int ok = 1;
-    __threadfence();
-    atomicAdd(gb.count, 1ull);
-    if (ld_acquire_u64(gb.count) < target) {
+    red_release_add_u64(gb.count, 1ull);
+    unsigned long long v = ld_acquire_u64(gb.count);
+    if (v < target) {
       const unsigned long long t0 = globaltimer_ns();
       const unsigned long long limit = gb.limit_ns ? gb.limit_ns : kBarrierLimitNs;
-      unsigned spins = 0;
-      while (ld_acquire_u64(gb.count) < target) {
-        __nanosleep(32);
-        if (ld_relaxed_i32(gb.err) != 0) { ok = 0; break; }
-        if ((spins++ & 63u) == 0 && globaltimer_ns() - t0 > limit) {
-          atomicCAS(gb.err, 0, (int)DEV_ERR_BARRIER_TIMEOUT);
-          ok = 0;
+      for (unsigned spins = 1; (v = ld_acquire_u64(gb.count)) < target; ++spins) {
+        if (spins >= 256) __nanosleep(32);
+        if ((spins <= 2 || (spins & 63u) == 0) && globaltimer_ns() - t0 > limit) {
+          grid_fail(gb.count, gb.err, (int)DEV_ERR_BARRIER_TIMEOUT);
+          v = kBarPoison;
           break;
         }
       }
     }
-    __threadfence();
-    if (ld_relaxed_i32(gb.err) != 0) ok = 0;
-    s_ok = ok;
+    s_ok = v < kBarPoison;
   }
   __syncthreads();
   return s_ok != 0;

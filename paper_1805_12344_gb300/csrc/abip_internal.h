@@ -112,6 +112,7 @@ struct LdlView {
   double* zy = nullptr; double* zx = nullptr;                                        // M^{-1} w
   double* g1y = nullptr; double* g1x = nullptr; double* g2y = nullptr; double* g2x = nullptr;
   double* partials = nullptr;
+  unsigned long long* bar = nullptr;    // the launch's barrier counter (grid_fail)
   SolveCtl* ctl = nullptr;
 };
 

@@ -103,7 +103,7 @@ struct DeltaSolver {
     return ok;
   }
   __device__ void flag(int code) {
-    if (threadIdx.x == 0) atomicCAS(&C->err, 0, code);
+    if (threadIdx.x == 0) grid_fail(D.bar, &C->err, code);
   }
 
   // Grid totals of K slots plus E scalars derived from them by f(totals, extra) on

@@ -65,7 +65,7 @@ __device__ __forceinline__ void st_relaxed_f64(double* p, double v) {
 // Shared wait loop: until done() holds, bounded by the barrier wall-clock limit and left
 // as soon as any thread has flagged an error; false in both cases.
 template <typename Done>
-__device__ __forceinline__ bool ldl_spin_until(Done done, SolveCtl* C) {
+__device__ __forceinline__ bool ldl_spin_until(Done done, SolveCtl* C, unsigned long long* bar) {
   const unsigned long long t0 = globaltimer_ns();
   const unsigned long long limit = C->bar_limit_ns ? C->bar_limit_ns : kBarrierLimitNs;
   for (unsigned spins = 0;; ++spins) {
@@ -74,7 +74,7 @@ __device__ __forceinline__ bool ldl_spin_until(Done done, SolveCtl* C) {
     if ((spins & 31u) == 31u) {
       if (ld_relaxed_i32(&C->err) != 0) return false;
       if (globaltimer_ns() - t0 > limit) {
-        atomicCAS(&C->err, 0, (int)DEV_ERR_BARRIER_TIMEOUT);
+        grid_fail(bar, &C->err, (int)DEV_ERR_BARRIER_TIMEOUT);
         return false;
       }
     }
@@ -82,26 +82,29 @@ __device__ __forceinline__ bool ldl_spin_until(Done done, SolveCtl* C) {
 }
 
 // Factorisation: wait (this lane) until *f >= target.
-__device__ __noinline__ bool ldl_spin(const unsigned long long* f, unsigned long long target, SolveCtl* C) {
-  return ldl_spin_until([&] { return ld_acquire_u64(f) >= target; }, C);
+__device__ __noinline__ bool ldl_spin(const unsigned long long* f, unsigned long long target, SolveCtl* C,
+                                      unsigned long long* bar) {
+  return ldl_spin_until([&] { return ld_acquire_u64(f) >= target; }, C, bar);
 }
-__device__ __forceinline__ bool ldl_wait(const unsigned long long* f, unsigned long long target, SolveCtl* C) {
-  return ld_acquire_u64(f) >= target || ldl_spin(f, target, C);
+__device__ __forceinline__ bool ldl_wait(const unsigned long long* f, unsigned long long target, SolveCtl* C,
+                                         unsigned long long* bar) {
+  return ld_acquire_u64(f) >= target || ldl_spin(f, target, C, bar);
 }
 __device__ __forceinline__ void st_release(unsigned long long* f, unsigned long long v) {
   asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(f), "l"(v) : "memory");
 }
 
 // Sweeps: the value at p once it is no longer kLdlEmpty (kLdlEmpty if the wait failed).
-__device__ __noinline__ unsigned long long ldl_spin_value(const unsigned long long* p, SolveCtl* C) {
+__device__ __noinline__ unsigned long long ldl_spin_value(const unsigned long long* p, SolveCtl* C,
+                                                          unsigned long long* bar) {
   unsigned long long v = kLdlEmpty;
-  ldl_spin_until([&] { v = ld_relaxed_u64(p); return v != kLdlEmpty; }, C);
+  ldl_spin_until([&] { v = ld_relaxed_u64(p); return v != kLdlEmpty; }, C, bar);
   return v;
 }
-__device__ __forceinline__ bool ldl_take(const double* p, double& out, SolveCtl* C) {
+__device__ __forceinline__ bool ldl_take(const double* p, double& out, SolveCtl* C, unsigned long long* bar) {
   const unsigned long long* q = reinterpret_cast<const unsigned long long*>(p);
   unsigned long long v = ld_relaxed_u64(q);
-  if (v == kLdlEmpty) v = ldl_spin_value(q, C);
+  if (v == kLdlEmpty) v = ldl_spin_value(q, C, bar);
   out = __longlong_as_double((long long)v);
   return v != kLdlEmpty;
 }
@@ -129,7 +132,7 @@ __device__ __noinline__ void ldl_factor(const LdlView* __restrict__ V) {
     bool ok = true;
     for (int64_t r = F.Rp[j]; r < F.Rp[j + 1]; ++r) {
       const int k = F.Rk[r];
-      if (!__all_sync(0xffffffffu, ldl_wait(F.flag + k, 1ull, C))) { ok = false; break; }
+      if (!__all_sync(0xffffffffu, ldl_wait(F.flag + k, 1ull, C, V->bar))) { ok = false; break; }
       const int64_t pjk = F.Rpos[r];
       const double ljk = __ldcg(F.Lx + pjk);
       const double f = ljk * __ldcg(F.Dd + k);
@@ -148,13 +151,13 @@ __device__ __noinline__ void ldl_factor(const LdlView* __restrict__ V) {
         else found = false;
       }
       if (!__all_sync(0xffffffffu, found)) {
-        if (lane == 0) atomicCAS(&C->err, 0, (int)DEV_ERR_LDL);
+        if (lane == 0) grid_fail(V->bar, &C->err, (int)DEV_ERR_LDL);
         ok = false;
         break;
       }
     }
     if (ok && !(isfinite(d) && (pos ? d > 0.0 : d < 0.0))) {
-      if (lane == 0) atomicCAS(&C->err, 0, (int)DEV_ERR_LDL);
+      if (lane == 0) grid_fail(V->bar, &C->err, (int)DEV_ERR_LDL);
       ok = false;
     }
     if (!ok) return;
@@ -203,7 +206,7 @@ __device__ __forceinline__ void ldl_solve(const LdlView* __restrict__ V, unsigne
     for (int64_t r = F.Rp[p] + lane; r < F.Rp[p + 1]; r += 32) {
       const double l = __ldcg(F.Lx + F.Rpos[r]);
       double zk;
-      if (!ldl_take(zf + F.Rk[r], zk, C)) { ok = false; break; }
+      if (!ldl_take(zf + F.Rk[r], zk, C, V->bar)) { ok = false; break; }
       acc += l * zk;
     }
     if (!__all_sync(0xffffffffu, ok)) return;
@@ -217,11 +220,11 @@ __device__ __forceinline__ void ldl_solve(const LdlView* __restrict__ V, unsigne
     for (int64_t e = F.Lp[p] + lane; e < F.Lp[p + 1]; e += 32) {
       const double l = __ldcg(F.Lx + e);
       double wi;
-      if (!ldl_take(wb + F.Li[e], wi, C)) { ok = false; break; }
+      if (!ldl_take(wb + F.Li[e], wi, C, V->bar)) { ok = false; break; }
       acc += l * wi;
     }
     double zp = 0.0;
-    if (lane == 0 && ok) ok = ldl_take(zf + p, zp, C);
+    if (lane == 0 && ok) ok = ldl_take(zf + p, zp, C, V->bar);
     if (!__all_sync(0xffffffffu, ok)) return;
     acc = warp_sum(acc);
     if (lane == 0) {
@@ -383,7 +386,7 @@ struct Solver {
   }
 
   __device__ void flag(int code) {
-    if (threadIdx.x == 0) atomicCAS(&C->err, 0, code);
+    if (threadIdx.x == 0) grid_fail(D.bar, &C->err, code);
   }
 
   // PCG start (reading A10): 0 the previous solution, 1 the linear extrapolation
