@@ -21,10 +21,14 @@
 //    shared memory when it fits.
 // The same kernel serves the sparse direct projection of an LP with few rows (SPARSE): the
 // products with A run over its CSR rows and columns, L^{-1} stays dense.
-// One update has five barriers of the group: t | z_y | H^T z | x, s | products and test sums.
-// Measured, us per update, one CTA with triangular sweeps -> this kernel: 50 x 120 76.9 -> 11.1
-// (the chain of phases: 16 x 48 takes 10.0), 512 x 1154 1564 -> 26.4, the slowest of 64 LPs of
-// m 16 .. 256 621 -> 65.
+//  * H^T z, which fixes (t1, t2), needs no z: H^T M^{-1} w = (M^{-T} H)^T w, so its sums over
+//    w = (y, x + s) join the test sums and the scalars' own step runs on one warp beside the
+//    products of the others; the tests are decided the same way, beside t = L^{-1} q, which is
+//    dropped when the decision is not another update.
+// One update has four barriers of the group: products and all sums | t | z_y | x, s.
+// Measured, us per update, one CTA with triangular sweeps -> this kernel: 50 x 120 76.9 -> 9.8
+// (the chain of dependent FP64 operations: about 100 clocks each, four barriers of 500),
+// 512 x 1154 1564 -> 20 over the grid, the slowest of 64 LPs of m 16 .. 256 621 -> 60.
 #include <algorithm>
 
 #include <cooperative_groups.h>
@@ -39,7 +43,7 @@ namespace {
 
 constexpr int kThr = 256;
 constexpr int kWarps = kThr / 32;
-constexpr int kSums = 9;
+constexpr int kSums = 11;   // the nine of the tests and the two of H^T z
 
 enum Act : int { ACT_STEP = 0, ACT_WARM = 1, ACT_STOP = 2 };
 
@@ -66,13 +70,15 @@ __device__ __forceinline__ double sum_together(double (&a)[P], int lane) {
 
 // out(which, i, sum_j M[row0 + i][j] v_which[j]) for i < rows: R rows per warp at a time, NV
 // vectors; rows of M are ld (even) doubles, 16-byte aligned and zero-padded like v0, v1.
-template <int R, int NV, typename F>
+// By the warps from W0 on.
+template <int R, int NV, int W0, typename F>
 __device__ __forceinline__ void dots(const double* M, int64_t ld, int rows, const double* v0, const double* v1, F out) {
   constexpr int P = R * NV;
   constexpr int kShift = P == 16 ? 1 : P == 8 ? 2 : P == 4 ? 3 : P == 2 ? 4 : 5;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31, wid = (int)(threadIdx.x >> 5) - W0;
   const int nq = (int)(ld >> 1);
-  for (int g = wid * R; g < rows; g += kWarps * R) {
+  if (wid < 0) return;
+  for (int g = wid * R; g < rows; g += (kWarps - W0) * R) {
     double a[P];
 #pragma unroll
     for (int k = 0; k < P; ++k) a[k] = 0.0;
@@ -102,24 +108,27 @@ __device__ __forceinline__ void dots(const double* M, int64_t ld, int rows, cons
 }
 
 // rows per warp by the rows of the CTA: all warps busy first, then more sums per reduction
-template <int NV, typename F>
+template <int NV, int W0, typename F>
 __device__ __forceinline__ void dots_any(const double* M, int64_t ld, int rows, const double* v0, const double* v1, F out) {
-  if (rows > 4 * kWarps) dots<8, NV>(M, ld, rows, v0, v1, out);
-  else if (rows > 2 * kWarps) dots<4, NV>(M, ld, rows, v0, v1, out);
-  else if (rows > kWarps) dots<2, NV>(M, ld, rows, v0, v1, out);
-  else dots<1, NV>(M, ld, rows, v0, v1, out);
+  constexpr int W = kWarps - W0;
+  if (rows > 4 * W) dots<8, NV, W0>(M, ld, rows, v0, v1, out);
+  else if (rows > 2 * W) dots<4, NV, W0>(M, ld, rows, v0, v1, out);
+  else if (rows > W) dots<2, NV, W0>(M, ld, rows, v0, v1, out);
+  else dots<1, NV, W0>(M, ld, rows, v0, v1, out);
 }
 
 // out(k, sum_j M[k][j] v[j]) for the CTA's rows k < rows of a triangular M, row k being row
 // rank + size k of the matrix at M + k * stride: dealt out in turn, since the rows grow (LOWER)
 // or shrink in length.  Only the triangle is read, in pairs of columns and to the longest of
-// the R rows that a warp has at once (the entries beyond are stored zeros).
+// the R rows that a warp has at once (the entries beyond are stored zeros).  By all warps but
+// the first, which has the scalars' work meanwhile.
 template <int R, bool LOWER, typename F>
 __device__ __forceinline__ void tri_dots(const double* M, int64_t stride, int rows, int rank, int size, int nq,
                                          const double* v, F out) {
   constexpr int kShift = R == 8 ? 2 : R == 4 ? 3 : R == 2 ? 4 : 5;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  for (int g = wid * R; g < rows; g += kWarps * R) {
+  const int lane = threadIdx.x & 31, wid = (int)(threadIdx.x >> 5) - 1;
+  if (wid < 0) return;
+  for (int g = wid * R; g < rows; g += (kWarps - 1) * R) {
     double a[R];
     const double2* r[R];
 #pragma unroll
@@ -149,9 +158,10 @@ __device__ __forceinline__ void tri_dots(const double* M, int64_t stride, int ro
 template <bool LOWER, typename F>
 __device__ __forceinline__ void tri_any(const double* M, int64_t stride, int rows, int rank, int size, int nq,
                                         const double* v, F out) {
-  if (rows > 4 * kWarps) tri_dots<8, LOWER>(M, stride, rows, rank, size, nq, v, out);
-  else if (rows > 2 * kWarps) tri_dots<4, LOWER>(M, stride, rows, rank, size, nq, v, out);
-  else if (rows > kWarps) tri_dots<2, LOWER>(M, stride, rows, rank, size, nq, v, out);
+  constexpr int W = kWarps - 1;
+  if (rows > 4 * W) tri_dots<8, LOWER>(M, stride, rows, rank, size, nq, v, out);
+  else if (rows > 2 * W) tri_dots<4, LOWER>(M, stride, rows, rank, size, nq, v, out);
+  else if (rows > W) tri_dots<2, LOWER>(M, stride, rows, rank, size, nq, v, out);
   else tri_dots<1, LOWER>(M, stride, rows, rank, size, nq, v, out);
 }
 
@@ -193,6 +203,34 @@ struct Group {
   }
 };
 
+// barrier_step with the square root and the quotient refined from FP32 estimates: one coupled
+// step and a residual step each leave about 1e-16 relative, in half the dependent operations of
+// the library's (an update's critical path holds this chain).  Outside the FP32 range of the
+// discriminant, the closed form.
+__device__ __forceinline__ void barrier_step_fast(double omega, double c, double& x, double& s) {
+  const double disc = omega * omega + 4.0 * c;
+  if (!(disc > 1e-30 && disc < 1e30)) {
+    barrier_step<double>(omega, c, x, s);
+    return;
+  }
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"((float)disc));
+  const double rd = (double)r;
+  double g = disc * rd, h = 0.5 * rd;
+  const double e = 0.5 - g * h;
+  g += g * e;
+  h += h * e;
+  const double D = g + (disc - g * g) * h;
+  const double L = 0.5 * (fabs(omega) + D);   // the larger root; the smaller is c / L
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"((float)L));
+  double q = (double)r;
+  q += q * (1.0 - L * q);
+  const double t = c * q;
+  const double small = t + q * (c - L * t);
+  x = omega >= 0.0 ? L : small;
+  s = omega >= 0.0 ? small : L;
+}
+
 struct GroupArgs {
   DenseInst* insts;
   int count;
@@ -203,7 +241,7 @@ struct GroupArgs {
   GroupSparse sp;                 // SPARSE: A by rows and by columns
   // grid mode: published vectors (q, t, z_y: even(m) each; x, s: even(n) each), partial sums, barrier
   double* gvec;
-  double* gpart;                  // (kSums + 2) * grid
+  double* gpart;                  // kSums * grid
   unsigned long long* bar;
   int* err;
   unsigned long long bar_limit_ns;
@@ -213,20 +251,19 @@ struct Scal {
   double tau, kappa, theta, mu, t1, t2, itau, cmu, gk;
   int action, status, outer, ok;
   int64_t total;
-  double a[kSums];   // the test sums
+  double a[kSums];   // the sums
 };
 
 // The block's sums of NS values per thread (only the first `act` warps hold any), published
 // in the partial slots of every CTA: slots[r * NS + k] is CTA r's sum k.
-template <int NS, int P, bool GRID>
-__device__ __forceinline__ void publish_sums(const Group<GRID>& G, double (&acc)[P], int act, double* wsum, double* slots,
+template <int NS, bool GRID>
+__device__ __forceinline__ void publish_sums(const Group<GRID>& G, double (&acc)[16], int act, double* wsum, double* slots,
                                              double* gslots) {
-  constexpr int kShift = P == 16 ? 1 : 4;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   if (wid < act) {
-    const double v = sum_together<P>(acc, lane);
-    const int k = lane >> kShift;
-    if ((lane & ((1 << kShift) - 1)) == 0 && k < NS) wsum[k * kWarps + wid] = v;
+    const double v = sum_together<16>(acc, lane);
+    const int k = lane >> 1;
+    if ((lane & 1) == 0 && k < NS) wsum[k * kWarps + wid] = v;
   }
   __syncthreads();
   if constexpr (GRID) {
@@ -296,11 +333,12 @@ __device__ __forceinline__ void sparse_rows2(const int32_t* rp, const int32_t* c
     if (i < rows && (sub & 3) == 0) out(sub >> 2, i, v);
   }
 }
-// out(j, sum_i A_ij v[i]) for the CTA's columns, a thread per column
-template <typename F>
+// out(j, sum_i A_ij v[i]) for the CTA's columns, a thread per column, by the warps from W0 on
+template <int W0, typename F>
 __device__ __forceinline__ void sparse_cols(const int32_t* cp, const int32_t* ri, const double* cv, int cols,
                                             const double* v, F out) {
-  for (int j = threadIdx.x; j < cols; j += kThr) {
+  if (threadIdx.x < 32 * W0) return;
+  for (int j = threadIdx.x - 32 * W0; j < cols; j += kThr - 32 * W0) {
     double a = 0.0;
     for (int e = cp[j]; e < cp[j + 1]; ++e) a += cv[e] * v[ri[e]];
     out(j, a);
@@ -321,21 +359,23 @@ __device__ void solve_one(DenseInst& I, const GroupArgs& Q, Group<GRID>& G, doub
   double* zy = tv + mp;
   double* x = zy + mp;
   double* s = x + np;
-  double* hslot = s + np;                               // 2 * size
-  double* rslot = hslot + 2 * (GRID ? 1 : G.size);      // kSums * size
+  double* rslot = s + np;                               // kSums * size
   double* y = rslot + kSums * (GRID ? 1 : G.size);      // own rows
   double* Ax = y + mc;
   double* As = Ax + mc;
-  double* aty = As + mc;                                // own columns
+  double* k1y = As + mc;                                // M^{-T} h1, M^{-T} h2
+  double* k2y = k1y + mc;
+  double* aty = k2y + mc;                               // own columns
   double* v = aty + nc_;
-  double* top = v + nc_;
+  double* k1x = v + nc_;
+  double* k2x = k1x + nc_;
+  double* top = k2x + nc_;
   double* gq = Q.gvec;
   double* gtv = gq + mp;
   double* gzy = gtv + mp;
   double* gx = gzy + mp;
   double* gs = gx + np;
-  double* ghs = Q.gpart;
-  double* grs = Q.gpart + 2 * G.size;
+  double* grs = Q.gpart;
   const double* b = I.b + i0;
   const double* bbar = I.bbar + i0;
   const double* g1y = I.g1 + i0;
@@ -398,16 +438,16 @@ __device__ void solve_one(DenseInst& I, const GroupArgs& Q, Group<GRID>& G, doub
   // screens of the Sec. 4.1 tests without square roots and divisions; a sum that passes is
   // tested as written
   const double tp = eps * (1.0 + nb) * (1.0 + 1e-12), td = eps * (1.0 + nc) * (1.0 + 1e-12);
-  // start of Algorithm 2, or a state loaded by abip_set_state
+  const double tp2 = tp * tp, td2 = td * td, nb2 = nb * nb, nc2 = nc * nc;
   const bool resume = I.resume != 0;
   for (int i = threadIdx.x; i < mp; i += kThr) {
     q[i] = 0.0;
     tv[i] = 0.0;
-    zy[i] = (resume && i < m) ? I.y[i] : 0.0;
+    zy[i] = 0.0;
   }
-  for (int j = threadIdx.x; j < np; j += kThr) {
-    x[j] = j < n ? (resume ? I.x[j] : 1.0) : 0.0;
-    s[j] = j < n ? (resume ? I.s[j] : 1.0) : 0.0;
+  for (int j = n + threadIdx.x; j < np; j += kThr) {   // the padding
+    x[j] = 0.0;
+    s[j] = 0.0;
   }
   for (int i = threadIdx.x; i < mr; i += kThr) y[i] = resume ? I.y[i0 + i] : 0.0;
   for (int j = threadIdx.x; j < nr; j += kThr) aty[j] = 0.0;
@@ -423,98 +463,158 @@ __device__ void solve_one(DenseInst& I, const GroupArgs& Q, Group<GRID>& G, doub
     S.ok = 1;
   }
   __syncthreads();
-  if (resume) {   // A^T y of the loaded state, once (z_y's buffer holds y)
-    if constexpr (SPARSE) sparse_cols(cp, ri, cv, nr, zy, [&](int j, double d) { aty[j] = d; });
-    else dots_any<1>(ATr, mp, nr, zy, zy, [&](int, int j, double d) { aty[j] = d; });
-    __syncthreads();
-    for (int i = threadIdx.x; i < mp; i += kThr) zy[i] = 0.0;
-  }
-  const int items = nr + mr, act = min(kWarps, max(1, (items + 31) / 32));
-  bool first = true;   // the sums of a start or of a warm start: no test, no count
+  // rows of A times two vectors, and columns of A times one, over the CTA's share
+  auto rows_A = [&](const double* v0, const double* v1, auto out) {
+    if constexpr (SPARSE) sparse_rows2(rp, ci, va, mr, v0, v1, out);
+    else dots_any<2, 0>(Ar, np, mr, v0, v1, out);
+  };
+  // z_y = L^{-T} L^{-1} q of the published q, published; two barriers.  The first warp has
+  // `beside` and `beside2` to do meanwhile.
+  auto solve_G = [&](auto beside, auto beside2) -> bool {
+    if (wid == 0) beside();
+    tri_any<true>(Lr, tstride, tr, G.rank, G.size, mp >> 1, q, [&](int k, double d) { G.put(tv, gtv, G.rank + G.size * k, d); });
+    if (!G.sync()) return false;
+    if (S.action != ACT_STEP) return true;
+    G.fetch(tv, gtv, m);
+    if constexpr (GRID) __syncthreads();
+    if (wid == 0) beside2();
+    tri_any<false>(Ur, tstride, tr, G.rank, G.size, mp >> 1, tv, [&](int k, double d) { G.put(zy, gzy, G.rank + G.size * k, d); });
+    if (!G.sync()) return false;
+    G.fetch(zy, gzy, m);
+    if constexpr (GRID) __syncthreads();
+    return true;
+  };
+  const int rows0 = (nr + 31) & ~31;   // the CTA's rows start at a warp of their own
+  const int items = rows0 + mr, act = min(kWarps, max(1, (items + 31) / 32));
   if (!G.sync()) return;   // nobody publishes into a CTA that is still filling its copies
-  for (;;) {
-    // ---- products of the state, its test sums (residual_sums' order of quantities), and q
-    if constexpr (SPARSE) sparse_rows2(rp, ci, va, mr, x, s, [&](int w, int i, double d) { (w == 0 ? Ax : As)[i] = d; });
-    else dots_any<2>(Ar, np, mr, x, s, [&](int w, int i, double d) { (w == 0 ? Ax : As)[i] = d; });
+  // M^{-T} h = J M^{-1} J h, J = diag(I, -I): for h = [a; d], G g = a + A d and
+  // M^{-T} h = [g; d - A^T g].  The columns d of h1 and h2 stand in x and s meanwhile.
+  if (threadIdx.x == 0) S.action = ACT_STEP;
+  for (int j = threadIdx.x; j < n; j += kThr) { x[j] = I.c[j]; s[j] = -I.cbar[j]; }
+  __syncthreads();
+  rows_A(x, s, [&](int w, int i, double d) { (w == 0 ? Ax : As)[i] = d; });
+  __syncthreads();
+  for (int col = 0; col < 2; ++col) {
+    for (int i = threadIdx.x; i < mr; i += kThr) G.put(q, gq, i0 + i, col == 0 ? Ax[i] - b[i] : As[i] + bbar[i]);
+    if (!G.sync()) return;
+    G.fetch(q, gq, m);
     __syncthreads();
+    if (!solve_G([] {}, [] {})) return;
+    double* ky = col == 0 ? k1y : k2y;
+    double* kx = col == 0 ? k1x : k2x;
+    const double* d = col == 0 ? x : s;
+    for (int i = threadIdx.x; i < mr; i += kThr) ky[i] = zy[i0 + i];
+    auto put_k = [&](int j, double t) { kx[j] = d[j0 + j] - t; };
+    if constexpr (SPARSE) sparse_cols<0>(cp, ri, cv, nr, zy, put_k);
+    else dots_any<1, 0>(ATr, mp, nr, zy, zy, [&](int, int j, double t) { put_k(j, t); });
+    if (!G.sync()) return;   // z_y has been read
+  }
+  // start of Algorithm 2, or a state loaded by abip_set_state
+  for (int j = threadIdx.x; j < n; j += kThr) {
+    x[j] = resume ? I.x[j] : 1.0;
+    s[j] = resume ? I.s[j] : 1.0;
+  }
+  if (resume) {   // A^T y of the loaded state, once (z_y's buffer holds y)
+    for (int i = threadIdx.x; i < m; i += kThr) zy[i] = I.y[i];
+    __syncthreads();
+    if constexpr (SPARSE) sparse_cols<0>(cp, ri, cv, nr, zy, [&](int j, double d) { aty[j] = d; });
+    else dots_any<1, 0>(ATr, mp, nr, zy, zy, [&](int, int j, double d) { aty[j] = d; });
+  }
+  bool first = true;   // the sums of a start or of a warm start: no test, no count
+  if (!G.sync()) return;
+  for (;;) {
+    // ---- the sums over the columns, the products A x, A s, the sums over the rows, and q
     {
       double acc[16];
 #pragma unroll
       for (int k = 0; k < 16; ++k) acc[k] = 0.0;
       const double ta = S.tau, th = S.theta, it = S.itau;
-      for (int e = threadIdx.x; e < items; e += kThr) {
-        if (e < nr) {
-          const double at = aty[e], sj = s[j0 + e], cj = c[e], cb = cbar[e], xj = x[j0 + e];
-          const double as = at + sj;
-          const double rx = cj * ta - cb * th - as;
-          const double dr = as * it - cj;
-          acc[0] += rx * rx; acc[2] += dr * dr; acc[4] += as * as;
-          acc[7] += cj * xj; acc[8] += cb * xj;
-        } else {
-          const int i = e - nr;
-          const double ax = Ax[i], bi = b[i], bb = bbar[i], yi = y[i];
-          const double ry = ax - bi * ta + bb * th;
-          const double pr = ax * it - bi;
-          acc[0] += ry * ry; acc[1] += pr * pr; acc[3] += ax * ax;
-          acc[5] += bi * yi; acc[6] += bb * yi;
-          G.put(q, gq, i0 + i, yi - (ax + As[i]));
-        }
+      for (int e = threadIdx.x; e < nr; e += kThr) {
+        const double at = aty[e], sj = s[j0 + e], cj = c[e], cb = cbar[e], xj = x[j0 + e];
+        const double as = at + sj, w = xj + sj;
+        const double rx = cj * ta - cb * th - as;
+        const double dr = as * it - cj;
+        acc[0] += rx * rx; acc[2] += dr * dr; acc[4] += as * as;
+        acc[7] += cj * xj; acc[8] += cb * xj;
+        acc[9] += k1x[e] * w; acc[10] += k2x[e] * w;
       }
-      publish_sums<kSums, 16, GRID>(G, acc, act, wsum, rslot, grs);
+      rows_A(x, s, [&](int w, int i, double d) { (w == 0 ? Ax : As)[i] = d; });
+      __syncthreads();
+      for (int e = threadIdx.x; e < items; e += kThr) {
+        if (e < rows0) continue;
+        const int i = e - rows0;
+        const double ax = Ax[i], bi = b[i], bb = bbar[i], yi = y[i];
+        G.put(q, gq, i0 + i, yi - (ax + As[i]));
+        const double ry = ax - bi * ta + bb * th;
+        const double pr = ax * it - bi;
+        acc[0] += ry * ry; acc[1] += pr * pr; acc[3] += ax * ax;
+        acc[5] += bi * yi; acc[6] += bb * yi;
+        acc[9] += k1y[i] * yi; acc[10] += k2y[i] * yi;
+      }
+      publish_sums<kSums, GRID>(G, acc, act, wsum, rslot, grs);
     }
     if (!G.sync()) return;
     G.fetch(q, gq, m);
-    if (wid == 0) {
+    if constexpr (GRID) __syncthreads();
+    // ---- projection: z_y = G^{-1} (y - A (x + s)), beside it the decision on the sums and
+    // t = K^{-1} (w_{tau,theta} + H^T z)
+    auto decide = [&] {
       total_sums<kSums, GRID>(G, rslot, grs, S.a);
-      if (lane == 0) {
-        const double* a = S.a;
-        const double tau = S.tau;
-        const double rt = a[5] - a[7] + zbar * S.theta - S.kappa;
-        const double rth = -a[6] + a[8] - zbar * tau - xi;
-        const double inner2 = a[0] + rt * rt + rth * rth;
-        int st = 0, action = ACT_STEP;
-        if (!isfinite(inner2)) {
-          S.ok = 0;
-          action = ACT_STOP;
-        } else {
-          if (!first) {
-            S.total += 1;
-            if (P.stop_rule == 0) {
-              if (a[1] <= tp * tp && a[2] <= td * td) {
-                const double ps = sqrt(a[1]) / (1.0 + nb), ds = sqrt(a[2]) / (1.0 + nc);
-                const double gp = fabs(a[7] / tau - a[5] / tau) / (1.0 + fabs(a[7] / tau) + fabs(a[5] / tau));
-                if (ps <= eps && ds <= eps && gp <= eps) st = ABIP_OPTIMAL;
-              }
-              const double pe = eps * a[5], de = eps * a[7];
-              if (st == 0 && a[5] > 0 && a[4] * (nb * nb) <= pe * pe * (1.0 + 1e-11) && sqrt(a[4]) <= pe / nb)
-                st = ABIP_PRIMAL_INFEASIBLE;
-              if (st == 0 && a[7] < 0 && a[3] * (nc * nc) <= de * de * (1.0 + 1e-11) && sqrt(a[3]) <= -de / nc)
-                st = ABIP_DUAL_INFEASIBLE;
+      if (lane != 0) return;
+      const double* a = S.a;
+      const double tau = S.tau;
+      const double rt = a[5] - a[7] + zbar * S.theta - S.kappa;
+      const double rth = -a[6] + a[8] - zbar * tau - xi;
+      const double inner2 = a[0] + rt * rt + rth * rth;
+      int st = 0, action = ACT_STEP;
+      if (!isfinite(inner2)) {
+        S.ok = 0;
+        action = ACT_STOP;
+      } else {
+        if (!first) {
+          S.total += 1;
+          if (P.stop_rule == 0) {
+            if (a[1] <= tp2 && a[2] <= td2) {
+              const double ps = sqrt(a[1]) / (1.0 + nb), ds = sqrt(a[2]) / (1.0 + nc);
+              const double gp = fabs(a[7] / tau - a[5] / tau) / (1.0 + fabs(a[7] / tau) + fabs(a[5] / tau));
+              if (ps <= eps && ds <= eps && gp <= eps) st = ABIP_OPTIMAL;
             }
-            if (st == 0 && S.total >= P.max_admm) st = ABIP_MAX_ITER;
+            const double pe = eps * a[5], de = eps * a[7];
+            if (st == 0 && a[5] > 0 && a[4] * nb2 <= pe * pe * (1.0 + 1e-11) && sqrt(a[4]) <= pe / nb)
+              st = ABIP_PRIMAL_INFEASIBLE;
+            if (st == 0 && a[7] < 0 && a[3] * nc2 <= de * de * (1.0 + 1e-11) && sqrt(a[3]) <= -de / nc)
+              st = ABIP_DUAL_INFEASIBLE;
           }
-          if (st == 0 && inner2 <= S.mu) {
-            double rho = 0.0;
-            if (P.gamma_max > 0.0)
-              rho = fmax(sqrt(a[1]) / (1.0 + nb),
-                         fmax(sqrt(a[2]) / (1.0 + nc),
-                              fabs(a[7] / tau - a[5] / tau) / (1.0 + fabs(a[7] / tau) + fabs(a[5] / tau))));
-            S.gk = adaptive_gamma(P.gamma, P.gamma_max, eps, rho);
-            S.mu *= S.gk;
-            S.outer += 1;
-            action = ACT_WARM;
-            if (P.stop_rule == 1 && S.mu < eps) st = ABIP_OPTIMAL;
-            else if (S.outer >= kMaxOuter) st = ABIP_MAX_ITER;   // mu has underflowed
-          }
-          if (st != 0) {
-            S.status = st;
-            action = ACT_STOP;
-          }
+          if (st == 0 && S.total >= P.max_admm) st = ABIP_MAX_ITER;
         }
-        S.action = action;
+        if (st == 0 && inner2 <= S.mu) {
+          double rho = 0.0;
+          if (P.gamma_max > 0.0)
+            rho = fmax(sqrt(a[1]) / (1.0 + nb),
+                       fmax(sqrt(a[2]) / (1.0 + nc),
+                            fabs(a[7] / tau - a[5] / tau) / (1.0 + fabs(a[7] / tau) + fabs(a[5] / tau))));
+          S.gk = adaptive_gamma(P.gamma, P.gamma_max, eps, rho);
+          S.mu *= S.gk;
+          S.outer += 1;
+          action = ACT_WARM;
+          if (P.stop_rule == 1 && S.mu < eps) st = ABIP_OPTIMAL;
+          else if (S.outer >= kMaxOuter) st = ABIP_MAX_ITER;   // mu has underflowed
+        }
+        if (st != 0) {
+          S.status = st;
+          action = ACT_STOP;
+        }
       }
-    }
-    __syncthreads();
+      S.action = action;
+    };
+    auto scalars = [&] {
+      if (lane != 0) return;
+      const double v1 = S.tau + S.kappa + S.a[9], v2 = S.theta + xi + S.a[10];
+      S.t1 = Ki0 * v1 + Ki1 * v2;
+      S.t2 = Ki2 * v1 + Ki3 * v2;
+      S.cmu = S.mu / P.beta;
+    };
+    if (!solve_G(decide, scalars)) return;
     if (S.action == ACT_STOP) break;
     if (S.action == ACT_WARM) {
       const double gk = S.gk, sg = sqrt(gk);
@@ -533,79 +633,43 @@ __device__ void solve_one(DenseInst& I, const GroupArgs& Q, Group<GRID>& G, doub
         S.itau = 1.0 / S.tau;
       }
       first = true;
-      // no CTA publishes q or its sums before all have read the last ones
+      // no CTA publishes q, t or its sums before all have read the last ones
       if (!G.sync()) return;
       continue;
     }
     first = false;
-    // ---- projection: z_y = G^{-1} (y - A (x + s)), z_x = x + s + A^T z_y, H^T z
-    tri_any<true>(Lr, tstride, tr, G.rank, G.size, mp >> 1, q, [&](int k, double d) { G.put(tv, gtv, G.rank + G.size * k, d); });
-    if (!G.sync()) return;
-    G.fetch(tv, gtv, m);
-    if constexpr (GRID) __syncthreads();
-    tri_any<false>(Ur, tstride, tr, G.rank, G.size, mp >> 1, tv, [&](int k, double d) { G.put(zy, gzy, G.rank + G.size * k, d); });
-    if (!G.sync()) return;
-    G.fetch(zy, gzy, m);
-    if constexpr (GRID) __syncthreads();
-    if constexpr (SPARSE) sparse_cols(cp, ri, cv, nr, zy, [&](int j, double d) { v[j] = d; });
-    else dots_any<1>(ATr, mp, nr, zy, zy, [&](int, int j, double d) { v[j] = d; });
-    __syncthreads();
-    {
-      double acc[2] = {0.0, 0.0};
-      for (int e = threadIdx.x; e < items; e += kThr) {
-        if (e < nr) {
-          const double z = x[j0 + e] + s[j0 + e] + v[e];
-          acc[0] += c[e] * z;
-          acc[1] -= cbar[e] * z;
-        } else {
-          const int i = e - nr;
-          const double z = zy[i0 + i];
-          acc[0] -= b[i] * z;
-          acc[1] += bbar[i] * z;
-        }
-      }
-      publish_sums<2, 2, GRID>(G, acc, act, wsum, hslot, ghs);
-    }
-    if (!G.sync()) return;
-    if (wid == 0) {
-      __shared__ double hz[2];
-      total_sums<2, GRID>(G, hslot, ghs, hz);
-      if (lane == 0) {
-        const double v1 = S.tau + S.kappa + hz[0], v2 = S.theta + xi + hz[1];
-        S.t1 = Ki0 * v1 + Ki1 * v2;
-        S.t2 = Ki2 * v1 + Ki3 * v2;
-        S.cmu = S.mu / P.beta;
-      }
-    }
-    __syncthreads();
-    // ---- relaxation, barrier and dual steps (Eqs. Simple-Update:*), and A^T y by linearity;
-    // the scalars' own step on the last warp
+    // ---- A^T z_y, relaxation, barrier and dual steps (Eqs. Simple-Update:*), A^T y by
+    // linearity; the step of tau, kappa and theta on the first warp
     const double t1 = S.t1, t2 = S.t2, cmu = S.cmu;
-    for (int e = threadIdx.x; e < items; e += kThr) {
-      if (e < nr) {
-        const int j = j0 + e;
-        const double x0 = x[j], s0 = s[j];
-        const double ux = x0 + s0 + v[e] - g1x[e] * t1 - g2x[e] * t2;
-        double xn, sn;
-        barrier_step<double>(alpha * ux + a1 * x0 - s0, cmu, xn, sn);
-        G.put(x, gx, j, xn);
-        G.put(s, gs, j, sn);
-        // A^T g1y = g1x - c and A^T g2y = g2x + cbar (M g = h)
-        aty[e] = alpha * (v[e] - (g1x[e] - c[e]) * t1 - (g2x[e] + cbar[e]) * t2) + a1 * aty[e];
-      } else {
-        const int i = e - nr;
-        const double uy = zy[i0 + i] - g1y[i] * t1 - g2y[i] * t2;
-        y[i] = alpha * uy + a1 * y[i];
-      }
-    }
-    if (threadIdx.x == kThr - 1) {
+    if (threadIdx.x == 0) {
       const double th = alpha * t1 + a1 * S.tau;
       double tn, kn;
-      barrier_step<double>(th - S.kappa, cmu, tn, kn);
+      barrier_step_fast(th - S.kappa, cmu, tn, kn);
       S.tau = tn;
       S.kappa = kn;
       S.theta = alpha * t2 + a1 * S.theta;
       S.itau = 1.0 / tn;
+    }
+    if constexpr (SPARSE) sparse_cols<1>(cp, ri, cv, nr, zy, [&](int j, double d) { v[j] = d; });
+    else dots_any<1, 1>(ATr, mp, nr, zy, zy, [&](int, int j, double d) { v[j] = d; });
+    __syncthreads();
+    for (int e = threadIdx.x; e < items; e += kThr) {
+      if (e < nr) {
+        const int j = j0 + e;
+        const double x0 = x[j], s0 = s[j], vj = v[e];
+        const double gx1 = g1x[e], gx2 = g2x[e];
+        // A^T g1y = g1x - c and A^T g2y = g2x + cbar (M g = h)
+        aty[e] = alpha * (vj - (gx1 - c[e]) * t1 - (gx2 + cbar[e]) * t2) + a1 * aty[e];
+        const double ux = x0 + s0 + vj - gx1 * t1 - gx2 * t2;
+        double xn, sn;
+        barrier_step_fast(alpha * ux + a1 * x0 - s0, cmu, xn, sn);
+        G.put(x, gx, j, xn);
+        G.put(s, gs, j, sn);
+      } else if (e >= rows0) {
+        const int i = e - rows0;
+        const double uy = zy[i0 + i] - g1y[i] * t1 - g2y[i] * t2;
+        y[i] = alpha * uy + a1 * y[i];
+      }
     }
     if (!G.sync()) return;
     G.fetch(x, gx, n);
@@ -692,7 +756,7 @@ struct SmemPlan {
 
 size_t base_doubles(int m, int n, int C, bool grid) {
   const size_t mp = (m + 1) / 2 * 2, np = (n + 1) / 2 * 2, mc = (m + C - 1) / C, nc = (n + C - 1) / C;
-  return 3 * mp + 2 * np + (2 + kSums) * (size_t)(grid ? 1 : C) + 3 * mc + 2 * nc;
+  return 3 * mp + 2 * np + kSums * (size_t)(grid ? 1 : C) + 5 * mc + 4 * nc;
 }
 size_t vec_doubles(int m, int n, int C) { return 4 * (size_t)((m + C - 1) / C) + 4 * (size_t)((n + C - 1) / C) + 2; }
 size_t mat_doubles(int m, int n, int C) {
@@ -812,7 +876,7 @@ int plan_sparse_group(int m, int n, const int32_t* rp, const int32_t* cp, int sm
 
 size_t dense_group_scratch(int m, int n, int sms) {
   const size_t mp = (m + 1) / 2 * 2, np = (n + 1) / 2 * 2;
-  return 3 * mp + 2 * np + (size_t)(kSums + 2) * sms + 4;
+  return 3 * mp + 2 * np + (size_t)kSums * sms + 4;
 }
 
 cudaError_t launch_dense_group(DenseInst* inst, int count, const DenseParams& prm, int* queue, const int* order,
@@ -824,7 +888,7 @@ cudaError_t launch_dense_group(DenseInst* inst, int count, const DenseParams& pr
     Q.bar = reinterpret_cast<unsigned long long*>(scratch + scratch_len - 2);
     Q.err = reinterpret_cast<int*>(scratch + scratch_len - 1);
     Q.gpart = scratch;
-    Q.gvec = scratch + (size_t)(kSums + 2) * plan.ctas + ((kSums + 2) * (size_t)plan.ctas & 1);
+    Q.gvec = scratch + (size_t)kSums * plan.ctas + (kSums * (size_t)plan.ctas & 1);
     const ClusterFn f = grid_fn(plan.sparse != 0);
     cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
     if (e != cudaSuccess) return e;
