@@ -472,8 +472,8 @@ struct DenseHostInst {
 
 constexpr size_t kDenseSmemLimit = 200 * 1024;
 
-// shared memory of the dense solve: 5m + 3n elements; the mixed path also needs the
-// FP64 size because an instance may finish in FP64 after escalation
+// Shared memory of a dense solve by one CTA, which is also the limit of what the dense path takes
+// (a group's share is smaller).
 size_t dense_solve_smem(int m, int n, bool mixed = false) {
   // FP64: y, zy, w, Ax, As (m) and x, s, zx (n) doubles.  Mixed (FP64 state, FP32
   // changes): y, Ax, As, zy, q_prev (m) and x, s, A^T y, A^T zy (n) doubles, plus
@@ -493,18 +493,19 @@ int dense_alloc(abip_handle* h, const std::vector<DenseHostInst>& hi, void** are
   const int count = (int)hi.size();
   auto layout = [&](Arena& ar, std::vector<DenseInst>& d) {
     DenseInst* di = ar.take<DenseInst>(count);
-    int* q = ar.take<int>(2);
+    int* q = ar.take<int>(abip::kDenseBuckets);
     if (ar.base) { *dinst = di; *queue = q; }
     d.assign(count, DenseInst{});
     for (int k = 0; k < count; ++k) {
       const int m = hi[k].m, n = hi[k].n;
       DenseInst& I = d[k];
       I.m = m; I.n = n;
-      I.ld = group ? n + (n & 1) : n;
+      const bool f64 = group && !mixed;   // the FP64 group kernel's copies
+      I.ld = f64 ? n + (n & 1) : n;
       I.A = ar.take<double>((size_t)m * I.ld);
-      I.AT = group ? ar.take<double>((size_t)n * (m + (m & 1))) : nullptr;
-      I.Li = group ? ar.take<double>((size_t)m * (m + (m & 1))) : nullptr;
-      I.LiT = group ? ar.take<double>((size_t)m * (m + (m & 1))) : nullptr;
+      I.AT = f64 ? ar.take<double>((size_t)n * (m + (m & 1))) : nullptr;
+      I.Li = f64 ? ar.take<double>((size_t)m * (m + (m & 1))) : nullptr;
+      I.LiT = f64 ? ar.take<double>((size_t)m * (m + (m & 1))) : nullptr;
       I.b = ar.take<double>(m); I.c = ar.take<double>(n);
       I.L = ar.take<double>((size_t)m * m);
       I.bbar = ar.take<double>(m); I.cbar = ar.take<double>(n);
@@ -522,7 +523,7 @@ int dense_alloc(abip_handle* h, const std::vector<DenseHostInst>& hi, void** are
         I.Af = nullptr; I.ATf = nullptr; I.Ginvf = nullptr;
       }
     }
-    if (group && count == 1) {
+    if (group && !mixed && count == 1) {
       h->gscratch_len = abip::dense_group_scratch(hi[0].m, hi[0].n, abip::dense_max_ctas(h->device));
       h->gscratch = ar.take<double>(h->gscratch_len);
     }
@@ -583,19 +584,127 @@ DenseParams dense_params(const abip_params& p) {
                      p.bb_max_redo, p.eps_cor, p.eps_penalty, p.gamma_max};
 }
 
-// The solve launch: by groups of CTAs with h->gplan when h->group, else one CTA per instance.
+// CTAs per instance, and the hand-out order (ord, for a batch): by CTAs, then largest first (m n +
+// m^2) or, without `largest_first`, as given.  An instance's CTAs do not depend on the order.
+//
+// One LP: a cluster while a CTA keeps more than kClusterWork operations (of 2 per clock, the
+// FP64 rate: 2.5k clocks, about what an update's barriers cost), and in FP64 the whole grid from
+// 8e5 operations on, where its 152 SMs outweigh its dearer barriers (us per update, cluster of
+// 16 / grid: 200 x 600 20.6 / 23.7, 256 x 1024 25.2 / 24.2, 512 x 1154 50.7 / 26.4).
+// A batch: by work too, with the share chosen so that the CTAs of all instances are about two
+// per SM (FP64, 64 LPs of m 16 .. 256, 200 updates: 14.4 ms; 1 per SM 17.2, 3 15.4; the same
+// size for all 48 / 26 / 23 / 12.6 ms with 1 / 2 / 4 / 8; 128 LPs 24.8, 61 / 49 / 25 / 26).  The time of a batch is that of its slowest instance, so the large ones get the
+// CTAs; instances of one cluster size form a bucket, and the buckets' launches run side by
+// side.  A batch of more instances than that is one bucket of single CTAs.
+constexpr double kClusterWork = 5000.0;
+bool plan_buckets(abip_handle* h, const std::vector<std::pair<int, int>>& sizes, bool largest_first, bool mixed, int sms,
+                  std::vector<int>& ord) {
+  const int count = (int)sizes.size();
+  std::vector<double> work(count);
+  for (int k = 0; k < count; ++k) {
+    const double mm = sizes[k].first, nn = sizes[k].second;
+    // mixed: 16 m n + 4 m^2 bytes of matrices at 64 bytes per clock from L2, beside the steps and sums
+    work[k] = mixed ? (12.0 * mm * nn + 4.0 * mm * mm) / 32.0 + 60.0 * mm + 90.0 * nn
+                    : 3.0 * mm * nn + mm * mm + 80.0 * (mm + nn);
+  }
+  h->buckets.clear();
+  if (!mixed && count == 1 && work[0] > 8e5) {
+    abip::DenseBucket b{{}, 0, 1};
+    if (abip::plan_dense_grid(sizes[0].first, sizes[0].second, sms, b.plan)) {
+      h->buckets.push_back(b);
+      return true;
+    }
+  }
+  auto ctas = [](double w, double share) {
+    int C = 1;
+    while (C < 16 && w / C > share) C *= 2;
+    return C;
+  };
+  double share = kClusterWork;
+  int64_t total = 0;
+  for (;; share *= 1.2) {
+    total = 0;
+    for (int k = 0; k < count; ++k) total += ctas(work[k], share);
+    if (total <= 2 * (int64_t)sms || total == count) break;
+  }
+  std::vector<int> C(count), m(count), n(count);
+  for (int k = 0; k < count; ++k) C[k] = ctas(work[k], share);
+  ord.resize(count);
+  for (int k = 0; k < count; ++k) ord[k] = k;
+  std::stable_sort(ord.begin(), ord.end(), [&](int a, int b) {
+    if (C[a] != C[b] || !largest_first) return C[a] > C[b];
+    const double ca = (double)sizes[a].first * sizes[a].second + (double)sizes[a].first * sizes[a].first;
+    const double cb = (double)sizes[b].first * sizes[b].second + (double)sizes[b].first * sizes[b].first;
+    return ca > cb;
+  });
+  for (int k = 0; k < count; ++k) { m[k] = sizes[ord[k]].first; n[k] = sizes[ord[k]].second; }
+  const size_t budget = total > sms ? 100 * 1024 : 223 * 1024;
+  for (int k = 0; k < count;) {
+    int e = k + 1;
+    while (e < count && C[ord[e]] == C[ord[k]]) ++e;
+    abip::DenseBucket b{{}, k, e - k};
+    const int ok = mixed ? abip::plan_dense_mixed(&m[k], &n[k], b.count, C[ord[k]], budget, b.plan)
+                         : abip::plan_dense_cluster(&m[k], &n[k], b.count, C[ord[k]], budget, b.plan);
+    if (!ok) return false;
+    h->buckets.push_back(b);
+    k = e;
+  }
+  return true;
+}
+
+// The launches of a solve by groups: the buckets side by side, joined on st.
+cudaError_t launch_buckets(abip_handle* h, DenseInst* dinst, int* queue, const DenseParams& dp, cudaStream_t st,
+                           const int* order, int variant) {
+  const int nb = (int)h->buckets.size();
+  auto one = [&](int i, cudaStream_t on) {
+    const abip::DenseBucket& b = h->buckets[i];
+    const int* ord = order ? order + b.first : nullptr;
+    if (dp.mixed) return abip::launch_dense_mixed(dinst, b.count, dp, queue + i, ord, b.plan, variant, on);
+    return abip::launch_dense_group(dinst, b.count, dp, queue + i, ord, b.plan, h->gsp, variant, h->gscratch, h->gscratch_len,
+                                    (unsigned long long)h->prm.barrier_limit_ns, on);
+  };
+  if (nb == 1) return one(0, st);
+  cudaEvent_t fork = nullptr, join[abip::kDenseBuckets] = {};
+  cudaStream_t side[abip::kDenseBuckets] = {};
+  cudaError_t e = cudaEventCreateWithFlags(&fork, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = cudaEventRecord(fork, st);
+  for (int i = 0; i < nb && e == cudaSuccess; ++i) {
+    if (i == 0) {
+      e = one(0, st);
+      continue;
+    }
+    e = cudaStreamCreateWithFlags(&side[i], cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(side[i], fork, 0);
+    if (e == cudaSuccess) e = one(i, side[i]);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&join[i], cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventRecord(join[i], side[i]);
+  }
+  for (int i = 1; i < nb; ++i)
+    if (join[i]) {
+      const cudaError_t w = cudaStreamWaitEvent(st, join[i], 0);
+      if (e == cudaSuccess) e = w;
+      cudaEventDestroy(join[i]);
+    } else if (side[i]) {
+      cudaStreamSynchronize(side[i]);   // a launch without its event: waited for here
+    }
+  for (int i = 1; i < nb; ++i)
+    if (side[i]) cudaStreamDestroy(side[i]);   // freed once its work is done
+  if (fork) cudaEventDestroy(fork);
+  return e;
+}
+
+// The solve launch: by groups of CTAs (h->buckets) when h->group, else one CTA per instance.
 int dense_run_solve(abip_handle* h, DenseInst* dinst, int* queue, int count, int grid, size_t smem,
                     const DenseParams& dp, cudaStream_t st, const int* order = nullptr, int variant = 0) {
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
-  cudaMemsetAsync(queue, 0, 8, st);
-  const bool grid_mode = h->group && h->gplan.grid_mode;
+  cudaMemsetAsync(queue, 0, sizeof(int) * abip::kDenseBuckets, st);
+  const bool grid_mode = h->group && h->buckets[0].plan.grid_mode;
   double* words = grid_mode ? h->gscratch + h->gscratch_len - 2 : nullptr;   // barrier counter, error word
   if (words) cudaMemsetAsync(words, 0, 16, st);
   cudaEventRecord(e0, st);
-  cudaError_t e = h->group ? abip::launch_dense_group(dinst, count, dp, queue, order, h->gplan, h->gsp, variant,
-                                                      h->gscratch, h->gscratch_len, (unsigned long long)h->prm.barrier_limit_ns, st)
+  cudaError_t e = h->group ? launch_buckets(h, dinst, queue, dp, st, order, variant)
                            : abip::launch_dense_solve(dinst, count, dp, queue, order, grid, smem, variant, st);
   cudaEventRecord(e1, st);
   int derr = 0;
@@ -608,7 +717,7 @@ int dense_run_solve(abip_handle* h, DenseInst* dinst, int* queue, int count, int
   if (e != cudaSuccess) return fail(h, ABIP_E_CUDA, std::string("dense solve: ") + cudaGetErrorString(e));
   if (derr != 0) return fail(h, device_error_code(derr), std::string("solve: ") + device_error_str(derr));
   h->kernel_s = ms * 1e-3;
-  h->launches = 1;
+  h->launches = h->group ? (int64_t)h->buckets.size() : 1;
   return ABIP_OK;
 }
 
@@ -648,7 +757,7 @@ void setup_direct(abip_handle* h, const HostCSR& A) {
   const size_t scratch_len = abip::dense_group_scratch(m, n, sms);
   auto layout = [&](Arena& ar) {
     dinst = ar.take<DenseInst>(1);
-    queue = ar.take<int>(2);
+    queue = ar.take<int>(abip::kDenseBuckets);
     I.L = ar.take<double>((size_t)m * m);
     I.Li = ar.take<double>((size_t)m * mp);
     I.LiT = ar.take<double>((size_t)m * mp);
@@ -703,7 +812,7 @@ void setup_direct(abip_handle* h, const HostCSR& A) {
   h->hinst = I;
   h->dinst = dinst;
   h->queue = queue;
-  h->gplan = plan;
+  h->buckets = {abip::DenseBucket{plan, 0, 1}};
   h->gsp = sp;
   h->gscratch = scratch;
   h->gscratch_len = scratch_len;
@@ -1101,19 +1210,19 @@ int abip_setup(const abip_matrix* A, const double* b, const double* c, const abi
       hi[0].m = m; hi[0].n = n; hi[0].b = hb; hi[0].c = hc;
       rc = read_matrix_dense(h, A, hi[0].A);
       std::vector<DenseInst> hd;
-      h->group = !h->mixed && !prm.bb_beta &&
-                 abip::plan_dense_group(&m, &n, 1, abip::dense_max_ctas(h->device), h->gplan) != 0;
+      std::vector<int> ord;
+      h->group = !prm.bb_beta && plan_buckets(h, {{m, n}}, true, h->mixed != 0, abip::dense_max_ctas(h->device), ord);
       if (rc == ABIP_OK) {
         rc = dense_alloc(h, hi, &h->arena, &h->dinst, &h->queue, hd, h->mixed != 0, prm.bb_beta != 0, h->group);
-        if (rc == ABIP_E_OOM && h->group) {   // without the group's copies of A^T and the factor's inverse
+        if (rc == ABIP_E_OOM && h->group && !h->mixed) {   // without the group's copies of A^T and the factor's inverse
           h->group = false;
           rc = dense_alloc(h, hi, &h->arena, &h->dinst, &h->queue, hd, false, false, false);
         }
       }
       if (rc == ABIP_OK) {
         h->hinst = hd[0];
-        rc = dense_run_setup(h, h->dinst, h->queue, 1, 1, dense_setup_smem(m, n), m, h->group ? n : 0,
-                             h->mixed || h->group, 0);
+        rc = dense_run_setup(h, h->dinst, h->queue, 1, 1, dense_setup_smem(m, n), m,
+                             h->group && !h->mixed ? n : 0, h->mixed || h->group, 0);
       }
       if (rc == ABIP_OK) {
         cudaMemcpy(&h->hinst, h->dinst, sizeof(DenseInst), cudaMemcpyDeviceToHost);
@@ -1259,28 +1368,36 @@ int abip_solve_batch(int32_t count, const abip_matrix* A, const double* const* b
   int* queue = nullptr;
   std::vector<DenseInst> hd;
   const int sms = abip::dense_max_ctas(tmp.device);
+  // hand-out order: largest first (the batch's wall time is its slowest instance), or as given
+  std::vector<int> ord;
   {
-    std::vector<int> ms(count), ns(count);
-    for (int k = 0; k < count; ++k) { ms[k] = hi[k].m; ns[k] = hi[k].n; }
-    tmp.group = !mixed && !prm.bb_beta && abip::plan_dense_group(ms.data(), ns.data(), count, sms, tmp.gplan) != 0;
+    std::vector<std::pair<int, int>> sizes(count);
+    for (int k = 0; k < count; ++k) sizes[k] = {hi[k].m, hi[k].n};
+    const bool largest_first = prm.batch_order == 1;
+    tmp.group = !prm.bb_beta && plan_buckets(&tmp, sizes, largest_first, mixed, sms, ord);
+    if (!tmp.group) {   // one CTA per instance
+      ord.clear();
+      if (largest_first && count > 1) {
+        ord.resize(count);
+        for (int k = 0; k < count; ++k) ord[k] = k;
+        std::stable_sort(ord.begin(), ord.end(), [&](int a, int b) {
+          const double ca = (double)hi[a].m * hi[a].n + (double)hi[a].m * hi[a].m;
+          const double cb = (double)hi[b].m * hi[b].n + (double)hi[b].m * hi[b].m;
+          return ca > cb;
+        });
+      }
+    }
   }
+  if (mixed && !tmp.group) return fail(nullptr, ABIP_E_UNSUPPORTED, "an instance does not fit the shared memory of a cluster");
   tmp.prm = prm;
   int rc = dense_alloc(&tmp, hi, &arena, &dinst, &queue, hd, mixed, prm.bb_beta != 0, tmp.group);
-  if (rc == ABIP_E_OOM && tmp.group) {   // without the group's copies of A^T and the factor's inverse
+  if (rc == ABIP_E_OOM && tmp.group && !mixed) {   // without the group's copies of A^T and the factor's inverse
     tmp.group = false;
     rc = dense_alloc(&tmp, hi, &arena, &dinst, &queue, hd, mixed, false, false);
   }
   if (rc) return fail(nullptr, rc, tmp.err);
-  // hand-out order: largest first (the batch's wall time is its slowest instance)
   int* order = nullptr;
-  if (prm.batch_order == 1 && count > 1) {
-    std::vector<int> ord(count);
-    for (int k = 0; k < count; ++k) ord[k] = k;
-    std::stable_sort(ord.begin(), ord.end(), [&](int a, int b) {
-      const double ca = (double)hi[a].m * hi[a].n + (double)hi[a].m * hi[a].m;
-      const double cb = (double)hi[b].m * hi[b].n + (double)hi[b].m * hi[b].m;
-      return ca > cb;
-    });
+  if (!ord.empty()) {
     if (cudaMalloc(&order, count * sizeof(int)) != cudaSuccess) {
       cudaGetLastError();
       cudaFree(arena);
@@ -1289,8 +1406,13 @@ int abip_solve_batch(int32_t count, const abip_matrix* A, const double* const* b
     cudaMemcpy(order, ord.data(), count * sizeof(int), cudaMemcpyHostToDevice);
   }
   const DenseParams dp = dense_params(prm);
-  rc = dense_run_setup(&tmp, dinst, queue, count, std::min(count, sms * 4), smem_setup, mmax, tmp.group ? nmax : 0,
-                       mixed || tmp.group, st);
+  rc = dense_run_setup(&tmp, dinst, queue, count, std::min(count, sms * 4), smem_setup, mmax,
+                       tmp.group && !mixed ? nmax : 0, mixed || tmp.group, st);
+  auto ctas_per_sm = [&](int v) {
+    if (!tmp.group) return abip::dense_solve_ctas_per_sm(smem_solve, v);
+    const abip::DenseGroupPlan& p = tmp.buckets[0].plan;
+    return mixed ? abip::dense_mixed_ctas_per_sm(p, v) : abip::dense_group_ctas_per_sm(p, v);
+  };
   // occupancy variant: 0, or the autotuner's (cached, or timed on this batch)
   int variant = 0, tuned = 0;
   if (!rc && prm.autotune) {
@@ -1309,8 +1431,7 @@ int abip_solve_batch(int32_t count, const abip_matrix* A, const double* const* b
       probe.bb = 0;
       double best_s = 1e300;
       for (int v = 0; v < abip::kDenseVariants && !rc; ++v) {
-        const int per_v = tmp.group ? abip::dense_group_ctas_per_sm(tmp.gplan, v)
-                                    : abip::dense_solve_ctas_per_sm(mixed, smem_solve, v);
+        const int per_v = ctas_per_sm(v);
         if (per_v < 1) continue;
         rc = dense_run_solve(&tmp, dinst, queue, count, std::min(count, sms * per_v), smem_solve, probe, st, order, v);
         if (!rc && tmp.kernel_s < best_s) { best_s = tmp.kernel_s; variant = v; }
@@ -1321,8 +1442,7 @@ int abip_solve_batch(int32_t count, const abip_matrix* A, const double* const* b
       tune_store(tc);
     }
   }
-  const int per = std::max(1, tmp.group ? abip::dense_group_ctas_per_sm(tmp.gplan, variant)
-                                        : abip::dense_solve_ctas_per_sm(mixed, smem_solve, variant));
+  const int per = std::max(1, ctas_per_sm(variant));
   const int grid = std::min(count, sms * per);
   if (!rc) rc = dense_run_solve(&tmp, dinst, queue, count, grid, smem_solve, dp, st, order, variant);
   if (!rc) {

@@ -244,7 +244,7 @@ struct DenseParams {
   double beta, gamma, alpha, eps;
   int64_t max_admm;
   int32_t warmstart, stop_rule;
-  int32_t mixed;          // 1: FP32 iterates with FP64 termination decisions
+  int32_t mixed;          // 1: FP64 state, FP32 products of changes
   int32_t check_every;    // mixed: minimum spacing of FP64 confirmations (updates)
   int32_t bb;             // 1: Barzilai-Borwein beta at each outer iteration (FP64 path)
   int32_t bb_max_redo;
@@ -283,8 +283,11 @@ struct DenseGroupPlan {
   size_t smem;
   int sparse;                // 1: products with A over its CSR rows and columns (GroupSparse)
 };
-// the plan for a batch (sizes m[k], n[k]); 0 if no group holds its vectors in shared memory
-int plan_dense_group(const int* m, const int* n, int count, int sms, DenseGroupPlan& plan);
+// the plan of one LP over the cooperative grid, and of `count` LPs by clusters of C CTAs (more
+// where their vectors do not fit); 0 if no group holds the vectors in shared memory.  budget:
+// bytes of shared memory that copies of matrices and vectors may fill
+int plan_dense_grid(int m, int n, int sms, DenseGroupPlan& plan);
+int plan_dense_cluster(const int* m, const int* n, int count, int C, size_t budget, DenseGroupPlan& plan);
 // Rows up to which the sparse direct projection forms L^{-1}: m^2 multiply-adds over the SMs per
 // update against two sweeps along the elimination tree at about 2.8 us per dependent link
 // (grid flow, us per update, sweeps / inverse: m = 255 309 / 12, 1023 631 / 23, 1599 903 / 29),
@@ -299,11 +302,24 @@ cudaError_t launch_dense_group(DenseInst* inst, int count, const DenseParams& pr
                                const DenseGroupPlan& plan, const GroupSparse& sp, int variant, double* scratch,
                                size_t scratch_len, unsigned long long limit_ns, cudaStream_t st);
 int dense_group_ctas_per_sm(const DenseGroupPlan& plan, int variant);
+
+// Mixed-precision solve by clusters of CTAs (dense_mixed.cu): the same results for every size
+int plan_dense_mixed(const int* m, const int* n, int count, int C, size_t budget, DenseGroupPlan& plan);
+cudaError_t launch_dense_mixed(DenseInst* inst, int count, const DenseParams& prm, int* queue, const int* order,
+                               const DenseGroupPlan& plan, int variant, cudaStream_t st);
+int dense_mixed_ctas_per_sm(const DenseGroupPlan& plan, int variant);
+
+// The instances [first, first + count) of the hand-out order, solved with one plan.
+constexpr int kDenseBuckets = 5;   // cluster sizes 1, 2, 4, 8, 16
+struct DenseBucket {
+  DenseGroupPlan plan;
+  int first, count;
+};
 // Occupancy variants of the dense solve kernel (the batch autotuner's choice)
 constexpr int kDenseVariants = 3;
 cudaError_t launch_dense_solve(DenseInst* inst, int count, DenseParams prm, int* queue, const int* order,
                                int grid, size_t smem, int variant, cudaStream_t st);
-int dense_solve_ctas_per_sm(bool mixed, size_t smem, int variant);
+int dense_solve_ctas_per_sm(size_t smem, int variant);
 int dense_max_ctas(int device);
 cudaError_t launch_dense_backward(BackwardInst* insts, int count, int grid, cudaStream_t st);
 inline size_t backward_work_doubles(int m, int n) { return 2 * (size_t)m + 4 * (size_t)n + 5 * ((size_t)m + n + 2); }
@@ -394,8 +410,8 @@ struct abip_handle {
   int grid = 0;
   // dense path
   abip::DenseInst* dinst = nullptr;   // device, one entry
-  bool group = false;                 // FP64 solve by a group of CTAs (gplan)
-  abip::DenseGroupPlan gplan{};
+  bool group = false;                 // solve by groups of CTAs (buckets; one for one LP)
+  std::vector<abip::DenseBucket> buckets;
   double* gscratch = nullptr;         // its grid mode's scratch, gscratch_len doubles
   size_t gscratch_len = 0;
   // sparse direct projection of an LP with few rows: path 0 with group set, its own arena

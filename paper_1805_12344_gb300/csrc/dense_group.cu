@@ -35,38 +35,19 @@
 
 #include "abip_device.cuh"
 #include "abip_internal.h"
+#include "dense_device.cuh"
 
 namespace cg = cooperative_groups;
 
 namespace abip {
 namespace {
 
-constexpr int kThr = 256;
-constexpr int kWarps = kThr / 32;
+using dense::kWarps;
+using dense::sum_together;
+constexpr int kThr = dense::kThreads;
 constexpr int kSums = 11;   // the nine of the tests and the two of H^T z
 
 enum Act : int { ACT_STEP = 0, ACT_WARM = 1, ACT_STOP = 2 };
-
-// Sums of P per-lane values over the warp, P a power of two <= 32: halving exchanges, then a
-// butterfly over the rest.  Lane l receives the sum of value l >> (5 - log2 P).
-template <int P>
-__device__ __forceinline__ double sum_together(double (&a)[P], int lane) {
-  int o = 16;
-#pragma unroll
-  for (int h = P / 2; h > 0; h >>= 1, o >>= 1) {
-    const bool up = (lane & o) != 0;
-#pragma unroll
-    for (int k = 0; k < h; ++k) {
-      const double send = up ? a[k] : a[k + h];
-      const double keep = up ? a[k + h] : a[k];
-      a[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-    }
-  }
-  double v = a[0];
-#pragma unroll
-  for (; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
 
 // out(which, i, sum_j M[row0 + i][j] v_which[j]) for i < rows: R rows per warp at a time, NV
 // vectors; rows of M are ld (even) doubles, 16-byte aligned and zero-padded like v0, v1.
@@ -744,8 +725,9 @@ __global__ void __launch_bounds__(kThr, 1) dense_grid_kernel(GroupArgs Q) {
 using ClusterFn = void (*)(GroupArgs);
 ClusterFn cluster_fn(int variant, bool sparse) {
   if (sparse) return dense_cluster_kernel<1, true>;
-  return variant == 2 ? dense_cluster_kernel<3, false> : variant == 1 ? dense_cluster_kernel<2, false>
-                                                                      : dense_cluster_kernel<1, false>;
+  // a batch plans two CTAs per SM, so that is the default
+  return variant == 2 ? dense_cluster_kernel<3, false> : variant == 1 ? dense_cluster_kernel<1, false>
+                                                                      : dense_cluster_kernel<2, false>;
 }
 ClusterFn grid_fn(bool sparse) { return sparse ? dense_grid_kernel<true> : dense_grid_kernel<false>; }
 
@@ -789,6 +771,10 @@ constexpr size_t kSmemMax = 224 * 1024;
 
 cudaError_t cluster_config(ClusterFn f, int C, size_t smem, cudaLaunchConfig_t& cfg, cudaLaunchAttribute* at) {
   cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
+  // one split of the SM's memory for every launch, so that buckets of different shared memory
+  // run side by side on an SM (a mixed batch of 128 LPs, 200 updates: 17.9 -> 11.7 ms)
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
   if (e == cudaSuccess && C > 8) e = cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   cfg.blockDim = dim3(kThr);
   cfg.gridDim = dim3((unsigned)C);
@@ -804,39 +790,16 @@ cudaError_t cluster_config(ClusterFn f, int C, size_t smem, cudaLaunchConfig_t& 
 
 }  // namespace
 
-int plan_dense_group(const int* m, const int* n, int count, int sms, DenseGroupPlan& plan) {
-  plan = DenseGroupPlan{};
-  // FP64 operations of one update of the largest instance: its products, and about 80 a
-  // column and row for the steps and sums
-  int64_t wmax = 0;
-  for (int k = 0; k < count; ++k)
-    wmax = std::max(wmax, 3 * (int64_t)m[k] * n[k] + (int64_t)m[k] * m[k] + 80 * (int64_t)(m[k] + n[k]));
-  // CTAs per instance: up to two CTAs per SM over the batch, while a CTA keeps more than 5000
-  // operations (2.5k clocks; the four barriers cost about as much).  Measured, us per update
-  // with 1 / 2 / 4 / 8 / 16 CTAs: 16 x 48 11.6 / 10.6 / 10.0 / 10.1 / 10.9; 50 x 120 19.0 /
-  // 13.5 / 11.9 / 11.1 / 11.1; 100 x 300 53 / 31 / 19.7 / 14.5 / 13.1; 512 x 1154 578 / 298 /
-  // 153 / 83 / 51; 64 LPs of m 16 .. 256 222 / 117 / 65 / 98 / 163.
-  int C = 1;
-  while (C < 16 && 2 * C * (int64_t)count <= 2 * sms && wmax / C > 5000) C *= 2;
-  // One LP over the whole grid: its barriers cost more than a cluster's, its 152 SMs take over
-  // from 16 at about 8e5 operations (cluster of 16 / grid: 200 x 600 20.6 / 23.7 us, 256 x
-  // 1024 25.2 / 24.2, 300 x 900 30.8 / 24.5, 512 x 1154 50.7 / 26.4).
-  plan.grid_mode = count == 1 && wmax > 800000;
-  if (plan.grid_mode) {
-    const SmemPlan s = plan_smem(m, n, count, sms, true, kSmemMax - 16);
-    plan.ctas = sms;
-    plan.smem = s.bytes;
-    plan.cache_vec = s.cache_vec;
-    plan.cache_mat = s.cache_mat;
-    return 1;
-  }
+int plan_dense_grid(int m, int n, int sms, DenseGroupPlan& plan) {
+  const SmemPlan s = plan_smem(&m, &n, 1, sms, true, kSmemMax - 16);
+  plan = DenseGroupPlan{sms, 1, s.cache_vec, s.cache_mat, s.bytes, 0};
+  return s.bytes <= kSmemMax;
+}
+
+int plan_dense_cluster(const int* m, const int* n, int count, int C, size_t budget, DenseGroupPlan& plan) {
   for (;; C *= 2) {
-    const size_t budget = C * (int64_t)count > sms ? 100 * 1024 : kSmemMax - 16;
     const SmemPlan s = plan_smem(m, n, count, C, false, budget);
-    plan.ctas = C;
-    plan.smem = s.bytes;
-    plan.cache_vec = s.cache_vec;
-    plan.cache_mat = s.cache_mat;
+    plan = DenseGroupPlan{C, 0, s.cache_vec, s.cache_mat, s.bytes, 0};
     if (s.bytes <= kSmemMax) return 1;
     if (C >= 8) return 0;
   }

@@ -15,13 +15,13 @@
 
 #include "abip_device.cuh"
 #include "abip_internal.h"
+#include "dense_device.cuh"
 
 namespace abip {
 
 namespace {
 
-constexpr int kThreads = 256;
-constexpr int kWarps = kThreads / 32;
+using namespace dense;
 
 // next instance id from the work queue (thread 0), broadcast to the CTA; `order` (may be
 // null) lists the instances in the order they are handed out
@@ -34,59 +34,6 @@ __device__ __forceinline__ int next_instance(int* queue, int count, const int* o
   }
   __syncthreads();
   return s_id;
-}
-
-// w <- L^{-1} w, L lower triangular (row-major, leading dimension m), w in shared memory.
-template <typename T>
-__device__ void trsv_lower(const T* __restrict__ L, int m, T* w) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  for (int kb = 0; kb < m; kb += 32) {
-    const int nb = min(32, m - kb);
-    if (wid == 0) {
-      T wl = lane < nb ? w[kb + lane] : T(0);
-      for (int j = 0; j < nb; ++j) {
-        if (lane == j) wl = wl / L[(size_t)(kb + j) * m + kb + j];
-        const T wj = __shfl_sync(0xffffffffu, wl, j);
-        if (lane > j && lane < nb) wl -= L[(size_t)(kb + lane) * m + kb + j] * wj;
-      }
-      if (lane < nb) w[kb + lane] = wl;
-    }
-    __syncthreads();
-    const T wb = lane < nb ? w[kb + lane] : T(0);
-    for (int i = kb + nb + wid; i < m; i += kWarps) {
-      T a = lane < nb ? L[(size_t)i * m + kb + lane] * wb : T(0);
-      a = warp_sum(a);
-      if (lane == 0) w[i] -= a;
-    }
-    __syncthreads();
-  }
-}
-
-// w <- L^{-T} w.
-template <typename T>
-__device__ void trsv_lower_t(const T* __restrict__ L, int m, T* w) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int nblk = (m + 31) / 32;
-  for (int bk = nblk - 1; bk >= 0; --bk) {
-    const int kb = bk * 32;
-    const int nb = min(32, m - kb);
-    if (wid == 0) {
-      T wl = lane < nb ? w[kb + lane] : T(0);
-      for (int j = nb - 1; j >= 0; --j) {
-        if (lane == j) wl = wl / L[(size_t)(kb + j) * m + kb + j];
-        const T zj = __shfl_sync(0xffffffffu, wl, j);
-        if (lane < j) wl -= L[(size_t)(kb + j) * m + kb + lane] * zj;
-      }
-      if (lane < nb) w[kb + lane] = wl;
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < kb; i += kThreads) {
-      T a = T(0);
-      for (int j = 0; j < nb; ++j) a += L[(size_t)(kb + j) * m + i] * w[kb + j];
-      w[i] -= a;
-    }
-    __syncthreads();
-  }
 }
 
 // out[i] = sum_j A_ij v_j (warp per row, accumulated in Acc); optional second vector.
@@ -632,318 +579,7 @@ __device__ void dense_solve_one(DenseInst& I, const DenseParams& P, T* sm, doubl
 // accuracy floor.  Every kDeltaRefresh updates, and whenever the Sec. 4.1 tests pass on
 // the maintained sums with a factor-4 margin, the products are recomputed exactly in
 // FP64; the tests are decided on the exact sums.
-constexpr int kDeltaRefresh = 100;
-
-// o0[i] += sum_j M[i][j] v0[j] (and o1 with v1) for rows i < rows: each warp takes four
-// rows at a time (rows w, w + 8, w + 16, w + 24 of a group of 32), float4 loads, FP32
-// accumulation, so that four rows' loads are in flight per warp.  M rows are ldm floats
-// (a multiple of 4, zero padded); v0, v1 hold ldm floats, 16-byte aligned.  f0
-// (optional) receives the FP32 row sums.
-template <bool TWO>
-__device__ void rows_f32(const float* __restrict__ M, int ldm, int rows, const float* v0, const float* v1,
-                         double* o0, double* o1, float* f0) {
-  constexpr int R = 4;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int nq = ldm / 4;
-  const float4* p0 = reinterpret_cast<const float4*>(v0);
-  const float4* p1 = reinterpret_cast<const float4*>(v1);
-  for (int g = 0; g < rows; g += R * kWarps) {
-    float a0[R], a1[R];
-    const float4* r[R];
-#pragma unroll
-    for (int q = 0; q < R; ++q) {
-      a0[q] = 0.f;
-      a1[q] = 0.f;
-      const int i = g + wid + q * kWarps;
-      r[q] = reinterpret_cast<const float4*>(M + (size_t)min(i, rows - 1) * ldm);
-    }
-    for (int t = lane; t < nq; t += 32) {
-      const float4 x = p0[t];
-      float4 z = x;
-      if (TWO) z = p1[t];
-#pragma unroll
-      for (int q = 0; q < R; ++q) {
-        const float4 a = r[q][t];
-        a0[q] += a.x * x.x + a.y * x.y + a.z * x.z + a.w * x.w;
-        if (TWO) a1[q] += a.x * z.x + a.y * z.y + a.z * z.z + a.w * z.w;
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < R; ++q) {
-      const int i = g + wid + q * kWarps;
-      const float s0 = warp_sum(a0[q]);
-      const float s1 = TWO ? warp_sum(a1[q]) : 0.f;
-      if (lane == 0 && i < rows) {
-        o0[i] += (double)s0;
-        if (TWO) o1[i] += (double)s1;
-        if (f0) f0[i] = s0;
-      }
-    }
-  }
-}
-
-__device__ void dense_solve_delta(DenseInst& I, const DenseParams& P, unsigned char* smraw, double* red) {
-  const int m = I.m, n = I.n;
-  const int64_t ld = I.ld;
-  double* y = reinterpret_cast<double*>(smraw);
-  double* Ax = y + m;
-  double* As = Ax + m;
-  double* zy = As + m;
-  double* qp = zy + m;
-  double* x = qp + m;
-  double* s = x + n;
-  double* ATy = s + n;
-  double* ATz = ATy + n;
-  const int mp = I.ldtf, np = I.ldf;
-  float* dy = reinterpret_cast<float*>(smraw + (((size_t)(5 * m + 4 * n) * 8 + 15) / 16) * 16);
-  float* dq = dy + mp;
-  float* dz = dq + mp;
-  float* dx = dz + mp;
-  float* ds = dx + np;
-  const double alpha = P.alpha, beta = P.beta, gamma = P.gamma, eps = P.eps;
-  const double zbar = I.zbar, xi = -(double)n - 1.0, nb = I.nb, nc = I.nc;
-  const double Ki0 = I.Kinv[0], Ki1 = I.Kinv[1], Ki2 = I.Kinv[2], Ki3 = I.Kinv[3];
-  double tau = 1.0, kappa = 1.0, theta = 1.0, mu = beta;
-  int64_t total = 0;
-  int outer = 0, status = 0;
-  if (I.resume) {
-    for (int i = threadIdx.x; i < m; i += kThreads) y[i] = I.y[i];
-    for (int j = threadIdx.x; j < n; j += kThreads) { x[j] = I.x[j]; s[j] = I.s[j]; }
-    tau = I.r_tau; kappa = I.r_kappa; theta = I.r_theta; mu = I.r_mu;
-    total = I.r_iters;
-    outer = I.r_outer;
-  } else {
-    for (int i = threadIdx.x; i < m; i += kThreads) y[i] = 0.0;
-    for (int j = threadIdx.x; j < n; j += kThreads) { x[j] = 1.0; s[j] = 1.0; }
-  }
-  // the padding of the FP32 vectors meets zero padding of the FP32 matrices
-  for (int i = threadIdx.x; i < 3 * mp + 2 * np; i += kThreads) dy[i] = 0.f;
-  __syncthreads();
-  int64_t since_refresh = 0, next_confirm = 0;
-  double inner2 = 0, pres = 0, dres = 0, dgap = 0, ctx = 0, bty = 0;
-
-  // exact FP64 products of the current state
-  auto refresh = [&]() {
-    gemv_rows<true, double>(I.A, ld, m, n, x, s, Ax, As);
-    __syncthreads();
-    for (int i = threadIdx.x; i < m; i += kThreads) {
-      const double q = y[i] - (Ax[i] + As[i]);
-      qp[i] = q;
-      zy[i] = q;
-    }
-    __syncthreads();
-    trsv_lower<double>(I.L, m, zy);
-    trsv_lower_t<double>(I.L, m, zy);
-    for (int j = threadIdx.x; j < n; j += kThreads) {
-      double a0 = 0.0, a1 = 0.0;
-      for (int i = 0; i < m; ++i) {
-        const double aij = I.A[(size_t)i * ld + j];
-        a0 += aij * y[i];
-        a1 += aij * zy[i];
-      }
-      ATy[j] = a0;
-      ATz[j] = a1;
-    }
-    __syncthreads();
-    since_refresh = 0;
-  };
-  // the nine sums from the maintained products (as residual_sums)
-  auto sums = [&](double (&out)[9]) {
-    double acc[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
-    const double itau = 1.0 / tau;
-    for (int i = threadIdx.x; i < m; i += kThreads) {
-      const double ax = Ax[i], bi = I.b[i], yi = y[i], bb = I.bbar[i];
-      const double ry = ax - bi * tau + bb * theta;
-      const double pr = ax * itau - bi;
-      acc[0] += ry * ry; acc[1] += pr * pr; acc[3] += ax * ax;
-      acc[5] += bi * yi; acc[6] += bb * yi;
-    }
-    for (int j = threadIdx.x; j < n; j += kThreads) {
-      const double aty = ATy[j], sj = s[j], cj = I.c[j], cb = I.cbar[j], xj = x[j];
-      const double rx = -aty + cj * tau - cb * theta - sj;
-      const double dr = (aty + sj) * itau - cj;
-      acc[0] += rx * rx; acc[2] += dr * dr; acc[4] += (aty + sj) * (aty + sj);
-      acc[7] += cj * xj; acc[8] += cb * xj;
-    }
-#pragma unroll
-    for (int k = 0; k < 9; ++k) out[k] = acc[k];
-    block_allsum<9>(out, red);
-  };
-  auto tests = [&](const double (&a)[9], double margin) -> int {
-    const double ps = sqrt(a[1]) / (1.0 + nb), dsn = sqrt(a[2]) / (1.0 + nc);
-    const double gp = fabs(a[7] / tau - a[5] / tau) / (1.0 + fabs(a[7] / tau) + fabs(a[5] / tau));
-    if (ps <= margin * eps && dsn <= margin * eps && gp <= margin * eps) return ABIP_OPTIMAL;
-    if (a[5] > 0 && sqrt(a[4]) <= margin * eps * a[5] / nb) return ABIP_PRIMAL_INFEASIBLE;
-    if (a[7] < 0 && sqrt(a[3]) <= margin * eps * (-a[7]) / nc) return ABIP_DUAL_INFEASIBLE;
-    return 0;
-  };
-  auto absorb = [&](const double (&a)[9]) {
-    bty = a[5];
-    ctx = a[7];
-    const double rt = a[5] - a[7] + zbar * theta - kappa;
-    const double rth = -a[6] + a[8] - zbar * tau - xi;
-    inner2 = a[0] + rt * rt + rth * rth;
-    pres = sqrt(a[1]) / (1.0 + nb);
-    dres = sqrt(a[2]) / (1.0 + nc);
-    dgap = fabs(ctx / tau - bty / tau) / (1.0 + fabs(ctx / tau) + fabs(bty / tau));
-  };
-  auto evaluate = [&](bool final_test) -> bool {
-    double a[9];
-    sums(a);
-    absorb(a);
-    if (!isfinite(inner2)) return false;
-    if (!final_test || P.stop_rule != 0) return true;
-    if (total >= next_confirm && tests(a, 4.0) != 0) {
-      refresh();
-      sums(a);
-      absorb(a);
-      status = tests(a, 1.0);
-      next_confirm = total + P.check_every;
-    }
-    return true;
-  };
-  // maintained products after a change (dy, dx, ds) of the iterate
-  auto maintain = [&]() {
-    rows_f32<true>(I.Af, np, m, dx, ds, Ax, As, nullptr);
-    rows_f32<false>(I.ATf, mp, n, dy, dy, ATy, ATy, nullptr);
-    __syncthreads();
-  };
-
-  refresh();
-  bool ok = evaluate(false);
-  while (ok) {
-    if (inner2 <= mu) {
-      const double gk = adaptive_gamma(gamma, P.gamma_max, eps, fmax(pres, fmax(dres, dgap)));
-      mu *= gk;
-      ++outer;
-      if (P.stop_rule == 1 && mu < eps) { status = ABIP_OPTIMAL; break; }
-      if (outer >= kMaxOuter) { status = ABIP_MAX_ITER; break; }
-      const double sg = sqrt(gk);
-      for (int j = threadIdx.x; j < n; j += kThreads) {
-        const double x0 = x[j], s0 = s[j];
-        if (P.warmstart == 1) { x[j] = x0 * sg; s[j] = s0 * sg; }
-        else if (x0 >= s0) s[j] = s0 * gk;
-        else x[j] = x0 * gk;
-        dx[j] = (float)(x[j] - x0);
-        ds[j] = (float)(s[j] - s0);
-      }
-      if (P.warmstart == 1) { tau *= sg; kappa *= sg; }
-      else if (tau >= kappa) kappa *= gk;
-      else tau *= gk;
-      for (int i = threadIdx.x; i < m; i += kThreads) {
-        const double y0 = y[i];
-        y[i] = y0 * sg;
-        dy[i] = (float)(y[i] - y0);
-      }
-      theta *= sg;
-      __syncthreads();
-      maintain();
-      ok = evaluate(false);
-      continue;
-    }
-    // projection on the change of q = y - A(x + s)
-    for (int i = threadIdx.x; i < m; i += kThreads) {
-      const double q = y[i] - (Ax[i] + As[i]);
-      dq[i] = (float)(q - qp[i]);
-      qp[i] = q;
-    }
-    __syncthreads();
-    // zy += G^{-1} dq (dz keeps the FP32 change), A^T zy += A^T dz
-    rows_f32<false>(I.Ginvf, mp, m, dq, dq, zy, zy, dz);
-    __syncthreads();
-    rows_f32<false>(I.ATf, mp, n, dz, dz, ATz, ATz, nullptr);
-    __syncthreads();
-    double hz[2] = {0.0, 0.0};
-    for (int j = threadIdx.x; j < n; j += kThreads) {
-      const double z = x[j] + s[j] + ATz[j];
-      hz[0] += I.c[j] * z;
-      hz[1] -= I.cbar[j] * z;
-    }
-    for (int i = threadIdx.x; i < m; i += kThreads) {
-      hz[0] -= I.b[i] * zy[i];
-      hz[1] += I.bbar[i] * zy[i];
-    }
-    block_allsum<2>(hz, red);
-    const double v1 = tau + kappa + hz[0], v2 = theta + xi + hz[1];
-    const double t1 = Ki0 * v1 + Ki1 * v2, t2 = Ki2 * v1 + Ki3 * v2;
-    const double cmu = mu / beta;
-    for (int i = threadIdx.x; i < m; i += kThreads) {
-      const double uy = zy[i] - I.g1[i] * t1 - I.g2[i] * t2;
-      const double y0 = y[i];
-      y[i] = alpha * uy + (1.0 - alpha) * y0;
-      dy[i] = (float)(y[i] - y0);
-    }
-    for (int j = threadIdx.x; j < n; j += kThreads) {
-      const double z = x[j] + s[j] + ATz[j];
-      const double ux = z - I.g1[m + j] * t1 - I.g2[m + j] * t2;
-      const double x0 = x[j], s0 = s[j];
-      const double xh = alpha * ux + (1.0 - alpha) * x0;
-      double xn, sn;
-      barrier_step_newton(xh - s0, cmu, xn, sn);   // few FP64 operations (the FP64 pipe binds here)
-      x[j] = xn;
-      s[j] = sn;
-      dx[j] = (float)(xn - x0);
-      ds[j] = (float)(sn - s0);
-    }
-    {
-      const double th_ = alpha * t1 + (1.0 - alpha) * tau;
-      double tn, kn;
-      barrier_step<double>(th_ - kappa, mu / beta, tn, kn);
-      tau = tn;
-      kappa = kn;
-      theta = alpha * t2 + (1.0 - alpha) * theta;
-    }
-    __syncthreads();
-    maintain();
-    ++total;
-    if (++since_refresh >= kDeltaRefresh) refresh();
-    ok = evaluate(true);
-    if (status != 0) break;
-    if (total >= P.max_admm) { status = ABIP_MAX_ITER; break; }
-  }
-  // outputs: raw state and the scaled candidate or certificate (Sec. 4.1)
-  double sx = 1.0 / tau, sy = 1.0 / tau;
-  if (status == ABIP_PRIMAL_INFEASIBLE) { sx = 1.0; sy = 1.0 / bty; }
-  if (status == ABIP_DUAL_INFEASIBLE) { sx = -1.0 / ctx; sy = 1.0; }
-  for (int i = threadIdx.x; i < m; i += kThreads) {
-    I.y[i] = y[i];
-    if (I.out_y) I.out_y[i] = y[i] * sy;
-  }
-  for (int j = threadIdx.x; j < n; j += kThreads) {
-    I.x[j] = x[j];
-    I.s[j] = s[j];
-    if (I.out_x) I.out_x[j] = x[j] * sx;
-    if (I.out_s) I.out_s[j] = s[j] * sy;
-  }
-  if (threadIdx.x == 0) {
-    I.tau = tau; I.kappa = kappa; I.theta = theta; I.mu = mu;
-    I.resume = 0;
-    I.pres = pres; I.dres = dres; I.dgap = dgap; I.ctx = ctx; I.bty = bty; I.obj = ctx / tau;
-    I.admm_iters = total; I.outer_iters = outer; I.status = status;
-    I.fp32_iters_lo = (int32_t)(total & 0x7fffffff);
-    I.fp32_iters_hi = (int32_t)(total >> 31);
-    if (!ok) I.err = DEV_ERR_NONFINITE;
-  }
-  __syncthreads();
-}
-
-// Solve kernels, one CTA per instance at a time.  MINB (resident CTAs per SM the
-// compiler plans registers for) is the knob of the batch autotuner: the variants run the
-// same arithmetic and differ only in occupancy.
-template <int MINB>
-__global__ void __launch_bounds__(kThreads, MINB) dense_solve_mixed_kernel(DenseInst* insts, int count,
-                                                                           DenseParams P, int* queue,
-                                                                           const int* order) {
-  extern __shared__ double sm_raw[];
-  __shared__ double red[32 * 9];
-  for (;;) {
-    const int id = next_instance(queue, count, order);
-    if (id < 0) return;
-    DenseInst& I = insts[id];
-    if (I.err != 0) continue;
-    dense_solve_delta(I, P, reinterpret_cast<unsigned char*>(sm_raw), red);
-  }
-}
+// The kernel is in dense_mixed.cu.
 
 template <typename T, int MINB>
 __global__ void __launch_bounds__(kThreads, MINB) dense_solve_kernel(DenseInst* insts, int count, DenseParams P,
@@ -1477,14 +1113,11 @@ cudaError_t launch_dense_setup(DenseInst* inst, int count, int* queue, int grid,
   return e;
 }
 
-// the solve kernel of a precision and an occupancy variant (0, 1, 2: MINB 1, 2, 3 for FP64
-// and 2, 3, 4 for mixed precision), with its dynamic shared memory limit raised
+// the FP64 solve kernel of an occupancy variant (0, 1, 2: MINB 1, 2, 3), with its dynamic shared
+// memory limit raised
 using DenseSolveFn = void (*)(DenseInst*, int, DenseParams, int*, const int*);
-DenseSolveFn dense_solve_fn(bool mixed, int variant) {
-  DenseSolveFn f;
-  if (mixed) f = variant == 2 ? dense_solve_mixed_kernel<4> : variant == 1 ? dense_solve_mixed_kernel<3>
-                                                                             : dense_solve_mixed_kernel<2>;
-  else f = variant == 2 ? dense_solve_kernel<double, 3> : variant == 1 ? dense_solve_kernel<double, 2>
+DenseSolveFn dense_solve_fn(int variant) {
+  const DenseSolveFn f = variant == 2 ? dense_solve_kernel<double, 3> : variant == 1 ? dense_solve_kernel<double, 2>
                                                                          : dense_solve_kernel<double, 1>;
   cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDenseSmemMax);
   return f;
@@ -1492,16 +1125,16 @@ DenseSolveFn dense_solve_fn(bool mixed, int variant) {
 
 cudaError_t launch_dense_solve(DenseInst* inst, int count, DenseParams prm, int* queue, const int* order,
                                int grid, size_t smem, int variant, cudaStream_t st) {
-  // the caller sizes smem for the largest instance: (5m + 3n) doubles (FP64), 48m + 40n bytes (mixed)
-  DenseSolveFn f = dense_solve_fn(prm.mixed != 0, variant);
+  // the caller sizes smem for the largest instance: (5m + 3n) doubles
+  DenseSolveFn f = dense_solve_fn(variant);
   cudaGetLastError();
   f<<<grid, kThreads, smem, st>>>(inst, count, prm, queue, order);
   return cudaGetLastError();
 }
 
-int dense_solve_ctas_per_sm(bool mixed, size_t smem, int variant) {
+int dense_solve_ctas_per_sm(size_t smem, int variant) {
   int per = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, dense_solve_fn(mixed, variant), kThreads, smem);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, dense_solve_fn(variant), kThreads, smem);
   return per;
 }
 
@@ -1611,12 +1244,12 @@ extern "C" ABIP_API int abip_solve_dense_noalloc(int32_t m, int32_t n, const dou
   cudaMemcpyAsync(dinst, &I, sizeof(I), cudaMemcpyHostToDevice, st);
   cudaMemsetAsync(queue, 0, 2 * sizeof(int), st);
   const size_t smem_setup = std::max((size_t)(2 * 32 * 33), (size_t)(2 * m + n)) * sizeof(double);
-  abip::dense_setup_kernel<true><<<1, abip::kThreads, smem_setup, st>>>(dinst, 1, queue);
+  abip::dense_setup_kernel<true><<<1, abip::dense::kThreads, smem_setup, st>>>(dinst, 1, queue);
   cudaMemsetAsync(queue, 0, 2 * sizeof(int), st);
   abip::DenseParams dp{prm.beta, prm.gamma, prm.alpha, prm.eps, prm.max_admm_iters, prm.warmstart,
                        prm.stop_rule, 0, 1, 0, 0, 0.0, 0.0, prm.gamma_max};
   const size_t smem_solve = (size_t)(5 * m + 3 * n) * sizeof(double);
-  abip::dense_solve_kernel<double, 1><<<1, abip::kThreads, smem_solve, st>>>(dinst, 1, dp, queue, nullptr);
+  abip::dense_solve_kernel<double, 1><<<1, abip::dense::kThreads, smem_solve, st>>>(dinst, 1, dp, queue, nullptr);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaMemcpyAsync(&I, dinst, sizeof(I), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
