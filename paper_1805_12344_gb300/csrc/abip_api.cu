@@ -465,9 +465,14 @@ int solve_grid_path(abip_handle* h, cudaStream_t st) {
 // dense CTA path (single instance and batches)
 // ---------------------------------------------------------------------------
 
+// One dense LP of a call: values read to the host and checked there (A row-major m x n), or, with
+// `dev`, the caller's device arrays, which are copied on the device and checked there.
 struct DenseHostInst {
   int m, n;
-  std::vector<double> A, b, c;   // A row-major m x n
+  std::vector<double> A, b, c;
+  const abip_matrix* dev = nullptr;
+  const double* dev_b = nullptr;
+  const double* dev_c = nullptr;
 };
 
 constexpr size_t kDenseSmemLimit = 200 * 1024;
@@ -491,10 +496,18 @@ size_t dense_setup_smem(int m, int n) { return (size_t)(2 * m + n) * sizeof(doub
 int dense_alloc(abip_handle* h, const std::vector<DenseHostInst>& hi, void** arena_out, DenseInst** dinst,
                 int** queue, std::vector<DenseInst>& hdesc, bool mixed = false, bool bb = false, bool group = false) {
   const int count = (int)hi.size();
+  abip::DenseSource* dsrc = nullptr;
+  int* flags = nullptr;
+  std::vector<abip::DenseSource> src(count);
+  auto is_f32 = [&](int k) { return hi[k].dev && hi[k].dev->dtype == ABIP_F32; };
   auto layout = [&](Arena& ar, std::vector<DenseInst>& d) {
     DenseInst* di = ar.take<DenseInst>(count);
     int* q = ar.take<int>(abip::kDenseBuckets);
     if (ar.base) { *dinst = di; *queue = q; }
+    dsrc = ar.take<abip::DenseSource>(count);
+    flags = ar.take<int>(count);
+    for (int k = 0; k < count; ++k)
+      src[k] = {is_f32(k) ? ar.take<float>((size_t)hi[k].m * hi[k].n) : nullptr, hi[k].n};
     d.assign(count, DenseInst{});
     for (int k = 0; k < count; ++k) {
       const int m = hi[k].m, n = hi[k].n;
@@ -539,32 +552,52 @@ int dense_alloc(abip_handle* h, const std::vector<DenseHostInst>& hi, void** are
   Arena ar;
   ar.base = static_cast<char*>(mem);
   layout(ar, hdesc);
-  cudaMemset(mem, 0, probe.off);
+  cudaError_t e = cudaMemsetAsync(mem, 0, probe.off, 0);
+  // the inputs, on the default stream as every copy of a call's inputs; host arrays return read
+  auto copy = [&](const double* dst, const double* from, size_t len, cudaMemcpyKind kind) {
+    if (e == cudaSuccess) e = cudaMemcpyAsync(const_cast<double*>(dst), from, len * 8, kind, 0);
+  };
+  auto copy2d = [&](const void* dst, size_t dld, const void* from, size_t sld, size_t width, size_t rows, cudaMemcpyKind kind) {
+    if (e != cudaSuccess) return;
+    if (dld == width && sld == width) e = cudaMemcpyAsync(const_cast<void*>(dst), from, width * rows, kind, 0);
+    else e = cudaMemcpy2DAsync(const_cast<void*>(dst), dld, from, sld, width, rows, kind, 0);
+  };
   for (int k = 0; k < count; ++k) {
     const DenseInst& I = hdesc[k];
-    if (I.ld == I.n)
-      cudaMemcpy((void*)I.A, hi[k].A.data(), hi[k].A.size() * 8, cudaMemcpyHostToDevice);
-    else
-      cudaMemcpy2D((void*)I.A, I.ld * 8, hi[k].A.data(), (size_t)I.n * 8, (size_t)I.n * 8, I.m, cudaMemcpyHostToDevice);
-    cudaMemcpy((void*)I.b, hi[k].b.data(), hi[k].m * 8, cudaMemcpyHostToDevice);
-    cudaMemcpy((void*)I.c, hi[k].c.data(), hi[k].n * 8, cudaMemcpyHostToDevice);
-    if (mixed) {   // padded FP32 copies of A and A^T (padding stays 0 from the memset)
-      const int m = hi[k].m, n = hi[k].n;
-      std::vector<float> f((size_t)m * I.ldf, 0.f), ft((size_t)n * I.ldtf, 0.f);
-      for (int i = 0; i < m; ++i)
-        for (int j = 0; j < n; ++j) {
-          const float v = (float)hi[k].A[(size_t)i * n + j];
-          f[(size_t)i * I.ldf + j] = v;
-          ft[(size_t)j * I.ldtf + i] = v;
-        }
-      cudaMemcpy((void*)I.Af, f.data(), f.size() * 4, cudaMemcpyHostToDevice);
-      cudaMemcpy((void*)I.ATf, ft.data(), ft.size() * 4, cudaMemcpyHostToDevice);
+    const size_t n = I.n, m = I.m;
+    if (const abip_matrix* A = hi[k].dev) {
+      if (src[k].f32) copy2d(src[k].f32, n * 4, A->val, (size_t)A->ld * 4, n * 4, m, cudaMemcpyDeviceToDevice);
+      else copy2d(I.A, I.ld * 8, A->val, (size_t)A->ld * 8, n * 8, m, cudaMemcpyDeviceToDevice);
+      copy(I.b, hi[k].dev_b, m, cudaMemcpyDeviceToDevice);
+      copy(I.c, hi[k].dev_c, n, cudaMemcpyDeviceToDevice);
+    } else {
+      copy2d(I.A, I.ld * 8, hi[k].A.data(), n * 8, n * 8, m, cudaMemcpyHostToDevice);
+      copy(I.b, hi[k].b.data(), m, cudaMemcpyHostToDevice);
+      copy(I.c, hi[k].c.data(), n, cudaMemcpyHostToDevice);
     }
   }
-  cudaMemcpy(*dinst, hdesc.data(), sizeof(DenseInst) * count, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(dsrc, src.data(), sizeof(abip::DenseSource) * count, cudaMemcpyHostToDevice, 0);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(*dinst, hdesc.data(), sizeof(DenseInst) * count, cudaMemcpyHostToDevice, 0);
+  int mmax = 0, nmax = 0;
+  for (int k = 0; k < count; ++k) { mmax = std::max(mmax, hi[k].m); nmax = std::max(nmax, hi[k].n); }
+  if (e == cudaSuccess) e = abip::launch_dense_ingest(*dinst, dsrc, flags, count, mmax, nmax, abip::dense_max_ctas(h->device), 0);
+  std::vector<int> bad(count, 0);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(bad.data(), flags, sizeof(int) * count, cudaMemcpyDeviceToHost, 0);
+  const cudaError_t es = cudaStreamSynchronize(0);
+  if (e == cudaSuccess) e = es;
+  int rc = ABIP_OK;
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    rc = fail(h, ABIP_E_CUDA, std::string("dense copies: ") + cudaGetErrorString(e));
+  }
+  for (int k = 0; k < count && rc == ABIP_OK; ++k)
+    if (bad[k]) rc = fail(h, ABIP_E_INVALID_ARG, std::string(bad[k] & 1 ? "A has" : "b or c has") + " non-finite entries" +
+                                                     (count > 1 ? " (instance " + std::to_string(k) + ")" : ""));
+  if (rc != ABIP_OK) {
+    cudaFree(mem);
+    return rc;
+  }
   *arena_out = mem;
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return fail(h, ABIP_E_CUDA, std::string("dense copies: ") + cudaGetErrorString(e));
   return ABIP_OK;
 }
 
@@ -987,6 +1020,21 @@ int read_matrix_csr(abip_handle* h, const abip_matrix* A, HostCSR& out, bool& f3
   return ABIP_OK;
 }
 
+// Whether a dense A with its b and c is read where it is: device memory of this device, all three
+// (anything else goes through the host, with that route's errors).
+bool stays_on_device(const abip_matrix* A, const double* b, const double* c, int device) {
+  if (A->fmt != ABIP_DENSE_ROWMAJOR || !A->on_device) return false;
+  for (const void* p : {A->val, (const void*)b, (const void*)c}) {
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    if (at.type != cudaMemoryTypeDevice || at.device != device) return false;
+  }
+  return true;
+}
+
 int validate_matrix(abip_handle* h, const abip_matrix* A) {
   if (!A) return fail(h, ABIP_E_INVALID_ARG, "A is NULL");
   if (A->m < 1 || A->n < A->m) return fail(h, ABIP_E_DIM, "need 1 <= m <= n");
@@ -1158,12 +1206,17 @@ int abip_setup(const abip_matrix* A, const double* b, const double* c, const abi
   const int m = A->m, n = A->n;
   std::vector<double> hb, hc;
   const bool dev = A->on_device != 0;
-  if (fetch(b, m, dev, hb) != cudaSuccess || fetch(c, n, dev, hc) != cudaSuccess) {
-    rc = fail(h, ABIP_E_CUDA, "reading b, c");
-    g_err = h->err; delete h; return rc;
-  }
-  if (!finite_all(hb.data(), m) || !finite_all(hc.data(), n)) {
-    g_err = "b or c has non-finite entries"; delete h; return ABIP_E_INVALID_ARG;
+  // a dense A for the dense path stays on the device it is on
+  const bool dense = prm.linsys == ABIP_LINSYS_DENSE_CHOL || (prm.linsys < 0 && A->fmt != ABIP_CSR);
+  const bool stays = dense && stays_on_device(A, b, c, h->device);
+  if (!stays) {
+    if (fetch(b, m, dev, hb) != cudaSuccess || fetch(c, n, dev, hc) != cudaSuccess) {
+      rc = fail(h, ABIP_E_CUDA, "reading b, c");
+      g_err = h->err; delete h; return rc;
+    }
+    if (!finite_all(hb.data(), m) || !finite_all(hc.data(), n)) {
+      g_err = "b or c has non-finite entries"; delete h; return ABIP_E_INVALID_ARG;
+    }
   }
   if (cudaEventCreate(&h->ev0) != cudaSuccess || cudaEventCreate(&h->ev1) != cudaSuccess) {
     cudaGetLastError();
@@ -1207,8 +1260,14 @@ int abip_setup(const abip_matrix* A, const double* b, const double* c, const abi
       rc = fail(h, ABIP_E_UNSUPPORTED, "dense Cholesky path needs 40m + 24n bytes (FP64) or 48m + 40n bytes (mixed) of shared memory, at most 200 KB; use linsys = PCG");
     else {
       std::vector<DenseHostInst> hi(1);
-      hi[0].m = m; hi[0].n = n; hi[0].b = hb; hi[0].c = hc;
-      rc = read_matrix_dense(h, A, hi[0].A);
+      hi[0].m = m; hi[0].n = n;
+      if (stays) {
+        hi[0].dev = A; hi[0].dev_b = b; hi[0].dev_c = c;
+        if (A->ld < n) rc = fail(h, ABIP_E_DIM, "ld < n");
+      } else {
+        hi[0].b = hb; hi[0].c = hc;
+        rc = read_matrix_dense(h, A, hi[0].A);
+      }
       std::vector<DenseInst> hd;
       std::vector<int> ord;
       h->group = !prm.bb_beta && plan_buckets(h, {{m, n}}, true, h->mixed != 0, abip::dense_max_ctas(h->device), ord);
@@ -1351,13 +1410,18 @@ int abip_solve_batch(int32_t count, const abip_matrix* A, const double* const* b
       return fail(nullptr, ABIP_E_UNSUPPORTED, "instance " + std::to_string(k) + ": needs 40m + 24n bytes (FP64) or "
                                                   "48m + 40n bytes (mixed) of shared memory, at most 200 KB");
     hi[k].m = m; hi[k].n = n;
-    rc = read_matrix_dense(&tmp, &A[k], hi[k].A);
-    if (rc) return fail(nullptr, rc, "instance " + std::to_string(k) + ": " + tmp.err);
-    const bool dev = A[k].on_device != 0;
-    if (fetch(b[k], m, dev, hi[k].b) != cudaSuccess || fetch(c[k], n, dev, hi[k].c) != cudaSuccess)
-      return fail(nullptr, ABIP_E_CUDA, "reading b, c");
-    if (!finite_all(hi[k].b.data(), m) || !finite_all(hi[k].c.data(), n))
-      return fail(nullptr, ABIP_E_INVALID_ARG, "instance " + std::to_string(k) + ": non-finite b or c");
+    if (stays_on_device(&A[k], b[k], c[k], tmp.device)) {
+      if (A[k].ld < n) return fail(nullptr, ABIP_E_DIM, "instance " + std::to_string(k) + ": ld < n");
+      hi[k].dev = &A[k]; hi[k].dev_b = b[k]; hi[k].dev_c = c[k];
+    } else {
+      rc = read_matrix_dense(&tmp, &A[k], hi[k].A);
+      if (rc) return fail(nullptr, rc, "instance " + std::to_string(k) + ": " + tmp.err);
+      const bool dev = A[k].on_device != 0;
+      if (fetch(b[k], m, dev, hi[k].b) != cudaSuccess || fetch(c[k], n, dev, hi[k].c) != cudaSuccess)
+        return fail(nullptr, ABIP_E_CUDA, "reading b, c");
+      if (!finite_all(hi[k].b.data(), m) || !finite_all(hi[k].c.data(), n))
+        return fail(nullptr, ABIP_E_INVALID_ARG, "instance " + std::to_string(k) + ": non-finite b or c");
+    }
     smem_solve = std::max(smem_solve, dense_solve_smem(m, n, mixed));
     smem_setup = std::max(smem_setup, dense_setup_smem(m, n));
     mmax = std::max(mmax, m);

@@ -266,6 +266,15 @@ struct GroupSparse {
 // sparse form takes G = I + A A^T of one instance from A by rows and columns (L zeroed).
 cudaError_t launch_sparse_factor(DenseInst* inst, int m, const GroupSparse& sp, int sms, cudaStream_t st);
 cudaError_t launch_dense_factor(DenseInst* inst, int count, int mmax, int sms, cudaStream_t st);
+// Where an instance's A came from: FP32 values staged on the device (f32, ld), else FP64 in place.
+struct DenseSource {
+  const float* f32;
+  int64_t ld;
+};
+// Every instance's A as FP64 (from an FP32 source), its FP32 copies Af and ATf (where not
+// null), and a look at A, b and c: flags[k] gets bit 0 (A) or 1 (b, c) for a non-finite entry.
+cudaError_t launch_dense_ingest(const DenseInst* inst, const DenseSource* src, int* flags, int count, int mmax, int nmax,
+                                int sms, cudaStream_t st);
 // from L of every instance: the explicit inverse of G (FP32, Ginvf), or L^{-1} and L^{-T} (Li, LiT)
 cudaError_t launch_dense_inverse(DenseInst* inst, int count, int mmax, int sms, cudaStream_t st);
 // A^T of every instance (AT)

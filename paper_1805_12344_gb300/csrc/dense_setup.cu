@@ -342,6 +342,49 @@ __global__ void __launch_bounds__(kThr) inverse_tiles_kernel(const DenseInst* __
   }
 }
 
+// What a dense instance needs of its inputs, by 32 x 32 tiles of A: the FP64 values of an FP32
+// source, the FP32 copies of A and A^T of the mixed path (padding is zero already), and a test
+// of every value (bound by the tile's one read of A).
+__global__ void __launch_bounds__(kThr) ingest_kernel(const DenseInst* __restrict__ insts, const DenseSource* __restrict__ src,
+                                                      int* __restrict__ flags) {
+  __shared__ double T[32][33];
+  const DenseInst& I = insts[blockIdx.y];
+  const DenseSource S = src[blockIdx.y];
+  const int m = I.m, n = I.n;
+  const int tm = (m + 31) / 32, tiles = tm * ((n + 31) / 32);
+  const int lane = threadIdx.x & 31, row = threadIdx.x >> 5;
+  double* A = const_cast<double*>(I.A);
+  float* Af = const_cast<float*>(I.Af);
+  float* ATf = const_cast<float*>(I.ATf);
+  bool bad = false;
+  for (int t = blockIdx.x; t < tiles; t += gridDim.x) {
+    const int i0 = (t % tm) * 32, j0 = (t / tm) * 32;
+    for (int r = row; r < 32; r += kThr / 32) {
+      const int i = i0 + r, j = j0 + lane;
+      double v = 0.0;
+      if (i < m && j < n) {
+        v = S.f32 ? (double)S.f32[(size_t)i * S.ld + j] : A[(size_t)i * I.ld + j];
+        bad |= !isfinite(v);
+        if (S.f32) A[(size_t)i * I.ld + j] = v;
+        if (Af) Af[(size_t)i * I.ldf + j] = (float)v;
+      }
+      T[r][lane] = v;
+    }
+    __syncthreads();
+    if (ATf)
+      for (int r = row; r < 32; r += kThr / 32)
+        if (j0 + r < n && i0 + lane < m) ATf[(size_t)(j0 + r) * I.ldtf + i0 + lane] = (float)T[lane][r];
+    __syncthreads();
+  }
+  if (bad) atomicOr(flags + blockIdx.y, 1);
+  if (blockIdx.x == 0) {
+    bool vec = false;
+    for (int i = threadIdx.x; i < m; i += kThr) vec |= !isfinite(I.b[i]);
+    for (int j = threadIdx.x; j < n; j += kThr) vec |= !isfinite(I.c[j]);
+    if (vec) atomicOr(flags + blockIdx.y, 2);
+  }
+}
+
 // A^T, rows padded to an even length (the padding is zero already), 32 x 32 tiles
 __global__ void __launch_bounds__(kThr) transpose_tiles_kernel(const DenseInst* __restrict__ insts) {
   __shared__ double T[32][33];
@@ -414,6 +457,17 @@ cudaError_t launch_sparse_factor(DenseInst* inst, int m, const GroupSparse& sp, 
   gram_sparse_kernel<<<std::max(1, std::min(4 * sms, (m + 7) / 8)), kThr, 0, st>>>(inst, sp);
   const cudaError_t e = cudaGetLastError();
   return e != cudaSuccess ? e : launch_cholesky(inst, 1, m, sms, st);
+}
+
+cudaError_t launch_dense_ingest(const DenseInst* inst, const DenseSource* src, int* flags, int count, int mmax, int nmax,
+                                int sms, cudaStream_t st) {
+  const int64_t tiles = (int64_t)((mmax + 31) / 32) * ((nmax + 31) / 32);
+  for (int k0 = 0; k0 < count; k0 += 32768) {
+    const int cnt = std::min(32768, count - k0);
+    const int gx = (int)std::max<int64_t>(1, std::min<int64_t>(tiles, (8 * sms + cnt - 1) / cnt));
+    ingest_kernel<<<dim3(gx, cnt), kThr, 0, st>>>(inst + k0, src + k0, flags + k0);
+  }
+  return cudaGetLastError();
 }
 
 cudaError_t launch_dense_transpose(DenseInst* inst, int count, int mmax, int nmax, int sms, cudaStream_t st) {

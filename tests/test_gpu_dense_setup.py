@@ -54,3 +54,31 @@ def test_batch_first_iterates(abip, count):
             m, n = lps[k].A.shape
             got = np.concatenate([ys[k], xs[k]]) * infos[k]["tau"]
             assert _rel(got, ref[:m + n]) <= tol, (k, precision)
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_device_inputs_equal_host_inputs(abip, precision):
+    """A, b, c on the device (FP32 or FP64 A, odd sizes) give the bits of the same values from the host."""
+    lp = W.planted_dense_f32(33, 71, seed=11)
+    A, b, c = (torch.from_numpy(v).cuda() for v in (lp.A, lp.b, lp.c))
+    states = []
+    for args in ((lp.A, lp.b, lp.c), (A, b, c), (A.float(), b, c)):
+        s = abip.Solver(*args, precision=precision, max_admm_iters=30)
+        s.solve()
+        states.append(s.state())
+        s.close()
+    assert np.array_equal(states[0], states[1]) and np.array_equal(states[0], states[2])
+
+
+@pytest.mark.parametrize("which", [0, 1, 2])
+def test_non_finite_device_input_is_refused(abip, which):
+    lp = W.planted_dense(33, 71, seed=12)
+    good = [torch.from_numpy(v).cuda() for v in (lp.A, lp.b, lp.c)]
+    bad = [t.clone() for t in good]
+    bad[which].view(-1)[-1] = float("inf")
+    with pytest.raises(abip.AbipError) as e:
+        abip.Solver(*bad)
+    assert e.value.code == abip.ABIP_E_INVALID_ARG
+    with pytest.raises(abip.AbipError) as e:
+        abip.abip_solve_batch(*[list(p) for p in zip(good, bad)])
+    assert e.value.code == abip.ABIP_E_INVALID_ARG
