@@ -331,7 +331,7 @@ cudaError_t launch_dense_solve(DenseInst* inst, int count, DenseParams prm, int*
 int dense_solve_ctas_per_sm(size_t smem, int variant);
 int dense_max_ctas(int device);
 cudaError_t launch_dense_backward(BackwardInst* insts, int count, int grid, cudaStream_t st);
-inline size_t backward_work_doubles(int m, int n) { return 2 * (size_t)m + 4 * (size_t)n + 5 * ((size_t)m + n + 2); }
+inline size_t backward_work_doubles(int m, int n) { return 2 * (size_t)m + 8 * (size_t)n + 7 * ((size_t)m + n + 2) + 4; }
 
 // shared by the allocation-free entry point (defined in abip_api.cu)
 int check_params_internal(const abip_params& p, std::string& why);
