@@ -37,18 +37,20 @@ constexpr int kSumRowGroups = kThr / kMaxBatch;
 // ---------------------------------------------------------------------------
 // SIMT GEMM:  Cpart[z] = op(A)[M x K_z] * W[K_z x N], K split into gridDim.z chunks.
 // op(A) = A (row-major, lda) or A^T.  W row-major (ldw).  Cpart: gridDim.z x M x N.
-// 256 threads as 16 x 16, each TM x TN outputs at rows tr + 16u, columns tc + 16v.
+// 256 threads as 16 x 16, each TM x TN outputs at rows tr + 16u, columns tc + 16v.  Every output
+// is one chain over its chunk in increasing order, whatever the tile, so the tile is free to
+// follow the shape (gemm_tile) without moving a bit; the chunks follow GemmCfg alone.
 // ---------------------------------------------------------------------------
 template <typename T> struct GemmCfg;
 template <> struct GemmCfg<float> { static constexpr int TM = 8, TN = 4, BK = 16; };
 template <> struct GemmCfg<double> { static constexpr int TM = 4, TN = 4, BK = 16; };
 
-template <typename T, bool TRANS>
+template <typename T, bool TRANS, int TM, int TN>
 __global__ void __launch_bounds__(kThr) gemm_kernel(const T* __restrict__ A, int64_t lda, int M, int N, int K,
                                                     const T* __restrict__ W, int64_t ldw, T* __restrict__ Cp,
                                                     int kchunk, const int* __restrict__ gate) {
   if (gate && *gate == 0) return;
-  constexpr int TM = GemmCfg<T>::TM, TN = GemmCfg<T>::TN, BK = GemmCfg<T>::BK;
+  constexpr int BK = GemmCfg<T>::BK;
   constexpr int BM = 16 * TM, BN = 16 * TN;
   __shared__ T As[BK][BM + 1];
   __shared__ T Ws[BK][BN + 1];
@@ -892,7 +894,6 @@ __global__ void output_kernel(ShView<T> V, const ShInst* __restrict__ insts, dou
 // ---------------------------------------------------------------------------
 struct GemmPlan {
   int splits = 1, kchunk = 0;
-  dim3 grid;
 };
 
 template <typename T>
@@ -906,8 +907,48 @@ GemmPlan plan_gemm(int M, int N, int K, int sms) {
   const int kchunk = ((kblocks + splits - 1) / splits) * BK;
   g.splits = (K + kchunk - 1) / kchunk;
   g.kchunk = kchunk;
-  g.grid = dim3((M + BM - 1) / BM, (N + BN - 1) / BN, g.splits);
   return g;
+}
+
+template <typename T, int TM, int TN>
+void launch_gemm_tile(bool trans, const T* A, int64_t lda, int M, int N, int K, const T* W, int64_t ldw, T* work,
+                      const GemmPlan& g, const int* gate, cudaStream_t st) {
+  const dim3 grid((M + 16 * TM - 1) / (16 * TM), (N + 16 * TN - 1) / (16 * TN), g.splits);
+  if (trans) gemm_kernel<T, true, TM, TN><<<grid, kThr, 0, st>>>(A, lda, M, N, K, W, ldw, work, g.kchunk, gate);
+  else gemm_kernel<T, false, TM, TN><<<grid, kThr, 0, st>>>(A, lda, M, N, K, W, ldw, work, g.kchunk, gate);
+}
+
+// The tile of a product: GemmCfg's while its CTAs fill the SMs twice; else smaller ones, down to
+// 16 x 16 outputs (a CTA's time is its tile's chain count, so halving the tile of a launch that
+// leaves SMs idle halves the launch), and no wider than the right-hand sides need.  Measured,
+// FP64, 256 x 512 with 64 instances: 64 x 64 tiles give 16 to 64 CTAs of 70 us each per product
+// on 152 SMs, 381 us per cycle of four products; with this rule 164.  500 x 5000, one instance
+// (64-wide tiles for one column): FP64 1269 -> 376 us, mixed 132 -> 108.
+template <typename T>
+void launch_gemm(bool trans, const T* A, int64_t lda, int M, int N, int K, const T* W, int64_t ldw, T* work,
+                 const GemmPlan& g, int sms, const int* gate, cudaStream_t st) {
+  constexpr int TM = GemmCfg<T>::TM, TN = GemmCfg<T>::TN;
+  int tm = TM, tn = TN;
+  auto ctas = [&](int a, int b) { return ((M + 16 * a - 1) / (16 * a)) * ((N + 16 * b - 1) / (16 * b)) * g.splits; };
+  while (tn > 1 && N <= 8 * tn) tn /= 2;
+  while (ctas(tm, tn) < 2 * sms && (tm > 1 || tn > 1)) {
+    if (tm >= tn && tm > 1) tm /= 2;
+    else tn /= 2;
+  }
+  auto go = [&](auto a, auto b) {
+    launch_gemm_tile<T, decltype(a)::value, decltype(b)::value>(trans, A, lda, M, N, K, W, ldw, work, g, gate, st);
+  };
+  auto with_tn = [&](auto a) {
+    if (tn == 4) go(a, std::integral_constant<int, 4>{});
+    else if (tn == 2) go(a, std::integral_constant<int, 2>{});
+    else go(a, std::integral_constant<int, 1>{});
+  };
+  if constexpr (TM == 8) {
+    if (tm == 8) { with_tn(std::integral_constant<int, 8>{}); return; }
+  }
+  if (tm == 4) with_tn(std::integral_constant<int, 4>{});
+  else if (tm == 2) with_tn(std::integral_constant<int, 2>{});
+  else with_tn(std::integral_constant<int, 1>{});
 }
 
 template <typename T>
@@ -916,8 +957,7 @@ cudaError_t gemm(bool trans, const T* A, int64_t lda, int M, int N, int K, const
                  const T* F = nullptr, int64_t lde = 0, const int* gate = nullptr) {
   const GemmPlan g = plan_gemm<T>(M, N, K, sms);
   if ((size_t)g.splits * M * N > work_elems) return cudaErrorInvalidValue;
-  if (trans) gemm_kernel<T, true><<<g.grid, kThr, 0, st>>>(A, lda, M, N, K, W, ldw, work, g.kchunk, gate);
-  else gemm_kernel<T, false><<<g.grid, kThr, 0, st>>>(A, lda, M, N, K, W, ldw, work, g.kchunk, gate);
+  launch_gemm<T>(trans, A, lda, M, N, K, W, ldw, work, g, sms, gate, st);
   const size_t MN = (size_t)M * N;
   const int rb = (int)std::min<size_t>((MN + kThr - 1) / kThr, (size_t)sms * 8);
   reduce_kernel<T><<<std::max(rb, 1), kThr, 0, st>>>(work, g.splits, M, N, out, diag, E, F, lde, gate);
@@ -930,8 +970,7 @@ cudaError_t gemm_acc(bool trans, const float* A, int64_t lda, int M, int N, int 
                      cudaStream_t st) {
   const GemmPlan g = plan_gemm<float>(M, N, K, sms);
   if ((size_t)g.splits * M * N > work_elems) return cudaErrorInvalidValue;
-  if (trans) gemm_kernel<float, true><<<g.grid, kThr, 0, st>>>(A, lda, M, N, K, W, ldw, work, g.kchunk, nullptr);
-  else gemm_kernel<float, false><<<g.grid, kThr, 0, st>>>(A, lda, M, N, K, W, ldw, work, g.kchunk, nullptr);
+  launch_gemm<float>(trans, A, lda, M, N, K, W, ldw, work, g, sms, nullptr, st);
   const size_t MN = (size_t)M * N;
   const int rb = (int)std::min<size_t>((MN + kThr - 1) / kThr, (size_t)sms * 8);
   accum_kernel<<<std::max(rb, 1), kThr, 0, st>>>(work, g.splits, M, N, B, acc64, out32, mask);
