@@ -202,6 +202,7 @@ struct DenseInst {
   // FP64 path by a group of CTAs (null elsewhere): A^T (n rows), L^{-1} and L^{-T} (m rows
   // each), rows padded with zeros to an even length; A's ld is even then
   double* AT; double* Li; double* LiT;
+  double* Ginv;                // the explicit inverse of G (m x m), shared-A batch only
   double zbar, nb, nc;
   double Kinv[4];
   // results
@@ -275,7 +276,8 @@ struct DenseSource {
 // null), and a look at A, b and c: flags[k] gets bit 0 (A) or 1 (b, c) for a non-finite entry.
 cudaError_t launch_dense_ingest(const DenseInst* inst, const DenseSource* src, int* flags, int count, int mmax, int nmax,
                                 int sms, cudaStream_t st);
-// from L of every instance: the explicit inverse of G (FP32, Ginvf), or L^{-1} and L^{-T} (Li, LiT)
+// from L of every instance: the explicit inverse of G (FP32 Ginvf, FP64 Ginv), or
+// L^{-1} and L^{-T} (Li, LiT)
 cudaError_t launch_dense_inverse(DenseInst* inst, int count, int mmax, int sms, cudaStream_t st);
 // A^T of every instance (AT)
 cudaError_t launch_dense_transpose(DenseInst* inst, int count, int mmax, int nmax, int sms, cudaStream_t st);

@@ -336,8 +336,11 @@ __global__ void __launch_bounds__(kThr) inverse_tiles_kernel(const DenseInst* __
     }
     for (int e = threadIdx.x; e < m * Q; e += kThr) {
       const int q = e / m, i = e % m;
-      if (c0 + q < m) I.Ginvf[(size_t)(c0 + q) * I.ldtf + i] = (float)W[i * Q + q];
+      if (c0 + q < m && I.Ginvf) I.Ginvf[(size_t)(c0 + q) * I.ldtf + i] = (float)W[i * Q + q];
     }
+    if (I.Ginv)
+      for (int e = threadIdx.x; e < m * Q; e += kThr)
+        if (c0 + e % Q < m) I.Ginv[(size_t)(e / Q) * m + c0 + e % Q] = W[e];
     __syncthreads();
   }
 }

@@ -19,6 +19,7 @@
 //             dual update (Eqs. Simple-Update:*, Sec. 4.2)
 #include "abip_internal.h"
 #include "abip_device.cuh"
+#include "dense_device.cuh"
 #include "tc_gemm.cuh"
 
 #include <algorithm>
@@ -48,10 +49,11 @@ template <> struct GemmCfg<double> { static constexpr int TM = 4, TN = 4, BK = 1
 template <typename T, bool TRANS, int TM, int TN>
 __global__ void __launch_bounds__(kThr) gemm_kernel(const T* __restrict__ A, int64_t lda, int M, int N, int K,
                                                     const T* __restrict__ W, int64_t ldw, T* __restrict__ Cp,
-                                                    int kchunk, const int* __restrict__ gate) {
+                                                    int kchunk, const int* __restrict__ gate, int lower) {
   if (gate && *gate == 0) return;
   constexpr int BK = GemmCfg<T>::BK;
   constexpr int BM = 16 * TM, BN = 16 * TN;
+  if (lower && (int)blockIdx.y * BN >= ((int)blockIdx.x + 1) * BM) return;   // above the diagonal: not read
   __shared__ T As[BK][BM + 1];
   __shared__ T Ws[BK][BN + 1];
   const int tid = threadIdx.x, tr = tid / 16, tc = tid % 16;
@@ -62,26 +64,37 @@ __global__ void __launch_bounds__(kThr) gemm_kernel(const T* __restrict__ A, int
   for (int u = 0; u < TM; ++u)
 #pragma unroll
     for (int v = 0; v < TN; ++v) acc[u][v] = T(0);
-  for (int j0 = jb; j0 < je; j0 += BK) {
-    if (!TRANS) {
-      for (int e = tid; e < BM * BK; e += kThr) {
-        const int r = e / BK, q = e % BK;
-        const int gi = i0 + r, gj = j0 + q;
-        As[q][r] = (gi < M && gj < je) ? A[(size_t)gi * lda + gj] : T(0);
-      }
-    } else {
-      for (int e = tid; e < BM * BK; e += kThr) {
-        const int q = e / BM, r = e % BM;
-        const int gi = i0 + r, gj = j0 + q;
-        As[q][r] = (gi < M && gj < je) ? A[(size_t)gj * lda + gi] : T(0);
-      }
+  // the next step's tiles are on their way in registers while this step computes
+  constexpr int NA = (BM * BK + kThr - 1) / kThr, NW = (BN * BK + kThr - 1) / kThr;
+  T pa[NA], pw[NW];
+  auto load = [&](int j0) {
+#pragma unroll
+    for (int t = 0; t < NA; ++t) {
+      const int e = tid + t * kThr;
+      const int r = TRANS ? e % BM : e / BK, q = TRANS ? e / BM : e % BK;
+      const int gi = i0 + r, gj = j0 + q;
+      pa[t] = (e < BM * BK && gi < M && gj < je) ? A[TRANS ? (size_t)gj * lda + gi : (size_t)gi * lda + gj] : T(0);
     }
-    for (int e = tid; e < BK * BN; e += kThr) {
-      const int q = e / BN, cc = e % BN;
-      const int gj = j0 + q, gk = k0 + cc;
-      Ws[q][cc] = (gj < je && gk < N) ? W[(size_t)gj * ldw + gk] : T(0);
+#pragma unroll
+    for (int t = 0; t < NW; ++t) {
+      const int e = tid + t * kThr, gj = j0 + e / BN, gk = k0 + e % BN;
+      pw[t] = (e < BK * BN && gj < je && gk < N) ? W[(size_t)gj * ldw + gk] : T(0);
+    }
+  };
+  load(jb);
+  for (int j0 = jb; j0 < je; j0 += BK) {
+#pragma unroll
+    for (int t = 0; t < NA; ++t) {
+      const int e = tid + t * kThr;
+      if (e < BM * BK) As[TRANS ? e / BM : e % BK][TRANS ? e % BM : e / BK] = pa[t];
+    }
+#pragma unroll
+    for (int t = 0; t < NW; ++t) {
+      const int e = tid + t * kThr;
+      if (e < BK * BN) Ws[e / BN][e % BN] = pw[t];
     }
     __syncthreads();
+    if (j0 + BK < je) load(j0 + BK);
 #pragma unroll
     for (int q = 0; q < BK; ++q) {
       T a[TM], w[TN];
@@ -390,8 +403,9 @@ __global__ void bf16_copies_kernel(const double* __restrict__ A, int m, int n, i
 // 0 .. m+n-1 (rows < m are y-type, the rest x-type); thread (rg, k) handles instance
 // k and rows rg, rg + 4, ...; partials[cta][k][NS] in double.
 // ---------------------------------------------------------------------------
+// by_sum: partials[(k NS + q) gridDim + cta], so that partials_total_kernel reads rows
 template <int NS>
-__device__ void store_partials(double (&acc)[NS], double* sm, double* partials, int B) {
+__device__ void store_partials(double (&acc)[NS], double* sm, double* partials, int B, bool by_sum = false) {
   const int k = threadIdx.x % kMaxBatch, rg = threadIdx.x / kMaxBatch;
 #pragma unroll
   for (int q = 0; q < NS; ++q) sm[(rg * kMaxBatch + k) * NS + q] = acc[q];
@@ -401,7 +415,7 @@ __device__ void store_partials(double (&acc)[NS], double* sm, double* partials, 
     for (int q = 0; q < NS; ++q) {
       double v = sm[k * NS + q];
       for (int g = 1; g < kSumRowGroups; ++g) v += sm[(g * kMaxBatch + k) * NS + q];
-      partials[((size_t)blockIdx.x * kMaxBatch + k) * NS + q] = v;
+      partials[by_sum ? ((size_t)k * NS + q) * gridDim.x + blockIdx.x : ((size_t)blockIdx.x * kMaxBatch + k) * NS + q] = v;
     }
   }
 }
@@ -430,90 +444,86 @@ __global__ void __launch_bounds__(kThr) sums_kernel(ShView<T> V, const ShInst* _
   double acc[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
   const RowRange rr = my_rows(m + n);
   if (k < B) {
-    const double ta = st[k].tau, th = st[k].theta;
-    for (int r = rr.r0 + rg; r < rr.r1; r += kSumRowGroups) {
-      if (r < m) {
-        const size_t e = (size_t)r * B + k;
-        const double ax = (double)V.AXS[(size_t)r * 2 * B + k], as = (double)V.AXS[(size_t)r * 2 * B + B + k];
-        const double bi = (double)V.b[e], bb = (double)V.bbar[e], yi = (double)V.Y[e];
-        const double ry = ax - bi * ta + bb * th;
-        const double pr = ax / ta - bi;
-        acc[0] += ry * ry; acc[1] += pr * pr; acc[3] += ax * ax;
-        acc[5] += bi * yi; acc[6] += bb * yi;
-        if (Q) Q[e] = (T)(yi - (ax + as));
-        if (dQ) dQ[e] = (float)((yi - (ax + as)) - Qprev[e]);
-      } else {
-        const int j = r - m;
-        const size_t e = (size_t)j * B + k;
-        const double aty = (double)V.ATY[e];
-        const double xj = (double)V.XS[(size_t)j * 2 * B + k], sj = (double)V.XS[(size_t)j * 2 * B + B + k];
-        const double cj = (double)V.c[e], cb = (double)V.cbar[e];
+    const double ta = st[k].tau, th = st[k].theta, it = 1.0 / ta;   // one quotient, not two per row
+    int r = rr.r0 + rg;
+    for (; r < rr.r1 && r < m; r += kSumRowGroups) {
+      const size_t e = (size_t)r * B + k;
+      const double ax = (double)V.AXS[(size_t)r * 2 * B + k], as = (double)V.AXS[(size_t)r * 2 * B + B + k];
+      const double bi = (double)V.b[e], bb = (double)V.bbar[e], yi = (double)V.Y[e];
+      const double ry = ax - bi * ta + bb * th;
+      const double pr = ax * it - bi;
+      acc[0] += ry * ry; acc[1] += pr * pr; acc[3] += ax * ax;
+      acc[5] += bi * yi; acc[6] += bb * yi;
+      if (Q) Q[e] = (T)(yi - (ax + as));
+      if (dQ) dQ[e] = (float)((yi - (ax + as)) - Qprev[e]);
+    }
+    // columns, four rows' loads in flight
+    constexpr int U = 4;
+    for (; r < rr.r1; r += U * kSumRowGroups) {
+      double v[U][5];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int j = min(r + u * kSumRowGroups, rr.r1 - 1) - m;
+        const size_t e = (size_t)j * B + k, ex = (size_t)j * 2 * B + k;
+        v[u][0] = (double)V.ATY[e]; v[u][1] = (double)V.XS[ex]; v[u][2] = (double)V.XS[ex + B];
+        v[u][3] = (double)V.c[e]; v[u][4] = (double)V.cbar[e];
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        if (r + u * kSumRowGroups >= rr.r1) break;
+        const double aty = v[u][0], xj = v[u][1], sj = v[u][2], cj = v[u][3], cb = v[u][4];
         const double rx = -aty + cj * ta - cb * th - sj;
-        const double dr = (aty + sj) / ta - cj;
+        const double dr = (aty + sj) * it - cj;
         acc[0] += rx * rx; acc[2] += dr * dr; acc[4] += (aty + sj) * (aty + sj);
         acc[7] += cj * xj; acc[8] += cb * xj;
       }
     }
   }
-  store_partials<9>(acc, sm, partials, B);
+  store_partials<9>(acc, sm, partials, B, true);
 }
 
-// H^T z for the projection result: hz0 = c^T zx - b^T zy, hz1 = -cbar^T zx + bbar^T zy.
-template <typename T>
-__global__ void __launch_bounds__(kThr) hz_kernel(ShView<T> V, double* partials) {
+// ZX = X + S + A^T ZY, H^T z (hz0 = c^T zx - b^T zy, hz1 = -cbar^T zx + bbar^T zy) and, in mixed
+// precision (Qprev not null), Qprev = Q for the instances that take this update (their ZY now
+// matches Q).
+__global__ void __launch_bounds__(kThr) hz_kernel(ShView<double> V, const double* __restrict__ ATZY, double* Qprev,
+                                                  const ShInst* __restrict__ insts, double* partials) {
   __shared__ double sm[kThr * 2];
   const int m = V.m, n = V.n, B = V.B;
   const int k = threadIdx.x % kMaxBatch, rg = threadIdx.x / kMaxBatch;
   double acc[2] = {0, 0};
   const RowRange rr = my_rows(m + n);
   if (k < B) {
-    for (int r = rr.r0 + rg; r < rr.r1; r += kSumRowGroups) {
-      if (r < m) {
-        const size_t e = (size_t)r * B + k;
-        const double z = (double)V.ZY[e];
-        acc[0] -= (double)V.b[e] * z;
-        acc[1] += (double)V.bbar[e] * z;
-      } else {
-        const size_t e = (size_t)(r - m) * B + k;
-        const double z = (double)V.ZX[e];
-        acc[0] += (double)V.c[e] * z;
-        acc[1] -= (double)V.cbar[e] * z;
+    const bool step = Qprev && insts[k].action == SH_STEP;
+    int r = rr.r0 + rg;
+    for (; r < rr.r1 && r < m; r += kSumRowGroups) {
+      const size_t e = (size_t)r * B + k;
+      const double z = V.ZY[e];
+      acc[0] -= V.b[e] * z;
+      acc[1] += V.bbar[e] * z;
+      if (step) Qprev[e] = V.Q[e];
+    }
+    constexpr int U = 4;   // columns, four rows' loads in flight
+    for (; r < rr.r1; r += U * kSumRowGroups) {
+      double v[U][5];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int j = min(r + u * kSumRowGroups, rr.r1 - 1) - m;
+        const size_t e = (size_t)j * B + k, ex = (size_t)j * 2 * B + k;
+        v[u][0] = V.XS[ex]; v[u][1] = V.XS[ex + B]; v[u][2] = ATZY[e];
+        v[u][3] = V.c[e]; v[u][4] = V.cbar[e];
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int ru = r + u * kSumRowGroups;
+        if (ru >= rr.r1) break;
+        const double z = v[u][0] + v[u][1] + v[u][2];
+        V.ZX[(size_t)(ru - m) * B + k] = z;
+        acc[0] += v[u][3] * z;
+        acc[1] -= v[u][4] * z;
       }
     }
   }
-  store_partials<2>(acc, sm, partials, B);
-}
-
-// Mixed path: ZX = X + S + (A^T ZY maintained in FP64), H^T z from ZY and ZX, and
-// Qprev = Q for the instances that take this update (their ZY now matches Q).
-__global__ void __launch_bounds__(kThr) hz_delta_kernel(ShView<double> V, const double* __restrict__ ATZY,
-                                                        double* Qprev, const ShInst* __restrict__ insts,
-                                                        double* partials) {
-  __shared__ double sm[kThr * 2];
-  const int m = V.m, n = V.n, B = V.B;
-  const int k = threadIdx.x % kMaxBatch, rg = threadIdx.x / kMaxBatch;
-  double acc[2] = {0, 0};
-  const RowRange rr = my_rows(m + n);
-  if (k < B) {
-    const bool step = insts[k].action == SH_STEP;
-    for (int r = rr.r0 + rg; r < rr.r1; r += kSumRowGroups) {
-      if (r < m) {
-        const size_t e = (size_t)r * B + k;
-        const double z = V.ZY[e];
-        acc[0] -= V.b[e] * z;
-        acc[1] += V.bbar[e] * z;
-        if (step) Qprev[e] = V.Q[e];
-      } else {
-        const int j = r - m;
-        const size_t e = (size_t)j * B + k;
-        const double z = V.XS[(size_t)j * 2 * B + k] + V.XS[(size_t)j * 2 * B + B + k] + ATZY[e];
-        V.ZX[e] = z;
-        acc[0] += V.c[e] * z;
-        acc[1] -= V.cbar[e] * z;
-      }
-    }
-  }
-  store_partials<2>(acc, sm, partials, B);
+  store_partials<2>(acc, sm, partials, B, true);
 }
 
 // End of an FP64 refresh: the exact Q becomes the reference for later deltas.
@@ -535,23 +545,29 @@ __device__ void total_partials(const double* partials, int nparts, int k, double
     for (int q = 0; q < NS; ++q) out[q] += partials[((size_t)p * kMaxBatch + k) * NS + q];
 }
 
-// totals[k][q] = sum over the reduction CTAs of partials[cta][k][q]: one CTA per instance,
-// fixed assignment of partials to threads and a fixed-order block reduction.
+// totals[k][q] = sum over the reduction CTAs of partials[k][q][cta]: one CTA per instance, fixed
+// assignment of partials to threads and a fixed-order block reduction (block_sum's additions,
+// the sums of a warp taken together).
 template <int NS>
 __global__ void __launch_bounds__(kThr) partials_total_kernel(const double* __restrict__ partials, int nparts,
                                                               double* __restrict__ totals) {
-  __shared__ double red[32 * NS];
-  const int k = blockIdx.x;
-  double v[NS];
+  constexpr int P = NS > 2 ? 16 : 2, kShift = NS > 2 ? 1 : 4;
+  __shared__ double red[kThrWarps * NS];
+  const int k = blockIdx.x, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  double v[P];
 #pragma unroll
-  for (int q = 0; q < NS; ++q) v[q] = 0.0;
+  for (int q = 0; q < P; ++q) v[q] = 0.0;
   for (int p = threadIdx.x; p < nparts; p += kThr)
 #pragma unroll
-    for (int q = 0; q < NS; ++q) v[q] += partials[((size_t)p * kMaxBatch + k) * NS + q];
-  block_sum<NS>(v, red);
-  if (threadIdx.x == 0)
-#pragma unroll
-    for (int q = 0; q < NS; ++q) totals[k * NS + q] = v[q];
+    for (int q = 0; q < NS; ++q) v[q] += partials[((size_t)k * NS + q) * nparts + p];
+  const double t = dense::sum_together<P>(v, lane);
+  const int q = lane >> kShift;
+  if ((lane & ((1 << kShift) - 1)) == 0 && q < NS) red[q * kThrWarps + wid] = t;
+  __syncthreads();
+  if (threadIdx.x < NS) {
+    const double* w = red + threadIdx.x * kThrWarps;
+    totals[k * NS + threadIdx.x] = ((w[0] + w[4]) + (w[2] + w[6])) + ((w[1] + w[5]) + (w[3] + w[7]));
+  }
 }
 
 // Sec. 4.1 tests on the nine sums; 0 = none passes.
@@ -686,7 +702,7 @@ __global__ void ctrl_step_kernel(ShInst* insts, int B, int n, const double* part
 // Elementwise part of the update (STEP) or of the warm start (WARM), per (row, instance).
 // Mixed path (dXS non-null): also the FP32 changes of x and s (zero where the instance
 // did not move), the input of the maintained product A [dX dS].
-//   ATZY, ATG1, ATG2 (mixed path, else null): A^T y of the new state follows from the
+//   ATZY, ATG1, ATG2: A^T y of the new state follows from the
 //   update's linearity in y: y <- alpha (zy - g1y t1 - g2y t2) + (1 - alpha) y gives
 //   A^T y <- alpha (A^T zy - (A^T g1y) t1 - (A^T g2y) t2) + (1 - alpha) A^T y, with A^T zy
 //   maintained for the projection and A^T g1y, A^T g2y formed once at setup; the warm
@@ -726,7 +742,7 @@ __global__ void update_kernel(ShView<T> V, const ShInst* __restrict__ insts, ShP
         else barrier_step<T>(xh - *sp, (T)I.cmu, xn, sn);
         *xp = xn;
         *sp = sn;
-        if (ATG1) V.ATY[q] = a * (ATZY[q] - ATG1[q] * t1 - ATG2[q] * t2) + a1 * V.ATY[q];
+        V.ATY[q] = a * (ATZY[q] - ATG1[q] * t1 - ATG2[q] * t2) + a1 * V.ATY[q];
       }
     } else if (act == SH_WARM) {
       const T sg = (T)sqrt(I.gam), g = (T)I.gam;
@@ -739,7 +755,7 @@ __global__ void update_kernel(ShView<T> V, const ShInst* __restrict__ insts, ShP
         if (P.warmstart == 1) { *xp *= sg; *sp *= sg; }
         else if (*xp >= *sp) *sp *= g;
         else *xp *= g;
-        if (ATG1) V.ATY[(size_t)j * B + k] *= sg;
+        V.ATY[(size_t)j * B + k] *= sg;
       }
     }
     if ((act == SH_STEP || act == SH_WARM) && r >= m && dXS) {
@@ -912,10 +928,10 @@ GemmPlan plan_gemm(int M, int N, int K, int sms) {
 
 template <typename T, int TM, int TN>
 void launch_gemm_tile(bool trans, const T* A, int64_t lda, int M, int N, int K, const T* W, int64_t ldw, T* work,
-                      const GemmPlan& g, const int* gate, cudaStream_t st) {
+                      const GemmPlan& g, const int* gate, bool lower, cudaStream_t st) {
   const dim3 grid((M + 16 * TM - 1) / (16 * TM), (N + 16 * TN - 1) / (16 * TN), g.splits);
-  if (trans) gemm_kernel<T, true, TM, TN><<<grid, kThr, 0, st>>>(A, lda, M, N, K, W, ldw, work, g.kchunk, gate);
-  else gemm_kernel<T, false, TM, TN><<<grid, kThr, 0, st>>>(A, lda, M, N, K, W, ldw, work, g.kchunk, gate);
+  if (trans) gemm_kernel<T, true, TM, TN><<<grid, kThr, 0, st>>>(A, lda, M, N, K, W, ldw, work, g.kchunk, gate, lower);
+  else gemm_kernel<T, false, TM, TN><<<grid, kThr, 0, st>>>(A, lda, M, N, K, W, ldw, work, g.kchunk, gate, lower);
 }
 
 // The tile of a product: GemmCfg's while its CTAs fill the SMs twice; else smaller ones, down to
@@ -926,7 +942,7 @@ void launch_gemm_tile(bool trans, const T* A, int64_t lda, int M, int N, int K, 
 // (64-wide tiles for one column): FP64 1269 -> 376 us, mixed 132 -> 108.
 template <typename T>
 void launch_gemm(bool trans, const T* A, int64_t lda, int M, int N, int K, const T* W, int64_t ldw, T* work,
-                 const GemmPlan& g, int sms, const int* gate, cudaStream_t st) {
+                 const GemmPlan& g, int sms, const int* gate, cudaStream_t st, bool lower = false) {
   constexpr int TM = GemmCfg<T>::TM, TN = GemmCfg<T>::TN;
   int tm = TM, tn = TN;
   auto ctas = [&](int a, int b) { return ((M + 16 * a - 1) / (16 * a)) * ((N + 16 * b - 1) / (16 * b)) * g.splits; };
@@ -936,7 +952,7 @@ void launch_gemm(bool trans, const T* A, int64_t lda, int M, int N, int K, const
     else tn /= 2;
   }
   auto go = [&](auto a, auto b) {
-    launch_gemm_tile<T, decltype(a)::value, decltype(b)::value>(trans, A, lda, M, N, K, W, ldw, work, g, gate, st);
+    launch_gemm_tile<T, decltype(a)::value, decltype(b)::value>(trans, A, lda, M, N, K, W, ldw, work, g, gate, lower, st);
   };
   auto with_tn = [&](auto a) {
     if (tn == 4) go(a, std::integral_constant<int, 4>{});
@@ -954,10 +970,10 @@ void launch_gemm(bool trans, const T* A, int64_t lda, int M, int N, int K, const
 template <typename T>
 cudaError_t gemm(bool trans, const T* A, int64_t lda, int M, int N, int K, const T* W, int64_t ldw, T* out,
                  T* work, size_t work_elems, int sms, cudaStream_t st, T diag = T(0), const T* E = nullptr,
-                 const T* F = nullptr, int64_t lde = 0, const int* gate = nullptr) {
+                 const T* F = nullptr, int64_t lde = 0, const int* gate = nullptr, bool lower = false) {
   const GemmPlan g = plan_gemm<T>(M, N, K, sms);
   if ((size_t)g.splits * M * N > work_elems) return cudaErrorInvalidValue;
-  launch_gemm<T>(trans, A, lda, M, N, K, W, ldw, work, g, sms, gate, st);
+  launch_gemm<T>(trans, A, lda, M, N, K, W, ldw, work, g, sms, gate, st, lower);
   const size_t MN = (size_t)M * N;
   const int rb = (int)std::min<size_t>((MN + kThr - 1) / kThr, (size_t)sms * 8);
   reduce_kernel<T><<<std::max(rb, 1), kThr, 0, st>>>(work, g.splits, M, N, out, diag, E, F, lde, gate);
@@ -1086,6 +1102,9 @@ int shared_batch_run(const SharedBatchArgs& a, std::vector<SharedBatchResult>& o
   // CTAs of the per-instance column reductions (their partials are totalled per instance
   // by partials_total_kernel before the control kernels read them)
   const int red_ctas = std::max(1, std::min(sms * 2, (m + n + 63) / 64));
+  // of the cycles in FP64: about two rows per thread (256 x 512: 12 CTAs took 31 us for the sums
+  // and 13 us for H^T z); the mixed path keeps the order of its sums
+  const int red_cyc = mixed ? red_ctas : std::max(1, std::min(sms * 2, (m + n + 7) / 8));
   const size_t wk64 = std::max({gemm_work<double>(m, m, n, sms), gemm_work<double>(m, 2 * B, n, sms),
                                 gemm_work<double>(m, 2 * B, m, sms), gemm_work<double>(n, 2 * B, m, sms),
                                 gemm_work<double>(n, B, m, sms), gemm_work<double>(m, B, m, sms)});
@@ -1108,6 +1127,7 @@ int shared_batch_run(const SharedBatchArgs& a, std::vector<SharedBatchResult>& o
   float *A32 = nullptr, *Ginv32 = nullptr, *work32 = nullptr, *dXS = nullptr, *dQ = nullptr,
         *dZY = nullptr;
   ShInst* insts = nullptr;
+  DenseInst* dinv = nullptr;
   int *flags = nullptr, *derr = nullptr;
   Bump bp;
   auto layout = [&]() {
@@ -1118,9 +1138,10 @@ int shared_batch_run(const SharedBatchArgs& a, std::vector<SharedBatchResult>& o
     Ginv64 = bp.take<double>((size_t)m * m);
     Ae = bp.take<double>(m);
     work64 = bp.take<double>(wk64);
-    partials = bp.take<double>((size_t)red_ctas * kMaxBatch * 9);
+    partials = bp.take<double>((size_t)std::max(red_ctas, red_cyc) * kMaxBatch * 9);
     totals = bp.take<double>((size_t)kMaxBatch * 9);
     insts = bp.take<ShInst>(kMaxBatch);
+    dinv = bp.take<DenseInst>(1);
     flags = bp.take<int>(8);
     derr = bp.take<int>(8);
     W2 = bp.take<double>((size_t)n * 2 * B);
@@ -1145,10 +1166,10 @@ int shared_batch_run(const SharedBatchArgs& a, std::vector<SharedBatchResult>& o
       AT16 = bp.take<__nv_bfloat16>(terms * aplane);
       WT16 = bp.take<__nv_bfloat16>(3 * std::max((size_t)2 * B * n, (size_t)B * m));
     }
+    ATZY = bp.take<double>((size_t)n * B);
+    ATG1 = bp.take<double>((size_t)n * B);
+    ATG2 = bp.take<double>((size_t)n * B);
     if (mixed) {
-      ATZY = bp.take<double>((size_t)n * B);
-      ATG1 = bp.take<double>((size_t)n * B);
-      ATG2 = bp.take<double>((size_t)n * B);
       Qprev = bp.take<double>((size_t)m * B);
       A32 = bp.take<float>((size_t)(tc ? 1 : m) * (tc ? 1 : n));
       Ginv32 = bp.take<float>((size_t)m * m);
@@ -1203,11 +1224,19 @@ int shared_batch_run(const SharedBatchArgs& a, std::vector<SharedBatchResult>& o
   setup_ctrl_kernel<<<1, kMaxBatch, 0, st>>>(insts, B, partials, red_ctas, 0, a.prm);
   // G = I + A A^T (Sec. 4.4), its Cholesky factor and the explicit inverse
   transpose_kernel<double><<<dim3((n + 31) / 32, (m + 31) / 32), dim3(32, 8), 0, st>>>(A64, m, n, AT64);
-  ck(gemm<double>(false, A64, n, m, m, n, AT64, m, G, work64, wk64, sms, st, 1.0), "Gram");
+  // (the factorisation and what follows read its lower triangle only)
+  ck(gemm<double>(false, A64, n, m, m, n, AT64, m, G, work64, wk64, sms, st, 1.0, nullptr, nullptr, 0, nullptr, true), "Gram");
   ck(cholesky_blocked(G, m, derr, st), "Cholesky");
   const size_t inv_smem = (size_t)m * 8;
   ck(cudaFuncSetAttribute(inverse_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)inv_smem), "smem");
-  inverse_kernel<<<std::min(m, sms * 2), kThr, inv_smem, st>>>(G, m, Ginv64);
+  if (m <= 6400) {   // column tiles in shared memory (the same operations per column)
+    DenseInst I{};
+    I.m = m; I.L = G; I.Ginv = Ginv64;
+    ck(cudaMemcpyAsync(dinv, &I, sizeof(I), cudaMemcpyHostToDevice, st), "inverse");
+    ck(launch_dense_inverse(dinv, 1, m, sms, st), "inverse");
+  } else {
+    inverse_kernel<<<std::min(m, sms * 2), kThr, inv_smem, st>>>(G, m, Ginv64);
+  }
   // M^{-1} h1, M^{-1} h2 for every instance: z_y = G^{-1}(a - A d), z_x = d + A^T z_y
   setup_rhs_kernel<<<eb, kThr, 0, st>>>(V, W2, nullptr, nullptr, 0);
   ck(gemm<double>(false, A64, n, m, 2 * B, n, W2, 2 * B, P2, work64, wk64, sms, st), "A W2");
@@ -1219,10 +1248,11 @@ int shared_batch_run(const SharedBatchArgs& a, std::vector<SharedBatchResult>& o
   setup_sums_kernel<<<red_ctas, kThr, 0, st>>>(V, Ae, partials, 1);
   setup_ctrl_kernel<<<1, kMaxBatch, 0, st>>>(insts, B, partials, red_ctas, 1, a.prm);
   init_state_kernel<double><<<eb, kThr, 0, st>>>(V);
+  // A^T g1y, A^T g2y per instance: the y-parts of M^{-1} h1, M^{-1} h2 (rows 0..m-1 of G1, G2)
+  ck(gemm<double>(true, A64, n, n, B, m, V.G1, B, ATG1, work64, wk64, sms, st), "A^T G1");
+  ck(gemm<double>(true, A64, n, n, B, m, V.G2, B, ATG2, work64, wk64, sms, st), "A^T G2");
+  if (!mixed) ck(cudaMemsetAsync(V.ATY, 0, (size_t)n * B * 8, st), "memset");   // y = 0
   if (mixed) {
-    // A^T g1y, A^T g2y per instance: the y-parts of M^{-1} h1, M^{-1} h2 (rows 0..m-1 of G1, G2)
-    ck(gemm<double>(true, A64, n, n, B, m, V.G1, B, ATG1, work64, wk64, sms, st), "A^T G1");
-    ck(gemm<double>(true, A64, n, n, B, m, V.G2, B, ATG2, work64, wk64, sms, st), "A^T G2");
     const int cb = sms * 8;
     if (tc) {
       bf16_copies_kernel<<<cb, kThr, 0, st>>>(A64, m, n, terms, A16, AT16);
@@ -1255,8 +1285,8 @@ int shared_batch_run(const SharedBatchArgs& a, std::vector<SharedBatchResult>& o
                     gate), "refresh A [X S]");
     ck(gemm<double>(true, A64, n, n, B, m, V.Y, B, V.ATY, work64, wk64, sms, st, 0.0, nullptr, nullptr, 0, gate),
        "refresh A^T Y");
-    sums_kernel<double><<<red_ctas, kThr, 0, st>>>(V, insts, partials, V.Q, gate, nullptr, nullptr);
-    partials_total_kernel<9><<<B, kThr, 0, st>>>(partials, red_ctas, totals);
+    sums_kernel<double><<<red_cyc, kThr, 0, st>>>(V, insts, partials, V.Q, gate, nullptr, nullptr);
+    partials_total_kernel<9><<<B, kThr, 0, st>>>(partials, red_cyc, totals);
     ctrl_confirm_kernel<<<1, kMaxBatch, 0, st>>>(insts, B, totals, 1, a.prm, flags);
     ck(gemm<double>(false, Ginv64, m, m, B, m, V.Q, B, V.ZY, work64, wk64, sms, st, 0.0, nullptr, nullptr, 0, gate),
        "refresh Ginv Q");
@@ -1266,26 +1296,25 @@ int shared_batch_run(const SharedBatchArgs& a, std::vector<SharedBatchResult>& o
     launches += 12;
   };
   // ---- Algorithm 2, all instances in lockstep
+  // A^T Y follows from the update's linearity (update_kernel), as in mixed precision
   auto cycle64 = [&]() {
     ck(gemm<double>(false, A64, n, m, 2 * B, n, V.XS, 2 * B, V.AXS, work64, wk64, sms, st), "A [X S]");
-    ck(gemm<double>(true, A64, n, n, B, m, V.Y, B, V.ATY, work64, wk64, sms, st), "A^T Y");
-    sums_kernel<double><<<red_ctas, kThr, 0, st>>>(V, insts, partials, V.Q, nullptr, nullptr, nullptr);
-    partials_total_kernel<9><<<B, kThr, 0, st>>>(partials, red_ctas, totals);
+    sums_kernel<double><<<red_cyc, kThr, 0, st>>>(V, insts, partials, V.Q, nullptr, nullptr, nullptr);
+    partials_total_kernel<9><<<B, kThr, 0, st>>>(partials, red_cyc, totals);
     ctrl_eval_kernel<<<1, kMaxBatch, 0, st>>>(insts, B, n, totals, 1, a.prm, flags);
     ck(gemm<double>(false, Ginv64, m, m, B, m, V.Q, B, V.ZY, work64, wk64, sms, st), "Ginv Q");
-    ck(gemm<double>(true, A64, n, n, B, m, V.ZY, B, V.ZX, work64, wk64, sms, st, 0.0, V.XS, V.XS + B, 2 * B),
-       "A^T ZY");
-    hz_kernel<double><<<red_ctas, kThr, 0, st>>>(V, partials);
-    partials_total_kernel<2><<<B, kThr, 0, st>>>(partials, red_ctas, totals);
+    ck(gemm<double>(true, A64, n, n, B, m, V.ZY, B, ATZY, work64, wk64, sms, st), "A^T ZY");
+    hz_kernel<<<red_cyc, kThr, 0, st>>>(V, ATZY, nullptr, insts, partials);
+    partials_total_kernel<2><<<B, kThr, 0, st>>>(partials, red_cyc, totals);
     ctrl_step_kernel<<<1, kMaxBatch, 0, st>>>(insts, B, n, totals, 1, a.prm);
-    update_kernel<double><<<eb, kThr, 0, st>>>(V, insts, a.prm, nullptr, nullptr, nullptr, nullptr);
-    launches += 15;
+    update_kernel<double><<<eb, kThr, 0, st>>>(V, insts, a.prm, nullptr, ATZY, ATG1, ATG2);
+    launches += 13;
   };
   // with_refresh: this cycle's number is a multiple of a.prm.refresh, so ctrl_eval_kernel
   // opens the gate of the FP64 refresh; other cycles leave its kernels out altogether
   auto cycle_mixed = [&](bool with_refresh) {
-    sums_kernel<double><<<red_ctas, kThr, 0, st>>>(V, insts, partials, V.Q, nullptr, Qprev, dQ);
-    partials_total_kernel<9><<<B, kThr, 0, st>>>(partials, red_ctas, totals);
+    sums_kernel<double><<<red_cyc, kThr, 0, st>>>(V, insts, partials, V.Q, nullptr, Qprev, dQ);
+    partials_total_kernel<9><<<B, kThr, 0, st>>>(partials, red_cyc, totals);
     ctrl_eval_kernel<<<1, kMaxBatch, 0, st>>>(insts, B, n, totals, 1, a.prm, flags);
     launches += 3;
     if (with_refresh) refresh();
@@ -1295,8 +1324,8 @@ int shared_batch_run(const SharedBatchArgs& a, std::vector<SharedBatchResult>& o
                        derr + 1, st),
                "A^T dZY");
     else ck(gemm_acc(true, A32, n, n, B, m, dZY, B, B, ATZY, nullptr, nullptr, work32, wk32, sms, st), "A^T dZY");
-    hz_delta_kernel<<<red_ctas, kThr, 0, st>>>(V, ATZY, Qprev, insts, partials);
-    partials_total_kernel<2><<<B, kThr, 0, st>>>(partials, red_ctas, totals);
+    hz_kernel<<<red_cyc, kThr, 0, st>>>(V, ATZY, Qprev, insts, partials);
+    partials_total_kernel<2><<<B, kThr, 0, st>>>(partials, red_cyc, totals);
     ctrl_step_kernel<<<1, kMaxBatch, 0, st>>>(insts, B, n, totals, 1, a.prm);
     update_kernel<double><<<eb, kThr, 0, st>>>(V, insts, a.prm, dXS, ATZY, ATG1, ATG2);
     // maintained products of the new state: AX, AS += A [dX dS] (A^T Y in update_kernel)
