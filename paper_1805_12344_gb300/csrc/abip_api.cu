@@ -1564,16 +1564,33 @@ int abip_solve_batch_shared(int32_t count, const abip_matrix* A, const double* c
   int rc = validate_matrix(&tmp, A);
   if (rc) return fail(nullptr, rc, tmp.err);
   const int m = A->m, n = A->n;
-  std::vector<double> Ah;
-  rc = read_matrix_dense(&tmp, A, Ah);
-  if (rc) return fail(nullptr, rc, tmp.err);
-  std::vector<std::vector<double>> hb(count), hc(count);
-  for (int k = 0; k < count; ++k) {
+  for (int k = 0; k < count; ++k)
     if (!b[k] || !c[k]) return fail(nullptr, ABIP_E_INVALID_ARG, "instance " + std::to_string(k) + ": b or c is NULL");
-    if (fetch(b[k], m, is_device_ptr(b[k]), hb[k]) != cudaSuccess || fetch(c[k], n, is_device_ptr(c[k]), hc[k]) != cudaSuccess)
-      return fail(nullptr, ABIP_E_CUDA, "reading b, c");
-    if (!finite_all(hb[k].data(), m) || !finite_all(hc[k].data(), n))
-      return fail(nullptr, ABIP_E_INVALID_ARG, "instance " + std::to_string(k) + ": non-finite b or c");
+  // A: read to the host and checked there, or copied and checked on the device it is on
+  std::vector<double> Ah;
+  double* Ad = nullptr;
+  struct Free { double** p; ~Free() { if (*p) cudaFree(*p); } } free_Ad{&Ad};
+  int look = 0;
+  cudaPointerAttributes at{};
+  const bool on_dev = A->on_device && cudaPointerGetAttributes(&at, A->val) == cudaSuccess &&
+                      at.type == cudaMemoryTypeDevice && at.device == tmp.device;
+  cudaGetLastError();
+  if (on_dev) {
+    if (A->ld < n) return fail(nullptr, ABIP_E_DIM, "ld < n");
+    if (cudaMalloc(&Ad, (size_t)m * n * 8) != cudaSuccess) {
+      cudaGetLastError();
+      Ad = nullptr;
+      return fail(nullptr, ABIP_E_OOM, "shared batch: cannot allocate A");
+    }
+    const cudaError_t e = abip::shared_read_matrix(A->val, A->dtype == ABIP_F32, A->ld, m, n, Ad, &look);
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      return fail(nullptr, e == cudaErrorMemoryAllocation ? ABIP_E_OOM : ABIP_E_CUDA, std::string("reading A: ") + cudaGetErrorString(e));
+    }
+    if (look & abip::SH_NONFINITE) return fail(nullptr, ABIP_E_INVALID_ARG, "A has non-finite entries");
+  } else {
+    rc = read_matrix_dense(&tmp, A, Ah);
+    if (rc) return fail(nullptr, rc, tmp.err);
   }
   abip::ShParams sp{};
   sp.beta = prm.beta; sp.gamma = prm.gamma; sp.alpha = prm.alpha; sp.eps = prm.eps;
@@ -1584,24 +1601,24 @@ int abip_solve_batch_shared(int32_t count, const abip_matrix* A, const double* c
   if (prm.precision == ABIP_PREC_MIXED_BF16) {
     // the tensor-core products take A as bfloat16 terms: one when A is exact in bfloat16,
     // three otherwise (they hold A's FP32 value exactly); A must lie in the FP32 range
-    sp.tc = 1;
     for (const double v : Ah) {
       const float f = (float)v;
-      if (!std::isfinite(f))
-        return fail(nullptr, ABIP_E_INVALID_ARG, "ABIP_PREC_MIXED_BF16 needs A within the FP32 range");
       uint32_t u;
       std::memcpy(&u, &f, 4);
-      if ((double)f != v || (u & 0xFFFFu) != 0) sp.tc = 3;
+      if (!std::isfinite(f)) look |= abip::SH_BEYOND_F32;
+      if ((double)f != v || (u & 0xFFFFu) != 0) look |= abip::SH_NOT_BF16;
     }
+    if (look & abip::SH_BEYOND_F32)
+      return fail(nullptr, ABIP_E_INVALID_ARG, "ABIP_PREC_MIXED_BF16 needs A within the FP32 range");
+    sp.tc = look & abip::SH_NOT_BF16 ? 3 : 1;
   }
   sp.n = n;
   sp.confirm_gap = std::max<int64_t>(prm.check_every, 20);
   sp.refresh = 192;   // a multiple of the 16-cycle groups of the shared-A solve loop
   for (int k0 = 0; k0 < count; k0 += 64) {
     const int cnt = std::min(64, count - k0);
-    std::vector<const double*> bp(cnt), cp(cnt);
-    for (int k = 0; k < cnt; ++k) { bp[k] = hb[k0 + k].data(); cp[k] = hc[k0 + k].data(); }
-    abip::SharedBatchArgs args{m, n, cnt, Ah.data(), bp.data(), cp.data(), sp, static_cast<cudaStream_t>(stream)};
+    abip::SharedBatchArgs args{m, n, cnt, Ad ? nullptr : Ah.data(), Ad, b + k0, c + k0, sp, static_cast<cudaStream_t>(stream), k0,
+                               x ? x + k0 : nullptr, y ? y + k0 : nullptr, s ? s + k0 : nullptr};
     std::vector<abip::SharedBatchResult> res;
     std::string err;
     rc = abip::shared_batch_run(args, res, err);
@@ -1620,15 +1637,7 @@ int abip_solve_batch_shared(int32_t count, const abip_matrix* A, const double* c
         f.beta = prm.beta;
         f.setup_s = res[k].setup_s; f.solve_s = el; f.kernel_s = res[k].kernel_s; f.launches = res[k].launches;
       }
-      auto put = [&](double* dst, const std::vector<double>& v) {
-        if (rc == ABIP_OK && dst && cudaMemcpy(dst, v.data(), v.size() * 8, cudaMemcpyDefault) != cudaSuccess)
-          rc = fail(nullptr, ABIP_E_CUDA, "output copy");
-      };
-      if (x) put(x[id], res[k].x);
-      if (y) put(y[id], res[k].y);
-      if (s) put(s[id], res[k].s);
     }
-    if (rc) return rc;
   }
   return ABIP_OK;
 }

@@ -380,16 +380,26 @@ struct ShView {
 
 struct SharedBatchArgs {
   int m, n, count;                 // count <= 64
-  const double* A;                 // host, m x n row-major FP64
-  const double* const* b;          // host, count vectors of m
-  const double* const* c;          // host, count vectors of n
+  const double* A;                 // host, m x n row-major FP64, or null
+  const double* A_dev;             // device, the same (used in place)
+  const double* const* b;          // count vectors of m, host or device
+  const double* const* c;          // count vectors of n, host or device
   ShParams prm;
   cudaStream_t stream;
+  int first;                       // number of the first instance (messages)
+  double* const* x;                // outputs, each host or device, entries (and arrays) may be null
+  double* const* y;
+  double* const* s;
 };
+
+// What the shared-A batch asks of its matrix (bits): an entry that is not finite, one beyond FP32's
+// range, one that is no bfloat16 value.
+enum ShLook : int { SH_NONFINITE = 1, SH_BEYOND_F32 = 2, SH_NOT_BF16 = 4 };
+// A on the device (device source, FP64 or FP32, ld) as m x n FP64 in dst, and its SH_* bits in *look
+cudaError_t shared_read_matrix(const void* src, bool f32, int64_t ld, int m, int n, double* dst, int* look);
 
 struct SharedBatchResult {
   ShInst inst;
-  std::vector<double> x, y, s;     // scaled outputs (Sec. 4.1)
   double setup_s;                  // device time of the setup (Gram, Cholesky, inverse, M^{-1} H)
   double kernel_s;                 // device time of the iterations
   int64_t launches;

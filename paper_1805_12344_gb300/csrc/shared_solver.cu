@@ -905,6 +905,27 @@ __global__ void output_kernel(ShView<T> V, const ShInst* __restrict__ insts, dou
   }
 }
 
+// flags[k] = 1 where column k of an [len x B] array holds a value that is not finite
+__global__ void finite_columns_kernel(const double* __restrict__ v, size_t len, int B, int* flags) {
+  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < len * B; e += (size_t)gridDim.x * blockDim.x)
+    if (!isfinite(v[e])) atomicOr(flags + (int)(e % B), 1);
+}
+
+// A's values (from an FP32 source: converted) and its SH_* bits
+__global__ void look_kernel(const float* __restrict__ src, double* __restrict__ A, size_t len, int* look) {
+  int bits = 0;
+  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < len; e += (size_t)gridDim.x * blockDim.x) {
+    const double v = src ? (double)src[e] : A[e];
+    if (src) A[e] = v;
+    const float f = (float)v;
+    if (!isfinite(v)) bits |= SH_NONFINITE;
+    if (!isfinite(f)) bits |= SH_BEYOND_F32;
+    if ((double)f != v || (__float_as_uint(f) & 0xFFFFu) != 0) bits |= SH_NOT_BF16;
+  }
+  bits = __reduce_or_sync(0xffffffffu, bits);
+  if ((threadIdx.x & 31) == 0 && bits) atomicOr(look, bits);
+}
+
 // ---------------------------------------------------------------------------
 // Host side
 // ---------------------------------------------------------------------------
@@ -1074,6 +1095,25 @@ struct Bump {
 
 }  // namespace
 
+cudaError_t shared_read_matrix(const void* src, bool f32, int64_t ld, int m, int n, double* dst, int* look) {
+  const size_t w = f32 ? 4 : 8, len = (size_t)m * n;
+  float* stage = nullptr;
+  int* dlook = nullptr;
+  cudaError_t e = cudaMalloc(&dlook, sizeof(int));
+  if (e == cudaSuccess && f32) e = cudaMalloc(&stage, len * 4);
+  if (e == cudaSuccess) e = cudaMemsetAsync(dlook, 0, sizeof(int), 0);
+  if (e == cudaSuccess)
+    e = cudaMemcpy2DAsync(f32 ? (void*)stage : (void*)dst, n * w, src, (size_t)ld * w, n * w, m, cudaMemcpyDeviceToDevice, 0);
+  if (e == cudaSuccess) {
+    look_kernel<<<1216, kThr>>>(stage, dst, len, dlook);
+    e = cudaGetLastError();
+  }
+  if (e == cudaSuccess) e = cudaMemcpy(look, dlook, sizeof(int), cudaMemcpyDeviceToHost);
+  if (stage) cudaFree(stage);
+  if (dlook) cudaFree(dlook);
+  return e;
+}
+
 // One chunk of <= 64 instances sharing A.
 int shared_batch_run(const SharedBatchArgs& a, std::vector<SharedBatchResult>& out, std::string& err) {
   const int m = a.m, n = a.n, B = a.count;
@@ -1128,11 +1168,11 @@ int shared_batch_run(const SharedBatchArgs& a, std::vector<SharedBatchResult>& o
         *dZY = nullptr;
   ShInst* insts = nullptr;
   DenseInst* dinv = nullptr;
-  int *flags = nullptr, *derr = nullptr;
+  int *flags = nullptr, *derr = nullptr, *bad = nullptr;
   Bump bp;
   auto layout = [&]() {
     bp.off = 0;
-    A64 = bp.take<double>((size_t)m * n);
+    A64 = a.A_dev ? const_cast<double*>(a.A_dev) : bp.take<double>((size_t)m * n);
     AT64 = bp.take<double>((size_t)n * m);
     G = bp.take<double>((size_t)m * m);
     Ginv64 = bp.take<double>((size_t)m * m);
@@ -1144,6 +1184,7 @@ int shared_batch_run(const SharedBatchArgs& a, std::vector<SharedBatchResult>& o
     dinv = bp.take<DenseInst>(1);
     flags = bp.take<int>(8);
     derr = bp.take<int>(8);
+    bad = bp.take<int>(kMaxBatch);
     W2 = bp.take<double>((size_t)n * 2 * B);
     P2 = bp.take<double>((size_t)m * 2 * B);
     R = bp.take<double>((size_t)m * 2 * B);
@@ -1204,18 +1245,36 @@ int shared_batch_run(const SharedBatchArgs& a, std::vector<SharedBatchResult>& o
   cudaEventCreate(&es);
   cudaEventCreate(&e1);
   // ---- inputs: A (m x n FP64) and the per-instance vectors in [len x B] layout
+  // (each vector to a row of Xo, Yo, which are transposed and looked over on the device)
+  if (a.A) ck(cudaMemcpyAsync(A64, a.A, (size_t)m * n * 8, cudaMemcpyHostToDevice, st), "upload A");
+  for (int k = 0; k < B; ++k) {
+    ck(cudaMemcpyAsync(Yo + (size_t)k * m, a.b[k], (size_t)m * 8, cudaMemcpyDefault, st), "upload b");
+    ck(cudaMemcpyAsync(Xo + (size_t)k * n, a.c[k], (size_t)n * 8, cudaMemcpyDefault, st), "upload c");
+  }
+  transpose_kernel<double><<<dim3((m + 31) / 32, (B + 31) / 32), dim3(32, 8), 0, st>>>(Yo, B, m, V.b);
+  transpose_kernel<double><<<dim3((n + 31) / 32, (B + 31) / 32), dim3(32, 8), 0, st>>>(Xo, B, n, V.c);
+  ck(cudaMemsetAsync(derr, 0, 8 * sizeof(int), st), "memset");
+  ck(cudaMemsetAsync(flags, 0, 8 * sizeof(int), st), "memset");
+  ck(cudaMemsetAsync(bad, 0, kMaxBatch * sizeof(int), st), "memset");
+  finite_columns_kernel<<<eb, kThr, 0, st>>>(V.b, m, B, bad);
+  finite_columns_kernel<<<eb, kThr, 0, st>>>(V.c, n, B, bad);
   {
-    std::vector<double> hb((size_t)m * B), hc((size_t)n * B);
-    for (int k = 0; k < B; ++k) {
-      for (int i = 0; i < m; ++i) hb[(size_t)i * B + k] = a.b[k][i];
-      for (int j = 0; j < n; ++j) hc[(size_t)j * B + k] = a.c[k][j];
+    int hbad[kMaxBatch] = {};
+    ck(cudaMemcpyAsync(hbad, bad, B * sizeof(int), cudaMemcpyDeviceToHost, st), "look");
+    ck(cudaStreamSynchronize(st), "upload");
+    for (int k = 0; k < B && rc == ABIP_OK; ++k)
+      if (hbad[k]) {
+        err = "instance " + std::to_string(a.first + k) + ": non-finite b or c";
+        rc = ABIP_E_INVALID_ARG;
+      }
+    if (rc != ABIP_OK) {
+      cudaEventDestroy(e0);
+      cudaEventDestroy(es);
+      cudaEventDestroy(e1);
+      cudaFree(arena);
+      if (owned) cudaStreamDestroy(owned);
+      return rc;
     }
-    ck(cudaMemcpyAsync(A64, a.A, (size_t)m * n * 8, cudaMemcpyHostToDevice, st), "upload A");
-    ck(cudaMemcpyAsync(V.b, hb.data(), hb.size() * 8, cudaMemcpyHostToDevice, st), "upload b");
-    ck(cudaMemcpyAsync(V.c, hc.data(), hc.size() * 8, cudaMemcpyHostToDevice, st), "upload c");
-    ck(cudaMemsetAsync(derr, 0, 8 * sizeof(int), st), "memset");
-    ck(cudaMemsetAsync(flags, 0, 8 * sizeof(int), st), "memset");
-    ck(cudaStreamSynchronize(st), "upload");   // the host staging vectors go out of scope here
   }
   cudaEventRecord(e0, st);
   // ---- setup (FP64): embedding constants (Eq. bar-b-c-z-re)
@@ -1417,12 +1476,17 @@ int shared_batch_run(const SharedBatchArgs& a, std::vector<SharedBatchResult>& o
   if (rc == ABIP_OK) {
     output_kernel<double><<<eb, kThr, 0, st>>>(V, insts, Xo, Yo, So);
     cudaEventRecord(e1, st);
+    // instance by instance, in buffers that the iterations no longer need
+    double *xt = V.ZX, *st_ = ATZY, *yt = V.Q;
+    auto turn = [&](const double* from, int len, double* to) {
+      transpose_kernel<double><<<dim3((B + 31) / 32, (len + 31) / 32), dim3(32, 8), 0, st>>>(from, len, B, to);
+    };
+    turn(Xo, n, xt);
+    turn(So, n, st_);
+    turn(Yo, m, yt);
     std::vector<ShInst> hi(B);
-    std::vector<double> hx((size_t)n * B), hy((size_t)m * B), hs((size_t)n * B);
+    ck(cudaGetLastError(), "outputs");
     ck(cudaMemcpyAsync(hi.data(), insts, sizeof(ShInst) * B, cudaMemcpyDeviceToHost, st), "results");
-    ck(cudaMemcpyAsync(hx.data(), Xo, hx.size() * 8, cudaMemcpyDeviceToHost, st), "x");
-    ck(cudaMemcpyAsync(hy.data(), Yo, hy.size() * 8, cudaMemcpyDeviceToHost, st), "y");
-    ck(cudaMemcpyAsync(hs.data(), So, hs.size() * 8, cudaMemcpyDeviceToHost, st), "s");
     ck(cudaStreamSynchronize(st), "outputs");
     float ms_setup = 0.f, ms_iter = 0.f;
     cudaEventElapsedTime(&ms_setup, e0, es);
@@ -1435,14 +1499,21 @@ int shared_batch_run(const SharedBatchArgs& a, std::vector<SharedBatchResult>& o
       r.kernel_s = ms_iter * 1e-3;
       r.launches = launches;
       r.tensor_cores = tc;
-      r.x.resize(n); r.y.resize(m); r.s.resize(n);
-      for (int j = 0; j < n; ++j) { r.x[j] = hx[(size_t)j * B + k]; r.s[j] = hs[(size_t)j * B + k]; }
-      for (int i = 0; i < m; ++i) r.y[i] = hy[(size_t)i * B + k];
       if (hi[k].err != 0) {
-        err = "shared batch instance " + std::to_string(k) + ": non-finite reduction";
+        err = "shared batch instance " + std::to_string(a.first + k) + ": non-finite reduction";
         rc = ABIP_E_NUMERICAL;
       }
     }
+    auto put = [&](double* const* dst, int k, const double* from, int len) {
+      if (rc == ABIP_OK && dst && dst[k])
+        ck(cudaMemcpyAsync(dst[k], from + (size_t)k * len, (size_t)len * 8, cudaMemcpyDefault, st), "output copy");
+    };
+    for (int k = 0; k < B; ++k) {
+      put(a.x, k, xt, n);
+      put(a.y, k, yt, m);
+      put(a.s, k, st_, n);
+    }
+    ck(cudaStreamSynchronize(st), "output copies");
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(es);

@@ -82,3 +82,24 @@ def test_non_finite_device_input_is_refused(abip, which):
     with pytest.raises(abip.AbipError) as e:
         abip.abip_solve_batch(*[list(p) for p in zip(good, bad)])
     assert e.value.code == abip.ABIP_E_INVALID_ARG
+
+
+@pytest.mark.parametrize("precision", [0, 1, 2])
+def test_shared_batch_device_inputs_equal_host_inputs(abip, precision):
+    """The shared-A batch reads a device A (FP32 or FP64), b and c in place: the bits of the host route."""
+    lps = W.basis_pursuit(40, 90, batch=5, seed=21)
+    prm = abip.default_params(precision=precision, max_admm_iters=40)
+    A32 = lps.A.astype(np.float32)
+    runs = []
+    for A, on in ((lps.A, False), (torch.from_numpy(lps.A).cuda(), True), (torch.from_numpy(A32).cuda(), True)):
+        vec = (lambda v: torch.from_numpy(v).cuda()) if on else (lambda v: v)
+        infos, xs, ys, ss = abip.abip_solve_batch_shared(A, [vec(v) for v in lps.bs], [vec(v) for v in lps.cs], prm)
+        runs.append(np.concatenate([np.concatenate(t) for t in (xs, ys, ss)]))
+    assert np.array_equal(runs[0], runs[1]) and np.array_equal(runs[0], runs[2])
+    bad = [torch.from_numpy(v).cuda() for v in lps.bs]
+    bad[3][-1] = float("nan")
+    for A, b in ((torch.full((40, 180), float("inf"), device="cuda", dtype=torch.float64), lps.bs),
+                 (torch.from_numpy(lps.A).cuda(), bad)):
+        with pytest.raises(abip.AbipError) as e:
+            abip.abip_solve_batch_shared(A, b, lps.cs, prm)
+        assert e.value.code == abip.ABIP_E_INVALID_ARG
