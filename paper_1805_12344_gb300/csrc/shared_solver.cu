@@ -1120,8 +1120,7 @@ int shared_batch_run(const SharedBatchArgs& a, std::vector<SharedBatchResult>& o
   const bool mixed = a.prm.mixed != 0;
   if (B < 1 || B > kMaxBatch) { err = "shared batch: a chunk holds 1..64 instances"; return ABIP_E_INVALID_ARG; }
   // the update cycles are captured in a CUDA graph, which the legacy default stream cannot
-  // record: without a caller stream the solve runs on its own (it is synchronous, and its
-  // inputs are staged through host memory first)
+  // record: without a caller stream the solve runs on its own
   cudaStream_t st = a.stream;
   cudaStream_t owned = nullptr;
   if (!st) {
@@ -1244,6 +1243,10 @@ int shared_batch_run(const SharedBatchArgs& a, std::vector<SharedBatchResult>& o
   cudaEventCreate(&e0);
   cudaEventCreate(&es);
   cudaEventCreate(&e1);
+  // b, c and the outputs may be device memory that work on the default stream (and on streams that
+  // it waits for) still fills or reads, and st waits for neither: that work ends first
+  ck(cudaMemsetAsync(derr, 0, 8 * sizeof(int), 0), "memset");
+  ck(cudaStreamSynchronize(0), "default stream");
   // ---- inputs: A (m x n FP64) and the per-instance vectors in [len x B] layout
   // (each vector to a row of Xo, Yo, which are transposed and looked over on the device)
   if (a.A) ck(cudaMemcpyAsync(A64, a.A, (size_t)m * n * 8, cudaMemcpyHostToDevice, st), "upload A");
@@ -1253,7 +1256,6 @@ int shared_batch_run(const SharedBatchArgs& a, std::vector<SharedBatchResult>& o
   }
   transpose_kernel<double><<<dim3((m + 31) / 32, (B + 31) / 32), dim3(32, 8), 0, st>>>(Yo, B, m, V.b);
   transpose_kernel<double><<<dim3((n + 31) / 32, (B + 31) / 32), dim3(32, 8), 0, st>>>(Xo, B, n, V.c);
-  ck(cudaMemsetAsync(derr, 0, 8 * sizeof(int), st), "memset");
   ck(cudaMemsetAsync(flags, 0, 8 * sizeof(int), st), "memset");
   ck(cudaMemsetAsync(bad, 0, kMaxBatch * sizeof(int), st), "memset");
   finite_columns_kernel<<<eb, kThr, 0, st>>>(V.b, m, B, bad);

@@ -103,3 +103,20 @@ def test_shared_batch_device_inputs_equal_host_inputs(abip, precision):
         with pytest.raises(abip.AbipError) as e:
             abip.abip_solve_batch_shared(A, b, lps.cs, prm)
         assert e.value.code == abip.ABIP_E_INVALID_ARG
+
+
+def test_shared_batch_waits_for_work_on_the_default_stream(abip):
+    """A on the host; b and c on the device, written on the default stream after a long kernel."""
+    lps = W.basis_pursuit(40, 90, batch=5, seed=22)
+    prm = abip.default_params(max_admm_iters=20)
+    want = np.concatenate(abip.abip_solve_batch_shared(lps.A, lps.bs, lps.cs, prm)[1])
+    src = [torch.from_numpy(v).cuda() for v in [*lps.bs, *lps.cs]]
+    dst = [torch.zeros_like(v) for v in src]
+    busy = torch.ones(8192, 8192, device="cuda")
+    torch.cuda.synchronize()
+    for _ in range(20):   # some 10 ms each
+        busy = busy @ busy * 1e-4
+    for d, v in zip(dst, src):
+        d.copy_(v)
+    got = np.concatenate(abip.abip_solve_batch_shared(lps.A, dst[:5], dst[5:], prm)[1])
+    assert np.array_equal(got, want)
