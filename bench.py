@@ -100,11 +100,11 @@ def algorithmic_bytes(m, n, nnz, admm_iters, cg_iters, vec_bytes, val_bytes=4):
 KERNEL_SOURCES = ("paper_1805_12344_gb300/csrc/grid_delta.cu", "paper_1805_12344_gb300/csrc/sell.cuh",
                   "paper_1805_12344_gb300/csrc/abip_device.cuh", "paper_1805_12344_gb300/csrc/sell_host.h")
 # DRAM bytes of one solve launch from ncu (dram__bytes_read.sum + dram__bytes_write.sum) at
-# 20 and 60 updates, caches flushed before the launch: 596.0 MB and 1585.0 MB, so
-# 101.5 MB fixed + 24.72 MB per update (profiles/grid_delta_kernel_solve_sparse_m100000.md);
+# 20 and 60 updates, caches flushed before the launch: 656.1 MB and 1764.2 MB, so
+# 102.1 MB fixed + 27.70 MB per update (profiles/grid_delta_kernel_solve_sparse_m100000.md);
 # valid while the sources above are the ones measured.
-TRAFFIC = {"sources_sha256": "c9e17702ca9d067a39c456c66b8e70d58bde0a93626023c2521eb21554d8e93f",
-           "dram_bytes_fixed": 101535488, "dram_bytes_per_update": 24724185.6}
+TRAFFIC = {"sources_sha256": "c3d55137c3f226b8c13ff8983d783882c82a8304c5220eb08a06d3e14d3779e2",
+           "dram_bytes_fixed": 102076288, "dram_bytes_per_update": 27701600.0}
 
 
 def kernel_sources_hash():
