@@ -281,8 +281,21 @@ int setup_grid_path(abip_handle* h, G& g, const HostCSR& A, const std::vector<do
   h->grid = grid;
 
   constexpr bool delta = std::is_same<G, abip::GridDelta>::value;
-  const double per_lane = delta ? 32.0 : 16.0;
-  const HostSell SA = to_sell(A, sell_lanes(A, per_lane)), ST = to_sell(AT, sell_lanes(AT, per_lane));
+  // FP64: more lanes per row, down to 4 entries per lane, while all rows' lanes fit in two thirds of
+  // the grid's threads: a phase of a small LP lasts as long as one lane's chain of L2 round trips,
+  // and the other threads idle.  Measured (25 entries per row of A, us per update; lanes of at most
+  // 16 entries / of 4): m = 300 485 / 405, 2000 522 / 433, 8000 506 / 473, 16000 543 / 533; with
+  // nearly all threads in use they cost more than they save (24000 615 / 642, 40000 789 / 951).
+  // Mixed precision keeps its lanes: a sum in another order changes the rounding of the FP32
+  // changes, and x by 1e-6 to 1e-5 of itself (FP64: 4e-14).
+  auto lanes = [&](const HostCSR& M) {
+    int L = sell_lanes(M, delta ? 32.0 : 16.0);
+    const double mean = M.m > 0 ? (double)M.rp[M.m] / M.m : 0.0;
+    const int64_t room = (int64_t)grid * abip::kGridThreads * 2 / 3;
+    while (!delta && L < 32 && mean > 4.0 * L && 2 * (int64_t)L * M.m <= room) L *= 2;
+    return L;
+  };
+  const HostSell SA = to_sell(A, lanes(A)), ST = to_sell(AT, lanes(AT));
   const int wpc = abip::kGridThreads / 32;
   const std::vector<int32_t> wpA = warp_partition(SA, grid * wpc), wpT = warp_partition(ST, grid * wpc);
 
