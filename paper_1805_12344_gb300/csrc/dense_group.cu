@@ -698,6 +698,7 @@ __global__ void __launch_bounds__(kThr, MINB) dense_cluster_kernel(GroupArgs Q) 
   __shared__ int s_id;
   cg::cluster_group cl = cg::this_cluster();
   Group<false> G(GridBarrier{});
+  cl.sync();   // no CTA writes to a peer (s_id below) that may not have started
   for (;;) {
     if (G.rank == 0 && threadIdx.x == 0) {
       const int k = atomicAdd(Q.queue, 1);

@@ -537,6 +537,7 @@ __global__ void __launch_bounds__(kThr, MINB) dense_mixed_kernel(MixArgs Q) {
   __shared__ MixScal S;
   __shared__ int s_id;
   const cg::cluster_group cl = cg::this_cluster();
+  cl.sync();   // no CTA writes to a peer (s_id below) that may not have started
   for (;;) {
     if (cl.block_rank() == 0 && threadIdx.x == 0) {
       const int k = atomicAdd(Q.queue, 1);
