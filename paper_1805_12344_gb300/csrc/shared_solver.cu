@@ -358,16 +358,23 @@ __global__ void __launch_bounds__(kThr) inverse_kernel(const double* __restrict_
 template <typename T>
 __global__ void transpose_kernel(const double* __restrict__ A, int m, int n, T* __restrict__ AT) {
   __shared__ double t[32][33];
-  const int bx = blockIdx.x * 32, by = blockIdx.y * 32;
-  for (int r = threadIdx.y; r < 32; r += blockDim.y) {
-    const int i = by + r, j = bx + threadIdx.x;
-    t[r][threadIdx.x] = (i < m && j < n) ? A[(size_t)i * n + j] : 0.0;
+  const int bx = blockIdx.x * 32;
+  for (int by = blockIdx.y * 32; by < m; by += gridDim.y * 32) {
+    for (int r = threadIdx.y; r < 32; r += blockDim.y) {
+      const int i = by + r, j = bx + threadIdx.x;
+      t[r][threadIdx.x] = (i < m && j < n) ? A[(size_t)i * n + j] : 0.0;
+    }
+    __syncthreads();
+    for (int r = threadIdx.y; r < 32; r += blockDim.y) {
+      const int j = bx + r, i = by + threadIdx.x;
+      if (j < n && i < m) AT[(size_t)j * m + i] = (T)t[threadIdx.x][r];
+    }
+    __syncthreads();
   }
-  __syncthreads();
-  for (int r = threadIdx.y; r < 32; r += blockDim.y) {
-    const int j = bx + r, i = by + threadIdx.x;
-    if (j < n && i < m) AT[(size_t)j * m + i] = (T)t[threadIdx.x][r];
-  }
+}
+// AT (n x m) = A^T, A m x n row-major; a grid holds 65535 blocks of rows, the rest in a loop
+void launch_transpose(const double* A, int m, int n, double* AT, cudaStream_t st) {
+  transpose_kernel<double><<<dim3((n + 31) / 32, std::min((m + 31) / 32, 65535)), dim3(32, 8), 0, st>>>(A, m, n, AT);
 }
 
 template <typename T>
@@ -1254,8 +1261,8 @@ int shared_batch_run(const SharedBatchArgs& a, std::vector<SharedBatchResult>& o
     ck(cudaMemcpyAsync(Yo + (size_t)k * m, a.b[k], (size_t)m * 8, cudaMemcpyDefault, st), "upload b");
     ck(cudaMemcpyAsync(Xo + (size_t)k * n, a.c[k], (size_t)n * 8, cudaMemcpyDefault, st), "upload c");
   }
-  transpose_kernel<double><<<dim3((m + 31) / 32, (B + 31) / 32), dim3(32, 8), 0, st>>>(Yo, B, m, V.b);
-  transpose_kernel<double><<<dim3((n + 31) / 32, (B + 31) / 32), dim3(32, 8), 0, st>>>(Xo, B, n, V.c);
+  launch_transpose(Yo, B, m, V.b, st);
+  launch_transpose(Xo, B, n, V.c, st);
   ck(cudaMemsetAsync(flags, 0, 8 * sizeof(int), st), "memset");
   ck(cudaMemsetAsync(bad, 0, kMaxBatch * sizeof(int), st), "memset");
   finite_columns_kernel<<<eb, kThr, 0, st>>>(V.b, m, B, bad);
@@ -1284,7 +1291,7 @@ int shared_batch_run(const SharedBatchArgs& a, std::vector<SharedBatchResult>& o
   setup_sums_kernel<<<red_ctas, kThr, 0, st>>>(V, Ae, partials, 0);
   setup_ctrl_kernel<<<1, kMaxBatch, 0, st>>>(insts, B, partials, red_ctas, 0, a.prm);
   // G = I + A A^T (Sec. 4.4), its Cholesky factor and the explicit inverse
-  transpose_kernel<double><<<dim3((n + 31) / 32, (m + 31) / 32), dim3(32, 8), 0, st>>>(A64, m, n, AT64);
+  launch_transpose(A64, m, n, AT64, st);
   // (the factorisation and what follows read its lower triangle only)
   ck(gemm<double>(false, A64, n, m, m, n, AT64, m, G, work64, wk64, sms, st, 1.0, nullptr, nullptr, 0, nullptr, true), "Gram");
   ck(cholesky_blocked(G, m, derr, st), "Cholesky");
@@ -1480,12 +1487,9 @@ int shared_batch_run(const SharedBatchArgs& a, std::vector<SharedBatchResult>& o
     cudaEventRecord(e1, st);
     // instance by instance, in buffers that the iterations no longer need
     double *xt = V.ZX, *st_ = ATZY, *yt = V.Q;
-    auto turn = [&](const double* from, int len, double* to) {
-      transpose_kernel<double><<<dim3((B + 31) / 32, (len + 31) / 32), dim3(32, 8), 0, st>>>(from, len, B, to);
-    };
-    turn(Xo, n, xt);
-    turn(So, n, st_);
-    turn(Yo, m, yt);
+    launch_transpose(Xo, n, B, xt, st);
+    launch_transpose(So, n, B, st_, st);
+    launch_transpose(Yo, m, B, yt, st);
     std::vector<ShInst> hi(B);
     ck(cudaGetLastError(), "outputs");
     ck(cudaMemcpyAsync(hi.data(), insts, sizeof(ShInst) * B, cudaMemcpyDeviceToHost, st), "results");
