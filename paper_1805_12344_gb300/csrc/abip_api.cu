@@ -1605,6 +1605,14 @@ int abip_solve_batch_shared(int32_t count, const abip_matrix* A, const double* c
     rc = read_matrix_dense(&tmp, A, Ah);
     if (rc) return fail(nullptr, rc, tmp.err);
   }
+  abip::SharedVectors vec;
+  int bad = -1;
+  const cudaError_t ev = vec.read(count, m, n, b, c, static_cast<cudaStream_t>(stream), bad);
+  if (ev != cudaSuccess) {
+    cudaGetLastError();
+    return fail(nullptr, ev == cudaErrorMemoryAllocation ? ABIP_E_OOM : ABIP_E_CUDA, std::string("reading b, c: ") + cudaGetErrorString(ev));
+  }
+  if (bad >= 0) return fail(nullptr, ABIP_E_INVALID_ARG, "instance " + std::to_string(bad) + ": non-finite b or c");
   abip::ShParams sp{};
   sp.beta = prm.beta; sp.gamma = prm.gamma; sp.alpha = prm.alpha; sp.eps = prm.eps;
   sp.gamma_max = prm.gamma_max;
@@ -1630,8 +1638,8 @@ int abip_solve_batch_shared(int32_t count, const abip_matrix* A, const double* c
   sp.refresh = 192;   // a multiple of the 16-cycle groups of the shared-A solve loop
   for (int k0 = 0; k0 < count; k0 += 64) {
     const int cnt = std::min(64, count - k0);
-    abip::SharedBatchArgs args{m, n, cnt, Ad ? nullptr : Ah.data(), Ad, b + k0, c + k0, sp, static_cast<cudaStream_t>(stream), k0,
-                               x ? x + k0 : nullptr, y ? y + k0 : nullptr, s ? s + k0 : nullptr};
+    abip::SharedBatchArgs args{m, n, cnt, Ad ? nullptr : Ah.data(), Ad, vec.b + (size_t)k0 * m, vec.c + (size_t)k0 * n, vec.on_host,
+                               sp, static_cast<cudaStream_t>(stream), k0, x ? x + k0 : nullptr, y ? y + k0 : nullptr, s ? s + k0 : nullptr};
     std::vector<abip::SharedBatchResult> res;
     std::string err;
     rc = abip::shared_batch_run(args, res, err);

@@ -382,14 +382,32 @@ struct SharedBatchArgs {
   int m, n, count;                 // count <= 64
   const double* A;                 // host, m x n row-major FP64, or null
   const double* A_dev;             // device, the same (used in place)
-  const double* const* b;          // count vectors of m, host or device
-  const double* const* c;          // count vectors of n, host or device
+  const double* b;                 // count x m and count x n, read and checked by SharedVectors
+  const double* c;
+  bool vectors_on_host;
   ShParams prm;
   cudaStream_t stream;
   int first;                       // number of the first instance (messages)
   double* const* x;                // outputs, each host or device, entries (and arrays) may be null
   double* const* y;
   double* const* s;
+};
+
+// The b and c of all instances, read whole before the first chunk is solved: a bad vector is refused
+// before anything is written, and an output may lie where a later chunk's input lay.  On the device,
+// or on the host where the device has no room for them.
+struct SharedVectors {
+  const double* b = nullptr;       // count x m
+  const double* c = nullptr;       // count x n
+  bool on_host = false;
+  double* dev = nullptr;
+  std::vector<double> host;
+  SharedVectors() = default;
+  SharedVectors(const SharedVectors&) = delete;
+  SharedVectors& operator=(const SharedVectors&) = delete;
+  ~SharedVectors();
+  // b[k] (m) and c[k] (n), each host or device; bad: the first instance with a value that is not finite, or -1
+  cudaError_t read(int count, int m, int n, const double* const* b, const double* const* c, cudaStream_t st, int& bad);
 };
 
 // What the shared-A batch asks of its matrix (bits): an entry that is not finite, one beyond FP32's

@@ -24,6 +24,7 @@
 
 #include <algorithm>
 #include <cstring>
+#include <exception>
 #include <type_traits>
 #include <vector>
 
@@ -912,10 +913,10 @@ __global__ void output_kernel(ShView<T> V, const ShInst* __restrict__ insts, dou
   }
 }
 
-// flags[k] = 1 where column k of an [len x B] array holds a value that is not finite
-__global__ void finite_columns_kernel(const double* __restrict__ v, size_t len, int B, int* flags) {
-  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < len * B; e += (size_t)gridDim.x * blockDim.x)
-    if (!isfinite(v[e])) atomicOr(flags + (int)(e % B), 1);
+// *first = the smallest row of a [count x len] array that holds a value that is not finite
+__global__ void finite_rows_kernel(const double* __restrict__ v, size_t count, size_t len, int* first) {
+  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < len * count; e += (size_t)gridDim.x * blockDim.x)
+    if (!isfinite(v[e])) atomicMin(first, (int)(e / len));
 }
 
 // A's values (from an FP32 source: converted) and its SH_* bits
@@ -1121,6 +1122,56 @@ cudaError_t shared_read_matrix(const void* src, bool f32, int64_t ld, int m, int
   return e;
 }
 
+cudaError_t SharedVectors::read(int count, int m, int n, const double* const* b, const double* const* c, cudaStream_t st,
+                                int& bad) {
+  const size_t nb = (size_t)count * m, nc = (size_t)count * n;
+  int* first = nullptr;
+  if (cudaMalloc(&dev, (nb + nc) * 8 + sizeof(int)) == cudaSuccess) {
+    first = reinterpret_cast<int*>(dev + nb + nc);
+  } else {
+    cudaGetLastError();
+    dev = nullptr;
+    try {
+      host.resize(nb + nc);
+    } catch (const std::exception&) {
+      return cudaErrorMemoryAllocation;
+    }
+  }
+  on_host = dev == nullptr;
+  double* to = on_host ? host.data() : dev;
+  this->b = to;
+  this->c = to + nb;
+  // device inputs may still be filled by work on the default stream, which st need not wait for
+  cudaError_t e = cudaStreamSynchronize(0);
+  for (int k = 0; k < count && e == cudaSuccess; ++k) {
+    e = cudaMemcpyAsync(to + (size_t)k * m, b[k], (size_t)m * 8, cudaMemcpyDefault, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(to + nb + (size_t)k * n, c[k], (size_t)n * 8, cudaMemcpyDefault, st);
+  }
+  bad = count;
+  if (!on_host) {
+    if (e == cudaSuccess) e = cudaMemcpyAsync(first, &bad, sizeof(int), cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) {
+      finite_rows_kernel<<<608, kThr, 0, st>>>(this->b, count, m, first);
+      finite_rows_kernel<<<608, kThr, 0, st>>>(this->c, count, n, first);
+      e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&bad, first, sizeof(int), cudaMemcpyDeviceToHost, st);
+  }
+  const cudaError_t es = cudaStreamSynchronize(st);
+  if (e == cudaSuccess) e = es;
+  if (on_host && e == cudaSuccess)
+    for (int k = 0; k < count && bad == count; ++k) {
+      for (int i = 0; i < m; ++i) if (!std::isfinite(this->b[(size_t)k * m + i])) bad = k;
+      for (int j = 0; j < n; ++j) if (!std::isfinite(this->c[(size_t)k * n + j])) bad = k;
+    }
+  if (bad == count) bad = -1;
+  return e;
+}
+
+SharedVectors::~SharedVectors() {
+  if (dev) cudaFree(dev);
+}
+
 // One chunk of <= 64 instances sharing A.
 int shared_batch_run(const SharedBatchArgs& a, std::vector<SharedBatchResult>& out, std::string& err) {
   const int m = a.m, n = a.n, B = a.count;
@@ -1174,7 +1225,7 @@ int shared_batch_run(const SharedBatchArgs& a, std::vector<SharedBatchResult>& o
         *dZY = nullptr;
   ShInst* insts = nullptr;
   DenseInst* dinv = nullptr;
-  int *flags = nullptr, *derr = nullptr, *bad = nullptr;
+  int *flags = nullptr, *derr = nullptr;
   Bump bp;
   auto layout = [&]() {
     bp.off = 0;
@@ -1190,7 +1241,6 @@ int shared_batch_run(const SharedBatchArgs& a, std::vector<SharedBatchResult>& o
     dinv = bp.take<DenseInst>(1);
     flags = bp.take<int>(8);
     derr = bp.take<int>(8);
-    bad = bp.take<int>(kMaxBatch);
     W2 = bp.take<double>((size_t)n * 2 * B);
     P2 = bp.take<double>((size_t)m * 2 * B);
     R = bp.take<double>((size_t)m * 2 * B);
@@ -1250,41 +1300,22 @@ int shared_batch_run(const SharedBatchArgs& a, std::vector<SharedBatchResult>& o
   cudaEventCreate(&e0);
   cudaEventCreate(&es);
   cudaEventCreate(&e1);
-  // b, c and the outputs may be device memory that work on the default stream (and on streams that
-  // it waits for) still fills or reads, and st waits for neither: that work ends first
+  // the outputs may be device memory that work on the default stream (and on streams that it waits
+  // for) still fills or reads, and st does not wait for it: that work ends first
   ck(cudaMemsetAsync(derr, 0, 8 * sizeof(int), 0), "memset");
   ck(cudaStreamSynchronize(0), "default stream");
   // ---- inputs: A (m x n FP64) and the per-instance vectors in [len x B] layout
-  // (each vector to a row of Xo, Yo, which are transposed and looked over on the device)
   if (a.A) ck(cudaMemcpyAsync(A64, a.A, (size_t)m * n * 8, cudaMemcpyHostToDevice, st), "upload A");
-  for (int k = 0; k < B; ++k) {
-    ck(cudaMemcpyAsync(Yo + (size_t)k * m, a.b[k], (size_t)m * 8, cudaMemcpyDefault, st), "upload b");
-    ck(cudaMemcpyAsync(Xo + (size_t)k * n, a.c[k], (size_t)n * 8, cudaMemcpyDefault, st), "upload c");
+  const double *bv = a.b, *cv = a.c;
+  if (a.vectors_on_host) {
+    ck(cudaMemcpyAsync(Yo, a.b, (size_t)m * B * 8, cudaMemcpyHostToDevice, st), "upload b");
+    ck(cudaMemcpyAsync(Xo, a.c, (size_t)n * B * 8, cudaMemcpyHostToDevice, st), "upload c");
+    bv = Yo;
+    cv = Xo;
   }
-  launch_transpose(Yo, B, m, V.b, st);
-  launch_transpose(Xo, B, n, V.c, st);
+  launch_transpose(bv, B, m, V.b, st);
+  launch_transpose(cv, B, n, V.c, st);
   ck(cudaMemsetAsync(flags, 0, 8 * sizeof(int), st), "memset");
-  ck(cudaMemsetAsync(bad, 0, kMaxBatch * sizeof(int), st), "memset");
-  finite_columns_kernel<<<eb, kThr, 0, st>>>(V.b, m, B, bad);
-  finite_columns_kernel<<<eb, kThr, 0, st>>>(V.c, n, B, bad);
-  {
-    int hbad[kMaxBatch] = {};
-    ck(cudaMemcpyAsync(hbad, bad, B * sizeof(int), cudaMemcpyDeviceToHost, st), "look");
-    ck(cudaStreamSynchronize(st), "upload");
-    for (int k = 0; k < B && rc == ABIP_OK; ++k)
-      if (hbad[k]) {
-        err = "instance " + std::to_string(a.first + k) + ": non-finite b or c";
-        rc = ABIP_E_INVALID_ARG;
-      }
-    if (rc != ABIP_OK) {
-      cudaEventDestroy(e0);
-      cudaEventDestroy(es);
-      cudaEventDestroy(e1);
-      cudaFree(arena);
-      if (owned) cudaStreamDestroy(owned);
-      return rc;
-    }
-  }
   cudaEventRecord(e0, st);
   // ---- setup (FP64): embedding constants (Eq. bar-b-c-z-re)
   rowsum_kernel<<<std::max(1, std::min(sms * 4, (m + 7) / 8)), kThr, 0, st>>>(A64, m, n, Ae);
