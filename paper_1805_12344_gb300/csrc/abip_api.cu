@@ -1605,14 +1605,6 @@ int abip_solve_batch_shared(int32_t count, const abip_matrix* A, const double* c
     rc = read_matrix_dense(&tmp, A, Ah);
     if (rc) return fail(nullptr, rc, tmp.err);
   }
-  abip::SharedVectors vec;
-  int bad = -1;
-  const cudaError_t ev = vec.read(count, m, n, b, c, static_cast<cudaStream_t>(stream), bad);
-  if (ev != cudaSuccess) {
-    cudaGetLastError();
-    return fail(nullptr, ev == cudaErrorMemoryAllocation ? ABIP_E_OOM : ABIP_E_CUDA, std::string("reading b, c: ") + cudaGetErrorString(ev));
-  }
-  if (bad >= 0) return fail(nullptr, ABIP_E_INVALID_ARG, "instance " + std::to_string(bad) + ": non-finite b or c");
   abip::ShParams sp{};
   sp.beta = prm.beta; sp.gamma = prm.gamma; sp.alpha = prm.alpha; sp.eps = prm.eps;
   sp.gamma_max = prm.gamma_max;
@@ -1633,6 +1625,14 @@ int abip_solve_batch_shared(int32_t count, const abip_matrix* A, const double* c
       return fail(nullptr, ABIP_E_INVALID_ARG, "ABIP_PREC_MIXED_BF16 needs A within the FP32 range");
     sp.tc = look & abip::SH_NOT_BF16 ? 3 : 1;
   }
+  abip::SharedVectors vec;
+  int bad = -1;
+  const cudaError_t ev = vec.read(count, m, n, b, c, static_cast<cudaStream_t>(stream), bad);
+  if (ev != cudaSuccess) {
+    cudaGetLastError();
+    return fail(nullptr, ev == cudaErrorMemoryAllocation ? ABIP_E_OOM : ABIP_E_CUDA, std::string("reading b, c: ") + cudaGetErrorString(ev));
+  }
+  if (bad >= 0) return fail(nullptr, ABIP_E_INVALID_ARG, "instance " + std::to_string(bad) + ": non-finite b or c");
   sp.n = n;
   sp.confirm_gap = std::max<int64_t>(prm.check_every, 20);
   sp.refresh = 192;   // a multiple of the 16-cycle groups of the shared-A solve loop

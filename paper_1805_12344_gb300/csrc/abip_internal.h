@@ -408,6 +408,9 @@ struct SharedVectors {
   ~SharedVectors();
   // b[k] (m) and c[k] (n), each host or device; bad: the first instance with a value that is not finite, or -1
   cudaError_t read(int count, int m, int n, const double* const* b, const double* const* c, cudaStream_t st, int& bad);
+
+ private:
+  cudaError_t read_host(int count, int m, int n, const double* const* b, const double* const* c, cudaStream_t st, int& bad);
 };
 
 // What the shared-A batch asks of its matrix (bits): an entry that is not finite, one beyond FP32's

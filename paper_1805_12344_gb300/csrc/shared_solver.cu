@@ -1125,47 +1125,66 @@ cudaError_t shared_read_matrix(const void* src, bool f32, int64_t ld, int m, int
 cudaError_t SharedVectors::read(int count, int m, int n, const double* const* b, const double* const* c, cudaStream_t st,
                                 int& bad) {
   const size_t nb = (size_t)count * m, nc = (size_t)count * n;
-  int* first = nullptr;
-  if (cudaMalloc(&dev, (nb + nc) * 8 + sizeof(int)) == cudaSuccess) {
-    first = reinterpret_cast<int*>(dev + nb + nc);
-  } else {
+  bad = count;
+  if (cudaMalloc(&dev, (nb + nc) * 8 + sizeof(int)) != cudaSuccess) {
     cudaGetLastError();
     dev = nullptr;
-    try {
-      host.resize(nb + nc);
-    } catch (const std::exception&) {
-      return cudaErrorMemoryAllocation;
-    }
+    on_host = true;
+    return read_host(count, m, n, b, c, st, bad);
   }
-  on_host = dev == nullptr;
-  double* to = on_host ? host.data() : dev;
-  this->b = to;
-  this->c = to + nb;
+  int* first = reinterpret_cast<int*>(dev + nb + nc);
+  this->b = dev;
+  this->c = dev + nb;
   // device inputs may still be filled by work on the default stream, which st need not wait for
   cudaError_t e = cudaStreamSynchronize(0);
   for (int k = 0; k < count && e == cudaSuccess; ++k) {
-    e = cudaMemcpyAsync(to + (size_t)k * m, b[k], (size_t)m * 8, cudaMemcpyDefault, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(to + nb + (size_t)k * n, c[k], (size_t)n * 8, cudaMemcpyDefault, st);
+    e = cudaMemcpyAsync(dev + (size_t)k * m, b[k], (size_t)m * 8, cudaMemcpyDefault, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(dev + nb + (size_t)k * n, c[k], (size_t)n * 8, cudaMemcpyDefault, st);
   }
-  bad = count;
-  if (!on_host) {
-    if (e == cudaSuccess) e = cudaMemcpyAsync(first, &bad, sizeof(int), cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) {
-      finite_rows_kernel<<<608, kThr, 0, st>>>(this->b, count, m, first);
-      finite_rows_kernel<<<608, kThr, 0, st>>>(this->c, count, n, first);
-      e = cudaGetLastError();
-    }
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&bad, first, sizeof(int), cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(first, &bad, sizeof(int), cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) {
+    finite_rows_kernel<<<608, kThr, 0, st>>>(this->b, count, m, first);
+    finite_rows_kernel<<<608, kThr, 0, st>>>(this->c, count, n, first);
+    e = cudaGetLastError();
   }
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&bad, first, sizeof(int), cudaMemcpyDeviceToHost, st);
   const cudaError_t es = cudaStreamSynchronize(st);
-  if (e == cudaSuccess) e = es;
-  if (on_host && e == cudaSuccess)
-    for (int k = 0; k < count && bad == count; ++k) {
-      for (int i = 0; i < m; ++i) if (!std::isfinite(this->b[(size_t)k * m + i])) bad = k;
-      for (int j = 0; j < n; ++j) if (!std::isfinite(this->c[(size_t)k * n + j])) bad = k;
-    }
   if (bad == count) bad = -1;
-  return e;
+  return e != cudaSuccess ? e : es;
+}
+
+// The same in host memory; of host vectors without a call to the device.
+cudaError_t SharedVectors::read_host(int count, int m, int n, const double* const* b, const double* const* c, cudaStream_t st,
+                                     int& bad) {
+  const size_t nb = (size_t)count * m;
+  try {
+    host.resize(nb + (size_t)count * n);
+  } catch (const std::exception&) {
+    return cudaErrorMemoryAllocation;
+  }
+  this->b = host.data();
+  this->c = host.data() + nb;
+  bad = -1;
+  auto take = [&](double* to, const double* from, int len, int k) -> cudaError_t {
+    cudaPointerAttributes at{};
+    if (cudaPointerGetAttributes(&at, from) == cudaSuccess && (at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged)) {
+      cudaError_t e = cudaStreamSynchronize(st);
+      if (e == cudaSuccess) e = cudaMemcpy(to, from, (size_t)len * 8, cudaMemcpyDefault);   // waits for the default stream
+      if (e != cudaSuccess) return e;
+    } else {
+      cudaGetLastError();
+      std::memcpy(to, from, (size_t)len * 8);
+    }
+    for (int i = 0; i < len && bad < 0; ++i)
+      if (!std::isfinite(to[i])) bad = k;
+    return cudaSuccess;
+  };
+  for (int k = 0; k < count; ++k) {
+    cudaError_t e = take(host.data() + (size_t)k * m, b[k], m, k);
+    if (e == cudaSuccess) e = take(host.data() + nb + (size_t)k * n, c[k], n, k);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 SharedVectors::~SharedVectors() {
