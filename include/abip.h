@@ -211,6 +211,9 @@ ABIP_API int abip_solve(abip_handle* h, double* x, double* y, double* s,
  * (on_device = 0) or device pointers (on_device = 1) per instance.  x, y, s:
  * arrays of `count` caller-allocated output pointers (same memory kind as the
  * inputs), entries may be NULL.  infos: `count` entries, may be NULL.
+ * An instance's result does not depend on the others: the bits are those of abip_setup and
+ * abip_solve on it alone.  (FP64 where the device has no room for another 8 m n + 16 m^2
+ * bytes per instance beside the data: another kernel, other last bits.)
  * Each instance needs 40m + 24n bytes (FP64) or 48m + 40n bytes (mixed) of shared
  * memory, at most 200 KB (ABIP_E_UNSUPPORTED otherwise); larger LPs go through
  * abip_setup with linsys = PCG.

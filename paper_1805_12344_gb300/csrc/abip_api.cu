@@ -526,6 +526,7 @@ int dense_alloc(abip_handle* h, const std::vector<DenseHostInst>& hi, void** are
       const int m = hi[k].m, n = hi[k].n;
       DenseInst& I = d[k];
       I.m = m; I.n = n;
+      I.parts = abip::dense_parts(m, n);
       const bool f64 = group && !mixed;   // the FP64 group kernel's copies
       I.ld = f64 ? n + (n & 1) : n;
       I.A = ar.take<double>((size_t)m * I.ld);
@@ -550,7 +551,7 @@ int dense_alloc(abip_handle* h, const std::vector<DenseHostInst>& hi, void** are
       }
     }
     if (group && !mixed && count == 1) {
-      h->gscratch_len = abip::dense_group_scratch(hi[0].m, hi[0].n, abip::dense_max_ctas(h->device));
+      h->gscratch_len = abip::dense_group_scratch(hi[0].m, hi[0].n);
       h->gscratch = ar.take<double>(h->gscratch_len);
     }
   };
@@ -631,18 +632,18 @@ DenseParams dense_params(const abip_params& p) {
 }
 
 // CTAs per instance, and the hand-out order (ord, for a batch): by CTAs, then largest first (m n +
-// m^2) or, without `largest_first`, as given.  An instance's CTAs do not depend on the order.
+// m^2) or, without `largest_first`, as given.  An instance's CTAs do not depend on the order, and
+// its result does not depend on its CTAs (the sums' order is the LP's own).
 //
 // One LP: a cluster while a CTA keeps more than kClusterWork operations (of 2 per clock, the
-// FP64 rate: 2.5k clocks, about what an update's barriers cost), and in FP64 the whole grid from
-// 8e5 operations on, where its 152 SMs outweigh its dearer barriers (us per update, cluster of
-// 16 / grid: 200 x 600 20.6 / 23.7, 256 x 1024 25.2 / 24.2, 512 x 1154 50.7 / 26.4).
+// FP64 rate: 2.5k clocks, about what an update's barriers cost), and in FP64 a grid of 144 CTAs from
+// kGridWork operations on, where their SMs outweigh the dearer barriers (us per update, cluster of
+// 16 / grid: 200 x 600 19 / 24, 256 x 1024 29 / 20, 300 x 900 34 / 21, 512 x 1154 57 / 22).
 // A batch: by work too, with the share chosen so that the CTAs of all instances are about two
 // per SM (FP64, 64 LPs of m 16 .. 256, 200 updates: 14.4 ms; 1 per SM 17.2, 3 15.4; the same
-// size for all 48 / 26 / 23 / 12.6 ms with 1 / 2 / 4 / 8; 128 LPs 24.8, 61 / 49 / 25 / 26).  The time of a batch is that of its slowest instance, so the large ones get the
-// CTAs; instances of one cluster size form a bucket, and the buckets' launches run side by
-// side.  A batch of more instances than that is one bucket of single CTAs.
-constexpr double kClusterWork = 5000.0;
+// size for all 48 / 26 / 23 / 12.6 ms with 1 / 2 / 4 / 8; 128 LPs 24.8, 61 / 49 / 25 / 26).  The time
+// of a batch is that of its slowest instance, so the large ones get the CTAs; instances of one
+// cluster size form a bucket, and the buckets' launches run side by side.  A batch of more instances than that is one bucket of single CTAs.
 bool plan_buckets(abip_handle* h, const std::vector<std::pair<int, int>>& sizes, bool largest_first, bool mixed, int sms,
                   std::vector<int>& ord) {
   const int count = (int)sizes.size();
@@ -651,30 +652,25 @@ bool plan_buckets(abip_handle* h, const std::vector<std::pair<int, int>>& sizes,
     const double mm = sizes[k].first, nn = sizes[k].second;
     // mixed: 16 m n + 4 m^2 bytes of matrices at 64 bytes per clock from L2, beside the steps and sums
     work[k] = mixed ? (12.0 * mm * nn + 4.0 * mm * mm) / 32.0 + 60.0 * mm + 90.0 * nn
-                    : 3.0 * mm * nn + mm * mm + 80.0 * (mm + nn);
+                    : abip::dense_work(sizes[k].first, sizes[k].second);
   }
   h->buckets.clear();
-  if (!mixed && count == 1 && work[0] > 8e5) {
+  if (!mixed && count == 1 && work[0] > abip::kGridWork) {
     abip::DenseBucket b{{}, 0, 1};
     if (abip::plan_dense_grid(sizes[0].first, sizes[0].second, sms, b.plan)) {
       h->buckets.push_back(b);
       return true;
     }
   }
-  auto ctas = [](double w, double share) {
-    int C = 1;
-    while (C < 16 && w / C > share) C *= 2;
-    return C;
-  };
-  double share = kClusterWork;
+  double share = abip::kClusterWork;
   int64_t total = 0;
   for (;; share *= 1.2) {
     total = 0;
-    for (int k = 0; k < count; ++k) total += ctas(work[k], share);
+    for (int k = 0; k < count; ++k) total += abip::cluster_ctas(work[k], share);
     if (total <= 2 * (int64_t)sms || total == count) break;
   }
   std::vector<int> C(count), m(count), n(count);
-  for (int k = 0; k < count; ++k) C[k] = ctas(work[k], share);
+  for (int k = 0; k < count; ++k) C[k] = abip::cluster_ctas(work[k], share);
   ord.resize(count);
   for (int k = 0; k < count; ++k) ord[k] = k;
   std::stable_sort(ord.begin(), ord.end(), [&](int a, int b) {
@@ -794,13 +790,14 @@ void setup_direct(abip_handle* h, const HostCSR& A) {
   const int sms = abip::dense_max_ctas(h->device);
   abip::DenseGroupPlan plan;
   abip::GroupSparse sp;
-  if (!abip::plan_sparse_group(m, n, rp.data(), cp.data(), sms, sp, plan)) return;
+  int parts = 1;
+  if (!abip::plan_sparse_group(m, n, rp.data(), cp.data(), sms, sp, plan, parts)) return;
   struct { int32_t *rp, *ci, *cp, *ri; double *va, *cv; } d;
   DenseInst I{};
   DenseInst* dinst = nullptr;
   int* queue = nullptr;
   double* scratch = nullptr;
-  const size_t scratch_len = abip::dense_group_scratch(m, n, sms);
+  const size_t scratch_len = abip::dense_group_scratch(m, n);
   auto layout = [&](Arena& ar) {
     dinst = ar.take<DenseInst>(1);
     queue = ar.take<int>(abip::kDenseBuckets);
@@ -839,6 +836,7 @@ void setup_direct(abip_handle* h, const HostCSR& A) {
   SolveCtl hc;
   up(&hc, h->ctl, sizeof(hc), cudaMemcpyDeviceToHost);
   I.m = m; I.n = n; I.ld = n;
+  I.parts = parts;
   I.b = g.b; I.c = g.c; I.bbar = g.bbar; I.cbar = g.cbar;
   I.y = g.y; I.x = g.x; I.s = g.s;
   I.out_x = h->stage; I.out_y = h->stage + n; I.out_s = h->stage + n + m;

@@ -202,6 +202,7 @@ struct DenseInst {
   // FP64 path by a group of CTAs (null elsewhere): A^T (n rows), L^{-1} and L^{-T} (m rows
   // each), rows padded with zeros to an even length; A's ld is even then
   double* AT; double* Li; double* LiT;
+  int parts;                   // parts of the group kernel's sums (dense_parts)
   double* Ginv;                // the explicit inverse of G (m x m), shared-A batch only
   double zbar, nb, nc;
   double Kinv[4];
@@ -294,6 +295,18 @@ struct DenseGroupPlan {
   size_t smem;
   int sparse;                // 1: products with A over its CSR rows and columns (GroupSparse)
 };
+// Multiply-adds of one FP64 update, 80 for the steps and sums of a row or column; the CTAs that an LP of
+// such work is worth when each keeps more than `share`: up to 16, a power of two.
+inline double dense_work(int m, int n) { return 3.0 * m * n + (double)m * m + 80.0 * ((double)m + n); }
+inline int cluster_ctas(double work, double share) {
+  int C = 1;
+  while (C < 16 && work / C > share) C *= 2;
+  return C;
+}
+constexpr double kClusterWork = 5000.0;   // least share of a CTA in a cluster
+constexpr double kGridWork = 8e5;         // one LP above it takes the whole grid (FP64)
+// parts of an LP's sums: cluster_ctas at the least share, so that every cluster size divides them
+int dense_parts(int m, int n);
 // the plan of one LP over the cooperative grid, and of `count` LPs by clusters of C CTAs (more
 // where their vectors do not fit); 0 if no group holds the vectors in shared memory.  budget:
 // bytes of shared memory that copies of matrices and vectors may fill
@@ -305,10 +318,11 @@ int plan_dense_cluster(const int* m, const int* n, int count, int C, size_t budg
 // and a setup that grows by m^3 / 3 multiply-adds (1599: 24 ms more).
 constexpr int kDirectMaxRows = 1600;
 // the plan for one sparse LP (host rp, cp); 0 where the sweeps serve it
-int plan_sparse_group(int m, int n, const int32_t* rp, const int32_t* cp, int sms, GroupSparse& sp, DenseGroupPlan& plan);
+int plan_sparse_group(int m, int n, const int32_t* rp, const int32_t* cp, int sms, GroupSparse& sp, DenseGroupPlan& plan,
+                      int& parts);
 // doubles of scratch of the grid mode; its last two are the barrier counter and the error
 // word, zeroed by the caller before each launch
-size_t dense_group_scratch(int m, int n, int sms);
+size_t dense_group_scratch(int m, int n);
 cudaError_t launch_dense_group(DenseInst* inst, int count, const DenseParams& prm, int* queue, const int* order,
                                const DenseGroupPlan& plan, const GroupSparse& sp, int variant, double* scratch,
                                size_t scratch_len, unsigned long long limit_ns, cudaStream_t st);

@@ -28,7 +28,7 @@
 // One update has four barriers of the group: products and all sums | t | z_y | x, s.
 // Measured, us per update, one CTA with triangular sweeps -> this kernel: 50 x 120 76.9 -> 9.8
 // (the chain of dependent FP64 operations: about 100 clocks each, four barriers of 500),
-// 512 x 1154 1564 -> 20 over the grid, the slowest of 64 LPs of m 16 .. 256 621 -> 60.
+// 512 x 1154 1564 -> 22 over the grid, the slowest of 64 LPs of m 16 .. 256 621 -> 60.
 #include <algorithm>
 
 #include <cooperative_groups.h>
@@ -46,6 +46,27 @@ using dense::kWarps;
 using dense::sum_together;
 constexpr int kThr = dense::kThreads;
 constexpr int kSums = 11;   // the nine of the tests and the two of H^T z
+
+// The order of the sums over rows and columns follows from the LP alone, whatever group solves it, so
+// that its bits do not follow the batch it is in.  The LP has P parts (DenseInst::parts, the most CTAs
+// that its work is worth in a cluster) of nine cells each: runs of rows and of columns.  A cell's sums
+// are chains in order, a part's nine are joined by a fixed tree and the parts by another.  A CTA owns
+// whole parts or, in the grid, a cell: 144 is the largest count up to the chip's 152 SMs that 16
+// parts divide.  Against sums in the order of the CTAs' own elements, us per update: 50 x 120 9.9 -> 9.8,
+// 512 x 1154 22.3 -> 22.1, 16 x 16 grid flow 11.5 -> 11.4; 32 x 32 and 39 x 39 on 144 CTAs instead of
+// 152 21.7 -> 22.6 and 27.8 -> 30.2.
+constexpr int kPerPart = 9, kMaxParts = 16;
+constexpr int kGridCtas = kPerPart * kMaxParts;
+// the first of `len` elements that rank r of a group of `size` owns; ranks past the parts own none
+__host__ __device__ __forceinline__ int own_start(int r, int size, int parts, bool grid, int len) {
+  const int C = grid ? kGridCtas : size < parts ? size : parts;
+  return (int)((int64_t)(r < C ? r : C) * len / C);
+}
+// most elements that a CTA owns
+__host__ __device__ __forceinline__ int own_room(int size, int parts, bool grid, int len) {
+  const int C = grid ? kGridCtas : size < parts ? size : parts;
+  return (len + C - 1) / C;
+}
 
 enum Act : int { ACT_STEP = 0, ACT_WARM = 1, ACT_STOP = 2 };
 
@@ -117,7 +138,7 @@ __device__ __forceinline__ void tri_dots(const double* M, int64_t stride, int ro
       a[u] = 0.0;
       r[u] = reinterpret_cast<const double2*>(M + (size_t)min(g + u, rows - 1) * stride);
     }
-    const int t0 = LOWER ? 0 : (rank + size * g) >> 1;
+    const int t0 = LOWER ? 0 : ((rank + size * g) >> 1) & ~31;   // a lane sums the same pairs in every group
     const int t1 = LOWER ? ((rank + size * min(g + R - 1, rows - 1)) >> 1) + 1 : nq;
 #pragma unroll(R >= 4 ? 1 : 4)
     for (int t = t0 + lane; t < t1; t += 32) {
@@ -184,14 +205,22 @@ struct Group {
   }
 };
 
+// a b + c d with the second product rounded: where two products meet, which of them a compiler
+// fuses would differ between the kernels below, and with it the bits
+__device__ __forceinline__ double two_products(double a, double b, double c, double d) {
+  return __fma_rn(a, b, __dmul_rn(c, d));
+}
+
 // barrier_step with the square root and the quotient refined from FP32 estimates: one coupled
 // step and a residual step each leave about 1e-16 relative, in half the dependent operations of
 // the library's (an update's critical path holds this chain).  Outside the FP32 range of the
 // discriminant, the closed form.
 __device__ __forceinline__ void barrier_step_fast(double omega, double c, double& x, double& s) {
-  const double disc = omega * omega + 4.0 * c;
+  const double disc = __fma_rn(omega, omega, 4.0 * c);
   if (!(disc > 1e-30 && disc < 1e30)) {
-    barrier_step<double>(omega, c, x, s);
+    const double L = 0.5 * (fabs(omega) + sqrt(disc)), small = c / L;
+    x = omega >= 0.0 ? L : small;
+    s = omega >= 0.0 ? small : L;
     return;
   }
   float r;
@@ -235,56 +264,55 @@ struct Scal {
   double a[kSums];   // the sums
 };
 
-// The block's sums of NS values per thread (only the first `act` warps hold any), published
-// in the partial slots of every CTA: slots[r * NS + k] is CTA r's sum k.
-template <int NS, bool GRID>
-__device__ __forceinline__ void publish_sums(const Group<GRID>& G, double (&acc)[16], int act, double* wsum, double* slots,
-                                             double* gslots) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (wid < act) {
-    const double v = sum_together<16>(acc, lane);
-    const int k = lane >> 1;
-    if ((lane & 1) == 0 && k < NS) wsum[k * kWarps + wid] = v;
-  }
-  __syncthreads();
+// the sum of a part's nine cells
+__device__ __forceinline__ double part_tree(const double (&v)[kPerPart]) {
+  return (((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]))) + v[8];
+}
+
+// The CTA's part sums, from its cells' (cs: [sum][cell], `cells` of them), into the slots of every CTA
+// of the cluster, [part][sum]; in a grid the CTA's one cell into the L2, [part / 2][cell][sum][part % 2].
+template <bool GRID>
+__device__ __forceinline__ void publish_sums(const Group<GRID>& G, const double* cs, int cells, double* slots, double* gslots) {
   if constexpr (GRID) {
-    if (threadIdx.x < NS) {
-      double v = wsum[threadIdx.x * kWarps];
-      for (int w = 1; w < act; ++w) v += wsum[threadIdx.x * kWarps + w];
-      __stcg(gslots + (size_t)threadIdx.x * G.size + G.rank, v);
-    }
+    const int p = G.rank / kPerPart, i = G.rank % kPerPart, k = threadIdx.x;
+    if (k < kSums) __stcg(gslots + ((p >> 1) * kPerPart + i) * 2 * kSums + 2 * k + (p & 1), cs[k]);
   } else {
+    const int parts = cells / kPerPart, t = threadIdx.x;
+    if (t >= parts * kSums) return;
+    const int k = t % kSums, pl = t / kSums;
+    double v[kPerPart];
+#pragma unroll
+    for (int i = 0; i < kPerPart; ++i) v[i] = cs[k * cells + pl * kPerPart + i];
+    const double sum = part_tree(v);
+    double* at = slots + (G.rank * parts + pl) * kSums + k;
     const cg::cluster_group cl = cg::this_cluster();
-    for (int t = threadIdx.x; t < NS * G.size; t += kThr) {
-      const int k = t % NS, r = t / NS;
-      double v = wsum[k * kWarps];
-      for (int w = 1; w < act; ++w) v += wsum[k * kWarps + w];
-      *cl.map_shared_rank(slots + G.rank * NS + k, r) = v;
-    }
+    for (int r = 0; r < G.size; ++r) *cl.map_shared_rank(at, r) = sum;
   }
 }
 
-// After the barrier: the NS totals into out (shared), by warp 0, in the same order in every CTA.
-template <int NS, bool GRID>
-__device__ __forceinline__ void total_sums(const Group<GRID>& G, const double* slots, const double* gslots, double* out) {
-  const int lane = threadIdx.x & 31;
+// After the barrier: the totals into out (shared), by warp 0, in the same order in every CTA.
+template <bool GRID>
+__device__ __forceinline__ void total_sums(const double* slots, const double* gslots, int parts, double* out) {
+  const int lane = threadIdx.x & 31, k = lane >> 1, h = lane & 1;
+  double p[kMaxParts / 2];   // parts h, h + 2, ..., 0 beyond the last
   if constexpr (GRID) {
-    double v[16];
 #pragma unroll
-    for (int k = 0; k < 16; ++k) v[k] = 0.0;
-    for (int i = lane; i < G.size; i += 32)
+    for (int q0 = 0; q0 < kMaxParts / 2; q0 += 4) {   // 36 loads in flight
+      double v[4][kPerPart];
 #pragma unroll
-      for (int k = 0; k < NS; ++k) v[k] += __ldcg(gslots + (size_t)k * G.size + i);
-    const double s = sum_together<16>(v, lane);
-    if ((lane & 1) == 0 && (lane >> 1) < NS) out[lane >> 1] = s;
+      for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int i = 0; i < kPerPart; ++i) v[q][i] = k < kSums ? __ldcg(gslots + ((q0 + q) * kPerPart + i) * 2 * kSums + lane) : 0.0;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) p[q0 + q] = part_tree(v[q]);
+    }
   } else {
-    const int k = lane >> 1, h = lane & 1;
-    double v = 0.0;
-    if (k < NS)
-      for (int r = h; r < G.size; r += 2) v += slots[r * NS + k];
-    v += __shfl_xor_sync(0xffffffffu, v, 1);
-    if (h == 0 && k < NS) out[k] = v;
+#pragma unroll
+    for (int q = 0; q < kMaxParts / 2; ++q) p[q] = k < kSums && 2 * q + h < parts ? slots[(2 * q + h) * kSums + k] : 0.0;
   }
+  double v = ((p[0] + p[1]) + (p[2] + p[3])) + ((p[4] + p[5]) + (p[6] + p[7]));
+  v += __shfl_xor_sync(0xffffffffu, v, 1);
+  if (h == 0 && k < kSums) out[k] = v;
   __syncwarp();
 }
 
@@ -328,27 +356,36 @@ __device__ __forceinline__ void sparse_cols(const int32_t* cp, const int32_t* ri
 
 // Algorithm 2 (with the relaxation of Sec. 4.2) for one instance by the group.
 template <bool GRID, bool SPARSE>
-__device__ void solve_one(DenseInst& I, const GroupArgs& Q, Group<GRID>& G, double* sm, double* wsum, Scal& S) {
+__device__ void solve_one(DenseInst& I, const GroupArgs& Q, Group<GRID>& G, double* sm, Scal& S) {
   const DenseParams& P = Q.P;
   const int m = I.m, n = I.n, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int mp = even(m), np = even(n);
-  const int mc = (m + G.size - 1) / G.size, nc_ = (n + G.size - 1) / G.size;
-  const int i0 = min(m, G.rank * mc), mr = min(m, i0 + mc) - i0;   // this CTA's rows
-  const int j0 = min(n, G.rank * nc_), nr = min(n, j0 + nc_) - j0; // this CTA's columns
+  const int parts = I.parts;
+  const int mc = own_room(G.size, parts, GRID, m), nc_ = own_room(G.size, parts, GRID, n);
+  const int i0 = own_start(G.rank, G.size, parts, GRID, m), mr = own_start(G.rank + 1, G.size, parts, GRID, m) - i0;   // its rows
+  const int j0 = own_start(G.rank, G.size, parts, GRID, n), nr = own_start(G.rank + 1, G.size, parts, GRID, n) - j0;   // columns
+  const int most = GRID ? 1 : kPerPart * (parts / min(G.size, parts));   // cells of a CTA that owns any
+  const int cells = GRID || G.rank < parts ? most : 0;
   double* q = sm;
   double* tv = q + mp;
   double* zy = tv + mp;
   double* x = zy + mp;
   double* s = x + np;
-  double* rslot = s + np;                               // kSums * size
-  double* y = rslot + kSums * (GRID ? 1 : G.size);      // own rows
+  double* rslot = s + np;                               // the parts' sums (a grid's lie in the L2)
+  double* cs = rslot + (GRID ? 0 : kSums * kMaxParts);  // the cells' sums
+  int* ct = reinterpret_cast<int*>(cs + kSums * most);
+  int* rt = ct + most + 1;
+  double* y = cs + (kSums + 1) * most + 1;              // own rows
   double* Ax = y + mc;
   double* As = Ax + mc;
   double* k1y = As + mc;                                // M^{-T} h1, M^{-T} h2
   double* k2y = k1y + mc;
   double* aty = k2y + mc;                               // own columns
   double* v = aty + nc_;
-  double* k1x = v + nc_;
+  double* rx = v + nc_;                                 // factors of the sums; of w = x + s in v, of the
+  double* dr = rx + nc_;                                // rows in the idle t and z_y
+  double* as = dr + nc_;
+  double* k1x = as + nc_;
   double* k2x = k1x + nc_;
   double* top = k2x + nc_;
   double* gq = Q.gvec;
@@ -466,7 +503,14 @@ __device__ void solve_one(DenseInst& I, const GroupArgs& Q, Group<GRID>& G, doub
     return true;
   };
   const int rows0 = (nr + 31) & ~31;   // the CTA's rows start at a warp of their own
-  const int items = rows0 + mr, act = min(kWarps, max(1, (items + 31) / 32));
+  const int items = rows0 + mr;
+  // where each cell of this CTA begins among its columns (ct) and rows, and after the last its end
+  for (int k = threadIdx.x; k <= cells; k += kThr) {
+    const int64_t at = GRID ? G.rank + k : kPerPart * (G.rank * (parts / min(G.size, parts))) + k;
+    ct[k] = (int)(at * n / (kPerPart * parts)) - j0;
+    rt[k] = (int)(at * m / (kPerPart * parts)) - i0;
+  }
+  const int inv_cells = (1 << 20) / max(cells, 1) + 1;   // t / cells = t inv_cells >> 20 for t < kSums cells <= 1584
   if (!G.sync()) return;   // nobody publishes into a CTA that is still filling its copies
   // M^{-T} h = J M^{-1} J h, J = diag(I, -I): for h = [a; d], G g = a + A d and
   // M^{-T} h = [g; d - A^T g].  The columns d of h1 and h2 stand in x and s meanwhile.
@@ -506,33 +550,50 @@ __device__ void solve_one(DenseInst& I, const GroupArgs& Q, Group<GRID>& G, doub
   for (;;) {
     // ---- the sums over the columns, the products A x, A s, the sums over the rows, and q
     {
-      double acc[16];
-#pragma unroll
-      for (int k = 0; k < 16; ++k) acc[k] = 0.0;
       const double ta = S.tau, th = S.theta, it = S.itau;
+      double *ry = tv, *pr = zy;
       for (int e = threadIdx.x; e < nr; e += kThr) {
-        const double at = aty[e], sj = s[j0 + e], cj = c[e], cb = cbar[e], xj = x[j0 + e];
-        const double as = at + sj, w = xj + sj;
-        const double rx = cj * ta - cb * th - as;
-        const double dr = as * it - cj;
-        acc[0] += rx * rx; acc[2] += dr * dr; acc[4] += as * as;
-        acc[7] += cj * xj; acc[8] += cb * xj;
-        acc[9] += k1x[e] * w; acc[10] += k2x[e] * w;
+        const double at = aty[e], sj = s[j0 + e], cj = c[e];
+        const double a = at + sj;
+        rx[e] = two_products(cj, ta, -cbar[e], th) - a;
+        dr[e] = a * it - cj;
+        as[e] = a;
+        v[e] = x[j0 + e] + sj;
       }
       rows_A(x, s, [&](int w, int i, double d) { (w == 0 ? Ax : As)[i] = d; });
       __syncthreads();
-      for (int e = threadIdx.x; e < items; e += kThr) {
-        if (e < rows0) continue;
-        const int i = e - rows0;
-        const double ax = Ax[i], bi = b[i], bb = bbar[i], yi = y[i];
-        G.put(q, gq, i0 + i, yi - (ax + As[i]));
-        const double ry = ax - bi * ta + bb * th;
-        const double pr = ax * it - bi;
-        acc[0] += ry * ry; acc[1] += pr * pr; acc[3] += ax * ax;
-        acc[5] += bi * yi; acc[6] += bb * yi;
-        acc[9] += k1y[i] * yi; acc[10] += k2y[i] * yi;
+      for (int i = threadIdx.x; i < mr; i += kThr) {
+        const double ax = Ax[i], bi = b[i];
+        G.put(q, gq, i0 + i, y[i] - (ax + As[i]));
+        ry[i] = ax - bi * ta + bbar[i] * th;
+        pr[i] = ax * it - bi;
       }
-      publish_sums<kSums, GRID>(G, acc, act, wsum, rslot, grs);
+      __syncthreads();
+      for (int t = threadIdx.x; t < kSums * cells; t += kThr) {   // a chain: sum k over a cell's columns, then its rows
+        const int k = t * inv_cells >> 20, cell = t - k * cells;
+        const double *pc = nullptr, *qc = nullptr, *p = nullptr, *pq = nullptr;
+        switch (k) {
+          case 0: pc = qc = rx; p = pq = ry; break;
+          case 1: p = pq = pr; break;
+          case 2: pc = qc = dr; break;
+          case 3: p = pq = Ax; break;
+          case 4: pc = qc = as; break;
+          case 5: p = b; pq = y; break;
+          case 6: p = bbar; pq = y; break;
+          case 7: pc = c; qc = x + j0; break;
+          case 8: pc = cbar; qc = x + j0; break;
+          case 9: pc = k1x; qc = v; p = k1y; pq = y; break;
+          default: pc = k2x; qc = v; p = k2y; pq = y; break;
+        }
+        double acc = 0.0;
+        if (pc)
+          for (int e = ct[cell]; e < ct[cell + 1]; ++e) acc += pc[e] * qc[e];
+        if (p)
+          for (int i = rt[cell]; i < rt[cell + 1]; ++i) acc += p[i] * pq[i];
+        cs[t] = acc;
+      }
+      __syncthreads();
+      publish_sums<GRID>(G, cs, cells, rslot, grs);
     }
     if (!G.sync()) return;
     G.fetch(q, gq, m);
@@ -540,7 +601,7 @@ __device__ void solve_one(DenseInst& I, const GroupArgs& Q, Group<GRID>& G, doub
     // ---- projection: z_y = G^{-1} (y - A (x + s)), beside it the decision on the sums and
     // t = K^{-1} (w_{tau,theta} + H^T z)
     auto decide = [&] {
-      total_sums<kSums, GRID>(G, rslot, grs, S.a);
+      total_sums<GRID>(rslot, grs, parts, S.a);
       if (lane != 0) return;
       const double* a = S.a;
       const double tau = S.tau;
@@ -591,8 +652,8 @@ __device__ void solve_one(DenseInst& I, const GroupArgs& Q, Group<GRID>& G, doub
     auto scalars = [&] {
       if (lane != 0) return;
       const double v1 = S.tau + S.kappa + S.a[9], v2 = S.theta + xi + S.a[10];
-      S.t1 = Ki0 * v1 + Ki1 * v2;
-      S.t2 = Ki2 * v1 + Ki3 * v2;
+      S.t1 = two_products(Ki0, v1, Ki1, v2);
+      S.t2 = two_products(Ki2, v1, Ki3, v2);
       S.cmu = S.mu / P.beta;
     };
     if (!solve_G(decide, scalars)) return;
@@ -623,12 +684,12 @@ __device__ void solve_one(DenseInst& I, const GroupArgs& Q, Group<GRID>& G, doub
     // linearity; the step of tau, kappa and theta on the first warp
     const double t1 = S.t1, t2 = S.t2, cmu = S.cmu;
     if (threadIdx.x == 0) {
-      const double th = alpha * t1 + a1 * S.tau;
+      const double th = two_products(alpha, t1, a1, S.tau);
       double tn, kn;
       barrier_step_fast(th - S.kappa, cmu, tn, kn);
       S.tau = tn;
       S.kappa = kn;
-      S.theta = alpha * t2 + a1 * S.theta;
+      S.theta = two_products(alpha, t2, a1, S.theta);
       S.itau = 1.0 / tn;
     }
     if constexpr (SPARSE) sparse_cols<1>(cp, ri, cv, nr, zy, [&](int j, double d) { v[j] = d; });
@@ -640,16 +701,16 @@ __device__ void solve_one(DenseInst& I, const GroupArgs& Q, Group<GRID>& G, doub
         const double x0 = x[j], s0 = s[j], vj = v[e];
         const double gx1 = g1x[e], gx2 = g2x[e];
         // A^T g1y = g1x - c and A^T g2y = g2x + cbar (M g = h)
-        aty[e] = alpha * (vj - (gx1 - c[e]) * t1 - (gx2 + cbar[e]) * t2) + a1 * aty[e];
+        aty[e] = two_products(alpha, vj - (gx1 - c[e]) * t1 - (gx2 + cbar[e]) * t2, a1, aty[e]);
         const double ux = x0 + s0 + vj - gx1 * t1 - gx2 * t2;
         double xn, sn;
-        barrier_step_fast(alpha * ux + a1 * x0 - s0, cmu, xn, sn);
+        barrier_step_fast(two_products(alpha, ux, a1, x0) - s0, cmu, xn, sn);
         G.put(x, gx, j, xn);
         G.put(s, gs, j, sn);
       } else if (e >= rows0) {
         const int i = e - rows0;
         const double uy = zy[i0 + i] - g1y[i] * t1 - g2y[i] * t2;
-        y[i] = alpha * uy + a1 * y[i];
+        y[i] = two_products(alpha, uy, a1, y[i]);
       }
     }
     if (!G.sync()) return;
@@ -693,7 +754,6 @@ __device__ void solve_one(DenseInst& I, const GroupArgs& Q, Group<GRID>& G, doub
 template <int MINB, bool SPARSE>
 __global__ void __launch_bounds__(kThr, MINB) dense_cluster_kernel(GroupArgs Q) {
   extern __shared__ __align__(16) double sm[];
-  __shared__ double wsum[kSums * kWarps];
   __shared__ Scal S;
   __shared__ int s_id;
   cg::cluster_group cl = cg::this_cluster();
@@ -709,7 +769,7 @@ __global__ void __launch_bounds__(kThr, MINB) dense_cluster_kernel(GroupArgs Q) 
     const int id = s_id;
     if (id < 0) return;   // the same in every CTA, after which none writes to another
     DenseInst& I = Q.insts[id];
-    if (I.err == 0) solve_one<false, SPARSE>(I, Q, G, sm, wsum, S);
+    if (I.err == 0) solve_one<false, SPARSE>(I, Q, G, sm, S);
     cl.sync();            // every CTA has read s_id and its copies
   }
 }
@@ -717,10 +777,9 @@ __global__ void __launch_bounds__(kThr, MINB) dense_cluster_kernel(GroupArgs Q) 
 template <bool SPARSE>
 __global__ void __launch_bounds__(kThr, 1) dense_grid_kernel(GroupArgs Q) {
   extern __shared__ __align__(16) double sm[];
-  __shared__ double wsum[kSums * kWarps];
   __shared__ Scal S;
   Group<true> G(GridBarrier{Q.bar, Q.err, Q.bar_limit_ns});
-  if (Q.insts[0].err == 0) solve_one<true, SPARSE>(Q.insts[0], Q, G, sm, wsum, S);
+  if (Q.insts[0].err == 0) solve_one<true, SPARSE>(Q.insts[0], Q, G, sm, S);
 }
 
 using ClusterFn = void (*)(GroupArgs);
@@ -737,30 +796,34 @@ struct SmemPlan {
   int cache_vec, cache_mat;
 };
 
-size_t base_doubles(int m, int n, int C, bool grid) {
-  const size_t mp = (m + 1) / 2 * 2, np = (n + 1) / 2 * 2, mc = (m + C - 1) / C, nc = (n + C - 1) / C;
-  return 3 * mp + 2 * np + kSums * (size_t)(grid ? 1 : C) + 5 * mc + 4 * nc;
+size_t base_doubles(int m, int n, int C, int parts, bool grid) {
+  const size_t mp = (m + 1) / 2 * 2, np = (n + 1) / 2 * 2, mc = own_room(C, parts, grid, m), nc = own_room(C, parts, grid, n);
+  const size_t cells = grid ? 1 : kPerPart * (parts / std::min(C, parts));
+  const size_t sums = (grid ? 0 : kSums * kMaxParts) + (kSums + 1) * cells + 1;
+  return 3 * mp + 2 * np + sums + 5 * mc + 7 * nc;
 }
-size_t vec_doubles(int m, int n, int C) { return 4 * (size_t)((m + C - 1) / C) + 4 * (size_t)((n + C - 1) / C) + 2; }
-size_t mat_doubles(int m, int n, int C) {
-  const size_t mp = (m + 1) / 2 * 2, np = (n + 1) / 2 * 2, mc = (m + C - 1) / C, nc = (n + C - 1) / C;
+size_t vec_doubles(size_t mc, size_t nc) { return 4 * mc + 4 * nc + 2; }
+size_t mat_doubles(int m, int n, size_t mc, size_t nc) {
+  const size_t mp = (m + 1) / 2 * 2, np = (n + 1) / 2 * 2;
   return mc * (np + 2 * mp) + nc * mp + 2;
 }
 
-size_t sparse_doubles(int m, int n, int C, int room_a, int room_at) {
-  const size_t mp = (m + 1) / 2 * 2, mc = (m + C - 1) / C, nc = (n + C - 1) / C;
+size_t sparse_doubles(int m, size_t mc, size_t nc, int room_a, int room_at) {
+  const size_t mp = (m + 1) / 2 * 2;
   return 2 * mc * mp + 2 + room_a + (room_a + mc + 2) / 2 + room_at + (room_at + nc + 2) / 2;
 }
 
 // the shared memory of a launch for the given sizes: the copies that fit the budget
 SmemPlan plan_smem(const int* m, const int* n, int count, int C, bool grid, size_t budget,
-                   const GroupSparse* sp = nullptr) {
+                   const GroupSparse* sp = nullptr, int sp_parts = 0) {
   size_t base = 0, vec = 0, mat = 0;
   for (int k = 0; k < count; ++k) {
-    const size_t b = base_doubles(m[k], n[k], C, grid), v = b + vec_doubles(m[k], n[k], C);
+    const int parts = sp ? sp_parts : dense_parts(m[k], n[k]);
+    const size_t mc = own_room(C, parts, grid, m[k]), nc = own_room(C, parts, grid, n[k]);
+    const size_t b = base_doubles(m[k], n[k], C, parts, grid), v = b + vec_doubles(mc, nc);
     base = std::max(base, b);
     vec = std::max(vec, v);
-    mat = std::max(mat, v + (sp ? sparse_doubles(m[k], n[k], C, sp->room_a, sp->room_at) : mat_doubles(m[k], n[k], C)));
+    mat = std::max(mat, v + (sp ? sparse_doubles(m[k], mc, nc, sp->room_a, sp->room_at) : mat_doubles(m[k], n[k], mc, nc)));
   }
   SmemPlan p{base * 8 + 16, 0, 0};
   if (vec * 8 <= budget) { p.bytes = vec * 8 + 16; p.cache_vec = 1; }
@@ -792,8 +855,9 @@ cudaError_t cluster_config(ClusterFn f, int C, size_t smem, cudaLaunchConfig_t& 
 }  // namespace
 
 int plan_dense_grid(int m, int n, int sms, DenseGroupPlan& plan) {
-  const SmemPlan s = plan_smem(&m, &n, 1, sms, true, kSmemMax - 16);
-  plan = DenseGroupPlan{sms, 1, s.cache_vec, s.cache_mat, s.bytes, 0};
+  if (sms < kGridCtas) return 0;
+  const SmemPlan s = plan_smem(&m, &n, 1, kGridCtas, true, kSmemMax - 16);
+  plan = DenseGroupPlan{kGridCtas, 1, s.cache_vec, s.cache_mat, s.bytes, 0};
   return s.bytes <= kSmemMax;
 }
 
@@ -807,28 +871,30 @@ int plan_dense_cluster(const int* m, const int* n, int count, int C, size_t budg
 }
 
 namespace {
-// most entries a CTA's share of the rows holds: ptr (len + 1) in shares of ceil(len / C) rows
-int share_room(const int32_t* ptr, int len, int C) {
-  const int per = (len + C - 1) / C;
+// most entries a CTA's rows hold: ptr (len + 1), C CTAs
+int share_room(const int32_t* ptr, int len, int C, int parts, bool grid) {
   int most = 0;
-  for (int r = 0; r < len; r += per) most = std::max(most, ptr[std::min(len, r + per)] - ptr[r]);
+  for (int r = 0; r < C; ++r)
+    most = std::max(most, ptr[own_start(r + 1, C, parts, grid, len)] - ptr[own_start(r, C, parts, grid, len)]);
   return most;
 }
 }  // namespace
 
-int plan_sparse_group(int m, int n, const int32_t* rp, const int32_t* cp, int sms, GroupSparse& sp, DenseGroupPlan& plan) {
+int dense_parts(int m, int n) { return cluster_ctas(dense_work(m, n), kClusterWork); }
+
+int plan_sparse_group(int m, int n, const int32_t* rp, const int32_t* cp, int sms, GroupSparse& sp, DenseGroupPlan& plan,
+                      int& parts) {
   plan = DenseGroupPlan{};
   plan.sparse = 1;
   if (m > kDirectMaxRows) return 0;
-  const int64_t w = 3 * (int64_t)rp[m] + (int64_t)m * m + 80 * (int64_t)(m + n);
-  plan.grid_mode = w > 800000;   // as for a dense LP
-  int C = 1;
-  while (C < 16 && w / C > 5000) C *= 2;
-  if (plan.grid_mode) C = sms;
-  for (;; C *= 2) {
-    sp.room_a = share_room(rp, m, C);
-    sp.room_at = share_room(cp, n, C);
-    const SmemPlan s = plan_smem(&m, &n, 1, C, plan.grid_mode != 0, kSmemMax - 16, &sp);
+  const double w = 3.0 * rp[m] + (double)m * m + 80.0 * (m + n);
+  parts = cluster_ctas(w, kClusterWork);
+  const bool grid = w > kGridWork && sms >= kGridCtas;   // as for a dense LP
+  plan.grid_mode = grid;
+  for (int C = grid ? kGridCtas : parts;; C *= 2) {
+    sp.room_a = share_room(rp, m, C, parts, grid);
+    sp.room_at = share_room(cp, n, C, parts, grid);
+    const SmemPlan s = plan_smem(&m, &n, 1, C, grid, kSmemMax - 16, &sp, parts);
     plan.ctas = C;
     plan.smem = s.bytes;
     plan.cache_vec = s.cache_vec;
@@ -838,9 +904,9 @@ int plan_sparse_group(int m, int n, const int32_t* rp, const int32_t* cp, int sm
   }
 }
 
-size_t dense_group_scratch(int m, int n, int sms) {
+size_t dense_group_scratch(int m, int n) {
   const size_t mp = (m + 1) / 2 * 2, np = (n + 1) / 2 * 2;
-  return 3 * mp + 2 * np + (size_t)kSums * sms + 4;
+  return 3 * mp + 2 * np + (size_t)kSums * kGridCtas + 4;
 }
 
 cudaError_t launch_dense_group(DenseInst* inst, int count, const DenseParams& prm, int* queue, const int* order,
@@ -852,7 +918,7 @@ cudaError_t launch_dense_group(DenseInst* inst, int count, const DenseParams& pr
     Q.bar = reinterpret_cast<unsigned long long*>(scratch + scratch_len - 2);
     Q.err = reinterpret_cast<int*>(scratch + scratch_len - 1);
     Q.gpart = scratch;
-    Q.gvec = scratch + (size_t)kSums * plan.ctas + (kSums * (size_t)plan.ctas & 1);
+    Q.gvec = scratch + (size_t)kSums * kGridCtas;   // even
     const ClusterFn f = grid_fn(plan.sparse != 0);
     cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
     if (e != cudaSuccess) return e;
