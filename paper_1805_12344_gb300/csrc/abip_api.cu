@@ -1282,6 +1282,7 @@ int abip_setup(const abip_matrix* A, const double* b, const double* c, const abi
       std::vector<DenseInst> hd;
       std::vector<int> ord;
       h->group = !prm.bb_beta && plan_buckets(h, {{m, n}}, true, h->mixed != 0, abip::dense_max_ctas(h->device), ord);
+      if (rc == ABIP_OK && h->mixed && !h->group) rc = fail(h, ABIP_E_UNSUPPORTED, "the LP does not fit the shared memory of a cluster");
       if (rc == ABIP_OK) {
         rc = dense_alloc(h, hi, &h->arena, &h->dinst, &h->queue, hd, h->mixed != 0, prm.bb_beta != 0, h->group);
         if (rc == ABIP_E_OOM && h->group && !h->mixed) {   // without the group's copies of A^T and the factor's inverse
@@ -1463,7 +1464,8 @@ int abip_solve_batch(int32_t count, const abip_matrix* A, const double* const* b
       }
     }
   }
-  if (mixed && !tmp.group) return fail(nullptr, ABIP_E_UNSUPPORTED, "an instance does not fit the shared memory of a cluster");
+  if (mixed && !tmp.group && sms > 0)   // (without a device the allocation says so)
+    return fail(nullptr, ABIP_E_UNSUPPORTED, "an instance does not fit the shared memory of a cluster");
   tmp.prm = prm;
   int rc = dense_alloc(&tmp, hi, &arena, &dinst, &queue, hd, mixed, prm.bb_beta != 0, tmp.group);
   if (rc == ABIP_E_OOM && tmp.group && !mixed) {   // without the group's copies of A^T and the factor's inverse

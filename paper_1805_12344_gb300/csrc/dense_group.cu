@@ -861,13 +861,33 @@ int plan_dense_grid(int m, int n, int sms, DenseGroupPlan& plan) {
   return s.bytes <= kSmemMax;
 }
 
-int plan_dense_cluster(const int* m, const int* n, int count, int C, size_t budget, DenseGroupPlan& plan) {
-  for (;; C *= 2) {
-    const SmemPlan s = plan_smem(m, n, count, C, false, budget);
-    plan = DenseGroupPlan{C, 0, s.cache_vec, s.cache_mat, s.bytes, 0};
-    if (s.bytes <= kSmemMax) return 1;
+namespace {
+// A cluster plan from C CTAs: more, up to 8, where `at` (the plan of a size) does not fit the shared
+// memory, then fewer where the device holds no cluster of that size.  16 CTAs need an SM each of one
+// GPC, which a partitioned device may not have.
+template <typename F>
+int settle_cluster(int C, ClusterFn f, DenseGroupPlan& plan, F at) {
+  for (; plan = at(C), plan.smem > kSmemMax; C *= 2)
     if (C >= 8) return 0;
+  for (; C >= 1; C /= 2) {
+    plan = at(C);
+    if (plan.smem > kSmemMax) return 0;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    int n = 0;
+    if (cluster_config(f, C, plan.smem, cfg, attr) == cudaSuccess && cudaOccupancyMaxActiveClusters(&n, f, &cfg) == cudaSuccess && n > 0)
+      return 1;
+    cudaGetLastError();
   }
+  return 0;
+}
+}  // namespace
+
+int plan_dense_cluster(const int* m, const int* n, int count, int C, size_t budget, DenseGroupPlan& plan) {
+  return settle_cluster(C, cluster_fn(count == 1 ? 1 : 0, false), plan, [&](int c) {
+    const SmemPlan s = plan_smem(m, n, count, c, false, budget);
+    return DenseGroupPlan{c, 0, s.cache_vec, s.cache_mat, s.bytes, 0};
+  });
 }
 
 namespace {
@@ -884,24 +904,19 @@ int dense_parts(int m, int n) { return cluster_ctas(dense_work(m, n), kClusterWo
 
 int plan_sparse_group(int m, int n, const int32_t* rp, const int32_t* cp, int sms, GroupSparse& sp, DenseGroupPlan& plan,
                       int& parts) {
-  plan = DenseGroupPlan{};
-  plan.sparse = 1;
   if (m > kDirectMaxRows) return 0;
   const double w = 3.0 * rp[m] + (double)m * m + 80.0 * (m + n);
   parts = cluster_ctas(w, kClusterWork);
   const bool grid = w > kGridWork && sms >= kGridCtas;   // as for a dense LP
-  plan.grid_mode = grid;
-  for (int C = grid ? kGridCtas : parts;; C *= 2) {
+  auto at = [&](int C) {
     sp.room_a = share_room(rp, m, C, parts, grid);
     sp.room_at = share_room(cp, n, C, parts, grid);
     const SmemPlan s = plan_smem(&m, &n, 1, C, grid, kSmemMax - 16, &sp, parts);
-    plan.ctas = C;
-    plan.smem = s.bytes;
-    plan.cache_vec = s.cache_vec;
-    plan.cache_mat = s.cache_mat;
-    if (s.bytes <= kSmemMax) return 1;
-    if (C >= 8) return 0;
-  }
+    return DenseGroupPlan{C, grid, s.cache_vec, s.cache_mat, s.bytes, 1};
+  };
+  if (!grid) return settle_cluster(parts, cluster_fn(1, true), plan, at);
+  plan = at(kGridCtas);
+  return plan.smem <= kSmemMax;
 }
 
 size_t dense_group_scratch(int m, int n) {

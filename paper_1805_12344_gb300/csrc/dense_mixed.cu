@@ -562,23 +562,6 @@ constexpr size_t kSmemMax = 224 * 1024;
 
 }  // namespace
 
-int plan_dense_mixed(const int* m, const int* n, int count, int C, size_t budget, DenseGroupPlan& plan) {
-  plan = DenseGroupPlan{};
-  for (;; C *= 2) {
-    size_t base = 0, at = 0;
-    for (int k = 0; k < count; ++k) {
-      const size_t d = mix_doubles(m[k], n[k], C) * 8, mp = (m[k] + 3) / 4 * 4;
-      base = std::max(base, d);
-      at = std::max(at, d + 16 + (size_t)Own::count(n[k], 256 / C, 0) * mp * 4);
-    }
-    plan.ctas = C;
-    plan.smem = at <= budget ? at : base;
-    plan.cache_mat = at <= budget;
-    if (plan.smem <= kSmemMax) return 1;
-    if (C >= 16) return 0;
-  }
-}
-
 static cudaError_t mixed_config(const DenseGroupPlan& plan, int variant, cudaLaunchConfig_t& cfg, cudaLaunchAttribute* at) {
   const MixFn f = mix_fn(variant);
   cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
@@ -597,6 +580,35 @@ static cudaError_t mixed_config(const DenseGroupPlan& plan, int variant, cudaLau
   cfg.attrs = at;
   cfg.numAttrs = 1;
   return e;
+}
+
+int plan_dense_mixed(const int* m, const int* n, int count, int C, size_t budget, DenseGroupPlan& plan) {
+  auto at = [&](int c) {
+    size_t base = 0, copy = 0;
+    for (int k = 0; k < count; ++k) {
+      const size_t d = mix_doubles(m[k], n[k], c) * 8, mp = (m[k] + 3) / 4 * 4;
+      base = std::max(base, d);
+      copy = std::max(copy, d + 16 + (size_t)Own::count(n[k], 256 / c, 0) * mp * 4);
+    }
+    plan = DenseGroupPlan{};
+    plan.ctas = c;
+    plan.smem = copy <= budget ? copy : base;
+    plan.cache_mat = copy <= budget;
+    return plan.smem <= kSmemMax;
+  };
+  for (; !at(C); C *= 2)
+    if (C >= 16) return 0;
+  // fewer CTAs where the device holds no cluster of that size (16 need an SM each of one GPC)
+  for (; C >= 1 && at(C); C /= 2) {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    int n_active = 0;
+    if (mixed_config(plan, 0, cfg, attr) == cudaSuccess && cudaOccupancyMaxActiveClusters(&n_active, mix_fn(0), &cfg) == cudaSuccess &&
+        n_active > 0)
+      return 1;
+    cudaGetLastError();
+  }
+  return 0;
 }
 
 cudaError_t launch_dense_mixed(DenseInst* inst, int count, const DenseParams& prm, int* queue, const int* order,

@@ -421,24 +421,29 @@ cudaError_t launch_inverse(DenseInst* inst, int count, int mmax, int sms, cudaSt
 cudaError_t launch_cholesky(DenseInst* inst, int count, int mmax, int sms, cudaStream_t st) {
   const int nt = (mmax + 31) / 32, tiles = nt * (nt + 1) / 2;
   // CTAs per factorisation: a power of two up to 16 while the SMs outnumber the CTAs and a
-  // CTA has more than one tile of the first trailing update
+  // CTA has more than one tile of the first trailing update, and a cluster of them fits the device
   int C = 1;
   while (C < 16 && 2 * C * count <= sms && 2 * C <= tiles) C *= 2;
-  if (C > 8) {
-    const cudaError_t e = cudaFuncSetAttribute(chol_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
-  }
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(std::min(count, 4 * sms) * C));
   cfg.blockDim = dim3(kThr);
   cfg.stream = st;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = (unsigned)C;
   at[0].val.clusterDim.y = 1;
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
+  for (;; C /= 2) {
+    at[0].val.clusterDim.x = (unsigned)C;
+    cfg.gridDim = dim3((unsigned)(std::min(count, 4 * sms) * C));
+    if (C == 1) break;
+    cudaError_t e = cudaSuccess;
+    if (C > 8) e = cudaFuncSetAttribute(chol_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    int n = 0;
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, chol_cluster_kernel, &cfg);
+    if (e == cudaSuccess && n > 0) break;
+    cudaGetLastError();
+  }
   return cudaLaunchKernelEx(&cfg, chol_cluster_kernel, inst, count);
 }
 
