@@ -118,7 +118,8 @@ typedef struct {
     int32_t check_every;    /* mixed precision: minimum number of ADMM updates between two exact FP64
                                confirmations of the Sec. 4.1 tests (each screen pass that comes
                                sooner waits); 1 = confirm whenever the screen passes */
-    int32_t grid_ctas;      /* 0: automatic; else the persistent grid size (tests) */
+    int32_t grid_ctas;      /* sparse paths: 0 automatic, else the persistent grid's CTAs (tests); the
+                               direct projection then runs its sweeps there at any size */
     int64_t barrier_limit_ns; /* sparse paths, and one large dense LP in FP64 (solved by the whole
                                  grid): wall-clock limit of one grid-barrier wait in the
                                  persistent kernel, and of one wait of the direct projection's

@@ -1257,7 +1257,7 @@ int abip_setup(const abip_matrix* A, const double* b, const double* c, const abi
       } else {
         const std::vector<double> lx0 = abip::ldl_host::initial_values(hA, sym);
         rc = setup_grid_path(h, h->gd64, hA, hb, hc, !f32, abip::grid_solver_max_ctas(!f32, h->device), &sym, &lx0);
-        if (rc == ABIP_OK) setup_direct(h, hA);
+        if (rc == ABIP_OK && prm.grid_ctas <= 0) setup_direct(h, hA);   // a grid size asks for the persistent grid
       }
     } else if (rc == ABIP_OK) {
       if (h->mixed)   // FP32 values: exact for float input, rounded for double input (FP64 refreshes see them)
