@@ -35,6 +35,7 @@
 
 #include "abip_device.cuh"
 #include "abip_internal.h"
+#include "barrier_refined.h"
 #include "dense_device.cuh"
 
 namespace cg = cooperative_groups;
@@ -211,34 +212,23 @@ __device__ __forceinline__ double two_products(double a, double b, double c, dou
   return __fma_rn(a, b, __dmul_rn(c, d));
 }
 
-// barrier_step with the square root and the quotient refined from FP32 estimates: one coupled
-// step and a residual step each leave about 1e-16 relative, in half the dependent operations of
-// the library's (an update's critical path holds this chain).  Outside the FP32 range of the
-// discriminant, the closed form.
+// barrier_step_refined from the hardware's estimates (2^-22.9 and one unit in the last place off at
+// most): half the dependent operations of the library's root and quotient, and an update's critical
+// path holds this chain.
 __device__ __forceinline__ void barrier_step_fast(double omega, double c, double& x, double& s) {
-  const double disc = __fma_rn(omega, omega, 4.0 * c);
-  if (!(disc > 1e-30 && disc < 1e30)) {
-    const double L = 0.5 * (fabs(omega) + sqrt(disc)), small = c / L;
-    x = omega >= 0.0 ? L : small;
-    s = omega >= 0.0 ? small : L;
-    return;
-  }
-  float r;
-  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"((float)disc));
-  const double rd = (double)r;
-  double g = disc * rd, h = 0.5 * rd;
-  const double e = 0.5 - g * h;
-  g += g * e;
-  h += h * e;
-  const double D = g + (disc - g * g) * h;
-  const double L = 0.5 * (fabs(omega) + D);   // the larger root; the smaller is c / L
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"((float)L));
-  double q = (double)r;
-  q += q * (1.0 - L * q);
-  const double t = c * q;
-  const double small = t + q * (c - L * t);
-  x = omega >= 0.0 ? L : small;
-  s = omega >= 0.0 ? small : L;
+  barrier_step_refined(
+      omega, c,
+      [](float v) {
+        float r;
+        asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+        return r;
+      },
+      [](float v) {
+        float r;
+        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+        return r;
+      },
+      x, s);
 }
 
 struct GroupArgs {
