@@ -894,7 +894,9 @@ int solve_direct(abip_handle* h, cudaStream_t st) {
 
 // ---------------------------------------------------------------------------
 // Batch autotuner: the occupancy variant of the dense solve kernel, chosen by timing a
-// short capped run of the batch itself, cached per (GPU, precision, batch shape)
+// short capped run of the batch itself, cached per (GPU, precision, kernel, batch shape): the
+// variants of the cluster kernels are not those of the one-CTA kernel, so the key names the
+// launches (the clusters' size and LPs each)
 // ---------------------------------------------------------------------------
 struct TuneCache {
   std::mutex mu;
@@ -907,14 +909,15 @@ TuneCache& tune_cache() {
   return c;
 }
 
-std::string tune_key(int device, bool mixed, const std::vector<DenseHostInst>& hi) {
+std::string tune_key(int device, bool mixed, const std::vector<DenseHostInst>& hi, bool group,
+                     const std::vector<abip::DenseBucket>& buckets) {
   cudaDeviceProp prop;
   if (cudaGetDeviceProperties(&prop, device) != cudaSuccess) {
     cudaGetLastError();
     std::strcpy(prop.name, "unknown");
   }
   double mn = 0.0;
-  int mmax = 0, nmax = 0;
+  int mmax = 0;
   for (const DenseHostInst& x : hi) {
     mn += (double)x.m * x.n;
     mmax = std::max(mmax, x.m);
@@ -923,6 +926,10 @@ std::string tune_key(int device, bool mixed, const std::vector<DenseHostInst>& h
   std::snprintf(buf, sizeof buf, "%s|%s|count=%d|mmax=%d|mn=%.1e", prop.name, mixed ? "mixed" : "f64",
                 (int)hi.size(), mmax, mn);
   std::string k(buf);
+  k += group ? "|clusters" : "|cta";
+  if (group)
+    for (const abip::DenseBucket& b : buckets)
+      k += (&b == &buckets[0] ? "=" : ",") + std::to_string(b.plan.ctas) + (b.plan.grid_mode ? "g" : "x") + std::to_string(b.count);
   for (char& ch : k)
     if (ch == '"' || ch == ':' || ch == '\\') ch = '_';
   return k;
@@ -1485,16 +1492,18 @@ int abip_solve_batch(int32_t count, const abip_matrix* A, const double* const* b
   const DenseParams dp = dense_params(prm);
   rc = dense_run_setup(&tmp, dinst, queue, count, std::min(count, sms * 4), smem_setup, mmax,
                        tmp.group && !mixed ? nmax : 0, mixed || tmp.group, st);
-  auto ctas_per_sm = [&](int v) {
+  auto ctas_per_sm = [&](int v) {   // of the launch that fits the fewest
     if (!tmp.group) return abip::dense_solve_ctas_per_sm(smem_solve, v);
-    const abip::DenseGroupPlan& p = tmp.buckets[0].plan;
-    return mixed ? abip::dense_mixed_ctas_per_sm(p, v) : abip::dense_group_ctas_per_sm(p, v);
+    int per = INT32_MAX;
+    for (const abip::DenseBucket& b : tmp.buckets)
+      per = std::min(per, mixed ? abip::dense_mixed_ctas_per_sm(b.plan, v) : abip::dense_group_ctas_per_sm(b.plan, v));
+    return per;
   };
   // occupancy variant: 0, or the autotuner's (cached, or timed on this batch)
   int variant = 0, tuned = 0;
   if (!rc && prm.autotune) {
     TuneCache& tc = tune_cache();
-    const std::string key = tune_key(tmp.device, mixed, hi);
+    const std::string key = tune_key(tmp.device, mixed, hi, tmp.group, tmp.buckets);
     {
       std::lock_guard<std::mutex> lock(tc.mu);
       if (!tc.loaded) tune_load(tc);
