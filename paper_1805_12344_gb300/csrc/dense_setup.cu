@@ -406,10 +406,12 @@ __global__ void __launch_bounds__(kThr) transpose_tiles_kernel(const DenseInst* 
   }
 }
 
+constexpr size_t kInverseSmemMax = 200 * 1024;   // beside at most 25 KB of static shared memory
 template <int Q>
 cudaError_t launch_inverse(DenseInst* inst, int count, int mmax, int sms, cudaStream_t st) {
   const size_t smem = (size_t)mmax * Q * sizeof(double);
-  cudaError_t e = cudaFuncSetAttribute(inverse_tiles_kernel<Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // one limit whatever the call needs: it is the process's, and other threads set it too
+  cudaError_t e = cudaFuncSetAttribute(inverse_tiles_kernel<Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kInverseSmemMax);
   if (e != cudaSuccess) return e;
   for (int k0 = 0; k0 < count; k0 += 32768) {   // gridDim.y is limited to 65535
     const int cnt = std::min(32768, count - k0);

@@ -302,6 +302,8 @@ cudaError_t cholesky_blocked(double* G, int m, int* err, cudaStream_t st) {
   return cudaGetLastError();
 }
 
+constexpr size_t kInverseSmemMax = 200 * 1024;
+
 // Column k of G^{-1} = L^{-T} L^{-1} e_k, one column per CTA pass (w in shared memory).
 __global__ void __launch_bounds__(kThr) inverse_kernel(const double* __restrict__ L, int m, double* __restrict__ Ginv) {
   extern __shared__ double w[];
@@ -1207,7 +1209,7 @@ int shared_batch_run(const SharedBatchArgs& a, std::vector<SharedBatchResult>& o
     }
     st = owned;
   }
-  if ((size_t)m * 8 > 200 * 1024) {
+  if ((size_t)m * 8 > kInverseSmemMax) {
     err = "shared batch: m <= 25600";
     if (owned) cudaStreamDestroy(owned);
     return ABIP_E_UNSUPPORTED;
@@ -1345,15 +1347,14 @@ int shared_batch_run(const SharedBatchArgs& a, std::vector<SharedBatchResult>& o
   // (the factorisation and what follows read its lower triangle only)
   ck(gemm<double>(false, A64, n, m, m, n, AT64, m, G, work64, wk64, sms, st, 1.0, nullptr, nullptr, 0, nullptr, true), "Gram");
   ck(cholesky_blocked(G, m, derr, st), "Cholesky");
-  const size_t inv_smem = (size_t)m * 8;
-  ck(cudaFuncSetAttribute(inverse_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)inv_smem), "smem");
   if (m <= 6400) {   // column tiles in shared memory (the same operations per column)
     DenseInst I{};
     I.m = m; I.L = G; I.Ginv = Ginv64;
     ck(cudaMemcpyAsync(dinv, &I, sizeof(I), cudaMemcpyHostToDevice, st), "inverse");
     ck(launch_dense_inverse(dinv, 1, m, sms, st), "inverse");
   } else {
-    inverse_kernel<<<std::min(m, sms * 2), kThr, inv_smem, st>>>(G, m, Ginv64);
+    ck(cudaFuncSetAttribute(inverse_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kInverseSmemMax), "smem");
+    inverse_kernel<<<std::min(m, sms * 2), kThr, (size_t)m * 8, st>>>(G, m, Ginv64);
   }
   // M^{-1} h1, M^{-1} h2 for every instance: z_y = G^{-1}(a - A d), z_x = d + A^T z_y
   setup_rhs_kernel<<<eb, kThr, 0, st>>>(V, W2, nullptr, nullptr, 0);
@@ -1377,8 +1378,7 @@ int shared_batch_run(const SharedBatchArgs& a, std::vector<SharedBatchResult>& o
       for (int N : {B, 2 * B}) {
         const TcKernel kern = tc_kernel_for(tc::tc2_stages(N, terms), terms);
         if (!kern) ck(cudaErrorInvalidValue, "tc stages");
-        else ck(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)tc::tc2_smem_bytes(N, terms)), "tc smem");
+        else ck(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc::kTcSmemMax), "tc smem");
       }
     } else {
       convert_kernel<float><<<cb, kThr, 0, st>>>(A64, A32, (size_t)m * n);

@@ -176,6 +176,7 @@ __host__ __device__ inline size_t tc2_stage_bytes(int N, int TA) {
 // shared-memory stages: as many as fit in the 227 KB a CTA may use (less 2 KB for the
 // 1024-byte alignment of the tiles and the static variables), at most 6
 constexpr size_t kTcSmemCap = 227 * 1024 - 2048;
+constexpr size_t kTcSmemMax = kTcSmemCap + 1024;   // the kernels' limit, whatever N needs
 __host__ __device__ inline int tc2_stages(int N, int TA) {
   const int s = static_cast<int>(kTcSmemCap / tc2_stage_bytes(N, TA));
   return s < 6 ? s : 6;
