@@ -101,8 +101,7 @@ KERNEL_SOURCES = ("paper_1805_12344_gb300/csrc/grid_delta.cu", "paper_1805_12344
                   "paper_1805_12344_gb300/csrc/abip_device.cuh", "paper_1805_12344_gb300/csrc/sell_host.h")
 # DRAM bytes of one solve launch from ncu (dram__bytes_read.sum + dram__bytes_write.sum) at
 # 20 and 60 updates, caches flushed before the launch: 656.1 MB and 1764.2 MB, so
-# 102.1 MB fixed + 27.70 MB per update (profiles/grid_delta_kernel_solve_sparse_m100000.md);
-# valid while the sources above are the ones measured.
+# 102.1 MB fixed + 27.70 MB per update; valid while the sources above are the ones measured.
 TRAFFIC = {"sources_sha256": "c3d55137c3f226b8c13ff8983d783882c82a8304c5220eb08a06d3e14d3779e2",
            "dram_bytes_fixed": 102076288, "dram_bytes_per_update": 27701600.0}
 

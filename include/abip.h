@@ -83,7 +83,9 @@ extern "C" {
                                        K = [I A^T; A -I] (Sec. 4.4): minimum-degree order and
                                        symbolic factor on the host (abip_ldl_analyze), numeric
                                        LDL^T once per setup and two triangular sweeps per update
-                                       on the GPU.  CSR or dense input, precision F64 only */
+                                       on the GPU; up to 1600 rows the inverse of G's Cholesky
+                                       factor takes the sweeps' place in the updates.  CSR or
+                                       dense input, precision F64 only */
 
 /* ---- data ----------------------------------------------------------------- */
 typedef struct {
@@ -206,9 +208,10 @@ ABIP_API int abip_solve(abip_handle* h, double* x, double* y, double* s,
                abip_info* info, void* stream);
 
 /*
- * Solve `count` independent dense LPs in one persistent launch (one CTA per
- * instance at a time, pulled from a device work queue, each with its own
- * convergence state).  A[i] (dense row-major), b[i], c[i]: host pointers
+ * Solve `count` independent dense LPs, each by a cluster of CTAs according to its
+ * size and the batch's (one CTA to 16; a single large LP in FP64 by the whole grid),
+ * pulled from device work queues, one per cluster size, each with its own
+ * convergence state (bb_beta: one CTA per instance).  A[i] (dense row-major), b[i], c[i]: host pointers
  * (on_device = 0) or device pointers (on_device = 1) per instance.  x, y, s:
  * arrays of `count` caller-allocated output pointers (same memory kind as the
  * inputs), entries may be NULL.  infos: `count` entries, may be NULL.
@@ -228,18 +231,20 @@ ABIP_API int abip_solve_batch(int32_t count, const abip_matrix* A, const double*
  * Solve `count` LPs  min c_k^T x  s.t.  A x = b_k,  x >= 0  that share one dense A
  * (e.g. basis pursuit with one dictionary and many measurements).  Algorithm 2 runs
  * for all instances in lockstep with per-instance convergence control; each update's
- * products are GEMMs over the instances (A [X S], A^T Y, G^{-1} Q, A^T Z_y with
- * G = I + A A^T of Sec. 4.4 inverted once from its FP64 Cholesky factor).
+ * products are GEMMs over the instances (A [X S], G^{-1} Q, A^T Z_y with
+ * G = I + A A^T of Sec. 4.4 inverted once from its FP64 Cholesky factor; A^T Y
+ * follows from them by the update's linearity).
  *   A: one dense row-major matrix (host or device, F32 or F64), 1 <= m <= n.
- *   b[k] (m), c[k] (n): host or device.  x, y, s: arrays of `count` caller-allocated
+ *   b[k] (m), c[k] (n): host or device; all are read before the first output is
+ *   written.  x, y, s: arrays of `count` caller-allocated
  *   output pointers (host or device; entries may be NULL), scaled as abip_solve's.
  *   infos: `count` entries or NULL.  p->precision: ABIP_PREC_F64 (FP64 throughout),
  *   ABIP_PREC_MIXED (FP64 state; the products are updated by FP32 GEMMs of the state's
- *   changes and recomputed in FP64 every 200 cycles and before every termination
+ *   changes and recomputed in FP64 every 192 cycles and before every termination
  *   decision) or ABIP_PREC_MIXED_BF16 (as MIXED with the products with A on the tensor
- *   cores: the changes are split into three bfloat16 terms, so the products keep FP32
- *   accuracy; A must be exactly representable in bfloat16, else ABIP_E_INVALID_ARG;
- *   shapes other than m, n multiples of 128 and count a multiple of 16 per chunk of 64
+ *   cores: the changes are split into three bfloat16 terms, and A into one where it is
+ *   exact in bfloat16, else three, so the products keep FP32 accuracy; an A beyond the
+ *   FP32 range is refused with ABIP_E_INVALID_ARG; shapes other than m, n multiples of 128 and count a multiple of 16 per chunk of 64
  *   use the FP32 GEMMs).
  * Instances are processed in chunks of 64.  Needs m <= 25600.  Errors: as
  * abip_solve_batch; ABIP_E_UNSUPPORTED for a CSR A.
@@ -257,8 +262,9 @@ ABIP_API int abip_solve_batch_shared(int32_t count, const abip_matrix* A, const 
  * xi = -n-1, x o s = tau kappa = mu / beta).  The final ADMM iterate is first
  * polished onto that point by damped Newton steps; then J^T lam = dL/dz is solved by
  * eliminating ds and dkappa, which leaves the reduced Jacobian
- * K = Q + diag(0, S X^-1, kappa / tau, 0) of order m + n + 2, factored by LU with
- * partial pivoting in FP64 (one step of iterative refinement), and
+ * K = Q + diag(0, S X^-1, kappa / tau, 0) of order m + n + 2, whose x_j with a dominant
+ * diagonal are eliminated next and the rest factored by LU with partial pivoting, in
+ * FP64 (two steps of iterative refinement against K), and
  * dL/dp = -lam^T dF/dp, counting the dependence of bbar, cbar, zbar on (A, b, c)
  * (Eq. bar-b-c-z-re).  The handle's state is left unchanged.
  *   dl_dx: n entries, dL/dx* (host or device).
@@ -315,7 +321,8 @@ ABIP_API int64_t abip_state_size(const abip_handle* h);
  * footprint): every scratch byte comes from one fixed array of 167,680 bytes that
  * the library holds on each device that loads it, until the process exits.  The
  * paper has no counterpart; this is the dense Cholesky path of abip_setup +
- * abip_solve for one instance, same kernels and same arithmetic.
+ * abip_solve for one instance by the one-CTA kernels (triangular sweeps for L^{-1};
+ * the result agrees with abip_solve's to rounding, not bit for bit).
  *   m, n, A (m x ld row-major FP64), b (m), c (n): inputs, device pointers.
  *   x (n), y (m), s (n): outputs, device pointers (same meaning as abip_solve).
  *   p: NULL for defaults; FP64 only.  info: host, may be NULL.  stream: cudaStream_t.

@@ -337,7 +337,7 @@ def abip_backward_batch(As: Sequence, bs: Sequence, cs: Sequence, xs: Sequence, 
 
 def abip_solve_batch(As: Sequence, bs: Sequence, cs: Sequence, params: Optional[abip_params] = None,
                      want_solution: bool = True, stream=None, device_out: bool = False):
-    """Solve dense LPs (numpy arrays or torch tensors) in one persistent launch.
+    """Solve dense LPs (numpy arrays or torch tensors) at once, each by a cluster of CTAs.
     Returns (infos, xs, ys, ss); the solutions are numpy arrays, or CUDA float64 tensors
     when `device_out`."""
     count = len(As)

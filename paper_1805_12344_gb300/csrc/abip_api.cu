@@ -643,7 +643,8 @@ DenseParams dense_params(const abip_params& p) {
 // per SM (FP64, 64 LPs of m 16 .. 256, 200 updates: 14.4 ms; 1 per SM 17.2, 3 15.4; the same
 // size for all 48 / 26 / 23 / 12.6 ms with 1 / 2 / 4 / 8; 128 LPs 24.8, 61 / 49 / 25 / 26).  The time
 // of a batch is that of its slowest instance, so the large ones get the CTAs; instances of one
-// cluster size form a bucket, and the buckets' launches run side by side.  A batch of more instances than that is one bucket of single CTAs.
+// cluster size form a bucket, and the buckets' launches run side by side.  A batch of more instances
+// than that is one bucket of single CTAs.
 bool plan_buckets(abip_handle* h, const std::vector<std::pair<int, int>>& sizes, bool largest_first, bool mixed, int sms,
                   std::vector<int>& ord) {
   const int count = (int)sizes.size();

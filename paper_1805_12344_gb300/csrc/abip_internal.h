@@ -314,7 +314,7 @@ int plan_dense_grid(int m, int n, int sms, DenseGroupPlan& plan);
 int plan_dense_cluster(const int* m, const int* n, int count, int C, size_t budget, DenseGroupPlan& plan);
 // Rows up to which the sparse direct projection forms L^{-1}: m^2 multiply-adds over the SMs per
 // update against two sweeps along the elimination tree at about 2.8 us per dependent link
-// (grid flow, us per update, sweeps / inverse: m = 255 309 / 12, 1023 631 / 23, 1599 903 / 29),
+// (grid flow, us per update, sweeps / inverse: m = 255 309 / 11, 1023 631 / 23, 1599 903 / 29),
 // and a setup that grows by m^3 / 3 multiply-adds (1599: 24 ms more).
 constexpr int kDirectMaxRows = 1600;
 // the plan for one sparse LP (host rp, cp); 0 where the sweeps serve it

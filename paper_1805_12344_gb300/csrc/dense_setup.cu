@@ -9,8 +9,7 @@
 // bits whatever the split: the mixed path rounds its changes to FP32, and a last-bit
 // difference in the factor would move those roundings.
 // Measured, setup of one 512 x 1154 L1-SVM, one CTA -> this split: FP64 91 -> 7 ms, mixed
-// precision (with the inverse) 585 -> 9 ms; a mixed batch of 192 LPs (m 16 .. 256) of 400
-// updates 232 -> 118 ms in all.
+// precision (with the inverse) 585 -> 9 ms.
 #include <algorithm>
 
 #include <cooperative_groups.h>

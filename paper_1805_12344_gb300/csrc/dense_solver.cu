@@ -891,8 +891,9 @@ __device__ void backward_one(BackwardInst& P, double* sm, double* red, int* redi
   //   core = K_cc + W D W^T,  W = [A_E; -c_E^T; cbar_E^T],  D = diag(1 / sigma_E).
   // On an L1-SVM near the optimum that leaves about 2 m of the m + n + 2 rows (n = 2.4 m: the
   // LU falls to a fifth of its operations).  Measured: the gradients of 32 L1-SVMs 96 x 226 60 ->
-  // 25 ms, one 512 x 1154 4.7 -> 1.8 s; errors as before (geometric mean of dc over 24 LPs of 96 x
-  // 226 against 64-bit dense solves 3.2e-14 -> 2.1e-14).
+  // 25 ms, one 512 x 1154 4.7 -> 1.8 s.  Errors stay at the rounding floor, where they go either way
+  // (against 64-bit dense solves: geometric mean of dc over 24 LPs of 96 x 226 3.2e-14 -> 2.1e-14; all
+  // gradients of 32 others 1.0e-13 -> 2.0e-13).
   int* where = ipiv + N;         // n: the core's row of x_j, or -1
   int* keep = where + n;         // n: the kept columns, in order
   double* colmax = reinterpret_cast<double*>(keep + n + (n & 1) + ((N + n) & 1));   // n: largest entry beside the diagonal

@@ -1,7 +1,7 @@
 // Algorithm 2 for a batch of LPs that share one dense A (different b_k, c_k).
 //
 // With B instances side by side every product of the ADMM update becomes a GEMM
-// with B (or 2B) right-hand columns: A [X S], A^T Y, G^{-1} Q and A^T Z_y.  The
+// with B (or 2B) right-hand columns: A [X S], G^{-1} Q and A^T Z_y.  The
 // projection's G^{-1} = (I + A A^T)^{-1} (Sec. 4.4) is formed explicitly once, from
 // the FP64 Cholesky factor, so that the per-update solve is one parallel GEMM
 // instead of two sequential triangular sweeps.  Every vector is stored row-major as
@@ -9,14 +9,14 @@
 // and per-instance column reductions all read contiguous memory.
 //
 // One update cycle (fixed launch sequence, per-instance masks):
-//   products  AXS = A [X S], ATY = A^T Y            (GEMM, split-K, deterministic)
+//   products  AXS = A [X S]                         (GEMM, split-K, deterministic)
 //   sums      the nine sums of the Sec. 4.1 tests and Eq. inner-stop, Q = Y - AX - AS
 //   control   per instance: tests after an update, inner stop ||Qu-v||^2 <= mu,
 //             mu decrease with warm start, or another update
 //   [mixed]   FP64 confirmation of FP32 screens that pass
 //   step      ZY = G^{-1} Q, ZX = X + S + A^T ZY    (GEMM)
 //             H^T z, t = K^{-1}(w_tau,theta + H^T z), relaxation, barrier prox,
-//             dual update (Eqs. Simple-Update:*, Sec. 4.2)
+//             dual update (Eqs. Simple-Update:*, Sec. 4.2), ATY = A^T Y by the update's linearity
 #include "abip_internal.h"
 #include "abip_device.cuh"
 #include "dense_device.cuh"
@@ -41,7 +41,7 @@ constexpr int kSumRowGroups = kThr / kMaxBatch;
 // op(A) = A (row-major, lda) or A^T.  W row-major (ldw).  Cpart: gridDim.z x M x N.
 // 256 threads as 16 x 16, each TM x TN outputs at rows tr + 16u, columns tc + 16v.  Every output
 // is one chain over its chunk in increasing order, whatever the tile, so the tile is free to
-// follow the shape (gemm_tile) without moving a bit; the chunks follow GemmCfg alone.
+// follow the shape (launch_gemm) without moving a bit; the chunks follow GemmCfg alone.
 // ---------------------------------------------------------------------------
 template <typename T> struct GemmCfg;
 template <> struct GemmCfg<float> { static constexpr int TM = 8, TN = 4, BK = 16; };
