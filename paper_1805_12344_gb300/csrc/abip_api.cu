@@ -1648,11 +1648,16 @@ int abip_solve_batch_shared(int32_t count, const abip_matrix* A, const double* c
   sp.refresh = 192;   // a multiple of the 16-cycle groups of the shared-A solve loop
   for (int k0 = 0; k0 < count; k0 += 64) {
     const int cnt = std::min(64, count - k0);
-    abip::SharedBatchArgs args{m, n, cnt, Ad ? nullptr : Ah.data(), Ad, vec.b + (size_t)k0 * m, vec.c + (size_t)k0 * n, vec.on_host,
-                               sp, static_cast<cudaStream_t>(stream), k0, x ? x + k0 : nullptr, y ? y + k0 : nullptr, s ? s + k0 : nullptr};
     std::vector<abip::SharedBatchResult> res;
     std::string err;
-    rc = abip::shared_batch_run(args, res, err);
+    auto run = [&] {
+      const abip::SharedBatchArgs args{m, n, cnt, Ad ? nullptr : Ah.data(), Ad, vec.b + (size_t)k0 * m, vec.c + (size_t)k0 * n,
+                                       vec.on_host, sp, static_cast<cudaStream_t>(stream), k0, x ? x + k0 : nullptr,
+                                       y ? y + k0 : nullptr, s ? s + k0 : nullptr};
+      return abip::shared_batch_run(args, res, err);
+    };
+    rc = run();
+    if (rc == ABIP_E_OOM && vec.to_host(count, m, n)) rc = run();   // nothing of the chunk has run
     if (rc) return fail(nullptr, rc, err);
     const double el = now_s() - t0;
     for (int k = 0; k < cnt; ++k) {

@@ -422,6 +422,8 @@ struct SharedVectors {
   ~SharedVectors();
   // b[k] (m) and c[k] (n), each host or device; bad: the first instance with a value that is not finite, or -1
   cudaError_t read(int count, int m, int n, const double* const* b, const double* const* c, cudaStream_t st, int& bad);
+  // from the device to the host, for a solve that needs their room; false if that fails
+  bool to_host(int count, int m, int n);
 
  private:
   cudaError_t read_host(int count, int m, int n, const double* const* b, const double* const* c, cudaStream_t st, int& bad);

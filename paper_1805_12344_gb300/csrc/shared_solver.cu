@@ -1155,6 +1155,26 @@ cudaError_t SharedVectors::read(int count, int m, int n, const double* const* b,
   return e != cudaSuccess ? e : es;
 }
 
+bool SharedVectors::to_host(int count, int m, int n) {
+  if (on_host) return false;
+  const size_t nb = (size_t)count * m, len = nb + (size_t)count * n;
+  try {
+    host.resize(len);
+  } catch (const std::exception&) {
+    return false;
+  }
+  if (cudaMemcpy(host.data(), dev, len * 8, cudaMemcpyDeviceToHost) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  cudaFree(dev);
+  dev = nullptr;
+  on_host = true;
+  b = host.data();
+  c = host.data() + nb;
+  return true;
+}
+
 // The same in host memory; of host vectors without a call to the device.
 cudaError_t SharedVectors::read_host(int count, int m, int n, const double* const* b, const double* const* c, cudaStream_t st,
                                      int& bad) {
