@@ -1,5 +1,5 @@
-// Dense ABIP in FP64 with a group of CTAs per LP: a thread-block cluster (2 .. 16 CTAs) per
-// instance of a batch, or the whole cooperative grid for one large LP.
+// Dense ABIP in FP64 with a group of CTAs per LP: a thread-block cluster (1 .. 16 CTAs) per
+// instance of a batch, or a cooperative grid for one large LP.
 //
 // What bounds it: the FP64 pipe, 2 FMA per clock and SM on this part, so an LP on one SM pays
 // its 3 m n + m^2 multiply-adds per update at 1/152 of the chip; and, for a small LP, the chain
